@@ -185,6 +185,75 @@ def run(state):
             for w, prepared, X, table, ids in items]
 
 
+def _rtn64(W, bits, group):
+    """Codes, zero-points and scales by Eq. 1: integer decisions, so taken in binary32, returned as
+    binary64 tensors [N, G, g], [N, G, 1], [N, G, 1]."""
+    N, K = W.shape
+    g = K if group in (0, K) else group
+    Wg = W.view(N, K // g, g)
+    lo, hi = Wg.amin(2, keepdim=True), Wg.amax(2, keepdim=True)
+    top = float(2 ** bits - 1)
+    s = (hi - lo) / top
+    s = torch.where(hi == lo, torch.ones_like(s), s)
+    z = torch.clamp(torch.round(-lo / s), 0.0, top)
+    q = torch.clamp(torch.round(Wg / s) + z, 0.0, top)
+    return q.double(), z.double(), s.double()
+
+
+def _adamw64(p, grad):
+    """First AdamW step from zero moments, no decay: new value, m, v."""
+    m, v = (1.0 - 0.9) * grad, (1.0 - 0.999) * grad * grad
+    return p - LR * (m / (1.0 - 0.9)) / (torch.sqrt(v / (1.0 - 0.999)) + 1e-8), m, v
+
+
+def exact(case, seed):
+    """What run() returns after prepare(case, seed), in binary64; the draws follow prepare()'s order."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    kind, T, bits, group = case["kind"], case["tokens"], case["bits"], case["group"]
+    out, acts = [], {}
+    for N, K, shared in _linears(case):
+        W = _weight(gen, N, K)
+        if kind == "quantize":
+            q, z, s = _rtn64(W, bits, group)
+            out.append((None, None, s.view(N, -1)))       # packed codes have no value in binary64
+            continue
+        if shared not in acts:
+            acts[shared] = _bf16(gen, T, K)
+        X = acts[shared].double()
+        q, z, s = _rtn64(W, bits, group)
+        del W
+        if kind in ("train", "train_zp"):
+            if kind == "train_zp":
+                z = (z.float() + 0.1 * torch.randn((N, z.shape[1]), generator=gen, device="cuda").view(z.shape)).double()
+            dY = _bf16(gen, T, N, 1e-2).double()
+            q -= z
+            W64 = (q * s).view(N, K)
+            Y, dX = X @ W64.T, dY @ W64
+            del W64
+            dW = (dY.T @ X).view(q.shape)
+            dS = (q * dW).sum(2)
+            s2, m, v = _adamw64(s.view(N, -1), dS)
+            if kind == "train":
+                out.append((Y, dX, dS, s2, m, v))
+            else:
+                dZ = -s.view(N, -1) * dW.sum(2)
+                out.append((Y, dX, dS, dZ, s2, _adamw64(z.view(N, -1), dZ)[0]))
+            continue
+        q -= z
+        if kind != "multitask":
+            out.append(X @ (q * s).view(N, K).T)
+            continue
+        s32 = s.float().view(N, -1)
+        table = s32 * (1.0 + 0.05 * torch.randn((TASKS,) + tuple(s32.shape), generator=gen, device="cuda"))
+        ids = torch.randint(0, TASKS, (T,), generator=gen, device="cuda", dtype=torch.int32)
+        Y = torch.empty((T, N), dtype=torch.float64, device="cuda")
+        for task in ids.unique().tolist():
+            Y[ids == task] = X[ids == task] @ (q * table[task].double().view(s.shape)).view(N, K).T
+        out.append(Y)
+    return out
+
+
 def work(case):
     kind, T, bits, group = case["kind"], case["tokens"], case["bits"], case["group"]
     byts = flops = 0
@@ -202,7 +271,9 @@ def work(case):
             # in: X, dY, Q, z, s, m, v; out: Y, dX, dS, s, m, v (twice the optimizer with zero-points)
             trained = 1 if kind == "train" else 2
             byts += x + 2 * T * N + Q + zs + 2 * T * N + 2 * T * K + trained * 24 * N * G
-            flops += 6 * T * N * K
+            # one scale per channel: its gradient is a dot product with the forward's sums
+            # (sum_t dY * Y / s), not a third contraction, when one call has both in hand
+            flops += (4 if kind == "train" and G == 1 else 6) * T * N * K
         else:
             tasks = min(TASKS, T) if kind == "multitask" else 1
             byts += x + Q + N * G * (1 + 4 * tasks) + 2 * T * N
