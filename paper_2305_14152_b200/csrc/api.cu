@@ -432,8 +432,8 @@ int drain_and_fail(HostPipe* hp, cudaStream_t st, int rc) {
 // way to the device (auxiliary stream `in`) while chunk c runs forward and dX on the
 // caller's stream and chunk c-1 returns Y and dX (auxiliary stream `out`); PCIe carries both
 // directions at once.  dS sums over all tokens, so it runs once after the last chunk, then
-// AdamW.  Forward and dX treat tokens independently, so chunking does not change a bit of
-// their results.  With several linears the copies in of the next linear run while the
+// AdamW.  Forward and dX treat tokens independently; chunking them changes at most the order in
+// which a contraction is summed.  With several linears the copies in of the next linear run while the
 // kernels of the current one are still busy.
 
 // Host-side checks of one linear of a host-buffer step; nothing is enqueued.

@@ -162,6 +162,10 @@ int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const v
                    void* dX, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
               cudaStream_t st);
+// forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels
+bool split_is_faster(const peqa_qweight_t* w, int T, bool trans);
+int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
+                 bool trans, cudaStream_t st);
 // adam != nullptr: the AdamW step on (w->scales, m, v) is applied where dS is produced
 struct DsAdam {
   AdamWConsts c;

@@ -879,12 +879,14 @@ int ds_piece(int g) { return gcd_int(g, 128); }
 
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
                cudaStream_t st) {
+  if (fwd_pair_supported(w) && split_is_faster(w, T, false)) return launch_split(w, zeros_f, g, X, T, Y, false, st);
   if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, st);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
               cudaStream_t st) {
+  if (dx_pair_supported(w) && split_is_faster(w, T, true)) return launch_split(w, zeros_f, g, dY, T, dX, true, st);
   if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }

@@ -1,0 +1,610 @@
+// Forward and dX of the PEQA layer for few tokens:
+//
+//   TRANS = false   Y[t,i]  = sum_j X[t,j]  * W_hat[i,j]     (Eq. 2)
+//   TRANS = true    dX[t,j] = sum_i dY[t,i] * W_hat[i,j]
+//
+// With a few hundred tokens the CTA-pair kernels (512 tokens x 256 outputs per tile) keep a
+// handful of SMs busy and multiply mostly padding.  What bounds such a call is rebuilding the
+// weights, so this kernel spreads exactly that over the whole chip: a tile is 128 outputs x up to
+// 256 tokens (the token side is the MMA "N" and is cut to a multiple of 16, so padding costs
+// nothing), and the contraction of a tile is cut across the CTAs of a thread-block cluster.
+//
+// A cluster of `csize` CTAs owns `q` <= csize tiles.  Their q * k_blocks stages, tile-major, are
+// cut into csize equal contiguous ranges, one per CTA; a range is never longer than a tile, so a
+// CTA works on at most two tiles and holds their partial sums in two tensor-memory accumulators.
+// When its stages are done a CTA copies its partial sums to its own shared memory (over the stage
+// buffers), the cluster synchronises, and every CTA adds up one slice of the rows of each tile,
+// reading the contributors' shared memory in rank order: no workspace, no atomics, and the result
+// does not depend on timing.
+//
+// Warps: 0 activation TMA, 1 MMA issuer, 2 tensor memory, 3 code TMA, 4-19 dequant.  The weights
+// are the MMA "A" operand (M = 128), rebuilt by the dequant warps in shared memory exactly as in
+// the single-CTA kernel of gemm_sm100.cu (K-major for the forward, MN-major for dX).  Four groups
+// of four warps take the half stages round-robin; scales and zero-points are fetched one turn ahead.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include "common.cuh"
+#include "dequant.cuh"
+#include "sm100_ptx.cuh"
+#include "tensor_map.cuh"
+
+namespace peqa {
+
+namespace {
+
+using namespace ptx;
+
+constexpr int SM_ROWS = 128;                  // outputs per tile (MMA M, TMEM lanes)
+constexpr int SM_BK = 128;                    // contraction elements per stage: two halves of 64
+constexpr int SM_HALF = 64;                   // (the reach of the 128-byte swizzle)
+constexpr int SM_MAX_NT = 256;                // tokens per tile
+constexpr int SM_A_BYTES = SM_ROWS * SM_HALF * 2;   // weights of one half
+constexpr int SM_PK_BYTES = 8192;             // packed codes of one stage
+constexpr int SM_PK_SLOTS = 4;
+constexpr int SM_MAX_STAGES = 4;
+constexpr int kSplitThreads = 640;
+constexpr int kSplitWorkers = 512;            // threads of the dequant warps
+constexpr int SM_DUMP_TOK = 128;              // tokens reduced per pass
+constexpr int SM_SMEM_LIMIT = 227 * 1024;
+constexpr int SM_SMEM_FIXED = SM_PK_SLOTS * SM_PK_BYTES + 1024 /*align*/ + 512 /*barriers*/;
+
+struct SplitBarriers {
+  uint64_t full[SM_MAX_STAGES];       // weight tile written and activation bytes landed
+  uint64_t empty[SM_MAX_STAGES];      // MMAs that read the stage completed
+  uint64_t full_pk[SM_PK_SLOTS];
+  uint64_t empty_pk[SM_PK_SLOTS];
+  uint64_t acc_full;                  // every MMA of this CTA completed
+  uint32_t tmem_base;
+  int abort_flag;
+  int wait_limit_us;    // must follow abort_flag (read by the bounded waits)
+};
+
+struct SplitParams {
+  const uint8_t* zeros;
+  const float* zeros_f;   // real-valued zero-points (App. K) or nullptr; replaces `zeros`
+  const float* scales;
+  __nv_bfloat16* out;     // [T, R]
+  int N, K, G, g, g_shift, T;
+  int R;                  // output features
+  int r_tiles, tiles;     // row tiles, row tiles * token tiles
+  int k_blocks;
+  int nt;                 // tokens per tile, a multiple of 16
+  int stages;
+  int q, cshift;          // tiles per cluster, log2 of the CTAs per cluster (q <= 1 << cshift)
+  int* status;
+};
+
+__device__ __forceinline__ int split_group_of(const SplitParams& p, int col) {
+  if (p.G == 1) return 0;
+  return p.g_shift >= 0 ? (col >> p.g_shift) : (col / p.g);
+}
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
+
+// Zero-point and scale of one 32-column unit; c: the constant term -delta * s of a real-valued
+// zero-point (ZF).
+struct UnitZS {
+  uint32_t z;
+  float s, c;
+};
+
+template <int BITS, bool ZF>
+__device__ __forceinline__ UnitZS split_load_zs(const SplitParams& p, int i, int col) {
+  UnitZS u;
+  u.z = 0u;
+  u.s = 0.0f;       // outside the matrix: code 0, zero-point 0, scale 0
+  u.c = 0.0f;
+  if (i < p.N && col < p.K) {
+    const size_t gi = (size_t)i * p.G + split_group_of(p, col);
+    u.s = __ldg(p.scales + gi);
+    if (ZF) {
+      float delta;
+      dq::split_zero_point<BITS>(__ldg(p.zeros_f + gi), u.z, delta);
+      u.c = -delta * u.s;
+    } else {
+      u.z = __ldg(p.zeros + gi);
+    }
+  }
+  return u;
+}
+
+template <int BITS, bool TRANS, bool FOLD, bool ZF>
+__global__ void __launch_bounds__(kSplitThreads, 1)
+qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constant__ CUtensorMap tmap_pk,
+              const SplitParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  const int half_bytes = SM_A_BYTES + p.nt * (SM_HALF * 2);     // weights, then activations
+  const int stage_bytes = 2 * half_bytes;
+  uint8_t* sm_pk = base + p.stages * stage_bytes;
+  SplitBarriers* bars = reinterpret_cast<SplitBarriers*>(sm_pk + SM_PK_SLOTS * SM_PK_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort_flag = &bars->abort_flag;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(smem_u32(&bars->full[s]), 8 + 1);     // the warps of two dequant groups, the TMA lane
+      mbar_init(smem_u32(&bars->empty[s]), 1);
+    }
+    for (int s = 0; s < SM_PK_SLOTS; ++s) {
+      mbar_init(smem_u32(&bars->full_pk[s]), 1);
+      mbar_init(smem_u32(&bars->empty_pk[s]), 8);
+    }
+    mbar_init(smem_u32(&bars->acc_full), 1);
+    bars->abort_flag = 0;
+    bars->wait_limit_us = p.status[4];
+    fence_mbar_init();
+    prefetch_tmap(&tmap_act);
+    prefetch_tmap(&tmap_pk);
+  }
+  if (warp == 2) {
+    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  // Set-up is done.  The next kernel of the stream may begin its own (programmatic launch);
+  // everything below touches memory that the preceding kernel may still be writing.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const uint32_t tmem_base = bars->tmem_base;
+
+  // ---- this CTA's stages: [lo, hi) of the cluster's list, tile0 first, then the next tile
+  const int csize = 1 << p.cshift;
+  const int rank = (int)(blockIdx.x & (csize - 1));
+  const int first_tile = (int)(blockIdx.x >> p.cshift) * p.q;
+  const int q = min(p.q, p.tiles - first_tile);
+  const int L = q * p.k_blocks;
+  auto range_lo = [&](int r) { return (r * L) >> p.cshift; };
+  const int lo = range_lo(rank), hi = range_lo(rank + 1);
+  const int n_it = hi - lo;
+  const int j0 = lo / p.k_blocks;                            // first tile of the range
+  const int split_at = (j0 + 1) * p.k_blocks - lo;           // local stages of the first tile
+  const int kb0 = lo - j0 * p.k_blocks;
+  // local stage -> k-block; row and token tile of the segment
+  auto kb_of = [&](int it) { return it < split_at ? kb0 + it : it - split_at; };
+  auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
+  auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles) * p.nt; };
+
+  if (warp == 0) {
+    // ------------------------------------------------ activation TMA (one lane)
+    if (lane == 0) {
+      const int ta = t0_of(0), tb = t0_of(split_at);
+      // self-test knob (peqa_selftest_configure): announce one byte more than will arrive, so
+      // that the stage never fills and the bounded waits have to end the kernel
+      const uint32_t starve = !TRANS && p.status[5] != 0 ? 1u : 0u;
+      int s = 0;
+      uint32_t ph = 1;
+      for (int it = 0; it < n_it; ++it) {
+        if (!mbar_wait(smem_u32(&bars->empty[s]), ph, abort_flag)) break;
+        const uint32_t bar = smem_u32(&bars->full[s]);
+        mbar_arrive_expect_tx(bar, p.nt * (SM_BK * 2) + starve);
+        const uint32_t dst = smem_u32(base + s * stage_bytes + SM_A_BYTES);
+        const int t0 = it < split_at ? ta : tb, col = kb_of(it) * SM_BK;
+        tma_load_2d(dst, &tmap_act, bar, col, t0);
+        tma_load_2d(dst + half_bytes, &tmap_act, bar, col + SM_HALF, t0);
+        if (++s == p.stages) { s = 0; ph ^= 1u; }
+      }
+    }
+  } else if (warp == 3) {
+    // ------------------------------------------ packed-code TMA (one lane)
+    // 128 rows x 128 columns of codes: the tile's rows and the stage's columns (forward), or the
+    // stage's rows and the tile's columns (dX)
+    if (lane == 0) {
+      const int ra = r0_of(0), rb = r0_of(split_at);
+      for (int it = 0; it < n_it; ++it) {
+        const int s = it % SM_PK_SLOTS;
+        if (!mbar_wait(smem_u32(&bars->empty_pk[s]), ((it / SM_PK_SLOTS) & 1u) ^ 1u, abort_flag)) break;
+        const uint32_t bar = smem_u32(&bars->full_pk[s]);
+        const int kb = kb_of(it), r0 = it < split_at ? ra : rb;
+        mbar_arrive_expect_tx(bar, 128 * 16 * BITS);
+        const uint32_t dst = smem_u32(sm_pk + s * SM_PK_BYTES);
+        if (!TRANS) tma_load_2d(dst, &tmap_pk, bar, kb * (4 * BITS), r0);
+        else tma_load_2d(dst, &tmap_pk, bar, (r0 >> 5) * BITS, kb * SM_BK);
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------- MMA issuer (one lane)
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16_f32(SM_ROWS, 16, TRANS ? 1 : 0, 0) +
+                             ((uint32_t)((p.nt - 16) >> 3) << 17);
+      // One thread issues everything, so its instructions per stage are the pace of the kernel:
+      // descriptors are advanced by additions (the address field counts 16-byte units).
+      const uint32_t a0 = smem_u32(base);
+      const uint64_t adesc0 = smem_desc_sw128(a0, TRANS ? 64 * 128 : 16, 1024);
+      const uint64_t bdesc0 = smem_desc_sw128(a0 + SM_A_BYTES, 16, 1024);
+      const uint64_t stage_inc = (uint64_t)(stage_bytes >> 4), half_inc = (uint64_t)(half_bytes >> 4);
+      const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
+      uint64_t adesc = adesc0, bdesc = bdesc0;
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int it = 0; it < n_it; ++it) {
+        if (!mbar_wait(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d = tmem_base + (it < split_at ? 0u : (uint32_t)SM_MAX_NT);
+        const bool fresh = it == 0 || it == split_at;
+#pragma unroll
+        for (int k = 0; k < SM_HALF / 16; ++k)
+          mma_bf16_ss(d, adesc + k * (TRANS ? 16 * 128 / 16 : 32 / 16), bdesc + k * (32 / 16), idesc,
+                      (fresh && k == 0) ? 0u : 1u);
+#pragma unroll
+        for (int k = 0; k < SM_HALF / 16; ++k)
+          mma_bf16_ss(d, adesc + half_inc + k * (TRANS ? 16 * 128 / 16 : 32 / 16), bdesc + half_inc + k * (32 / 16),
+                      idesc, 1u);
+        mma_commit(empty0 + s * 8);
+        adesc += stage_inc;
+        bdesc += stage_inc;
+        if (++s == p.stages) {
+          s = 0;
+          ph ^= 1u;
+          adesc = adesc0;
+          bdesc = bdesc0;
+        }
+      }
+      if (ok) mma_commit(smem_u32(&bars->acc_full));
+    }
+  } else if (warp >= 4) {
+    // ------------------------------------------------------- weight dequant
+    // A group takes every fourth half stage.  Forward: a thread is one weight row and both 32-column
+    // units of the half.  dX: lanes are 8 rows x 4 units; the thread's second unit is 32 rows
+    // further down.
+    const int grp = (warp - 4) >> 2;
+    const int half = grp & 1;
+    const int gw = (warp - 4) & 3;
+    const int u4 = lane >> 3;
+    const int rowl = TRANS ? gw * 8 + (lane & 7) : gw * 32 + lane;
+    const int swz = rowl & 7;                          // rows of a thread agree modulo 8
+    const int ra = r0_of(0), rb = r0_of(split_at);
+    auto load_zs = [&](int it, UnitZS (&u)[2]) {
+      if (it >= n_it) { u[0] = UnitZS{0u, 0.f, 0.f}; u[1] = u[0]; return; }
+      const int c0 = kb_of(it) * SM_BK + half * SM_HALF, r0 = it < split_at ? ra : rb;
+      if (TRANS) {
+        u[0] = split_load_zs<BITS, ZF>(p, c0 + rowl, r0 + 32 * u4);
+        u[1] = split_load_zs<BITS, ZF>(p, c0 + rowl + 32, r0 + 32 * u4);
+      } else {
+        u[0] = split_load_zs<BITS, ZF>(p, r0 + rowl, c0);
+        // the second unit shares the group unless groups are not multiples of 64 columns
+        if (p.G == 1 || (p.g & 63) == 0) u[1] = u[0];
+        else u[1] = split_load_zs<BITS, ZF>(p, r0 + rowl, c0 + 32);
+      }
+    };
+    auto turn = [&](int it, const UnitZS (&cur)[2], UnitZS (&next)[2]) -> bool {
+      load_zs(it + 2, next);
+      const int pq = it % SM_PK_SLOTS;
+      if (!mbar_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)) return false;
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(sm_pk + pq * SM_PK_BYTES);
+      uint32_t w[2][BITS];
+      if constexpr (!TRANS) {
+        if constexpr (BITS == 4) {
+          // 64-byte rows, 16-byte chunk c of row r at c ^ ((r >> 1) & 3): the code map's swizzle
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const uint4 v = *reinterpret_cast<const uint4*>(src + rowl * 16 + (((2 * half + k) ^ ((rowl >> 1) & 3)) << 2));
+            w[k][0] = v.x; w[k][1] = v.y; w[k][2] = v.z; w[k][3] = v.w;
+          }
+        } else {
+          // 48-byte rows, read whole (consecutive rows fall into different banks)
+          const uint4 a = *reinterpret_cast<const uint4*>(src + rowl * 12 + 4 * half);
+          const uint4 b = *reinterpret_cast<const uint4*>(src + rowl * 12 + 4 * half + 4);
+          const uint32_t w8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+          for (int e = 0; e < 3; ++e) {
+            w[0][e] = half ? w8[2 + e] : w8[e];
+            w[1][e] = half ? w8[5 + e] : w8[3 + e];
+          }
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t* r = src + (half * SM_HALF + rowl + 32 * k) * (4 * BITS) + u4 * BITS;
+          if constexpr (BITS == 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(r);
+            w[k][0] = v.x; w[k][1] = v.y; w[k][2] = v.z; w[k][3] = v.w;
+          } else {
+#pragma unroll
+            for (int e = 0; e < BITS; ++e) w[k][e] = r[e];
+          }
+        }
+      }
+      uint32_t o[2][16];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        if constexpr (ZF) dq::unit32_affine<BITS>(w[k], cur[k].z, cur[k].s, cur[k].c, o[k]);
+        else dq::unit32_natural<BITS, FOLD>(w[k], cur[k].z, cur[k].s, o[k]);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->empty_pk[pq]));
+      const int s = it % p.stages;
+      if (!mbar_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)) return false;
+      uint8_t* tile = base + s * stage_bytes + half * half_bytes;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        uint8_t* row_ptr = TRANS ? tile + (u4 >> 1) * (64 * 128) + (rowl + 32 * k) * 128 : tile + rowl * 128;
+        const int chunk0 = TRANS ? (u4 & 1) * 4 : 4 * k;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          *reinterpret_cast<uint4*>(row_ptr + (((chunk0 + c) ^ swz) << 4)) =
+              make_uint4(o[k][4 * c], o[k][4 * c + 1], o[k][4 * c + 2], o[k][4 * c + 3]);
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->full[s]));
+      return true;
+    };
+    // Two turns per loop, so that the values fetched ahead stay in the registers they were loaded
+    // into: a copy at the end of a turn would wait for the load.
+    UnitZS za[2], zb[2];
+    const int it0 = grp >> 1;
+    load_zs(it0, za);
+    for (int it = it0; it < n_it; it += 4) {
+      if (!turn(it, za, zb)) break;
+      if (it + 2 >= n_it || !turn(it + 2, zb, za)) break;
+    }
+  }
+
+  // ------------------------------------------------- partial sums -> outputs
+  // Passes of SM_DUMP_TOK tokens.  dump[seg][token][row], fp32, over the stage buffers (every MMA
+  // that read them has completed: acc_full).
+  const bool worker = warp >= 4;
+  bool ok = n_it > 0;
+  if (worker && ok) {
+    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag));
+    tc_fence_after();
+  }
+  __syncwarp();
+  float* dump = reinterpret_cast<float*>(base);
+  const int tok_pass = min(p.nt, SM_DUMP_TOK);
+  const int seg_floats = tok_pass * SM_ROWS;
+  const int wtid = (int)threadIdx.x - 128;                   // worker thread index
+  const int rows_per = SM_ROWS / csize;                      // rows of a tile this CTA finishes
+  const int vec_shift = 5 - p.cshift, vec_per = 1 << vec_shift;
+  const uint32_t dump_addr = smem_u32(dump);
+  for (int tp = 0; tp < p.nt; tp += SM_DUMP_TOK) {
+    if (worker && ok) {
+      const int quarter = warp & 3;
+      const int col = ((warp - 4) >> 2) * 32;                // tokens of the pass this warp copies
+      if (tp + col < p.nt) {
+#pragma unroll 1
+        for (int seg = 0; seg < 2; ++seg) {
+          if (seg == 1 && n_it <= split_at) break;
+          uint32_t v[32];
+          tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + seg * SM_MAX_NT + tp + col, v);
+          tmem_ld_wait();
+          float* d = dump + seg * seg_floats + col * SM_ROWS + quarter * 32 + lane;
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (tp + col + e < p.nt) d[e * SM_ROWS] = __uint_as_float(v[e]);
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    if (worker) {
+      const int toks = min(tok_pass, p.nt - tp);
+      for (int j = 0; j < q; ++j) {
+        const int tile = first_tile + j;
+        const int r0 = (tile % p.r_tiles) * SM_ROWS + rank * rows_per;
+        const int t0 = (tile / p.r_tiles) * p.nt + tp;
+        // contributors: the CTAs whose ranges meet [j * k_blocks, (j + 1) * k_blocks)
+        const int b0 = j * p.k_blocks, b1 = b0 + p.k_blocks;
+        uint32_t from = 0, second = 0;     // contributing ranks; those that hold it as second segment
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int rl = range_lo(r), rh = range_lo(r + 1);
+          if (r < csize && rl < b1 && rh > b0 && rh > rl) from |= 1u << r;
+          if (rl < b0) second |= 1u << r;
+        }
+        for (int idx = wtid; idx < toks * vec_per; idx += kSplitWorkers) {
+          const int t = idx >> vec_shift, rv = (idx & (vec_per - 1)) * 4;
+          const int row = r0 + rv;
+          if (t0 + t >= p.T || row >= p.R) continue;
+          const uint32_t off = dump_addr + (uint32_t)(t * SM_ROWS + rank * rows_per + rv) * 4u;
+          float4 v[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (from >> r & 1u)
+              v[r] = ld_cluster_f4(mapa_shared(off + (second >> r & 1u ? (uint32_t)seg_floats * 4u : 0u), (uint32_t)r));
+          }
+          float4 a = v[0];
+#pragma unroll
+          for (int r = 1; r < 8; ++r) {
+            a.x += v[r].x; a.y += v[r].y; a.z += v[r].z; a.w += v[r].w;
+          }
+          if (!FOLD) {
+            const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scales + row));   // one scale per channel
+            a.x *= sc.x; a.y *= sc.y; a.z *= sc.z; a.w *= sc.w;
+          }
+          __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
+          uint2 o;
+          o.x = *reinterpret_cast<uint32_t*>(&h0);
+          o.y = *reinterpret_cast<uint32_t*>(&h1);
+          *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t) * p.R + row) = o;
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();   // the buffers are read by the whole cluster until here
+  }
+
+  if (*abort_flag)        // let copies and MMAs already in flight finish before memory is released
+    for (int i = 0; i < 64; ++i) __nanosleep(1000);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 2) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0 && bars->abort_flag) {
+    atomicExch(p.status, (int)PEQA_ERR_DEVICE_TIMEOUT);
+    p.status[1] = (int)blockIdx.x;
+  }
+}
+
+template <int BITS, bool TRANS, bool FOLD, bool ZF>
+int launch_split_t(const CUtensorMap& ta, const CUtensorMap& tp, const SplitParams& p, size_t smem,
+                   cudaStream_t st) {
+  auto kern = qsplit_kernel<BITS, TRANS, FOLD, ZF>;
+  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  const int clusters = (p.tiles + p.q - 1) / p.q;
+  cfg.gridDim = dim3(clusters << p.cshift, 1, 1);
+  cfg.blockDim = dim3(kSplitThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1 << p.cshift;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, ta, tp, p));
+  return PEQA_OK;
+}
+
+// Token tile, tiles per cluster and CTAs per cluster with the smallest estimated time.
+//
+// Measured on this part (4096 x 4096 and 4096 x 11008, 17 to 1024 tokens): a stage of 128
+// contraction elements takes 0.60 us + 1.8 ns per token of the tile (the weights of a stage cost
+// the same however many tokens multiply them; past 80 tokens the MMAs show), a wave of CTAs
+// another 7 us (launch, first copies, the exchange of the sums).
+struct SplitPlan {
+  int nt, t_tiles, q, cshift;
+  long long ns;
+};
+SplitPlan plan_split(int r_tiles, int C, int T, int sms) {
+  SplitPlan best = {};
+  best.t_tiles = (T + SM_MAX_NT - 1) / SM_MAX_NT;
+  best.nt = ((T + best.t_tiles - 1) / best.t_tiles + 15) & ~15;
+  best.t_tiles = (T + best.nt - 1) / best.nt;
+  best.ns = -1;
+  const long long tiles = (long long)r_tiles * best.t_tiles;
+  const long long k_blocks = (C + SM_BK - 1) / SM_BK;
+  // clusters of 1, 2, 4, 8 CTAs that run at once (cudaOccupancyMaxActiveClusters on this part: 148,
+  // 74, 33, 15 -- the larger ones leave SMs of a GPC idle)
+  const int active[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
+  for (int ci = 0; ci < 4; ++ci) {
+    if (active[ci] < 1) continue;
+    for (int q = 1; q <= (1 << ci); ++q) {
+      const long long clusters = (tiles + q - 1) / q;
+      const long long waves = (clusters + active[ci] - 1) / active[ci];
+      const long long stages = (q * k_blocks + (1 << ci) - 1) >> ci;
+      const long long ns = waves * (stages * (600 + best.nt * 9 / 5) + 7000 + (ci ? 500 : 0) + 50 * ci);
+      if (best.ns < 0 || ns < best.ns) {
+        best.q = q;
+        best.cshift = ci;
+        best.ns = ns;
+      }
+    }
+  }
+  return best;
+}
+
+// The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs, 0.70 us per
+// stage of 64 whether the tile has one block of tokens or two (measured: 44 us for 4096 x 4096 and
+// 117 us for 4096 x 11008 at 17 to 256 tokens, 51 us for 4096 x 4096 at 512 and 1024), and the
+// launch and drain (256 x 256 at 64 tokens: forward 13.4 us, dX 7.6 us).
+long long pair_ns(int R, int C, int T, bool trans, int sms) {
+  const long long tiles = (long long)((R + 255) / 256) * ((T + 511) / 512);
+  const int pairs = sms / 2 > 0 ? sms / 2 : 1;
+  return (tiles + pairs - 1) / pairs * ((C + 63) / 64) * 700 + (trans ? 5000 : 9000);
+}
+
+}  // namespace
+
+// Whether a call is served faster by this kernel than by the pair kernels.  Both estimates are
+// within 15 % of what was measured on either side of the line (before / here, in us): 4096 x 11008
+// forward at 1001 tokens 133 / 99, its dX (86 row tiles: three waves) 102 / 138; 4096 x 4096
+// forward at 77 tokens 44 / 13, at 1024 50 / 44, at 2048 53 / 96; 22016 x 8192 at 256 tokens
+// forward 178 / 128, dX 215 / 93.  A tie goes to the pair kernels.
+bool split_is_faster(const peqa_qweight_t* w, int T, bool trans) {
+  const int R = trans ? w->in_features : w->out_features, C = trans ? w->out_features : w->in_features;
+  const int sms = sm_count_or(148);
+  const SplitPlan plan = plan_split((R + SM_ROWS - 1) / SM_ROWS, C, T, sms);
+  return plan.ns * 105 < pair_ns(R, C, T, trans, sms) * 100;
+}
+
+int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
+                 bool trans, cudaStream_t st) {
+  SplitParams p;
+  p.zeros = w->zeros;
+  p.zeros_f = zeros_f;
+  p.scales = w->scales;
+  p.out = static_cast<__nv_bfloat16*>(out);
+  p.N = w->out_features;
+  p.K = w->in_features;
+  p.g = g;
+  p.G = p.K / g;
+  p.g_shift = -1;
+  for (int b = 5; b < 31; ++b)
+    if ((1 << b) == g) p.g_shift = b;
+  p.T = T;
+  p.R = trans ? p.K : p.N;
+  const int C = trans ? p.N : p.K;
+  p.r_tiles = (p.R + SM_ROWS - 1) / SM_ROWS;
+  const SplitPlan plan = plan_split(p.r_tiles, C, T, sm_count_or(148));
+  p.nt = plan.nt;
+  p.q = plan.q;
+  p.cshift = plan.cshift;
+  p.tiles = p.r_tiles * plan.t_tiles;
+  p.k_blocks = (C + SM_BK - 1) / SM_BK;
+  const int stage_bytes = 2 * (SM_A_BYTES + p.nt * (SM_HALF * 2));
+  p.stages = (SM_SMEM_LIMIT - SM_SMEM_FIXED) / stage_bytes;
+  if (p.stages > SM_MAX_STAGES) p.stages = SM_MAX_STAGES;
+  const size_t smem = (size_t)p.stages * stage_bytes + SM_SMEM_FIXED;
+  PEQA_TRY(status_word(st, &p.status));
+  EncodeTiledFn enc = nullptr;
+  PEQA_TRY(tensor_map_encoder(&enc));
+  CUtensorMap ta, tp;
+  {
+    cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)T};
+    cuuint64_t strides[1] = {(cuuint64_t)C * 2};
+    cuuint32_t box[2] = {64, (cuuint32_t)p.nt};
+    cuuint32_t estr[2] = {1, 1};
+    if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(act), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cuda_fail(cudaErrorInvalidValue);
+  }
+  {
+    const int wpr = p.K * w->bits / 32;
+    cuuint64_t dims[2] = {(cuuint64_t)wpr, (cuuint64_t)p.N};
+    cuuint64_t strides[1] = {(cuuint64_t)wpr * 4};
+    cuuint32_t box[2] = {(cuuint32_t)(4 * w->bits), 128u};
+    cuuint32_t estr[2] = {1, 1};
+    if (enc(&tp, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(w->qweight), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            !trans && w->bits == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cuda_fail(cudaErrorInvalidValue);
+  }
+  const bool b4 = w->bits == 4;
+  if (trans) {
+    if (zeros_f) return b4 ? launch_split_t<4, true, true, true>(ta, tp, p, smem, st)
+                           : launch_split_t<3, true, true, true>(ta, tp, p, smem, st);
+    return b4 ? launch_split_t<4, true, true, false>(ta, tp, p, smem, st)
+              : launch_split_t<3, true, true, false>(ta, tp, p, smem, st);
+  }
+  if (zeros_f) return b4 ? launch_split_t<4, false, true, true>(ta, tp, p, smem, st)
+                         : launch_split_t<3, false, true, true>(ta, tp, p, smem, st);
+  if (p.G > 1) return b4 ? launch_split_t<4, false, true, false>(ta, tp, p, smem, st)
+                         : launch_split_t<3, false, true, false>(ta, tp, p, smem, st);
+  return b4 ? launch_split_t<4, false, false, false>(ta, tp, p, smem, st)
+            : launch_split_t<3, false, false, false>(ta, tp, p, smem, st);
+}
+
+}  // namespace peqa
