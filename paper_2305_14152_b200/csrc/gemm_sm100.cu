@@ -472,6 +472,7 @@ struct DsParams {
   int N, K, G, g, T;
   int wpr;
   int piece;         // columns per output piece: 32, 64 or 128; divides g
+  int vec_ok;        // out, out_z, adam_s, adam_m, adam_v are 16-byte aligned
   int i_tiles, j_tiles, k_blocks;
   int band, band_rows;   // tile order: tiles per band and which dimension is banded (see ds_tile)
   int* status;
@@ -503,26 +504,64 @@ __device__ __forceinline__ void ds_tile(const DsParams& p, int tile, int& it, in
 // leader's "full" barrier and tcgen05.commit releases the stage in both CTAs.
 constexpr int DS_STAGES = 6;
 constexpr int DS_STAGE_BYTES = 2 * (BM * BK * 2);                      // A 16 KiB + B half 16 KiB
-constexpr int DS_SMEM_BYTES = DS_STAGES * DS_STAGE_BYTES + 1024 + 512;
+constexpr int DS_PK_BYTES = BM * 128;                                    // packed codes of a CTA's 128 x 256 half tile
+constexpr int DS_SMEM_BYTES = DS_STAGES * DS_STAGE_BYTES + 2 * DS_PK_BYTES + 1024 + 512;
 
 struct DsBarriers {
   uint64_t full[DS_STAGES];     // leader: bytes of both CTAs landed
   uint64_t empty[DS_STAGES];    // each CTA: MMAs that read the stage completed
   uint64_t acc_full[2];         // each CTA: accumulator ready
   uint64_t acc_empty[2];        // leader: both CTAs' epilogues drained the accumulator
+  uint64_t pk_full[2];          // each CTA: packed codes of a tile landed
+  uint64_t pk_empty[2];         // each CTA: its epilogue warps have read them
   uint32_t tmem_base;
   int abort_flag;
   int wait_limit_us;    // must follow abort_flag (read by the bounded waits)
 };
 
-template <int BITS, bool DZ, bool ADAM>
+// A thread's pieces of one row (n <= 4 adjacent floats): one vector access when they are whole and
+// aligned.  The rows of a warp's lanes lie far apart, so every access touches 32 sectors and
+// their number is what counts.
+__device__ __forceinline__ void load_pieces(const float* src, int n, bool vec, float (&v)[4]) {
+  if (n == 4 && vec) {
+    const float4 t = *reinterpret_cast<const float4*>(src);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  } else if (n == 2 && vec) {
+    const float2 t = *reinterpret_cast<const float2*>(src);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k < n) v[k] = src[k];
+  }
+}
+__device__ __forceinline__ void store_pieces(float* dst, int n, bool vec, const float (&v)[4]) {
+  if (n == 4 && vec) *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  else if (n == 2 && vec) *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
+  else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k < n) dst[k] = v[k];
+  }
+}
+
+// PKTMA: the packed codes of a tile arrive by TMA (needs a 16-byte row pitch of the packed matrix);
+// otherwise the epilogue threads read them from global memory.  With few tokens the epilogue sets
+// the pace (a 256 x 256 tile has only T / 64 stages of MMAs), and what it cost was some thirty
+// accesses of 32 sectors per warp and tile -- codes, optimizer state and results, read row by row
+// after the accumulator was ready.  Codes by TMA a tile ahead, the rest as vectors requested before
+// the wait (gradient and AdamW, before -> after): 22016 x 8192 in groups of 64 at 40 tokens
+// 235 -> 122 us, 4096 x 4096 in groups of 32 at 77 tokens 42 -> 18 us, 4096 x 11008 per channel at
+// 77 tokens 44 -> 31 us; 8192 x 8192 in groups of 64 at 4096 tokens 427 -> 406 us.
+template <int BITS, bool DZ, bool ADAM, bool PKTMA>
 __global__ void __launch_bounds__(kDsThreads, 1)
 ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ CUtensorMap tmap_x,
-          const DsParams p) {
+          const __grid_constant__ CUtensorMap tmap_pk, const DsParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  DsBarriers* bars = reinterpret_cast<DsBarriers*>(base + DS_STAGES * DS_STAGE_BYTES);
+  uint8_t* sm_pk = base + DS_STAGES * DS_STAGE_BYTES;
+  DsBarriers* bars = reinterpret_cast<DsBarriers*>(sm_pk + 2 * DS_PK_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
@@ -536,12 +575,15 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars->acc_full[b]), 1);
       mbar_init(smem_u32(&bars->acc_empty[b]), 16);   // 8 epilogue warps in each of the 2 CTAs
+      mbar_init(smem_u32(&bars->pk_full[b]), 1);
+      mbar_init(smem_u32(&bars->pk_empty[b]), 8);
     }
     bars->abort_flag = 0;
     bars->wait_limit_us = p.status[4];
     fence_mbar_init();
     prefetch_tmap(&tmap_dy);
     prefetch_tmap(&tmap_x);
+    if (PKTMA) prefetch_tmap(&tmap_pk);
   }
   if (warp == 2) {
     tmem_alloc_pair(smem_u32(&bars->tmem_base), TMEM_COLS);
@@ -616,12 +658,26 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full[buf]), 3);
       }
     }
+  } else if (warp == 3) {
+    // packed codes of this CTA's 128 rows x 256 columns, a tile ahead of the epilogue (one lane)
+    if (PKTMA && lane == 0) {
+      int local = 0;
+      for (int tile = pair; tile < total_tiles; tile += n_pairs, ++local) {
+        int ti, tj;
+        ds_tile(p, tile, ti, tj);
+        const int ps = local & 1;
+        if (!mbar_wait(smem_u32(&bars->pk_empty[ps]), ((local >> 1) & 1u) ^ 1u, abort_flag)) break;
+        const uint32_t bar = smem_u32(&bars->pk_full[ps]);
+        mbar_arrive_expect_tx(bar, BM * 32 * BITS);
+        tma_load_2d(smem_u32(sm_pk + ps * DS_PK_BYTES), &tmap_pk, bar, tj * (8 * BITS), ti * (2 * BM) + (int)rank * BM);
+      }
+    }
   } else if (warp >= 4) {
     // Epilogue: thread = one weight row i (TMEM lane) and one 128-column half.
     const int quarter = warp & 3;
     const int half = (warp - 4) >> 2;
     const int npieces = p.K / p.piece;
-    const int chunks_per_piece = p.piece >> 5;
+    const int cpp = p.piece >> 5;                    // 32-column chunks per piece: 1, 2 or 4
     const uint32_t acc_empty_leader0 = mapa_shared(smem_u32(&bars->acc_empty[0]), 0);
     const uint32_t acc_empty_leader1 = mapa_shared(smem_u32(&bars->acc_empty[1]), 0);
     int local = 0;
@@ -630,38 +686,82 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
       int ti, tj;
       ds_tile(p, tile, ti, tj);
       const int i0 = ti * (2 * BM) + (int)rank * BM;
-      const int j0 = tj * BN;
+      const int c0 = tj * BN + half * 128;             // this thread's columns [c0, c0 + 128)
       const int buf = local & 1;
       const uint32_t acc_ph = (local >> 1) & 1u;
+      const int i = i0 + quarter * 32 + lane;
+      const bool row_ok = i < p.N;
+      // Zero-points and optimizer state of the tile do not depend on the accumulator: they are
+      // requested before the wait for it, one vector of the thread's pieces per array.
+      const bool live = row_ok && c0 < p.K;
+      const int n_pieces = live ? min(4 / cpp, (p.K - c0) / p.piece) : 0;
+      // the pieces of a thread are one aligned vector (m and v may have any 4-byte address)
+      const bool vec = p.vec_ok && (npieces & (4 / cpp - 1)) == 0;
+      const size_t e0 = (size_t)i * npieces + c0 / p.piece;  // first piece
+      uint32_t z[4] = {0u, 0u, 0u, 0u};
+      float zreal[4], sc[4], ms[4], mm[4], mv[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        zreal[k] = sc[k] = ms[k] = mm[k] = mv[k] = 0.0f;
+        if (k < n_pieces) {
+          const size_t gi = (size_t)i * p.G + (p.G == 1 ? 0 : (c0 + k * p.piece) / p.g);
+          if (DZ && p.zeros_f) zreal[k] = __ldg(p.zeros_f + gi);
+          else z[k] = __ldg(p.zeros + gi);
+          if (DZ && p.piece == p.g) sc[k] = __ldg(p.scales + gi);
+        }
+      }
+      if (ADAM) {
+        load_pieces(p.adam_s + e0, n_pieces, vec, ms);
+        load_pieces(p.adam_m + e0, n_pieces, vec, mm);
+        load_pieces(p.adam_v + e0, n_pieces, vec, mv);
+      }
+      // the packed codes of the tile (see warp 3)
+      uint32_t w[4][BITS];
+      if (PKTMA) {
+        const int ps = local & 1;
+        if (!mbar_wait(smem_u32(&bars->pk_full[ps]), acc_ph, abort_flag)) { ok = false; break; }
+        const uint8_t* src = sm_pk + ps * DS_PK_BYTES;
+        const int row = quarter * 32 + lane;
+        if constexpr (BITS == 4) {
+          // rows of 128 bytes, 16-byte chunk c at c ^ (row % 8): the code map's swizzle
+#pragma unroll
+          for (int cc = 0; cc < 4; ++cc) {
+            const uint4 v = *reinterpret_cast<const uint4*>(src + row * 128 + (((half * 4 + cc) ^ (row & 7)) << 4));
+            w[cc][0] = v.x; w[cc][1] = v.y; w[cc][2] = v.z; w[cc][3] = v.w;
+          }
+        } else {
+          const uint4* at = reinterpret_cast<const uint4*>(src + row * 96 + half * 48);
+          const uint4 a = at[0], b = at[1], c = at[2];
+          const uint32_t f[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+#pragma unroll
+          for (int cc = 0; cc < 4; ++cc)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) w[cc][q] = f[3 * cc + q];
+        }
+      } else {
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) {
+#pragma unroll
+          for (int q = 0; q < BITS; ++q)
+            w[cc][q] = row_ok && c0 + cc * 32 < p.K ? __ldg(p.qw + (size_t)i * p.wpr + ((c0 >> 5) + cc) * BITS + q) : 0u;
+        }
+      }
       if (!mbar_wait_cluster(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      const int i = i0 + quarter * 32 + lane;
       float acc = 0.0f, accz = 0.0f;
-#pragma unroll 1
+      float r[4] = {0.f, 0.f, 0.f, 0.f}, rz[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
-        const int col0 = j0 + half * 128 + cc * 32;
-        if (col0 >= p.K) break;
+        if (c0 + cc * 32 >= p.K) break;
+        const uint32_t zc = cpp == 1 ? z[cc] : cpp == 2 ? z[cc >> 1] : z[0];
+        const float zr = cpp == 1 ? zreal[cc] : cpp == 2 ? zreal[cc >> 1] : zreal[0];
         uint32_t v[32];
         tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * BN + half * 128 + cc * 32, v);
-        const bool row_ok = i < p.N;
-        uint32_t w[BITS];
-        uint32_t z = 0u;
-        float delta = 0.0f;   // real-valued zero-point = z + delta
-#pragma unroll
-        for (int q = 0; q < BITS; ++q) w[q] = 0u;
-        if (row_ok) {
-          const uint32_t* src = p.qw + (size_t)i * p.wpr + (col0 >> 5) * BITS;
-          if constexpr (BITS == 4) {
-            const uint4 q4 = __ldg(reinterpret_cast<const uint4*>(src));
-            w[0] = q4.x; w[1] = q4.y; w[2] = q4.z; w[3] = q4.w;
-          } else {
-            w[0] = __ldg(src); w[1] = __ldg(src + 1); w[2] = __ldg(src + 2);
-          }
-          if (DZ && p.zeros_f) dq::split_zero_point<BITS>(__ldg(p.zeros_f + (size_t)i * p.G + col0 / p.g), z, delta);
-          else z = __ldg(p.zeros + (size_t)i * p.G + col0 / p.g);
-        }
+        uint32_t zi = zc;
+        float delta = 0.0f;   // real-valued zero-point = zi + delta
+        if (DZ && p.zeros_f) dq::split_zero_point<BITS>(zr, zi, delta);
         uint32_t o[16];
-        dq::unit32_natural<BITS, false>(w, z, 0.0f, o);
+        dq::unit32_natural<BITS, false>(w[cc], zi, 0.0f, o);
         tmem_ld_wait();   // warp-wide: every lane executes it, ragged rows included
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
@@ -669,35 +769,41 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
           acc = fmaf(__uint_as_float(v[2 * q + 1]), __uint_as_float(o[q] & 0xFFFF0000u), acc);
           if (DZ) accz += __uint_as_float(v[2 * q]) + __uint_as_float(v[2 * q + 1]);
         }
-        if (((cc + 1) % chunks_per_piece) == 0) {
-          if (row_ok) {
-            // with a real-valued zero-point, sum (q - z) dW = sum (q - zi) dW - delta * sum dW;
-            // partial pieces are stored raw and corrected after they have been added
-            if (DZ && p.zeros_f && p.piece == p.g) acc = fmaf(-delta, accz, acc);
-            p.out[(size_t)i * npieces + col0 / p.piece] = acc;
-            if (ADAM) {
-              // pieces are whole groups here (the launcher only asks for this then): acc is
-              // the final dS of scale (i, group), owned by this thread alone
-              const size_t e = (size_t)i * npieces + col0 / p.piece;
-              float sv = p.adam_s[e], mv = p.adam_m[e], vv = p.adam_v[e];
-              adamw_update(sv, acc, mv, vv, p.adam);
-              p.adam_s[e] = sv;
-              p.adam_m[e] = mv;
-              p.adam_v[e] = vv;
-            }
-            if (DZ) {
-              // a piece that is a whole group is dZ itself: -s * sum of dW; otherwise the
-              // reduction kernel applies -s after adding the pieces
-              const float f = p.piece == p.g ? -__ldg(p.scales + (size_t)i * p.G + col0 / p.g) : 1.0f;
-              p.out_z[(size_t)i * npieces + col0 / p.piece] = f * accz;
-            }
-          }
+        if (((cc + 1) & (cpp - 1)) == 0) {
+          // with a real-valued zero-point, sum (q - z) dW = sum (q - zi) dW - delta * sum dW;
+          // partial pieces are stored raw and corrected after they have been added
+          if (DZ && p.zeros_f && p.piece == p.g) acc = fmaf(-delta, accz, acc);
+          if (cpp == 1) { r[cc] = acc; rz[cc] = accz; }
+          else if (cpp == 2) { r[cc >> 1] = acc; rz[cc >> 1] = accz; }
+          else { r[0] = acc; rz[0] = accz; }
           acc = 0.0f;
           accz = 0.0f;
         }
       }
+      store_pieces(p.out + e0, n_pieces, vec, r);
+      if (ADAM) {
+        // pieces are whole groups here (the launcher only asks for this then): r holds the final
+        // dS of this row's scales, owned by this thread alone
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (k < n_pieces) adamw_update(ms[k], r[k], mm[k], mv[k], p.adam);
+        store_pieces(p.adam_s + e0, n_pieces, vec, ms);
+        store_pieces(p.adam_m + e0, n_pieces, vec, mm);
+        store_pieces(p.adam_v + e0, n_pieces, vec, mv);
+      }
+      if (DZ) {
+        // a piece that is a whole group is dZ itself: -s * sum of dW; otherwise the reduction
+        // kernel applies -s after adding the pieces
+#pragma unroll
+        for (int k = 0; k < 4; ++k) rz[k] *= p.piece == p.g ? -sc[k] : 1.0f;
+        store_pieces(p.out_z + e0, n_pieces, vec, rz);
+      }
       tc_fence_before();
       __syncwarp();
+      // The code slot goes back only here, after results made from its words have been stored: an
+      // arrive right behind the reads overtook them when the load unit was busy, and the refill
+      // was read in their place.
+      if (PKTMA && lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[local & 1]));
       if (lane == 0) mbar_arrive_cluster(buf ? acc_empty_leader1 : acc_empty_leader0);
     }
   }
@@ -930,6 +1036,7 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   p.adam_m = adam ? adam->m : nullptr;
   p.adam_v = adam ? adam->v : nullptr;
   const bool adam_in_kernel = adam && direct;
+  p.vec_ok = aligned16(p.out) && aligned16(p.out_z) && aligned16(p.adam_s) && aligned16(p.adam_m) && aligned16(p.adam_v);
   p.i_tiles = (p.N + 2 * BM - 1) / (2 * BM);   // 256-row pair tiles
   p.j_tiles = (p.K + BN - 1) / BN;
   p.k_blocks = (T + BK - 1) / BK;
@@ -968,12 +1075,32 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-#define PEQA_DS_LAUNCH(B, Z, A)                                                                       \
+  const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;   // 4-bit: always; 3-bit: K % 128 == 0
+  CUtensorMap tmap_pk = tmap_x;
+  if (pktma) {
+    EncodeTiledFn enc = nullptr;
+    PEQA_TRY(tensor_map_encoder(&enc));
+    cuuint64_t dims[2] = {(cuuint64_t)p.wpr, (cuuint64_t)p.N};
+    cuuint64_t strides[1] = {(cuuint64_t)p.wpr * 4};
+    cuuint32_t box[2] = {8u * w->bits, (cuuint32_t)BM};
+    cuuint32_t estr[2] = {1, 1};
+    if (enc(&tmap_pk, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(w->qweight), dims, strides, box,
+            estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            w->bits == 4 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cuda_fail(cudaErrorInvalidValue);
+  }
+#define PEQA_DS_LAUNCH_T(B, Z, A, P)                                                                  \
   do {                                                                                               \
-    auto kern = ds_kernel<B, Z, A>;                                                                  \
+    auto kern = ds_kernel<B, Z, A, P>;                                                               \
     PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
                                    DS_SMEM_BYTES));                                                  \
-    PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, tmap_dy, tmap_x, p));                                   \
+    PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, tmap_dy, tmap_x, tmap_pk, p));                          \
+  } while (0)
+#define PEQA_DS_LAUNCH(B, Z, A)                     \
+  do {                                              \
+    if (B == 4 || pktma) PEQA_DS_LAUNCH_T(B, Z, A, true); \
+    else PEQA_DS_LAUNCH_T(B, Z, A, (B == 4));       \
   } while (0)
   if (w->bits == 4) {
     if (dZ) PEQA_DS_LAUNCH(4, true, false);
@@ -985,6 +1112,7 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
     else PEQA_DS_LAUNCH(3, false, false);
   }
 #undef PEQA_DS_LAUNCH
+#undef PEQA_DS_LAUNCH_T
   if (!direct) {
     const long long n_out = (long long)p.N * p.G;
     const int ppg = g / p.piece;

@@ -283,20 +283,20 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       load_zs(it + 2, next);
       const int pq = it % SM_PK_SLOTS;
       if (!mbar_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)) return false;
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(sm_pk + pq * SM_PK_BYTES);
+      const uint8_t* src = sm_pk + pq * SM_PK_BYTES;
       uint32_t w[2][BITS];
       if constexpr (!TRANS) {
         if constexpr (BITS == 4) {
           // 64-byte rows, 16-byte chunk c of row r at c ^ ((r >> 1) & 3): the code map's swizzle
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
-            const uint4 v = *reinterpret_cast<const uint4*>(src + rowl * 16 + (((2 * half + k) ^ ((rowl >> 1) & 3)) << 2));
+            const uint4 v = *reinterpret_cast<const uint4*>(src + rowl * 64 + (((2 * half + k) ^ ((rowl >> 1) & 3)) << 4));
             w[k][0] = v.x; w[k][1] = v.y; w[k][2] = v.z; w[k][3] = v.w;
           }
         } else {
           // 48-byte rows, read whole (consecutive rows fall into different banks)
-          const uint4 a = *reinterpret_cast<const uint4*>(src + rowl * 12 + 4 * half);
-          const uint4 b = *reinterpret_cast<const uint4*>(src + rowl * 12 + 4 * half + 4);
+          const uint4 a = *reinterpret_cast<const uint4*>(src + rowl * 48 + 16 * half);
+          const uint4 b = *reinterpret_cast<const uint4*>(src + rowl * 48 + 16 * half + 16);
           const uint32_t w8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
           for (int e = 0; e < 3; ++e) {
@@ -307,13 +307,13 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       } else {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-          const uint32_t* r = src + (half * SM_HALF + rowl + 32 * k) * (4 * BITS) + u4 * BITS;
+          const uint8_t* at = src + (half * SM_HALF + rowl + 32 * k) * (16 * BITS) + u4 * (4 * BITS);
           if constexpr (BITS == 4) {
-            const uint4 v = *reinterpret_cast<const uint4*>(r);
+            const uint4 v = *reinterpret_cast<const uint4*>(at);
             w[k][0] = v.x; w[k][1] = v.y; w[k][2] = v.z; w[k][3] = v.w;
           } else {
 #pragma unroll
-            for (int e = 0; e < BITS; ++e) w[k][e] = r[e];
+            for (int e = 0; e < BITS; ++e) w[k][e] = reinterpret_cast<const uint32_t*>(at)[e];
           }
         }
       }
@@ -323,8 +323,6 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         if constexpr (ZF) dq::unit32_affine<BITS>(w[k], cur[k].z, cur[k].s, cur[k].c, o[k]);
         else dq::unit32_natural<BITS, FOLD>(w[k], cur[k].z, cur[k].s, o[k]);
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->empty_pk[pq]));
       const int s = it % p.stages;
       if (!mbar_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)) return false;
       uint8_t* tile = base + s * stage_bytes + half * half_bytes;
@@ -339,7 +337,12 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->full[s]));
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&bars->full[s]));
+        // behind the stores of what was made from the codes: an arrive right behind the reads can
+        // overtake them when the load unit is busy, and the refill is read in their place
+        mbar_arrive(smem_u32(&bars->empty_pk[pq]));
+      }
       return true;
     };
     // Two turns per loop, so that the values fetched ahead stay in the registers they were loaded
