@@ -27,7 +27,9 @@
 // [bits*p, bits*p + bits) of the string read as a little-endian bit string.
 //
 // Work split.  One CTA per SM owns a contiguous range of 8-row groups and all
-// of K for them, so no sum crosses a CTA: no workspace, no atomics.  Row
+// of K for them, or, when the activations of more tokens would not fit beside
+// the rings, a cluster of CTAs owns the range, each with a slice of K, and their
+// sums meet in distributed shared memory (plan_prep): no workspace, no atomics.  Row
 // groups 2P and 2P+1 form a "pair", the 16 rows of a warp-level mma.m16n8k16
 // whose 8-wide side are the tokens (a range that starts or ends inside a pair
 // runs that group as a half pair).  The CTA's (pair, step) list, pair-major, is cut into sixteen
@@ -36,12 +38,15 @@
 // (one or two steps of a pair: 3 to 8 KiB of contiguous memory; streaming reads
 // on this part want few, large copies and well over 100 KiB in flight per SM)
 // and all lanes wait on the slot's mbarrier.  Codes reach the tensor core as the biased integers
-// (bias + q) they are after one logic operation; the zero-point and bias terms
-// come off the sum when a group (or the row) is complete:
+// (bias + q) they are after one logic operation; the bias terms come off the sum
+// step by step or group by group, the zero-point's with the group (or the row):
 //   y += s * (acc - z * sum_j x_j - sum_j bias_j x_j).
 // When a warp's range crosses into the next pair it parks its sums in shared
 // memory; at the end the parked sums of each pair are added in warp order, so
-// results do not depend on timing.
+// results do not depend on timing.  What that final pass needs per token, row and
+// pair (sums of x, zero-point and scale, contributing warps) lies ready in tables
+// by then: looked up per output it took twice as long as the main loop (12,000
+// cycles against 11,400 for 8 tokens at 8192 x 8192; 2,300 with the tables).
 //
 // Activations are staged in shared memory, all of K when they fit, otherwise in
 // chunks of steps with the per-output sums carried in shared memory.
@@ -73,8 +78,8 @@ constexpr int kPSmemLimit = 227 * 1024;
 constexpr int kPMaxSlots = 4;
 constexpr int kStepCols = 512;
 constexpr int kPBarBytes = kPWarps * kPMaxSlots * 8;              // the warps' mbarriers
-// + abort flag, wait limit and, per warp, the bounds of its steps and its first and last pair
-constexpr int kPHeadBytes = (kPBarBytes + 32 + 3 * (kPWarps + 1) * 4 + 127) / 128 * 128;
+// + abort flag, wait limit, the bounds of the warps' steps and, per token, the sums of x and bias * x
+constexpr int kPHeadBytes = (kPBarBytes + 32 + (kPWarps + 1) * 4 + 4 + 16 * 8 + 127) / 128 * 128;
 
 // Pitch (floats) of a row's tokens in the per-output tables of shared memory.
 __host__ __device__ inline int tok_pitch(int toks) { return toks + ((6 - (toks & 3)) & 3); }
@@ -95,9 +100,9 @@ struct PrepParams {
   int nchunks;
   int slots;                // ring slots per warp
   int sps;                  // steps per slot (1 or 2)
-  int maxseg;               // parked partial sums per warp and chunk
   int x_pitch;              // bytes between staged token rows
   int pairs_per_cta;
+  int cshift;               // log2 of the CTAs that share a range of rows, each with a slice of K
   int* status;
 };
 
@@ -120,6 +125,14 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void* src, ui
       : "memory");
 }
 
+// Asks for [src, src + bytes) in L2, shrunk to whole 16-byte units.
+__device__ __forceinline__ void prefetch_l2(const void* src, size_t bytes) {
+  const uint64_t a = (reinterpret_cast<uint64_t>(src) + 15) & ~(uint64_t)15;
+  const uint64_t e = (reinterpret_cast<uint64_t>(src) + bytes) & ~(uint64_t)15;
+  if (e > a)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
+}
+
 // 16 bytes of a ring slot.  Volatile at both compiler levels: the read must be issued before
 // the bulk copy that refills the slot, and neither the compiler nor the assembler can see
 // that the copy writes this memory, so an ordinary load could be moved behind it.
@@ -130,6 +143,54 @@ __device__ __forceinline__ uint4 ring_load(uint32_t addr) {
                : "r"(addr)
                : "memory");
   return v;
+}
+
+__device__ __forceinline__ float2 ld_cluster_f2(uint32_t cluster_addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
+  return v;
+}
+
+// Values of a step's quantization groups: the first `left` of TG adjacent entries (those beyond the
+// row's last group read as zero).  G: entries per row; when it is a multiple of TG they are one
+// aligned vector and never partly beyond the row.
+template <int TG>
+__device__ __forceinline__ void load_groups(const float* src, int left, bool row_ok, int G, float (&v)[TG]) {
+#pragma unroll
+  for (int q = 0; q < TG; ++q) v[q] = 0.0f;
+  if (!row_ok || left <= 0) return;
+  if (TG >= 2 && (G % TG) == 0 && (reinterpret_cast<uintptr_t>(src) & (TG >= 4 ? 15u : 7u)) == 0) {
+    if constexpr (TG >= 4) {
+#pragma unroll
+      for (int q = 0; q < TG / 4; ++q) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(src) + q);
+        v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
+      }
+    } else if constexpr (TG == 2) {
+      const float2 t = __ldg(reinterpret_cast<const float2*>(src));
+      v[0] = t.x; v[1] = t.y;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < TG; ++q)
+      if (q < left) v[q] = __ldg(src + q);
+  }
+}
+// The same for zero-points, four to a word.
+template <int TG>
+__device__ __forceinline__ void load_zero_bytes(const uint8_t* src, int left, bool row_ok, int G,
+                                                uint32_t (&v)[(TG + 3) / 4]) {
+#pragma unroll
+  for (int q = 0; q < (TG + 3) / 4; ++q) v[q] = 0u;
+  if (!row_ok || left <= 0) return;
+  if (TG >= 4 && (G % TG) == 0 && (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
+#pragma unroll
+    for (int q = 0; q < TG / 4; ++q) v[q] = __ldg(reinterpret_cast<const uint32_t*>(src) + q);
+  } else {
+#pragma unroll
+    for (int q = 0; q < TG; ++q)
+      if (q < left) v[q >> 2] |= (uint32_t)__ldg(src + q) << (8 * (q & 3));
+  }
 }
 
 // One lane's weights of one step: row r of the pair's two groups.
@@ -177,7 +238,8 @@ __host__ __device__ constexpr float column_bias(int cs) {
 // GSH: quantization groups of 32 << GSH columns (1: 64, 2: 128, 3: 256), or 0: one group
 // per row or groups that are multiples of 512 columns (the sums of a whole staged chunk of
 // steps are taken off at once, which needs the chunk to lie inside one group).
-template <int BITS, int NT, int GSH>
+// TASKS: grouped scales with a table per task (NT = 1 only).
+template <int BITS, int NT, int GSH, bool TASKS>
 __global__ void __launch_bounds__(kPThreads, 1)
 decode_prep_kernel(const PrepParams p) {
   constexpr int C = BITS;                            // 16-byte chunks per lane, step and group
@@ -192,28 +254,35 @@ decode_prep_kernel(const PrepParams p) {
   uint64_t* bars = reinterpret_cast<uint64_t*>(base);                        // [warps][kPMaxSlots]
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base + kPBarBytes);   // [0] flag, [1] limit
   int* wbound = const_cast<int*>(abort_flag) + 8;                            // [warps + 1] bounds of the chunk
-  int* wfirst = wbound + kPWarps + 1;                                        // [warps] first pair of the range
-  int* wlast = wfirst + kPWarps + 1;                                         // [warps] last pair, -1: no steps
+  float* tsum = reinterpret_cast<float*>(wbound + kPWarps + 2);              // [16] sum of a token's x (not GROUPED)
   const int toks = (p.M + 1) & ~1;                                           // tokens kept of a tile
   // pitch of a row's tokens in the per-output tables: toks rounded up to 2 mod 4, so that the
   // sixteen rows a warp reads for one token fall into sixteen different banks
   const int tp = tok_pitch(toks);
-  float* part = reinterpret_cast<float*>(base + kPHeadBytes);                // [warps][maxseg][16][tp]
-  float* yacc = part + (size_t)kPWarps * p.maxseg * 16 * tp;                 // [pairs][16][tp]
+  // a warp's range meets other warps' only in its first and its last pair: those sums are parked per
+  // warp, a pair in between is one warp's alone
+  // per pair: see share_bounds; per row: zero-point and scale
+  int* pwarps = reinterpret_cast<int*>(base + kPHeadBytes);                  // [pairs]
+  float2* rowzs = reinterpret_cast<float2*>(pwarps + ((p.pairs_per_cta + 3) & ~3));   // [pairs][16]
+  float* part = reinterpret_cast<float*>(rowzs + (size_t)p.pairs_per_cta * 16);       // [warps][2][16][tp]
+  float* ywhole = part + (size_t)kPWarps * 2 * 16 * tp;                      // [pairs][16][tp]
+  float* yacc = ywhole + (size_t)p.pairs_per_cta * 16 * tp;                  // [pairs][16][tp] (several chunks)
   float* sums = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * 16 * tp : 0);
   // sums, GROUPED: [groups of the chunk][TOKP][2] = (sum x, sum bias*x) per group and token;
-  // else [16 warps][TOKP][2]: every warp's share of the chunk's sums, added in warp order
-  const int sum_rows = GROUPED ? p.spc * GPS : kPWarps;
-  // cterm (GROUPED): [pairs][16][tp], the part of every output that does not depend on the weights
-  float* cterm = sums + (size_t)sum_rows * TOKP * 2;
+  // else [steps of the chunk][TOKP] minus the sum of bias * x, then [16 warps] shares of a token's sum of x
+  const size_t sum_floats = GROUPED ? (size_t)p.spc * GPS * TOKP * 2 : (size_t)p.spc * TOKP + kPWarps;
+  float* xshare = sums + (size_t)p.spc * TOKP;                           // (not GROUPED)
   uint8_t* xs = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(cterm + (GROUPED ? (size_t)p.pairs_per_cta * 16 * tp : 0)) + 127) &
-      ~static_cast<uintptr_t>(127));
+      (reinterpret_cast<uintptr_t>(sums + sum_floats) + 127) & ~static_cast<uintptr_t>(127));
   uint8_t* ring = xs + (((size_t)p.M * p.x_pitch + 127) & ~static_cast<size_t>(127));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r8 = lane >> 2, c4 = lane & 3;
-  const int rg0 = blockIdx.x * p.rg_per_cta;
+  // a cluster of 1 << cshift CTAs owns the rows, each of its CTAs steps [t_lo, t_lo + n_t) of K
+  const int rank = (int)(blockIdx.x & ((1u << p.cshift) - 1u));
+  const int t_lo = (p.T * rank) >> p.cshift;
+  const int n_t = ((p.T * (rank + 1)) >> p.cshift) - t_lo;
+  const int rg0 = (int)(blockIdx.x >> p.cshift) * p.rg_per_cta;
   const int rg_end = min(p.rgs, rg0 + p.rg_per_cta);
   // pairs are (2P, 2P+1) for the whole matrix; a range that starts (ends) at an odd row group
   // has a half pair in front (at the end)
@@ -240,13 +309,13 @@ decode_prep_kernel(const PrepParams p) {
 
   // ---- this warp's steps of a chunk: [bound(w), bound(w+1)) of the pair-major list, cut so
   // that the warps' costs are equal (a step of a full pair costs 4, of a half pair 3)
-  auto spc_of = [&](int ch) { return min(p.spc, p.T - ch * p.spc); };
+  auto spc_of = [&](int ch) { return min(p.spc, n_t - ch * p.spc); };
   auto bound = [&](int w, int spc_c) {
     // measured: a step of a half pair takes about three quarters of a full pair's step (half
     // the code extraction, the same MMAs and activation reads)
     constexpr int CF = 4, CH = 3;
     const int tot = (CH * (lead + trail) + CF * F) * spc_c;
-    int b = (int)(((long long)w * tot) / kPWarps);
+    int b = (int)((unsigned)(w * tot) / kPWarps);
     int at = 0;
     if (lead) {
       if (b <= CH * spc_c) return (b + CH / 2) / CH;
@@ -278,7 +347,7 @@ decode_prep_kernel(const PrepParams p) {
   auto issue_next = [&]() {
     if (i_ch >= p.nchunks) return;
     const int lp = i_lp, tl = i_tl;
-    const int t = i_ch * p.spc + tl;
+    const int t = t_lo + i_ch * p.spc + tl;
     const int n = (p.sps == 2 && i_lin + 1 < i_hi && tl + 1 < i_spc) ? 2 : 1;
     const int rg = pair_rg(lp);
     const int slot = i_slot;
@@ -306,6 +375,29 @@ decode_prep_kernel(const PrepParams p) {
       issue_seek();
     }
   };
+  // The warps' bounds in a chunk of spc_c steps and, per pair, the warps with steps of it and where the
+  // first of them leaves its sums: a range that starts in the pair has it as its first (0), else one
+  // that ends in it as its last (1), else the pair is that warp's alone (2).  Run by one warp.
+  auto share_bounds = [&](int spc_c) {
+    const int mine = bound(min(lane, kPWarps), spc_c);
+    if (lane <= kPWarps) wbound[lane] = mine;
+    for (int base_lp = 0; base_lp < npairs; base_lp += 32) {
+      const int lp = base_lp + lane;
+      const int l0 = lp * spc_c, l1 = l0 + spc_c;
+      uint32_t who = 0u, where = 0u;
+      int wl = 0;
+#pragma unroll
+      for (int w = 0; w < kPWarps; ++w) {
+        const int wh = __shfl_sync(0xffffffffu, mine, w + 1);
+        if (wh > wl && wl < l1 && wh > l0) {
+          if (who == 0u) where = wl >= l0 ? 0u : wh <= l1 ? 1u : 2u;
+          who |= 1u << w;
+        }
+        wl = wh;
+      }
+      if (lp < npairs) pwarps[lp] = (int)(who | where << kPWarps);
+    }
+  };
   // One slot per warp is requested while the preceding kernel drains; the others follow the
   // activation requests of the first chunk, which would otherwise queue behind a full ring of
   // weights on their way into this SM (the CTAs that start last wait longest for them).
@@ -317,13 +409,25 @@ decode_prep_kernel(const PrepParams p) {
   // everything below reads X or writes Y: the preceding kernel must have completed
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
+  // Grouped scales and zero-points are read a few at a time throughout the kernel: the rows' share of
+  // both is requested into L2 as a whole, so that those reads do not each wait for DRAM.
+  if (GROUPED && warp == 2) {
+    const size_t at = (size_t)rg0 * 8 * p.G, n = (size_t)(rg_end - rg0) * 8 * p.G;   // 8 rows: n % 8 == 0
+    const size_t lo = (n * rank >> p.cshift) & ~(size_t)15, hi = (n * (rank + 1) >> p.cshift) & ~(size_t)15;
+    const int tabs = p.task_ids ? min(p.n_tasks, 31) : 1;
+    if (hi > lo) {
+      if (lane < tabs) prefetch_l2(p.scales + (size_t)lane * p.N * p.G + at + lo, (hi - lo) * 4);
+      if (lane == 31) prefetch_l2(p.zeros + at + lo, hi - lo);
+    }
+  }
+
   int c_slot = 0;
   uint32_t c_phase = 0;                              // parity of the ring's current round
   bool ok = true;
 
   for (int ch = 0; ch < p.nchunks; ++ch) {
     const int spc_c = spc_of(ch);
-    const int col0 = ch * p.spc * kStepCols;                       // first column of the chunk
+    const int col0 = (t_lo + ch * p.spc) * kStepCols;              // first column of the chunk
     const int ccols = min(p.K - col0, spc_c * kStepCols);          // real columns in it
     if (ch > 0) __syncthreads();                                   // the previous chunk is no longer read
     // ---- stage X[:, chunk] (columns beyond K read as zero) and take, per token, the sum of x
@@ -331,15 +435,6 @@ decode_prep_kernel(const PrepParams p) {
     // pieces this thread staged itself, added up per warp (the warps' shares are added in
     // warp order when the rows are finished)
     const int pieces = spc_c * (kStepCols / 8);                    // 16-byte pieces per token
-    if (threadIdx.x <= kPWarps) {
-      const int wl = bound(threadIdx.x, spc_c);
-      wbound[threadIdx.x] = wl;
-      if (threadIdx.x < kPWarps) {
-        const int wh = bound(threadIdx.x + 1, spc_c);
-        wfirst[threadIdx.x] = wl / spc_c;
-        wlast[threadIdx.x] = wh > wl ? (wh - 1) / spc_c : -1;
-      }
-    }
     // bias of the two columns in word e of a piece whose run in the step is run % 4 == rq
     auto piece_sums = [&](const uint8_t* ptr, int rq, float& sx, float& sb) {
       const uint4 v = *reinterpret_cast<const uint4*>(ptr);
@@ -363,6 +458,18 @@ decode_prep_kernel(const PrepParams p) {
       if (pc * 8 < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)m * p.K + col0 + pc * 8);
       else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
     };
+    // zero-point and scale of a row, for the final sums (a table per task: scales are looked up there)
+    auto row_zs = [&](int r, uint32_t& z, float& sc) {
+      z = 0u;
+      sc = 0.0f;
+      const int lp = r >> 4, lr = r & 15;
+      if (r >= npairs * 16 || (!pair_full(lp) && lr >= 8)) return;
+      const size_t at = (size_t)(pair_rg(lp) * 8 + lr) * p.G + (p.G == 1 ? 0 : col0 / (p.K / p.G));
+      z = __ldg(p.zeros + at);
+      if (!p.task_ids) sc = __ldg(p.scales + at);
+    };
+    uint32_t z_own = 0u;
+    float s_own = 0.0f;
     if (GROUPED) {
       const int ngr = spc_c * GPS;
       constexpr int gpieces = RUNS_PER_GROUP * 4;                  // 16-byte pieces per group
@@ -372,6 +479,7 @@ decode_prep_kernel(const PrepParams p) {
       }
       if (ch == 0 && lane == 0)
         for (int s = 1; s < p.slots; ++s) issue_next();
+      if (warp == kPWarps - 1) share_bounds(spc_c);                          // while the activations are on their way
       asm volatile("cp.async.wait_all;" ::: "memory");
       for (int idx = threadIdx.x; idx < ngr * p.M; idx += kPThreads) {
         const int gi = idx / p.M, m = idx - gi * p.M;
@@ -384,92 +492,88 @@ decode_prep_kernel(const PrepParams p) {
       }
     } else {
       // A token belongs to 16 / Mp warps (Mp: M rounded up to a power of two); a warp copies
-      // every (16 / Mp)-th block of 32 pieces of its token and sums what it copied itself, so
-      // it needs no other warp's copies and reduces once.  run % 4 of a lane's pieces is fixed.
+      // every (16 / Mp)-th step of its token and sums what it copied itself, so
+      // it needs no other warp's copies.  run % 4 of a lane's pieces is fixed.
       int mp = 1;
       while (mp < p.M) mp <<= 1;
       const int wpt = kPWarps / mp;                                // warps per token
       const int tok = warp / wpt, sub = warp - tok * wpt;
       if (tok < p.M)
-        for (int pc = sub * 32 + lane; pc < pieces; pc += wpt * 32) stage_piece(tok, pc);
+        for (int st = sub; st < spc_c; st += wpt) {
+          stage_piece(tok, st * 64 + lane);
+          stage_piece(tok, st * 64 + 32 + lane);
+        }
       if (ch == 0 && lane == 0)
         for (int s = 1; s < p.slots; ++s) issue_next();
-      // this warp's row of the table: zero but for its own token
-      for (int i = lane; i < TOKP * 2; i += 32) sums[warp * TOKP * 2 + i] = 0.0f;
+      if (warp == kPWarps - 1) share_bounds(spc_c);                          // while the activations are on their way
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncwarp();
       if (tok < p.M) {
-        float sx = 0.0f, sb = 0.0f;
+        float sx = 0.0f;
         const uint8_t* row = xs + (size_t)tok * p.x_pitch;
-        for (int pc = sub * 32 + lane; pc < pieces; pc += wpt * 32)
-          piece_sums(row + pc * 16, (lane >> 2) & 3, sx, sb);
+        // steps by fours; the four sums fold into one register on the way down the lanes: 6
+        // shuffles instead of 20, lane 8 * j ends with the j-th
+        for (int st = sub; st < spc_c; st += 4 * wpt) {
+          float sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          sx += __shfl_xor_sync(0xffffffffu, sx, o);
-          sb += __shfl_xor_sync(0xffffffffu, sb, o);
+          for (int j = 0; j < 4; ++j)
+            if (st + j * wpt < spc_c) {
+              piece_sums(row + ((st + j * wpt) * 64 + lane) * 16, (lane >> 2) & 3, sx, sb[j]);
+              piece_sums(row + ((st + j * wpt) * 64 + 32 + lane) * 16, (lane >> 2) & 3, sx, sb[j]);
+            }
+          const bool u16 = lane & 16, u8 = lane & 8;
+          const float t0 = (u16 ? sb[2] : sb[0]) + __shfl_xor_sync(0xffffffffu, u16 ? sb[0] : sb[2], 16);
+          const float t1 = (u16 ? sb[3] : sb[1]) + __shfl_xor_sync(0xffffffffu, u16 ? sb[1] : sb[3], 16);
+          float t = (u8 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, u8 ? t0 : t1, 8);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          const int mine = st + (lane >> 3) * wpt;
+          if ((lane & 7) == 0 && mine < spc_c) sums[mine * TOKP + tok] = -t;
         }
-        if (lane == 0) {
-          sums[(warp * TOKP + tok) * 2] = sx;
-          sums[(warp * TOKP + tok) * 2 + 1] = sb;
-        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        if (lane == 0) xshare[warp] = sx;
       }
     }
     __syncthreads();
 
-    // ---- per-row terms: when every output of the CTA has a thread of its own, that thread fetches
-    // the row's zero-point and scale now, so that the final reduce does not wait for them
-    const bool own_output = !GROUPED && npairs * 16 * p.M <= kPThreads;
-    float z_own = 0.0f, s_own = 0.0f;
-    if (own_output && threadIdx.x < npairs * 16 * p.M) {
-      const int lp = threadIdx.x / (16 * p.M);
-      const int rem = threadIdx.x - lp * 16 * p.M;
-      const int m = rem >> 4, lr = rem & 15;
-      if (pair_full(lp) || lr < 8) {
-        const int row = pair_rg(lp) * 8 + lr;
-        const int gg = p.G == 1 ? 0 : col0 / (p.K / p.G);
-        z_own = (float)__ldg(p.zeros + (size_t)row * p.G + gg);
-        const float* tab = p.scales;
-        if (p.task_ids) tab += (size_t)min(max(__ldg(p.task_ids + m), 0), p.n_tasks - 1) * p.N * p.G;
-        s_own = __ldg(tab + (size_t)row * p.G + gg);
-      }
-    }
-
+    // a row per thread is fetched now and put down after the main loop, so that nothing waits for it
+    if (!GROUPED) row_zs((int)threadIdx.x, z_own, s_own);
     // ---- this warp's steps of the chunk
     const int lo = wbound[warp], hi = wbound[warp + 1];
-    int seg = 0, cur_pair = -1;
+    const int first_pair = lo / spc_c, last_pair = hi > lo ? (hi - 1) / spc_c : -1;
+    int cur_pair = -1;
     float acc[NT][4], acc2[NT][4], yv[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
-    auto fold = [&]() {
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          acc[nt][e] += acc2[nt][e];
-          acc2[nt][e] = 0.0f;
-        }
-    };
     auto park = [&]() {
-      fold();
-      float* mine = part + ((size_t)(warp * p.maxseg + seg) * 16) * tp;
+      float* mine = cur_pair == first_pair  ? part + (size_t)(warp * 2) * 16 * tp
+                    : cur_pair == last_pair ? part + (size_t)(warp * 2 + 1) * 16 * tp
+                                            : ywhole + (size_t)cur_pair * 16 * tp;
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         const int tk = nt * 8 + c4 * 2;
         const float* v = GROUPED ? yv[nt] : acc[nt];
-        if (seg < p.maxseg && tk < toks) {
+        if (tk < toks) {
           *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0], v[1]);
           *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2], v[3]);
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[nt][e] = yv[nt][e] = 0.0f;
       }
-      ++seg;
     };
     const uint8_t* xl = xs + (size_t)(r8 < p.M ? r8 : 0) * p.x_pitch + c4 * 16;
     const uint8_t* xh = xs + (size_t)(r8 + 8 < p.M ? r8 + 8 : 0) * p.x_pitch + c4 * 16;
 
+    // tasks of this lane's two tokens (grouped scales with a table per task)
+    int task_of[2] = {0, 0};
+    if (TASKS) {
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        if (c4 * 2 + e < p.M) task_of[e] = min(max(__ldg(p.task_ids + c4 * 2 + e), 0), p.n_tasks - 1);
+    }
     int lin = lo;
     int lp = lo / spc_c, tl = lo - lp * spc_c;
     while (ok && lin < hi) {
@@ -505,80 +609,55 @@ decode_prep_kernel(const PrepParams p) {
           if (lane == 0) issue_next();
         }
 
-        // scales of this lane's two rows for the groups of the step (GROUPED, one task): the
-        // sum of a group is only scaled here; its zero-point and bias terms, which do not depend
-        // on the weights, come off where the rows are finished
+        // scales (with a table per task: of this lane's two tokens) and zero-points of this lane's
+        // two rows for all groups of the step, requested before the first MMA: loaded one by one
+        // where a group ends, their latency was on the path of every group
         const int rowa = pair_rg(lp) * 8 + r8, rowb = rowa + 8;
-        const int gstep0 = ((ch * p.spc + tl) * GPS);              // first group of the step
-        float gsa[GPS], gsb[GPS];
-        if (GROUPED && !p.task_ids) {
-          const float* pa = p.scales + (size_t)rowa * p.G + gstep0;
-          const float* pb = p.scales + (size_t)rowb * p.G + gstep0;
-          if ((p.G % GPS) == 0 && gstep0 < p.G) {
-            // G is a multiple of the groups per step: whole, aligned vectors
-            if (GPS >= 4) {
+        const int gstep0 = (t_lo + ch * p.spc + tl) * GPS;         // first group of the step
+        constexpr int TG = GROUPED ? GPS : 1, NS = TASKS ? 2 : 1;
+        float gsa[NS][TG], gsb[NS][TG];
+        uint32_t gza[(TG + 3) / 4], gzb[(TG + 3) / 4];             // four zero-points to a word
+        if (GROUPED) {
+          load_zero_bytes<TG>(p.zeros + (size_t)rowa * p.G + gstep0, p.G - gstep0, true, p.G, gza);
+          load_zero_bytes<TG>(p.zeros + (size_t)rowb * p.G + gstep0, p.G - gstep0, has_b, p.G, gzb);
 #pragma unroll
-              for (int q = 0; q < GPS / 4; ++q) {
-                const float4 va = __ldg(reinterpret_cast<const float4*>(pa) + q);
-                const float4 vb = has_b ? __ldg(reinterpret_cast<const float4*>(pb) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                gsa[4 * q + 0] = va.x; gsa[4 * q + 1] = va.y; gsa[4 * q + 2] = va.z; gsa[4 * q + 3] = va.w;
-                gsb[4 * q + 0] = vb.x; gsb[4 * q + 1] = vb.y; gsb[4 * q + 2] = vb.z; gsb[4 * q + 3] = vb.w;
-              }
-            } else {
-              const float2 va = __ldg(reinterpret_cast<const float2*>(pa));
-              const float2 vb = has_b ? __ldg(reinterpret_cast<const float2*>(pb)) : make_float2(0.f, 0.f);
-              gsa[0] = va.x; gsa[GPS - 1] = va.y;
-              gsb[0] = vb.x; gsb[GPS - 1] = vb.y;
-            }
-          } else {
-#pragma unroll
-            for (int q = 0; q < GPS; ++q) {
-              const bool in = gstep0 + q < p.G;
-              gsa[q] = in ? __ldg(pa + q) : 0.0f;
-              gsb[q] = in && has_b ? __ldg(pb + q) : 0.0f;
-            }
+          for (int e = 0; e < NS; ++e) {
+            const float* tab = p.scales + (TASKS ? (size_t)task_of[e] * p.N * p.G : 0) + gstep0;
+            load_groups<TG>(tab + (size_t)rowa * p.G, p.G - gstep0, true, p.G, gsa[e]);
+            load_groups<TG>(tab + (size_t)rowb * p.G, p.G - gstep0, has_b, p.G, gsb[e]);
           }
         }
         // group gi of the step is complete: take z * sum x + sum bias * x off and scale
         auto flush = [&](int gi) {
-          fold();
-          const int gg = gstep0 + gi;                              // group index in the row
-          const float* sm = sums + ((size_t)(tl * GPS + gi) * TOKP) * 2;
-          if (!p.task_ids) {
-            const float sa = gsa[gi], sb = gsb[gi];
+          const int q = gi % TG;
+          const float za = (float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+          const float zb = (float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              yv[nt][0] = fmaf(sa, acc[nt][0], yv[nt][0]);
-              yv[nt][1] = fmaf(sa, acc[nt][1], yv[nt][1]);
-              yv[nt][2] = fmaf(sb, acc[nt][2], yv[nt][2]);
-              yv[nt][3] = fmaf(sb, acc[nt][3], yv[nt][3]);
+          for (int nt = 0; nt < NT; ++nt) {
+            const float4 sv = *reinterpret_cast<const float4*>(sums + ((size_t)(tl * GPS + gi) * TOKP + nt * 8 + c4 * 2) * 2);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float sx = e ? sv.z : sv.x, sbx = e ? sv.w : sv.y;
+              const float sa = gsa[e % NS][q], sb = gsb[e % NS][q];
+              yv[nt][e] = fmaf(sa, (acc[nt][e] - fmaf(za, sx, sbx)) + acc2[nt][e], yv[nt][e]);
+              yv[nt][2 + e] = fmaf(sb, (acc[nt][2 + e] - fmaf(zb, sx, sbx)) + acc2[nt][2 + e], yv[nt][2 + e]);
             }
-          } else if (gg < p.G) {
-            // every token has the scales of its own task (Sec. 3.3)
-            const float za = (float)__ldg(p.zeros + (size_t)rowa * p.G + gg);
-            const float zb = has_b ? (float)__ldg(p.zeros + (size_t)rowb * p.G + gg) : 0.0f;
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              const float4 sv = *reinterpret_cast<const float4*>(sm + (nt * 8 + c4 * 2) * 2);
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int tok = nt * 8 + c4 * 2 + e;
-                const int task = tok < p.M ? min(max(__ldg(p.task_ids + tok), 0), p.n_tasks - 1) : 0;
-                const float* tab = p.scales + (size_t)task * p.N * p.G;
-                const float sa = __ldg(tab + (size_t)rowa * p.G + gg);
-                const float sb = has_b ? __ldg(tab + (size_t)rowb * p.G + gg) : 0.0f;
-                const float sx = e ? sv.z : sv.x, sbx = e ? sv.w : sv.y;
-                yv[nt][e] = fmaf(sa, acc[nt][e] - fmaf(za, sx, sbx), yv[nt][e]);
-                yv[nt][2 + e] = fmaf(sb, acc[nt][2 + e] - fmaf(zb, sx, sbx), yv[nt][2 + e]);
-              }
-            }
+            for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = 0.0f;
           }
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
         };
 
+        if (!GROUPED) {
+          // one of the two accumulators of a step starts at minus the step's bias terms, so that what
+          // is carried from step to step is the small sum of q * x: carried along with the bias (up
+          // to 128 per column) it would lose bits of the result
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            const float2 b = *reinterpret_cast<const float2*>(sums + (size_t)tl * TOKP + nt * 8 + c4 * 2);
+            acc2[nt][0] = acc2[nt][2] = b.x;
+            acc2[nt][1] = acc2[nt][3] = b.y;
+          }
+        }
         const uint32_t* fa = reinterpret_cast<const uint32_t*>(w.a);
         const uint32_t* fb = reinterpret_cast<const uint32_t*>(w.b);
         const uint8_t* x0 = xl + (size_t)tl * (kStepCols * 2);
@@ -610,6 +689,12 @@ decode_prep_kernel(const PrepParams p) {
           if (GROUPED && RUNS_PER_GROUP == 4) flush(s);
           if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1)) flush(s >> 1);
         }
+        if (!GROUPED) {
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[nt][e] += acc2[nt][e];
+        }
         ++lin;
         if (++tl == spc_c) {
           tl = 0;
@@ -618,124 +703,112 @@ decode_prep_kernel(const PrepParams p) {
       }
     }
     if (cur_pair >= 0) park();
+    if (!GROUPED) {
+      if (warp == kPWarps - 1) {                       // the tokens' sums of x from their warps' shares
+        int mp = 1;
+        while (mp < p.M) mp <<= 1;
+        float t = lane < kPWarps ? xshare[lane] : 0.0f;
+        for (int o = kPWarps / mp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane < kPWarps && (lane & (kPWarps / mp - 1)) == 0) tsum[lane / (kPWarps / mp)] = t;
+      }
+      if (threadIdx.x < npairs * 16) rowzs[threadIdx.x] = make_float2((float)z_own, s_own);
+      for (int r = threadIdx.x + kPThreads; r < npairs * 16; r += kPThreads) {
+        row_zs(r, z_own, s_own);
+        rowzs[r] = make_float2((float)z_own, s_own);
+      }
+    }
     __syncthreads();
 
-    // ---- grouped scales of one task: the terms of the chunk's groups that do not depend on the
-    // weights, per row and token:  sum_g s[row, g] * (z[row, g] * sum x_g + sum bias * x_g).
-    // A warp takes rows warp, warp + 16, ...; the loads of all its rows are issued before the
-    // first is used (this pass is pure latency otherwise), a lane owns four adjacent groups.
     const bool last = ch + 1 == p.nchunks;
-    const bool group_terms = GROUPED && !p.task_ids;
-    if (group_terms) {
-      constexpr int RB = 8;                                        // rows of a warp in flight
-      const int nrows = npairs * 16;
-      const int g0 = ch * p.spc * GPS;
-      const int ng = min(p.G - g0, spc_c * GPS);
-      const bool vec = ((p.G | g0) & 3) == 0;                      // a lane's four scales are 16-byte aligned
-      for (int rbase = warp; rbase < nrows; rbase += kPWarps * RB) {
-        for (int gb = 0; gb < ng; gb += 128) {
-          const int gl = gb + 4 * lane;                            // this lane's first group of the block
-          float4 sv[RB];
-          uint32_t zv[RB];
-#pragma unroll
-          for (int i = 0; i < RB; ++i) {
-            const int r = rbase + i * kPWarps;
-            const int lp = r >> 4, lr = r & 15;
-            sv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            zv[i] = 0u;
-            if (r < nrows && (pair_full(lp) || lr < 8) && gl < ng) {
-              const size_t off = (size_t)(pair_rg(lp) * 8 + lr) * p.G + g0 + gl;
-              if (vec && gl + 4 <= ng) {
-                sv[i] = __ldg(reinterpret_cast<const float4*>(p.scales + off));
-                zv[i] = __ldg(reinterpret_cast<const uint32_t*>(p.zeros + off));
-              } else {
-                float t[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                  if (gl + e < ng) {
-                    t[e] = __ldg(p.scales + off + e);
-                    zv[i] |= (uint32_t)__ldg(p.zeros + off + e) << (8 * e);
-                  }
-                sv[i] = make_float4(t[0], t[1], t[2], t[3]);
-              }
-            }
-          }
-          // groups past the chunk's end carry s = 0; the sums read for them are the last group's
-          for (int m = 0; m < p.M; ++m) {
-            float2 sm[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              sm[e] = *reinterpret_cast<const float2*>(sums + ((size_t)min(gl + e, ng - 1) * TOKP + m) * 2);
-#pragma unroll
-            for (int i = 0; i < RB; ++i) {
-              const int r = rbase + i * kPWarps;
-              if (r >= nrows) break;                               // warp-uniform
-              const float s4[4] = {sv[i].x, sv[i].y, sv[i].z, sv[i].w};
-              float c = 0.0f;
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const float z = (float)((zv[i] >> (8 * e)) & 0xFFu);
-                c = fmaf(s4[e], fmaf(z, sm[e].x, sm[e].y), c);
-              }
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-              if (lane == 0) {
-                float* ct = cterm + (size_t)r * tp + m;
-                *ct = gb == 0 ? c : *ct + c;
-              }
-            }
-          }
-        }
-      }
-      __syncthreads();
-    }
-
-    // ---- add the parked sums of every pair in warp order
-    for (int idx = threadIdx.x; idx < npairs * 16 * p.M; idx += kPThreads) {
-      const int lp = idx / (16 * p.M);
-      const int rem = idx - lp * 16 * p.M;
-      const int m = rem >> 4, lr = rem & 15;
+    // ---- add the parked sums of every pair in warp order: a thread finishes two tokens of a row
+    const int mpairs = (p.M + 1) >> 1;
+    for (int idx = threadIdx.x; idx < npairs * 16 * mpairs; idx += kPThreads) {
+      const int lr = idx & 15, rest_i = idx >> 4;
+      const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
       if (!pair_full(lp) && lr >= 8) continue;                     // a half pair has eight rows
       const int row = pair_rg(lp) * 8 + lr;
-      float sum = group_terms ? -cterm[((size_t)lp * 16 + lr) * tp + m] : 0.0f;
-      // branch-free and unrolled, so that the sixteen reads do not wait for one another: a warp
-      // that has nothing parked for this pair reads a slot of its own (any value) and adds zero
+      const uint32_t pw = (uint32_t)pwarps[lp], who = pw & ((1u << kPWarps) - 1u), where = pw >> kPWarps;
+      float2 sum = make_float2(0.0f, 0.0f);
+      // branch-free and unrolled, so that the reads do not wait for one another; a further warp
+      // starts its range in the pair
+      const int wa = __ffs((int)who) - 1;
+      const float* own = (where == 2u ? ywhole + (size_t)lp * 16 * tp
+                                      : part + (size_t)(max(wa, 0) * 2 + (int)where) * 16 * tp) + lr * tp + m;
+      const uint32_t more = who & (who - 1u);
+      float2 v[kPWarps];
+      v[0] = *reinterpret_cast<const float2*>(own);
+#pragma unroll
+      for (int w = 1; w < kPWarps; ++w)
+        v[w] = more >> w & 1u ? *reinterpret_cast<const float2*>(part + ((size_t)(w * 2) * 16 + lr) * tp + m)
+                              : make_float2(0.0f, 0.0f);
 #pragma unroll
       for (int w = 0; w < kPWarps; ++w) {
-        const int sg = lp - wfirst[w];
-        const bool has = sg >= 0 && sg < p.maxseg && lp <= wlast[w];
-        const int sgc = min(max(sg, 0), p.maxseg - 1);
-        const float v = part[((size_t)(w * p.maxseg + sgc) * 16 + lr) * tp + m];
-        sum += has ? v : 0.0f;
+        sum.x += v[w].x;
+        sum.y += v[w].y;
       }
       if (!GROUPED) {
-        // the chunk lies inside one group: take its zero-point and bias terms off, then scale
-        float sx = 0.0f, sb = 0.0f;
-        for (int w = 0; w < kPWarps; ++w) {
-          sx += sums[(w * TOKP + m) * 2];
-          sb += sums[(w * TOKP + m) * 2 + 1];
-        }
-        float z = z_own, sc = s_own;
-        if (!own_output) {
+        // the chunk lies inside one group: take its zero-point term off, then scale
+        const float2 zs = rowzs[lp * 16 + lr];
+        const float t0 = tsum[m], t1 = tsum[m + 1];
+        float s0 = zs.y, s1 = zs.y;
+        if (p.task_ids) {
           const int gg = p.G == 1 ? 0 : col0 / (p.K / p.G);
-          z = (float)__ldg(p.zeros + (size_t)row * p.G + gg);
-          const float* tab = p.scales;
-          if (p.task_ids) tab += (size_t)min(max(__ldg(p.task_ids + m), 0), p.n_tasks - 1) * p.N * p.G;
-          sc = __ldg(tab + (size_t)row * p.G + gg);
+          const float* tab = p.scales + (size_t)row * p.G + gg;
+          const size_t per = (size_t)p.N * p.G;
+          s0 = __ldg(tab + (size_t)min(max(__ldg(p.task_ids + m), 0), p.n_tasks - 1) * per);
+          if (m + 1 < p.M) s1 = __ldg(tab + (size_t)min(max(__ldg(p.task_ids + m + 1), 0), p.n_tasks - 1) * per);
         }
-        sum -= fmaf(z, sx, sb);
-        sum *= sc;
+        sum.x = fmaf(-zs.x, t0, sum.x) * s0;
+        sum.y = fmaf(-zs.x, t1, sum.y) * s1;
       }
       if (p.nchunks > 1) {
-        float* ya = yacc + ((size_t)lp * 16 + lr) * tp + m;
-        if (ch > 0) sum += *ya;
+        float2* ya = reinterpret_cast<float2*>(yacc + ((size_t)lp * 16 + lr) * tp + m);
+        if (ch > 0) {
+          sum.x += ya->x;
+          sum.y += ya->y;
+        }
         if (!last) {
           *ya = sum;
           continue;
         }
+      } else if (p.cshift) {
+        // the pair's place in ywhole: read above by this thread alone
+        *reinterpret_cast<float2*>(ywhole + ((size_t)lp * 16 + lr) * tp + m) = sum;
+        continue;
       }
-      p.Y[(size_t)m * p.N + row] = __float2bfloat16_rn(sum);
+      p.Y[(size_t)m * p.N + row] = __float2bfloat16_rn(sum.x);
+      if (m + 1 < p.M) p.Y[(size_t)(m + 1) * p.N + row] = __float2bfloat16_rn(sum.y);
     }
+  }
+
+  // ---- the cluster's CTAs hold the sums over their slices of K: added in rank order, a share of
+  // the outputs per CTA
+  if (p.cshift) {
+    __syncwarp();
+    cluster_sync_all();
+    const int csize = 1 << p.cshift;
+    const uint32_t ysum = smem_u32(ywhole);
+    const int mpairs = (p.M + 1) >> 1;
+    for (int idx = (int)threadIdx.x + rank * kPThreads; idx < npairs * 16 * mpairs; idx += csize * kPThreads) {
+      const int lr = idx & 15, rest_i = idx >> 4;
+      const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
+      if (!pair_full(lp) && lr >= 8) continue;
+      const uint32_t at = ysum + (uint32_t)(((lp * 16 + lr) * tp + m) * 4);
+      float2 v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = r < csize ? ld_cluster_f2(mapa_shared(at, (uint32_t)r)) : make_float2(0.f, 0.f);
+      float2 sum = v[0];
+#pragma unroll
+      for (int r = 1; r < 8; ++r) {
+        sum.x += v[r].x;
+        sum.y += v[r].y;
+      }
+      __nv_bfloat16* y = p.Y + (size_t)m * p.N + pair_rg(lp) * 8 + lr;
+      y[0] = __float2bfloat16_rn(sum.x);
+      if (m + 1 < p.M) y[p.N] = __float2bfloat16_rn(sum.y);
+    }
+    __syncwarp();
+    cluster_sync_all();       // the sums are read by the whole cluster until here
   }
 
   if (!ok || abort_flag[0]) {
@@ -837,8 +910,9 @@ __global__ void prep_layout_kernel(const uint32_t* __restrict__ src, uint32_t* _
 }
 
 struct PrepPlan {
-  int rg_per_cta, grid, T, spc, nchunks, slots, sps, maxseg, x_pitch, pairs;
+  int rg_per_cta, grid, T, spc, nchunks, slots, sps, x_pitch, pairs, cshift;
   size_t smem;
+  long long ns;      // estimated time
 };
 
 int x_pitch_for(int steps) {
@@ -846,97 +920,125 @@ int x_pitch_for(int steps) {
   return raw + 64;                                                // pitch % 128 == 64
 }
 
-// Chooses how many steps of activations are staged at a time and the shape of the warps'
-// rings.  gcols: columns of one quantization group.
+// Chooses how many CTAs share a range of rows (each with a slice of K), how many steps of
+// activations are staged at a time and the shape of the warps' rings.  gcols: columns of one
+// quantization group.
+//
+// One CTA per range needs no exchange of sums, but it stages all of its K: from five to eight tokens
+// on, the activations do not fit beside the rings, and working through K in chunks costs a
+// staging, a parking and a reduce per chunk.  A cluster of 2, 4 or 8 CTAs stages a slice each and
+// adds its sums up through distributed shared memory.  The estimate, in ns, from timelines of
+// single CTAs: a warp's step of a pair 1600 (3000 with groups inside the step, a third more with
+// two token tiles), 10 per token and step staged, 2500 for the cluster's exchange, 1500 + 400 M per
+// further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 18.5 us, at 22016 x 8192
+// 65 / 46, in groups of 64 at 8192 x 8192 97 / 28.
 int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
   const int NT = M <= 8 ? 1 : 2, TOKP = 8 * NT;
   const int tp = tok_pitch((M + 1) & ~1);
   const int step_bytes = 2 * bits * 512;
-  plan->T = (K + kStepCols - 1) / kStepCols;
-  plan->rg_per_cta = (rgs + sms - 1) / sms;
-  plan->grid = (rgs + plan->rg_per_cta - 1) / plan->rg_per_cta;
-  plan->pairs = plan->rg_per_cta / 2 + 2;                         // incl. a half pair at either end
   const bool grouped = gcols < kStepCols;
   const int gps = grouped ? kStepCols / gcols : 0;
-  auto need = [&](int spc, int slots, int sps, int* maxseg) -> size_t {
-    const int nch = (plan->T + spc - 1) / spc;
-    // a warp's share of a chunk is at most pairs*spc*4/16 cost units, i.e. at most that / 3 + 2
-    // steps (all of them half-pair steps at cost 3): the pairs it touches
-    const int steps = plan->pairs * spc / 12 + 2;
-    *maxseg = (steps + spc - 1) / spc + 2;
-    if (*maxseg > plan->pairs) *maxseg = plan->pairs;
-    size_t b = 128 + kPHeadBytes;
-    b += (size_t)kPWarps * (*maxseg) * 16 * tp * 4;
-    if (nch > 1) b += (size_t)plan->pairs * 16 * tp * 4;
-    b += (size_t)(grouped ? spc * gps : kPWarps) * TOKP * 2 * 4 + 128;
-    if (grouped) b += (size_t)plan->pairs * 16 * tp * 4;
-    b += (((size_t)M * x_pitch_for(spc)) + 127) / 128 * 128;
-    b += (size_t)kPWarps * slots * sps * step_bytes;
-    return b;
-  };
   // a chunk must lie inside one quantization group unless the groups are applied per step
   const int steps_per_group = grouped ? 1 : gcols / kStepCols;     // one group per row: >= T
   const bool one_group = gcols >= K;
-  // ring shapes in order of preference: bytes in flight first, larger copies on a tie
-  const int shapes[5][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}, {1, 1}};   // {slots, steps per slot}
-  int seg = 0;
-  plan->spc = 0;
-  // all of K staged at once, with the best ring that fits ...
-  if (grouped || one_group) {
-    for (int i = 0; i < 4 && plan->spc == 0; ++i)
-      if (need(plan->T, shapes[i][0], shapes[i][1], &seg) <= (size_t)kPSmemLimit) {
-        plan->spc = plan->T;
-        plan->slots = shapes[i][0];
-        plan->sps = shapes[i][1];
+  // clusters of 1, 2, 4, 8 CTAs that run at once (the larger ones leave SMs of a GPC idle)
+  const int active[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
+  plan->ns = -1;
+  for (int ci = 0; ci < 4; ++ci)
+    for (int waves = 1; waves <= (ci ? 2 : 1); ++waves) {
+      PrepPlan c = {};
+      c.cshift = ci;
+      c.T = (K + kStepCols - 1) / kStepCols;
+      if (ci > 0 && (c.T < (1 << ci) || active[ci] < 1 || !(grouped || one_group))) continue;
+      const int Tl = (c.T + (1 << ci) - 1) >> ci;                     // most steps of a CTA
+      c.rg_per_cta = (rgs + active[ci] * waves - 1) / (active[ci] * waves);
+      c.grid = ((rgs + c.rg_per_cta - 1) / c.rg_per_cta) << ci;
+      // a range that starts and ends at an odd row group holds the most pairs
+      c.pairs = c.rg_per_cta / 2 + 1;
+      auto need = [&](int spc, int slots, int sps) -> size_t {
+        const size_t sums = (size_t)16 * tp * 4;                      // one pair's
+        size_t b = 128 + kPHeadBytes + (kPWarps * 2 + c.pairs) * sums;
+        if (spc < Tl) b += c.pairs * sums;
+        b += (size_t)((c.pairs + 3) & ~3) * 4 + (size_t)c.pairs * 16 * 8;
+        b += ((size_t)spc * (grouped ? 2 * gps : 1) * TOKP + kPWarps) * 4 + 128;
+        b += (((size_t)M * x_pitch_for(spc)) + 127) / 128 * 128;
+        b += (size_t)kPWarps * slots * sps * step_bytes;
+        return b;
+      };
+      // ring shapes in order of preference: bytes in flight first, larger copies on a tie
+      const int shapes[4][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}};   // {slots, steps per slot}
+      // all of the CTA's K staged at once, with the best ring that fits ...
+      if (grouped || one_group) {
+        for (int i = 0; i < 4 && c.spc == 0; ++i)
+          if (need(Tl, shapes[i][0], shapes[i][1]) <= (size_t)kPSmemLimit) {
+            c.spc = Tl;
+            c.slots = shapes[i][0];
+            c.sps = shapes[i][1];
+          }
       }
-  }
-  // ... else the largest chunk of steps beside a ring of two single steps
-  if (plan->spc == 0) {
-    for (int spc = plan->T; spc >= 1 && plan->spc == 0; --spc) {
-      if (!grouped && !one_group && (steps_per_group % spc) != 0) continue;
-      if (need(spc, 2, 1, &seg) <= (size_t)kPSmemLimit) {
-        plan->spc = spc;
-        plan->slots = 2;
-        plan->sps = 1;
+      // ... else (one CTA per range) the largest chunk of steps beside a ring of two single steps
+      if (c.spc == 0 && ci == 0) {
+        for (int spc = c.T; spc >= 1 && c.spc == 0; --spc) {
+          if (!grouped && !one_group && (steps_per_group % spc) != 0) continue;
+          if (need(spc, 2, 1) <= (size_t)kPSmemLimit) {
+            c.spc = spc;
+            c.slots = 2;
+            c.sps = 1;
+          }
+        }
       }
+      if (c.spc == 0) continue;
+      c.nchunks = (Tl + c.spc - 1) / c.spc;
+      c.x_pitch = x_pitch_for(c.spc);
+      c.smem = need(c.spc, c.slots, c.sps);
+      const long long steps = ((long long)c.rg_per_cta * Tl + 1) / 2;
+      const long long per_step = (grouped ? 3000 : 1600) * (NT == 2 ? 13 : 10) / 10;
+      c.ns = waves * ((steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * 10 + 4000 + (ci ? 2500 : 0) +
+                      (c.nchunks - 1) * (1500 + 400 * M)) + (waves - 1) * 10000;
+      if (plan->ns < 0 || c.ns < plan->ns) *plan = c;
     }
-  }
-  if (plan->spc == 0) return PEQA_ERR_TOO_LARGE;
-  plan->nchunks = (plan->T + plan->spc - 1) / plan->spc;
-  plan->x_pitch = x_pitch_for(plan->spc);
-  plan->smem = need(plan->spc, plan->slots, plan->sps, &seg);
-  plan->maxseg = seg;
-  return PEQA_OK;
+  return plan->ns < 0 ? PEQA_ERR_TOO_LARGE : PEQA_OK;
 }
 
-template <int BITS, int NT, int GSH>
+template <int BITS, int NT, int GSH, bool TASKS>
 int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto kern = decode_prep_kernel<BITS, NT, GSH>;
+  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS>;
   PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(kPThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1 << p.cshift;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = p.cshift ? 2 : 1;
   PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, p));
   return PEQA_OK;
 }
 
-template <int BITS, int NT>
+template <int BITS, int NT, bool TASKS>
 int launch_prep_g(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
   switch (gsh) {
-    case 1: return launch_prep_t<BITS, NT, 1>(p, grid, smem, st);
-    case 2: return launch_prep_t<BITS, NT, 2>(p, grid, smem, st);
-    case 3: return launch_prep_t<BITS, NT, 3>(p, grid, smem, st);
-    default: return launch_prep_t<BITS, NT, 0>(p, grid, smem, st);
+    case 1: return launch_prep_t<BITS, NT, 1, TASKS>(p, grid, smem, st);
+    case 2: return launch_prep_t<BITS, NT, 2, TASKS>(p, grid, smem, st);
+    case 3: return launch_prep_t<BITS, NT, 3, TASKS>(p, grid, smem, st);
+    default: return launch_prep_t<BITS, NT, 0, false>(p, grid, smem, st);   // tasks: looked up per row
   }
+}
+
+template <int BITS>
+int launch_prep_b(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
+  if (p.M > 8) return launch_prep_g<BITS, 2, false>(p, gsh, grid, smem, st);
+  return p.task_ids ? launch_prep_g<BITS, 1, true>(p, gsh, grid, smem, st)
+                    : launch_prep_g<BITS, 1, false>(p, gsh, grid, smem, st);
 }
 
 int check_prep_layer(const peqa_qweight_t* w) {
@@ -1014,11 +1116,14 @@ extern "C" int peqa_qlinear_decode_prepared(const peqa_qweight_t* w, const uint3
   }
   if (!aligned16(prepared) || !aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  if (M > 8) {
-    // Two launches of at most eight tokens each: the activations of eight tokens still fit
-    // beside the rings in fewer, larger chunks, and the second pass finds the weights in L2
-    // (measured: 64 us instead of 111 us for 16 tokens at 22016 x 8192, and a third of the
-    // time with scales in groups of 64).
+  PrepPlan plan;
+  PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan));
+  PrepPlan half = plan;
+  if (M > 8) PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, &half));
+  if (M > 8 && (task_ids || 2 * half.ns < plan.ns)) {
+    // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
+    // table per task (the scales of four tokens per lane do not fit in registers), and where
+    // sixteen tokens would be worked through in more chunks or waves.
     const int h = (M + 1) / 2;
     const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
     PEQA_TRY(peqa_qlinear_decode_prepared(w, prepared, X, h, Y, scale_table, n_tasks, task_ids, stream));
@@ -1026,8 +1131,6 @@ extern "C" int peqa_qlinear_decode_prepared(const peqa_qweight_t* w, const uint3
                                         static_cast<char*>(Y) + (size_t)h * N * 2, scale_table, n_tasks,
                                         task_ids ? task_ids + h : nullptr, stream);
   }
-  PrepPlan plan;
-  PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan));
   PrepParams p;
   p.P = reinterpret_cast<const uint8_t*>(prepared);
   p.zeros = w->zeros;
@@ -1047,13 +1150,12 @@ extern "C" int peqa_qlinear_decode_prepared(const peqa_qweight_t* w, const uint3
   p.nchunks = plan.nchunks;
   p.slots = plan.slots;
   p.sps = plan.sps;
-  p.maxseg = plan.maxseg;
   p.x_pitch = plan.x_pitch;
   p.pairs_per_cta = plan.pairs;
+  p.cshift = plan.cshift;
   cudaStream_t st = as_stream(stream);
   PEQA_TRY(status_word(st, &p.status));
   const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
-  // one tile of eight tokens per MMA (NT = 1) is the only instance: M <= 8 here
-  if (w->bits == 3) return launch_prep_g<3, 1>(p, gsh, plan.grid, plan.smem, st);
-  return launch_prep_g<4, 1>(p, gsh, plan.grid, plan.smem, st);
+  return w->bits == 3 ? launch_prep_b<3>(p, gsh, plan.grid, plan.smem, st)
+                      : launch_prep_b<4>(p, gsh, plan.grid, plan.smem, st);
 }
