@@ -2,6 +2,7 @@
 // CUDA error capture and the device status word.
 #pragma once
 
+#include <atomic>
 #include <math.h>
 
 #include <cuda_runtime.h>
@@ -29,6 +30,20 @@ inline int cuda_fail(cudaError_t e) {
     int _s = (expr);                \
     if (_s != PEQA_OK) return _s;   \
   } while (0)
+
+// Allows `kern` its dynamic shared memory on the current device, once per device: the attribute
+// stays with the function, and setting it again cost every launch 0.3 us on the host.  `done` is the kernel's
+// own record (a bit per device); `bytes` is the most it is ever launched with.
+template <typename Kern>
+int allow_smem(Kern kern, int bytes, std::atomic<uint64_t>& done) {
+  int dev = 0;
+  PEQA_CUDA(cudaGetDevice(&dev));
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_acquire) & bit) return PEQA_OK;
+  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  done.fetch_or(bit, std::memory_order_release);
+  return PEQA_OK;
+}
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

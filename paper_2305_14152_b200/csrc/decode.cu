@@ -407,7 +407,8 @@ template <int BITS, int NT, bool FOLD>
 int launch_decode_t(const CUtensorMap& tmap_q, const DecodeParams& p, int row_blocks, size_t smem,
                     cudaStream_t st) {
   auto kern = decode_kernel<BITS, NT, FOLD>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, 227 * 1024, done));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(row_blocks, p.split, 1);
   cfg.blockDim = dim3(kDecBlock, 1, 1);

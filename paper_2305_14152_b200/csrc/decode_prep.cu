@@ -1005,7 +1005,8 @@ int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
 template <int BITS, int NT, int GSH, bool TASKS>
 int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
   auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, kPSmemLimit, done));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(kPThreads, 1, 1);

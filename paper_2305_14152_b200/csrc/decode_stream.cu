@@ -499,7 +499,8 @@ int plan_stream(const peqa_qweight_t* w, int g, int M, StreamPlan* plan) {
 template <int BITS, int NT, bool GROUPED>
 int launch_stream_t(const StreamParams& p, int grid, size_t smem, cudaStream_t st) {
   auto kern = decode_stream_kernel<BITS, NT, GROUPED>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, 227 * 1024, done));
   kern<<<grid, kSBlock, smem, st>>>(p);
   PEQA_CUDA(cudaGetLastError());
   return PEQA_OK;

@@ -389,7 +389,8 @@ template <int BITS, bool ZF>
 int launch_dx_pair_t(const CUtensorMap& ta, const CUtensorMap& tq, const CUtensorMap& to, const DxParams& p, int pairs,
                      cudaStream_t st) {
   auto kern = qdx_pair_kernel<BITS, ZF>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, X_SMEM_BYTES));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, X_SMEM_BYTES, done));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   cfg.blockDim = dim3(kDxThreads, 1, 1);

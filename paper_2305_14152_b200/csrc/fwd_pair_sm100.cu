@@ -437,7 +437,8 @@ template <int BITS, bool FOLD, bool ZF>
 int launch_pair_t(const CUtensorMap& tx, const CUtensorMap& tq, const CUtensorMap& ty, const PairParams& p,
                   int pairs, cudaStream_t st) {
   auto kern = qfwd_pair_kernel<BITS, FOLD, ZF>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM_BYTES));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, P_SMEM_BYTES, done));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   cfg.blockDim = dim3(kPairThreads, 1, 1);

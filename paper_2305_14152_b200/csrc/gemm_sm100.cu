@@ -897,17 +897,12 @@ int sm_count(int* n) {
   return PEQA_OK;
 }
 
-template <typename Kern>
-int set_smem(Kern k) {
-  PEQA_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-  return PEQA_OK;
-}
-
 template <int BITS, bool TRANS, bool FOLD, bool PKTMA>
 int launch_qgemm_k(const CUtensorMap& tmap, const CUtensorMap& tmap_pk, const QGemmParams& p,
                    int grid, cudaStream_t st) {
   auto kern = qgemm_kernel<BITS, TRANS, FOLD, PKTMA>;
-  PEQA_TRY(set_smem(kern));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, SMEM_BYTES, done));
   kern<<<grid, kQgemmThreads, SMEM_BYTES, st>>>(tmap, tmap_pk, p);
   PEQA_CUDA(cudaGetLastError());
   return PEQA_OK;
@@ -1093,8 +1088,8 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
 #define PEQA_DS_LAUNCH_T(B, Z, A, P)                                                                  \
   do {                                                                                               \
     auto kern = ds_kernel<B, Z, A, P>;                                                               \
-    PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,                \
-                                   DS_SMEM_BYTES));                                                  \
+    static std::atomic<uint64_t> done{0};                                                            \
+    PEQA_TRY(allow_smem(kern, DS_SMEM_BYTES, done));                                                 \
     PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, tmap_dy, tmap_x, tmap_pk, p));                          \
   } while (0)
 #define PEQA_DS_LAUNCH(B, Z, A)                     \

@@ -459,7 +459,8 @@ template <int BITS, bool TRANS, bool FOLD, bool ZF>
 int launch_split_t(const CUtensorMap& ta, const CUtensorMap& tp, const SplitParams& p, size_t smem,
                    cudaStream_t st) {
   auto kern = qsplit_kernel<BITS, TRANS, FOLD, ZF>;
-  PEQA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  static std::atomic<uint64_t> done{0};
+  PEQA_TRY(allow_smem(kern, SM_SMEM_LIMIT, done));
   cudaLaunchConfig_t cfg = {};
   const int clusters = (p.tiles + p.q - 1) / p.q;
   cfg.gridDim = dim3(clusters << p.cshift, 1, 1);
