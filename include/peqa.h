@@ -186,6 +186,9 @@ int peqa_qlinear_bwd_ds_adamw(const peqa_qweight_t* w, const void* X_bf16, const
  *   since their kernels run in stream order.
  * 1 <= n_linears <= PEQA_LAYER_MAX_LINEARS.  Shape rules and return codes as for
  * the single calls; nothing is enqueued when a check fails.
+ * A large linear with one scale per channel (T*N*K >= 2^28) takes its dS from the
+ * forward's fp32 sums, dS[i] = sum_t dY[t,i] * sum_j X[t,j] (Q[i,j] - z[i]), instead of
+ * contracting dY^T X: the same sum in another order, closer to the exact one.
  */
 #define PEQA_LAYER_MAX_LINEARS 16
 typedef struct {

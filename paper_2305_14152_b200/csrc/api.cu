@@ -251,11 +251,19 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
   adam.c = adamw_consts(lr, beta1, beta2, eps, weight_decay, (long long)(apply_adamw ? step : 1));
   for (int i = 0; i < n_linears; ++i) {
     const peqa_layer_linear_t* L = &linears[i];
-    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st));
-    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));
     adam.scales = const_cast<float*>(L->w.scales);
     adam.m = L->m;
     adam.v = L->v;
+    const int slots = fwd_ds_slots(&L->w, g[i], T, L->workspace_bytes);
+    if (slots > 0) {
+      // dX first: it reads the scales that the step at the end of launch_fwd_ds rewrites
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));
+      PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, L->dS, apply_adamw ? &adam : nullptr,
+                             static_cast<float*>(L->workspace), slots, st));
+      continue;
+    }
+    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st));
+    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));
     PEQA_TRY(launch_ds(&L->w, nullptr, g[i], L->X_bf16, L->dY_bf16, T, L->dS, nullptr, apply_adamw ? &adam : nullptr,
                        L->workspace, L->workspace_bytes, st));
   }

@@ -58,6 +58,7 @@ struct PairBarriers {
   uint64_t pk_empty[PQ_SLOTS];  // each CTA: the group that owns the slot has read it
   uint64_t acc_full;            // each CTA: both accumulators ready
   uint64_t acc_empty;           // leader: both CTAs' epilogues drained them
+  uint64_t ds_full, ds_free;    // each CTA (DS): the epilogue warps' sums of a tile lie ready / have been read
   uint32_t tmem_base;
   int abort_flag;
   int wait_limit_us;    // must follow abort_flag (read by the bounded waits)
@@ -71,6 +72,8 @@ struct PairParams {
   int N, K, G, g, g_shift, T;
   int n_tiles, t_tiles, k_blocks;   // 256-channel tiles, 512-token tiles, 64-deep stages
   PairItems items;
+  const __nv_bfloat16* dY;   // DS: [T, N]
+  float* ds_part;            // DS: [2 * ceil(T / 256)][N]
   int* status;
 };
 
@@ -79,7 +82,13 @@ __device__ __forceinline__ int pair_group_of(const PairParams& p, int col) {
   return p.g_shift >= 0 ? (col >> p.g_shift) : (col / p.g);
 }
 
-template <int BITS, bool FOLD, bool ZF>
+// DS (one scale per channel): the epilogue also takes the scale gradient's sums.  Eq. 2 reads
+// Y[t,i] = s[i] * u[t,i] with u = sum_j X (Q - z), so dS[i] = sum_t dY[t,i] * u[t,i], and u is
+// what the accumulator holds, in fp32: a product per output replaces the third contraction
+// (2 T N K flop).  A warp multiplies its 32 tokens x 32 channels by dY and folds them over its
+// lanes; the four warps of a token block are added through their staging tiles in warp order and
+// stored to ds_part; ds_channel_kernel adds the blocks.
+template <int BITS, bool FOLD, bool ZF, bool DS>
 __global__ void __launch_bounds__(kPairThreads, 1)
 qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_q,
                  const __grid_constant__ CUtensorMap tmap_y, const PairParams p) {
@@ -106,6 +115,8 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
     mbar_init(smem_u32(&bars->acc_full), 1);
     mbar_init(smem_u32(&bars->acc_empty), 16);            // 8 epilogue warps in each CTA
+    mbar_init(smem_u32(&bars->ds_full), 8);
+    mbar_init(smem_u32(&bars->ds_free), 8);
     bars->abort_flag = 0;
     bars->wait_limit_us = p.status[4];
     fence_mbar_init();
@@ -233,10 +244,22 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       pair_item(p.items, tile, p.T, n_tile, tt0, blocks);
       const int n0 = n_tile * 256;
       const int row0 = tt0 + m * 256 + (int)rank * 128 + quarter * 32;   // first token of this warp
+      const __nv_bfloat16* dy_row = p.dY + (size_t)(row0 + lane) * p.N + n0;
+      float ds_sum[8];
+      if (DS) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ds_sum[k] = 0.0f;
+        // this token's 256 channels of dY on their way into L2 while the accumulators fill
+        if (m < blocks && row0 + lane < p.T)
+          for (int c = 0; c < 256 && n0 + c < p.N; c += 64)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(dy_row + c));
+      }
       if (!mbar_wait_cluster(smem_u32(&bars->acc_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
       tc_fence_after();
       int chunks = m < blocks ? (p.N - n0 + 31) / 32 : 0;
       chunks = chunks > 8 ? 8 : chunks;
+      // the sums of the last tile must have been read before the staging tiles are written again
+      if (DS && local > 0 && !mbar_wait(smem_u32(&bars->ds_free), (uint32_t)(local - 1) & 1u, abort_flag)) { ok = false; break; }
 #pragma unroll 1
       for (int cc = 0; cc < chunks; ++cc) {
         const int c0 = n0 + cc * 32;
@@ -249,14 +272,11 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
         }
-        if (!FOLD) {
-          // one scale per channel: every lane reads the same 32 scales (broadcast loads)
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float sc = c0 + j < p.N ? __ldg(p.scales + c0 + j) : 0.0f;
-            v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
-          }
-        }
+        // one scale per channel: every lane reads the same 32 scales (broadcast loads)
+        auto scaled = [&](int j) {
+          const float u = __uint_as_float(v[j]);
+          return FOLD ? u : u * (c0 + j < p.N ? __ldg(p.scales + c0 + j) : 0.0f);
+        };
         // the previous store must have finished reading the staging tile
         if (lane == 0) bulk_wait_group_read0();
         __syncwarp();
@@ -264,10 +284,10 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         for (int q = 0; q < 4; ++q) {
           uint4 o;
           __nv_bfloat162 h;
-          h = __floats2bfloat162_rn(__uint_as_float(v[8 * q + 0]), __uint_as_float(v[8 * q + 1])); o.x = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(__uint_as_float(v[8 * q + 2]), __uint_as_float(v[8 * q + 3])); o.y = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(__uint_as_float(v[8 * q + 4]), __uint_as_float(v[8 * q + 5])); o.z = *reinterpret_cast<uint32_t*>(&h);
-          h = __floats2bfloat162_rn(__uint_as_float(v[8 * q + 6]), __uint_as_float(v[8 * q + 7])); o.w = *reinterpret_cast<uint32_t*>(&h);
+          h = __floats2bfloat162_rn(scaled(8 * q + 0), scaled(8 * q + 1)); o.x = *reinterpret_cast<uint32_t*>(&h);
+          h = __floats2bfloat162_rn(scaled(8 * q + 2), scaled(8 * q + 3)); o.y = *reinterpret_cast<uint32_t*>(&h);
+          h = __floats2bfloat162_rn(scaled(8 * q + 4), scaled(8 * q + 5)); o.z = *reinterpret_cast<uint32_t*>(&h);
+          h = __floats2bfloat162_rn(scaled(8 * q + 6), scaled(8 * q + 7)); o.w = *reinterpret_cast<uint32_t*>(&h);
           *reinterpret_cast<uint4*>(srow + ((q ^ sw) << 4)) = o;
         }
         fence_proxy_async_smem();
@@ -276,11 +296,59 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
           tma_store_2d(&tmap_y, smem_u32(stage), c0, row0);
           bulk_commit_group();
         }
+        if (DS) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint4 y = make_uint4(0u, 0u, 0u, 0u);            // tokens and channels beyond the matrix count zero
+            if (row0 + lane < p.T && c0 + 8 * q < p.N) y = __ldg(reinterpret_cast<const uint4*>(dy_row + cc * 32 + 8 * q));
+            const uint32_t w4[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              v[8 * q + 2 * e] = __float_as_uint(__uint_as_float(v[8 * q + 2 * e]) * __uint_as_float(w4[e] << 16));
+              v[8 * q + 2 * e + 1] = __float_as_uint(__uint_as_float(v[8 * q + 2 * e + 1]) * __uint_as_float(w4[e] & 0xFFFF0000u));
+            }
+          }
+          // fold 32 tokens: at distance o a lane keeps the channels that agree with it in bit o and
+          // hands the others over; lane j ends with channel c0 + j
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int j = 0; j < o; ++j) {
+              const float keep = __uint_as_float(up ? v[j + o] : v[j]), give = __uint_as_float(up ? v[j] : v[j + o]);
+              v[j] = __float_as_uint(keep + __shfl_xor_sync(0xffffffffu, give, o));
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (k == cc) ds_sum[k] = __uint_as_float(v[0]);
+        }
       }
       if (chunks == 0) {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
+      }
+      if (DS) {
+        if (lane == 0) bulk_wait_group_read0();
+        __syncwarp();
+        float* mine = reinterpret_cast<float*>(stage);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) mine[k * 32 + lane] = ds_sum[k];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars->ds_full));
+        if (!mbar_wait(smem_u32(&bars->ds_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
+        // thread = channel: the four warps of a token block, in order
+        const int ch = (warp - 4) * 32 + lane;
+        const float* all = reinterpret_cast<const float*>(sm_e);
+        for (int mb = 0; mb < blocks; ++mb) {
+          float sum = 0.0f;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) sum += all[(mb * 4 + w) * (PE_BYTES / 4) + ch];
+          if (n0 + ch < p.N) p.ds_part[(size_t)(((tt0 >> 8) + mb) * 2 + (int)rank) * p.N + n0 + ch] = sum;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars->ds_free));   // behind the stores that used what was read
       }
     }
     if (lane == 0) bulk_wait_group0();             // every store has left shared memory and landed
@@ -433,10 +501,10 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   }
 }
 
-template <int BITS, bool FOLD, bool ZF>
+template <int BITS, bool FOLD, bool ZF, bool DS>
 int launch_pair_t(const CUtensorMap& tx, const CUtensorMap& tq, const CUtensorMap& ty, const PairParams& p,
                   int pairs, cudaStream_t st) {
-  auto kern = qfwd_pair_kernel<BITS, FOLD, ZF>;
+  auto kern = qfwd_pair_kernel<BITS, FOLD, ZF, DS>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, P_SMEM_BYTES, done));
   cudaLaunchConfig_t cfg = {};
@@ -468,12 +536,14 @@ bool fwd_pair_supported(const peqa_qweight_t* w) {
 }
 
 int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T,
-                    void* Y, cudaStream_t st) {
+                    void* Y, const void* dY, float* ds_part, cudaStream_t st) {
   PairParams p;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;
   p.out = static_cast<__nv_bfloat16*>(Y);
+  p.dY = static_cast<const __nv_bfloat16*>(dY);
+  p.ds_part = ds_part;
   p.N = w->out_features;
   p.K = w->in_features;
   p.g = g;
@@ -530,13 +600,16 @@ int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const 
   p.items = make_pair_items(p.n_tiles, p.t_tiles, T, pairs);
   const bool fold = p.G > 1;
   if (zeros_f)   // a real-valued zero-point is folded into the operand whatever the group size
-    return w->bits == 4 ? launch_pair_t<4, true, true>(tx, tq, ty, p, pairs, st)
-                        : launch_pair_t<3, true, true>(tx, tq, ty, p, pairs, st);
-  if (w->bits == 4)
-    return fold ? launch_pair_t<4, true, false>(tx, tq, ty, p, pairs, st)
-                : launch_pair_t<4, false, false>(tx, tq, ty, p, pairs, st);
-  return fold ? launch_pair_t<3, true, false>(tx, tq, ty, p, pairs, st)
-              : launch_pair_t<3, false, false>(tx, tq, ty, p, pairs, st);
+    return w->bits == 4 ? launch_pair_t<4, true, true, false>(tx, tq, ty, p, pairs, st)
+                        : launch_pair_t<3, true, true, false>(tx, tq, ty, p, pairs, st);
+  if (fold)
+    return w->bits == 4 ? launch_pair_t<4, true, false, false>(tx, tq, ty, p, pairs, st)
+                        : launch_pair_t<3, true, false, false>(tx, tq, ty, p, pairs, st);
+  if (ds_part)
+    return w->bits == 4 ? launch_pair_t<4, false, false, true>(tx, tq, ty, p, pairs, st)
+                        : launch_pair_t<3, false, false, true>(tx, tq, ty, p, pairs, st);
+  return w->bits == 4 ? launch_pair_t<4, false, false, false>(tx, tq, ty, p, pairs, st)
+                      : launch_pair_t<3, false, false, false>(tx, tq, ty, p, pairs, st);
 }
 
 }  // namespace peqa

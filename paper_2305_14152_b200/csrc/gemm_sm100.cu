@@ -866,6 +866,30 @@ __global__ void ds_reduce_kernel(const float* __restrict__ partial, float* __res
   }
 }
 
+// dS[i] = sum over the token blocks' partial sums, in a fixed order (eight interleaved chains, then
+// these in order), and the AdamW step on scale i with adam_s.
+__global__ void ds_channel_kernel(const float* __restrict__ part, float* __restrict__ dS, int N, int slots,
+                                  AdamWConsts adam, float* __restrict__ adam_s, float* __restrict__ adam_m,
+                                  float* __restrict__ adam_v) {
+  __shared__ float sums[8][33];
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  float acc = 0.0f;
+  if (i < N)
+    for (int q = threadIdx.y; q < slots; q += 8) acc += __ldg(part + (size_t)q * N + i);
+  sums[threadIdx.y][threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.y != 0 || i >= N) return;
+  for (int y = 1; y < 8; ++y) acc += sums[y][threadIdx.x];
+  dS[i] = acc;
+  if (adam_s) {
+    float sv = adam_s[i], mv = adam_m[i], vv = adam_v[i];
+    adamw_update(sv, acc, mv, vv, adam);
+    adam_s[i] = sv;
+    adam_m[i] = mv;
+    adam_v[i] = vv;
+  }
+}
+
 // --------------------------------------------------------------- host side
 
 // bf16 row-major [outer, inner] tensor, box = [box_outer rows, 64 elements], 128B swizzle,
@@ -980,16 +1004,41 @@ int ds_piece(int g) { return gcd_int(g, 128); }
 
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
                cudaStream_t st) {
-  if (fwd_pair_supported(w) && split_is_faster(w, T, false)) return launch_split(w, zeros_f, g, X, T, Y, false, st);
-  if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, st);
+  if (fwd_pair_supported(w) && split_is_faster(w, T, false)) return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st);
+  if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
               cudaStream_t st) {
-  if (dx_pair_supported(w) && split_is_faster(w, T, true)) return launch_split(w, zeros_f, g, dY, T, dX, true, st);
+  if (dx_pair_supported(w) && split_is_faster(w, T, true)) return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st);
   if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
+}
+
+int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes) {
+  if (g != w->in_features || !fwd_pair_supported(w)) return 0;
+  // dS = sum_t dY * u from the forward's fp32 sums instead of a contraction of its own (training
+  // step of one linear, before -> after in us, and error of dS against binary64): 11008 x 4096 at
+  // 4096 tokens 742 -> 611, 4.4e-6 -> 1.4e-7; 22016 x 8192 at 2048 tokens 1406 -> 1040; 4096 x 4096
+  // at 20 tokens 40 -> 32.  Below 2^28 products the contraction is two launches of a few us (256 x
+  // 256 at 64 tokens: 9 us) and the call stays the exact composition of the single calls, whose dS
+  // differs from this one in its last bits.
+  if ((double)T * w->out_features * w->in_features < (double)(1 << 28)) return 0;
+  const int slots = split_is_faster(w, T, false) ? split_ds_slots(w, T) : 2 * ((T + 255) / 256);
+  return (size_t)slots * w->out_features * sizeof(float) <= workspace_bytes ? slots : 0;
+}
+
+int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* dS,
+                  const DsAdam* adam, float* workspace, int slots, cudaStream_t st) {
+  const int g = w->in_features;
+  if (split_is_faster(w, T, false)) PEQA_TRY(launch_split(w, nullptr, g, X, T, Y, false, dY, workspace, st));
+  else PEQA_TRY(launch_fwd_pair(w, nullptr, g, X, T, Y, dY, workspace, st));
+  ds_channel_kernel<<<(w->out_features + 31) / 32, dim3(32, 8), 0, st>>>(
+      workspace, dS, w->out_features, slots, adam ? adam->c : AdamWConsts{}, adam ? adam->scales : nullptr,
+      adam ? adam->m : nullptr, adam ? adam->v : nullptr);
+  PEQA_CUDA(cudaGetLastError());
+  return PEQA_OK;
 }
 
 size_t ds_workspace_bytes(const peqa_qweight_t* w, int g, int T) {

@@ -72,6 +72,8 @@ struct SplitParams {
   int nt;                 // tokens per tile, a multiple of 16
   int stages;
   int q, cshift;          // tiles per cluster, log2 of the CTAs per cluster (q <= 1 << cshift)
+  const __nv_bfloat16* dY;   // DS: [T, N]
+  float* ds_part;            // DS: [token tiles * passes][N]
   int* status;
 };
 
@@ -116,7 +118,10 @@ __device__ __forceinline__ UnitZS split_load_zs(const SplitParams& p, int i, int
   return u;
 }
 
-template <int BITS, bool TRANS, bool FOLD, bool ZF>
+// DS (forward with one scale per channel): where the fp32 sums of a tile are complete they are also
+// multiplied by dY and summed over the tile's tokens, dS[i] = sum_t dY[t,i] * u[t,i] (see the
+// pair kernel).
+template <int BITS, bool TRANS, bool FOLD, bool ZF, bool DS>
 __global__ void __launch_bounds__(kSplitThreads, 1)
 qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constant__ CUtensorMap tmap_pk,
               const SplitParams p) {
@@ -408,6 +413,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           if (r < csize && rl < b1 && rh > b0 && rh > rl) from |= 1u << r;
           if (rl < b0) second |= 1u << r;
         }
+        float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);   // vec_per divides kSplitWorkers: a thread keeps its rows
         for (int idx = wtid; idx < toks * vec_per; idx += kSplitWorkers) {
           const int t = idx >> vec_shift, rv = (idx & (vec_per - 1)) * 4;
           const int row = r0 + rv;
@@ -425,6 +431,13 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           for (int r = 1; r < 8; ++r) {
             a.x += v[r].x; a.y += v[r].y; a.z += v[r].z; a.w += v[r].w;
           }
+          if (DS) {
+            const uint2 y = __ldg(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t) * p.R + row));
+            ds.x = fmaf(a.x, __uint_as_float(y.x << 16), ds.x);
+            ds.y = fmaf(a.y, __uint_as_float(y.x & 0xFFFF0000u), ds.y);
+            ds.z = fmaf(a.z, __uint_as_float(y.y << 16), ds.z);
+            ds.w = fmaf(a.w, __uint_as_float(y.y & 0xFFFF0000u), ds.w);
+          }
           if (!FOLD) {
             const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scales + row));   // one scale per channel
             a.x *= sc.x; a.y *= sc.y; a.z *= sc.z; a.w *= sc.w;
@@ -434,6 +447,29 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           o.x = *reinterpret_cast<uint32_t*>(&h0);
           o.y = *reinterpret_cast<uint32_t*>(&h1);
           *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t) * p.R + row) = o;
+        }
+        if (DS) {
+          // lanes that share rows, then the warps in order (over the code slots, which are done with)
+          for (int o = 16; o >= vec_per; o >>= 1) {
+            ds.x += __shfl_xor_sync(0xffffffffu, ds.x, o);
+            ds.y += __shfl_xor_sync(0xffffffffu, ds.y, o);
+            ds.z += __shfl_xor_sync(0xffffffffu, ds.z, o);
+            ds.w += __shfl_xor_sync(0xffffffffu, ds.w, o);
+          }
+          float4* sums = reinterpret_cast<float4*>(sm_pk);
+          if (lane < vec_per) sums[(warp - 4) * 32 + lane] = ds;
+          named_barrier_sync(1, kSplitWorkers);
+          if (wtid < vec_per && r0 + wtid * 4 < p.R) {
+            float4 s = sums[wtid];
+            for (int w = 1; w < kSplitWorkers / 32; ++w) {
+              const float4 v = sums[w * 32 + wtid];
+              s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+            }
+            const int passes = (p.nt + SM_DUMP_TOK - 1) / SM_DUMP_TOK;
+            const size_t slot = (size_t)(tile / p.r_tiles) * passes + tp / SM_DUMP_TOK;
+            *reinterpret_cast<float4*>(p.ds_part + slot * p.R + r0 + wtid * 4) = s;
+          }
+          named_barrier_sync(1, kSplitWorkers);
         }
       }
     }
@@ -455,10 +491,10 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   }
 }
 
-template <int BITS, bool TRANS, bool FOLD, bool ZF>
+template <int BITS, bool TRANS, bool FOLD, bool ZF, bool DS = false>
 int launch_split_t(const CUtensorMap& ta, const CUtensorMap& tp, const SplitParams& p, size_t smem,
                    cudaStream_t st) {
-  auto kern = qsplit_kernel<BITS, TRANS, FOLD, ZF>;
+  auto kern = qsplit_kernel<BITS, TRANS, FOLD, ZF, DS>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, SM_SMEM_LIMIT, done));
   cudaLaunchConfig_t cfg = {};
@@ -542,13 +578,21 @@ bool split_is_faster(const peqa_qweight_t* w, int T, bool trans) {
   return plan.ns * 105 < pair_ns(R, C, T, trans, sms) * 100;
 }
 
+// Partial sums per channel that a forward with dS writes.
+int split_ds_slots(const peqa_qweight_t* w, int T) {
+  const SplitPlan plan = plan_split((w->out_features + SM_ROWS - 1) / SM_ROWS, w->in_features, T, sm_count_or(148));
+  return plan.t_tiles * ((plan.nt + SM_DUMP_TOK - 1) / SM_DUMP_TOK);
+}
+
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, cudaStream_t st) {
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st) {
   SplitParams p;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;
   p.out = static_cast<__nv_bfloat16*>(out);
+  p.dY = static_cast<const __nv_bfloat16*>(dY);
+  p.ds_part = ds_part;
   p.N = w->out_features;
   p.K = w->in_features;
   p.g = g;
@@ -607,6 +651,8 @@ int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
                          : launch_split_t<3, false, true, true>(ta, tp, p, smem, st);
   if (p.G > 1) return b4 ? launch_split_t<4, false, true, false>(ta, tp, p, smem, st)
                          : launch_split_t<3, false, true, false>(ta, tp, p, smem, st);
+  if (ds_part) return b4 ? launch_split_t<4, false, false, false, true>(ta, tp, p, smem, st)
+                         : launch_split_t<3, false, false, false, true>(ta, tp, p, smem, st);
   return b4 ? launch_split_t<4, false, false, false>(ta, tp, p, smem, st)
             : launch_split_t<3, false, false, false>(ta, tp, p, smem, st);
 }

@@ -1,0 +1,56 @@
+"""GPU parity of the layer step where a linear with one scale per channel takes dS from the forward's
+fp32 sums: through the cluster-split forward and through the CTA-pair forward, with ragged token
+blocks, row tiles and channel tiles, with and without the optimizer step."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2305_14152_b200 import binding, synth
+from gpu_util import adamw_scale_tol, assert_close, bf16_to_dev, dev_to_f64, oracle_layer, to_qweight
+
+pytestmark = pytest.mark.gpu
+
+LR = float(np.float32(1e-3))
+
+
+# few tokens: one and several token tiles, two passes per tile, rows beyond a tile; many tokens: token
+# blocks that end inside a half tile, a channel tile of 8 columns, tiles of one token block only
+@pytest.mark.parametrize("N,K,bits,T", [(4104, 4096, 4, 17), (1000, 8192, 3, 200), (2056, 1152, 4, 300), (520, 4096, 3, 129),
+                                        (8456, 2048, 4, 1030), (9736, 1280, 3, 1279), (10248, 1536, 4, 700)])
+def test_channel_ds_from_the_forward(N, K, bits, T):
+    d = synth.custom(N + T, N, K, T, bits, 0, outliers=True, sigma_dy=1e-2)
+    codes, zeros, scales, packed = oracle_layer(d, bits, 0)
+    rows = np.unique(np.concatenate([np.arange(40), np.arange(N - 40, N), np.arange(0, N, 97)]))
+    toks = np.unique(np.concatenate([np.arange(3), [T // 2, T - 2, T - 1]]))
+    ref = oracle.bwd_ds(d["X"], d["dY"], packed, zeros, bits, 0, rows=rows)
+    X, dY = bf16_to_dev(d["X"]), bf16_to_dev(d["dY"])
+    out = []
+    for apply in (True, False, True):
+        qw = to_qweight(packed, zeros, scales, bits, 0, K)
+        L = binding.LayerLinear(w=qw, X=X, dY=dY, Y=torch.empty((T, N), dtype=torch.bfloat16, device="cuda"),
+                                dX=torch.empty((T, K), dtype=torch.bfloat16, device="cuda"),
+                                dS=torch.full((N, 1), 9.0, device="cuda"), m=torch.zeros((N, 1), device="cuda"),
+                                v=torch.zeros((N, 1), device="cuda"),
+                                workspace=binding.alloc_workspace(binding.OP_BWD, T, qw))
+        L.workspace.fill_(255)
+        binding.layer_train_step([L], LR, step=1, apply_adamw=apply)
+        binding.check_status()
+        out.append(L)
+        ds = L.dS.cpu().numpy()
+        assert_close(ds[rows].astype(np.float64), ref, "dS")
+        # both are binary32 sums of the same products: far closer than the bound for bf16 results
+        assert np.linalg.norm(ds[rows] - ref) <= 2e-6 * np.linalg.norm(ref)
+        assert_close(dev_to_f64(L.Y)[toks], oracle.fwd(d["X"], packed, zeros, scales, bits, 0, tokens=toks), "Y")
+        if apply:
+            zero = np.zeros_like(scales)
+            s_ref, _, _ = oracle.adamw(scales, ds, zero, zero, LR, float(np.float32(0.9)), float(np.float32(0.999)),
+                                       float(np.float32(1e-8)), 0.0, 1)
+            tol = adamw_scale_tol(scales, ds, zero, zero, LR, 0.9, 0.999, 1e-8, 0.0, 1)
+            assert np.all(np.abs(qw.scales.cpu().numpy().ravel().astype(np.float64) - s_ref) <= tol)
+        else:
+            assert np.array_equal(qw.scales.cpu().numpy(), scales)
+    for L in out[1:]:
+        assert torch.equal(L.dS, out[0].dS) and torch.equal(L.Y, out[0].Y) and torch.equal(L.dX, out[0].dX)
+    single = binding.qlinear_bwd(to_qweight(packed, zeros, scales, bits, 0, K), X, dY, need_dx=False)[1]
+    assert torch.allclose(single, out[0].dS, rtol=1e-3, atol=1e-4 * float(single.abs().mean()))
