@@ -469,6 +469,14 @@ int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
     split *= 2;
   }
   if (smem > 227 * 1024) return PEQA_ERR_TOO_LARGE;
+  const bool fold = p.G > 1;
+  // More than eight tokens need two token tiles per MMA here and twice the staging; the cluster-split
+  // forward, whose time hardly depends on the tokens, folds grouped scales into its operand
+  // as this kernel does.  In us, here / there: 8192 x 22016 in groups of 64 at 12 tokens 175 / 70,
+  // 22016 x 8192 in groups of 128 at 11 tokens 107 / 80, 4096 x 4096 in groups of 128 at 9 tokens
+  // 16 / 12; one scale per channel, 16 tokens: 8192 x 22016 107 / 60, 8192 x 8192 31 / 26, but
+  // 22016 x 8192 at 9 tokens 56 / 75 -- many rows are this kernel's better side.
+  if (M > 8 && (fold || p.K >= p.N)) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st);
   PEQA_TRY(status_word(st, &p.status));
   // packed matrix as uint32 [N, wpr]; box = 16 words x 128 rows, 64-byte swizzle
   CUtensorMap tmap_q;
@@ -484,17 +492,15 @@ int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cuda_fail(cudaErrorInvalidValue);
   }
-  const bool fold = p.G > 1;
-  if (w->bits == 4) {
-    if (NT == 1) return fold ? launch_decode_t<4, 1, true>(tmap_q, p, row_blocks, smem, st)
-                             : launch_decode_t<4, 1, false>(tmap_q, p, row_blocks, smem, st);
-    return fold ? launch_decode_t<4, 2, true>(tmap_q, p, row_blocks, smem, st)
-                : launch_decode_t<4, 2, false>(tmap_q, p, row_blocks, smem, st);
-  }
-  if (NT == 1) return fold ? launch_decode_t<3, 1, true>(tmap_q, p, row_blocks, smem, st)
-                           : launch_decode_t<3, 1, false>(tmap_q, p, row_blocks, smem, st);
-  return fold ? launch_decode_t<3, 2, true>(tmap_q, p, row_blocks, smem, st)
+  const bool b4 = w->bits == 4;
+  if (NT == 2)   // one scale per channel: grouped scales of so many tokens went the other way
+    return b4 ? launch_decode_t<4, 2, false>(tmap_q, p, row_blocks, smem, st)
               : launch_decode_t<3, 2, false>(tmap_q, p, row_blocks, smem, st);
+  if (fold)
+    return b4 ? launch_decode_t<4, 1, true>(tmap_q, p, row_blocks, smem, st)
+              : launch_decode_t<3, 1, true>(tmap_q, p, row_blocks, smem, st);
+  return b4 ? launch_decode_t<4, 1, false>(tmap_q, p, row_blocks, smem, st)
+            : launch_decode_t<3, 1, false>(tmap_q, p, row_blocks, smem, st);
 }
 
 }  // namespace peqa
