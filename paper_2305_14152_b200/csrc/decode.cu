@@ -322,7 +322,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmap_q, const DecodeParams p) 
         }
       }
     }
-    // the codes of this step are in registers and consumed: hand the slot back
+    // the codes of this step have been read: hand the slot back
+    ptx::fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->empty[slot]));
   }

@@ -347,8 +347,9 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
         dq::unit32_natural<BITS, true>(wa, z[0], sc[0], oa);
         dq::unit32_natural<BITS, true>(wb, z[1], sc[1], ob);
       }
+      fence_proxy_async_smem();                                   // the codes have been read
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // codes consumed: slot free
+      if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // slot free
       if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ((it / XSTAGES) & 1u) ^ 1u, abort_flag)) break;
       uint8_t* wbuf = base + s * XSTAGE_BYTES + XA_BYTES;
 #pragma unroll

@@ -462,8 +462,9 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         dq::unit32_natural<BITS, FOLD>(w[0], z[0], sc[0], o0);
         dq::unit32_natural<BITS, FOLD>(w[1], z[1], sc[1], o1);
       }
+      fence_proxy_async_smem();                                   // the codes have been read
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // codes consumed: slot free
+      if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // slot free
       if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ((it / PSTAGES) & 1u) ^ 1u, abort_flag)) break;
       uint8_t* wrow = base + s * PSTAGE_BYTES + PA_BYTES + row * 128;
 #pragma unroll

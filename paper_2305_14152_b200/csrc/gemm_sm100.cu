@@ -421,7 +421,8 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
 #pragma unroll
       for (int k = 0; k < UPT; ++k) dequant_unit<BITS, FOLD>(cur[k], p.zeros_f != nullptr, o[k]);
       if (PKTMA) {
-        // every lane has consumed its codes by now: hand the slot back
+        // every lane has read its codes by then: hand the slot back
+        fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars->empty_pk[it % PK_SLOTS]));
       }
@@ -799,10 +800,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         store_pieces(p.out_z + e0, n_pieces, vec, rz);
       }
       tc_fence_before();
+      if (PKTMA) fence_proxy_async_smem();           // the codes have been read: their slot goes back
       __syncwarp();
-      // The code slot goes back only here, after results made from its words have been stored: an
-      // arrive right behind the reads overtook them when the load unit was busy, and the refill
-      // was read in their place.
       if (PKTMA && lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[local & 1]));
       if (lane == 0) mbar_arrive_cluster(buf ? acc_empty_leader1 : acc_empty_leader0);
     }

@@ -79,8 +79,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
   }
 }
 
-// Generic-proxy writes to shared memory -> visible to the async proxy (TMA,
-// tensor core operand reads).
+// Orders this thread's earlier accesses to shared memory (generic proxy) before later ones of the
+// async proxy: its writes are then visible to TMA and to the tensor cores' operand reads, and its
+// reads are done when a copy refills what was read.  An mbarrier orders threads, not proxies, so a
+// buffer that threads read and a copy writes again is handed back as
+//   reads; fence_proxy_async_smem(); __syncwarp(); one lane arrives (or issues the copy).
+// Without the fence an arrive right behind the reads was overtaken by the refill (dS kernel, when
+// the load unit was busy).
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

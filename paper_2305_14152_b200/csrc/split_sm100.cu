@@ -340,12 +340,10 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           *reinterpret_cast<uint4*>(row_ptr + (((chunk0 + c) ^ swz) << 4)) =
               make_uint4(o[k][4 * c], o[k][4 * c + 1], o[k][4 * c + 2], o[k][4 * c + 3]);
       }
-      fence_proxy_async_smem();
+      fence_proxy_async_smem();       // the weights are written, the codes have been read
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(smem_u32(&bars->full[s]));
-        // behind the stores of what was made from the codes: an arrive right behind the reads can
-        // overtake them when the load unit is busy, and the refill is read in their place
         mbar_arrive(smem_u32(&bars->empty_pk[pq]));
       }
       return true;
