@@ -1121,13 +1121,20 @@ extern "C" int peqa_qlinear_decode_prepared(const peqa_qweight_t* w, const uint3
   if (!aligned16(prepared) || !aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
   PrepPlan plan;
-  PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan));
-  PrepPlan half = plan;
-  if (M > 8) PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, &half));
-  if (M > 8 && (task_ids || 2 * half.ns < plan.ns)) {
+  bool two = false;
+  if (M > 8) {
+    PrepPlan half;
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, &half));
+    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan) != PEQA_OK ||
+          2 * half.ns < plan.ns;
+  } else {
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan));
+  }
+  if (two) {
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
-    // table per task (the scales of four tokens per lane do not fit in registers), and where
-    // sixteen tokens would be worked through in more chunks or waves.
+    // table per task (the scales of four tokens per lane do not fit in registers), where all tokens
+    // at once would be worked through in more chunks or waves, and where their parked sums leave no
+    // room in shared memory (from about 42000 rows on for 16 tokens, 68000 for 12, 113000 for 9).
     const int h = (M + 1) / 2;
     const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
     PEQA_TRY(peqa_qlinear_decode_prepared(w, prepared, X, h, Y, scale_table, n_tasks, task_ids, stream));
