@@ -256,10 +256,10 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     adam.v = L->v;
     const int slots = fwd_ds_slots(&L->w, g[i], T, L->workspace_bytes);
     if (slots > 0) {
-      // dX first: it reads the scales that the step at the end of launch_fwd_ds rewrites
-      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));
-      PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, L->dS, apply_adamw ? &adam : nullptr,
-                             static_cast<float*>(L->workspace), slots, st));
+      float* ds_part = static_cast<float*>(L->workspace);
+      PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));   // before the scales change
+      PEQA_TRY(launch_ds_channel(&L->w, ds_part, slots, L->dS, apply_adamw ? &adam : nullptr, st));
       continue;
     }
     PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st));

@@ -169,13 +169,16 @@ __device__ __forceinline__ void pair_item(const PairItems& it, int item, int T, 
 // zeros_f != nullptr: real-valued zero-points [N, G] (App. K) replace w->zeros
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
                cudaStream_t st);
-// Forward and, from its fp32 sums, the scale gradient of a layer with one scale per channel (and the
-// AdamW step).  fwd_ds_slots: rows of N floats of scratch it needs, 0 when the layer or call is not
+// Forward and, from its fp32 sums, the scale gradient of a layer with one scale per channel in two
+// launches: the forward leaves partial sums per channel, launch_ds_channel adds them (and makes the
+// AdamW step).  fwd_ds_slots: rows of N floats of scratch that takes, 0 when the layer or call is not
 // served this way.
 int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes);
 struct DsAdam;
-int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* dS,
-                  const DsAdam* adam, float* workspace, int slots, cudaStream_t st);
+int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
+                  cudaStream_t st);
+int launch_ds_channel(const peqa_qweight_t* w, const float* ds_part, int slots, float* dS, const DsAdam* adam,
+                      cudaStream_t st);
 bool fwd_pair_supported(const peqa_qweight_t* w);
 // ds_part != nullptr (one scale per channel): sums of dY * u per channel, see fwd_pair_sm100.cu
 int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T,

@@ -1028,13 +1028,17 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes) 
   return (size_t)slots * w->out_features * sizeof(float) <= workspace_bytes ? slots : 0;
 }
 
-int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* dS,
-                  const DsAdam* adam, float* workspace, int slots, cudaStream_t st) {
+int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
+                  cudaStream_t st) {
   const int g = w->in_features;
-  if (split_is_faster(w, T, false)) PEQA_TRY(launch_split(w, nullptr, g, X, T, Y, false, dY, workspace, st));
-  else PEQA_TRY(launch_fwd_pair(w, nullptr, g, X, T, Y, dY, workspace, st));
+  if (split_is_faster(w, T, false)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st);
+  return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st);
+}
+
+int launch_ds_channel(const peqa_qweight_t* w, const float* ds_part, int slots, float* dS, const DsAdam* adam,
+                      cudaStream_t st) {
   ds_channel_kernel<<<(w->out_features + 31) / 32, dim3(32, 8), 0, st>>>(
-      workspace, dS, w->out_features, slots, adam ? adam->c : AdamWConsts{}, adam ? adam->scales : nullptr,
+      ds_part, dS, w->out_features, slots, adam ? adam->c : AdamWConsts{}, adam ? adam->scales : nullptr,
       adam ? adam->m : nullptr, adam ? adam->v : nullptr);
   PEQA_CUDA(cudaGetLastError());
   return PEQA_OK;

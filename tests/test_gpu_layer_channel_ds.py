@@ -54,3 +54,30 @@ def test_channel_ds_from_the_forward(N, K, bits, T):
         assert torch.equal(L.dS, out[0].dS) and torch.equal(L.Y, out[0].Y) and torch.equal(L.dX, out[0].dX)
     single = binding.qlinear_bwd(to_qweight(packed, zeros, scales, bits, 0, K), X, dY, need_dx=False)[1]
     assert torch.allclose(single, out[0].dS, rtol=1e-3, atol=1e-4 * float(single.abs().mean()))
+
+
+def _linear(N, K, T, bits):
+    d = synth.custom(N + T, N, K, T, bits, 0, outliers=True, sigma_dy=1e-2)
+    codes, zeros, scales, packed = oracle_layer(d, bits, 0)
+    qw = to_qweight(packed, zeros, scales, bits, 0, K)
+    L = binding.LayerLinear(w=qw, X=bf16_to_dev(d["X"]), dY=bf16_to_dev(d["dY"]),
+                            Y=torch.empty((T, N), dtype=torch.bfloat16, device="cuda"),
+                            dX=torch.empty((T, K), dtype=torch.bfloat16, device="cuda"),
+                            dS=torch.full((N, 1), 9.0, device="cuda"), m=torch.zeros((N, 1), device="cuda"),
+                            v=torch.zeros((N, 1), device="cuda"))
+    return d, packed, zeros, L
+
+
+# through the cluster-split forward and through the CTA-pair forward
+@pytest.mark.parametrize("T", [96, 2048])
+def test_y_and_dx_may_share_a_buffer(T):
+    """The forward is enqueued before dX: a caller that wants no Y may give both the same scratch."""
+    N = K = 2048
+    _, _, _, L = _linear(N, K, T, 4)
+    L.workspace = binding.alloc_workspace(binding.OP_BWD, T, L.w)
+    binding.layer_train_step([L], LR, step=1, apply_adamw=False)
+    dX, dS = L.dX, L.dS.clone()
+    L.Y = L.dX = torch.empty_like(dX)
+    binding.layer_train_step([L], LR, step=1, apply_adamw=True)
+    binding.check_status()
+    assert torch.equal(L.dX, dX) and torch.equal(L.dS, dS)
