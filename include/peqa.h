@@ -186,9 +186,13 @@ int peqa_qlinear_bwd_ds_adamw(const peqa_qweight_t* w, const void* X_bf16, const
  *   since their kernels run in stream order.
  * 1 <= n_linears <= PEQA_LAYER_MAX_LINEARS.  Shape rules and return codes as for
  * the single calls; nothing is enqueued when a check fails.
- * A large linear with one scale per channel (T*N*K >= 2^28) takes its dS from the
- * forward's fp32 sums, dS[i] = sum_t dY[t,i] * sum_j X[t,j] (Q[i,j] - z[i]), instead of
- * contracting dY^T X: the same sum in another order, closer to the exact one.
+ * A large linear with one scale per channel takes its dS from the forward's fp32
+ * sums, dS[i] = sum_t dY[t,i] * sum_j X[t,j] (Q[i,j] - z[i]), instead of contracting
+ * dY^T X: the same sum in another order, closer to the exact one.  Large means
+ * T*N*K >= 2^28; and the partial sums, one row of N floats per 128 tokens, have to fit
+ * the workspace of the size above, which holds K / 128 rows: T <= K, or a little less
+ * where T is not a multiple of 256.  Which way is taken depends on the shape and T
+ * alone, not on the workspace given.
  */
 #define PEQA_LAYER_MAX_LINEARS 16
 typedef struct {

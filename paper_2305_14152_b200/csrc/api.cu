@@ -254,7 +254,7 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     adam.scales = const_cast<float*>(L->w.scales);
     adam.m = L->m;
     adam.v = L->v;
-    const int slots = fwd_ds_slots(&L->w, g[i], T, L->workspace_bytes);
+    const int slots = fwd_ds_slots(&L->w, g[i], T);
     if (slots > 0) {
       float* ds_part = static_cast<float*>(L->workspace);
       PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));

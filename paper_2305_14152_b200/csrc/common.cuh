@@ -171,9 +171,9 @@ int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void*
                cudaStream_t st);
 // Forward and, from its fp32 sums, the scale gradient of a layer with one scale per channel in two
 // launches: the forward leaves partial sums per channel, launch_ds_channel adds them (and makes the
-// AdamW step).  fwd_ds_slots: rows of N floats of scratch that takes, 0 when the layer or call is not
-// served this way.
-int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes);
+// AdamW step).  fwd_ds_slots: rows of N floats that takes, at most ds_workspace_bytes; 0 when the
+// layer or T is not served this way.
+int fwd_ds_slots(const peqa_qweight_t* w, int g, int T);
 struct DsAdam;
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
                   cudaStream_t st);

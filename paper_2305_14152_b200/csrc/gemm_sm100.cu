@@ -1015,7 +1015,7 @@ int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }
 
-int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes) {
+int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
   if (g != w->in_features || !fwd_pair_supported(w)) return 0;
   // dS = sum_t dY * u from the forward's fp32 sums instead of a contraction of its own (training
   // step of one linear, before -> after in us, and error of dS against binary64): 11008 x 4096 at
@@ -1025,7 +1025,10 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T, size_t workspace_bytes) 
   // differs from this one in its last bits.
   if ((double)T * w->out_features * w->in_features < (double)(1 << 28)) return 0;
   const int slots = split_is_faster(w, T, false) ? split_ds_slots(w, T) : 2 * ((T + 255) / 256);
-  return (size_t)slots * w->out_features * sizeof(float) <= workspace_bytes ? slots : 0;
+  // The partial sums go to the workspace the caller was asked for, whose size does not depend on
+  // T (about T <= K fits).  Held against that size and not against the one that was given, so that
+  // the bits of dS depend on the shape and T alone and a pointer that is not needed is not used.
+  return (size_t)slots * w->out_features * sizeof(float) <= ds_workspace_bytes(w, g, T) ? slots : 0;
 }
 
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,

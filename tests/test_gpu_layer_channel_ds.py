@@ -81,3 +81,33 @@ def test_y_and_dx_may_share_a_buffer(T):
     binding.layer_train_step([L], LR, step=1, apply_adamw=True)
     binding.check_status()
     assert torch.equal(L.dX, dX) and torch.equal(L.dS, dS)
+
+
+@pytest.mark.parametrize("N,K,T", [(1024, 1024, 4096), (4104, 512, 1030), (2048, 2048, 2048)])
+def test_surplus_workspace_changes_no_bit(N, K, T):
+    # more tokens than columns in the first two: partial sums of the forward would only fit the larger one
+    d, packed, zeros, L = _linear(N, K, T, 4)
+    exact = binding.alloc_workspace(binding.OP_BWD, T, L.w)
+    out = []
+    for workspace in (exact, torch.empty(16 * exact.numel(), dtype=torch.uint8, device="cuda")):
+        L.workspace = workspace
+        binding.layer_train_step([L], LR, step=1, apply_adamw=False)
+        binding.check_status()
+        out.append(L.dS.clone())
+    assert torch.equal(out[0], out[1])
+    rows = np.arange(0, N, 131)
+    assert_close(out[0].cpu().numpy()[rows].astype(np.float64),
+                 oracle.bwd_ds(d["X"], d["dY"], packed, zeros, 4, 0, rows=rows), "dS")
+
+
+def test_a_workspace_that_is_not_needed_is_not_touched():
+    # one group of 128 columns is one piece: no scratch is asked for, so any pointer may be given
+    N, K, T = 2048, 128, 1024
+    d, packed, zeros, L = _linear(N, K, T, 4)
+    assert binding.workspace_bytes(binding.OP_BWD, T, L.w) == 0
+    scratch = torch.full((16 * N * 4 + 256,), 77, dtype=torch.uint8, device="cuda")
+    L.workspace = scratch[4:]
+    binding.layer_train_step([L], LR, step=1, apply_adamw=False)
+    binding.check_status()
+    assert torch.all(scratch == 77)
+    assert_close(L.dS.cpu().numpy().astype(np.float64), oracle.bwd_ds(d["X"], d["dY"], packed, zeros, 4, 0), "dS")
