@@ -73,3 +73,26 @@ def test_status_words_are_per_stream():
         binding.check_status()
     ref = oracle.fwd(d["X"], packed, zeros, scales, 4, 0)
     assert_close(dev_to_f64(Y), ref, "forward on the stream that had timed out")
+
+
+# few tokens go to the cluster-split forward, many to the CTA-pair forward
+@pytest.mark.parametrize("T", [64, 4096])
+def test_both_forwards_time_out(T):
+    d = synth.custom(5, 2560, 256, T, 4, 64)
+    codes, zeros, scales, packed = oracle_layer(d, 4, 64)
+    qw = to_qweight(packed, zeros, scales, 4, 64, 256)
+    X = bf16_to_dev(d["X"])
+    Y = binding.qlinear_fwd(qw, X)
+    binding.selftest_configure(wait_limit_us=1000, starve_forward=True)
+    try:
+        binding.qlinear_fwd(qw, X)
+        with pytest.raises(binding.PeqaError) as err:
+            binding.check_status()
+        assert err.value.status == -8                 # PEQA_ERR_DEVICE_TIMEOUT
+    finally:
+        binding.selftest_configure()
+    again = binding.qlinear_fwd(qw, X)
+    binding.check_status()
+    assert torch.equal(Y, again)
+    toks = np.array([0, T // 2, T - 1])
+    assert_close(dev_to_f64(Y)[toks], oracle.fwd(d["X"], packed, zeros, scales, 4, 64, tokens=toks), "Y")

@@ -42,6 +42,7 @@ def test_channel_ds_from_the_forward(N, K, bits, T):
         # both are binary32 sums of the same products: far closer than the bound for bf16 results
         assert np.linalg.norm(ds[rows] - ref) <= 2e-6 * np.linalg.norm(ref)
         assert_close(dev_to_f64(L.Y)[toks], oracle.fwd(d["X"], packed, zeros, scales, bits, 0, tokens=toks), "Y")
+        assert_close(dev_to_f64(L.dX)[toks], oracle.bwd_dx(d["dY"], packed, zeros, scales, K, bits, 0, tokens=toks), "dX")
         if apply:
             zero = np.zeros_like(scales)
             s_ref, _, _ = oracle.adamw(scales, ds, zero, zero, LR, float(np.float32(0.9)), float(np.float32(0.999)),
