@@ -46,11 +46,9 @@ constexpr int UMMA_K = 16;   // contraction elements per tcgen05.mma
 constexpr int STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;   // 16 KiB
 constexpr int B_BYTES = BN * BK * 2;   // 32 KiB
-constexpr int PK_BYTES = 4096;         // packed codes of one stage (qgemm)
-constexpr int PK_SLOTS = 8;            // their own, deeper ring: the codes run ahead of the operands
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int TMEM_COLS = 512;         // two fp32 accumulators of 256 columns
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + PK_SLOTS * PK_BYTES + 1024 /*align*/ + 512 /*barriers*/;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 512 /*barriers*/;
 
 constexpr int kQgemmThreads = 512;     // warps: 0 TMA, 1 MMA, 2 TMEM alloc, 4-7 epilogue, 8-15 dequant
 constexpr int kDequantThreads = 256;
@@ -60,8 +58,6 @@ constexpr int kDsThreads = 384;        // warps: 0 TMA, 1 MMA, 2 TMEM alloc, 4-1
 struct Barriers {
   uint64_t full_a[STAGES];   // dequantised weight tile written (qgemm only)
   uint64_t full_b[STAGES];   // TMA bytes landed
-  uint64_t full_pk[PK_SLOTS];   // packed codes landed (qgemm with TMA-staged codes)
-  uint64_t empty_pk[PK_SLOTS];  // all dequant warps have read the slot
   uint64_t empty[STAGES];    // MMAs that read the stage have completed
   uint64_t acc_full[2];      // accumulator ready for the epilogue
   uint64_t acc_empty[2];     // accumulator drained by the epilogue
@@ -73,7 +69,6 @@ struct Barriers {
 struct SmemView {
   uint8_t* a[STAGES];
   uint8_t* b[STAGES];
-  uint8_t* pk[PK_SLOTS];
   Barriers* bars;
 };
 
@@ -86,9 +81,7 @@ __device__ __forceinline__ SmemView carve_smem(uint8_t* raw) {
     v.a[s] = base + s * STAGE_BYTES;
     v.b[s] = base + s * STAGE_BYTES + A_BYTES;
   }
-#pragma unroll
-  for (int q = 0; q < PK_SLOTS; ++q) v.pk[q] = base + STAGES * STAGE_BYTES + q * PK_BYTES;
-  v.bars = reinterpret_cast<Barriers*>(base + STAGES * STAGE_BYTES + PK_SLOTS * PK_BYTES);
+  v.bars = reinterpret_cast<Barriers*>(base + STAGES * STAGE_BYTES);
   return v;
 }
 
@@ -126,23 +119,16 @@ __device__ __forceinline__ int group_of(const QGemmParams& p, int col) {
   return p.g_shift >= 0 ? (col >> p.g_shift) : (col / p.g);
 }
 
-// Weight row i, columns [col0, col0 + 32): zero-point and scale, plus the packed
-// words when WORDS is set (otherwise the caller takes them from shared memory).
-template <int BITS, bool WORDS = true>
+// Weight row i, columns [col0, col0 + 32): packed words, zero-point and scale.
+template <int BITS>
 __device__ __forceinline__ Unit<BITS> load_unit(const QGemmParams& p, int i, int col0) {
   Unit<BITS> u;
 #pragma unroll
   for (int q = 0; q < BITS; ++q) u.w[q] = 0u;
   if (i < p.N && col0 < p.K) {
-    if (WORDS) {
-      const uint32_t* src = p.qw + (size_t)i * p.wpr + (col0 >> 5) * BITS;
-      if constexpr (BITS == 4) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(src));
-        u.w[0] = v.x; u.w[1] = v.y; u.w[2] = v.z; u.w[3] = v.w;
-      } else {
-        u.w[0] = __ldg(src); u.w[1] = __ldg(src + 1); u.w[2] = __ldg(src + 2);
-      }
-    }
+    const uint32_t* src = p.qw + (size_t)i * p.wpr + (col0 >> 5) * BITS;
+#pragma unroll
+    for (int q = 0; q < BITS; ++q) u.w[q] = __ldg(src + q);
     const size_t gidx = (size_t)i * p.G + group_of(p, col0);
     u.s = __ldg(p.scales + gidx);
     u.c = 0.0f;
@@ -170,13 +156,11 @@ __device__ __forceinline__ void dequant_unit(const Unit<BITS>& u, bool zf, uint3
   else dq::unit32_natural<BITS, FOLD>(u.w, u.z, u.s, o);
 }
 
-// PKTMA: the packed codes of a stage arrive by TMA in shared memory (needs a
-// 16-byte row pitch of the packed matrix); otherwise the dequant threads read
-// them from global memory themselves.
-template <int BITS, bool TRANS, bool FOLD, bool PKTMA>
+// The fallback for packed rows whose pitch is not a multiple of 16 bytes (3-bit, K % 128 == 64): TMA
+// cannot fetch their codes, so the dequant threads read them from global memory.
+template <int BITS, bool TRANS, bool FOLD>
 __global__ void __launch_bounds__(kQgemmThreads, 1)
-qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
-             const __grid_constant__ CUtensorMap tmap_pk, const QGemmParams p) {
+qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   SmemView sm = carve_smem(smem_raw);
   Barriers* bars = sm.bars;
@@ -189,10 +173,6 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
       mbar_init(smem_u32(&bars->full_b[s]), 1);
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
-    for (int q = 0; q < PK_SLOTS; ++q) {
-      mbar_init(smem_u32(&bars->full_pk[q]), 1);
-      mbar_init(smem_u32(&bars->empty_pk[q]), (kDequantThreads / 32) / DQ_GROUPS);   // the warps of one group
-    }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&bars->acc_full[b]), 1);
       mbar_init(smem_u32(&bars->acc_empty[b]), 128);
@@ -201,7 +181,6 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
     bars->wait_limit_us = p.status[4];
     fence_mbar_init();
     prefetch_tmap(&tmap_act);
-    if (PKTMA) prefetch_tmap(&tmap_pk);
   }
   if (warp == 2) {
     tmem_alloc(smem_u32(&bars->tmem_base), TMEM_COLS);
@@ -228,32 +207,6 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
           const uint32_t bar = smem_u32(&bars->full_b[s]);
           mbar_arrive_expect_tx(bar, B_BYTES);
           tma_load_2d(smem_u32(sm.b[s]), &tmap_act, bar, kb * BK, t0);
-        }
-      }
-    }
-  } else if (warp == 3) {
-    // ------------------------------------------ packed-code TMA producer (one lane)
-    // forward: a box is 128 rows x 8 words holding the stage's 64 columns (3-bit: on odd
-    // k-blocks the 6 words start 2 words into the box, which keeps the box start
-    // 16-byte aligned); dX: 64 rows x the tile's 128 columns.
-    if (PKTMA && lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
-        const int w0 = (tile % p.r_tiles) * BM;   // first weight row (forward) / column (dX)
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int q = it % PK_SLOTS;
-          const uint32_t ph = (it / PK_SLOTS) & 1u;
-          if (!mbar_wait(smem_u32(&bars->empty_pk[q]), ph ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t pbar = smem_u32(&bars->full_pk[q]);
-          if (!TRANS) {
-            mbar_arrive_expect_tx(pbar, 128 * 32);
-            tma_load_2d(smem_u32(sm.pk[q]), &tmap_pk, pbar,
-                        BITS == 3 ? 6 * kb - 2 * (kb & 1) : 8 * kb, w0);
-          } else {
-            mbar_arrive_expect_tx(pbar, 64 * 16 * BITS);
-            tma_load_2d(smem_u32(sm.pk[q]), &tmap_pk, pbar, (w0 >> 5) * BITS, kb * BK);
-          }
         }
       }
     }
@@ -365,8 +318,8 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
     auto load_next = [&](Unit<BITS> (&u)[UPT]) {
 #pragma unroll
       for (int k = 0; k < UPT; ++k) {
-        if constexpr (!TRANS) u[k] = load_unit<BITS, !PKTMA>(p, pf_w0 + rowl[k], pf_kb * BK + col_off[k]);
-        else u[k] = load_unit<BITS, !PKTMA>(p, pf_kb * BK + rowl[k], pf_w0 + col_off[k]);
+        if constexpr (!TRANS) u[k] = load_unit<BITS>(p, pf_w0 + rowl[k], pf_kb * BK + col_off[k]);
+        else u[k] = load_unit<BITS>(p, pf_kb * BK + rowl[k], pf_w0 + col_off[k]);
       }
       pf_kb += DQ_GROUPS;
       while (pf_kb >= p.k_blocks) {
@@ -376,56 +329,14 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
       }
     };
     Unit<BITS> cur[UPT], nxt[UPT];
-    int cur_kb = pf_kb;                      // k-block of the stage about to be processed
     if ((uint32_t)grp < total_it) load_next(cur);
     for (uint32_t it = grp; it < total_it; it += DQ_GROUPS) {
-      const int next_kb = pf_kb;
       if (it + DQ_GROUPS < total_it) load_next(nxt);
       const int s = it % STAGES;
       const uint32_t ph = (it / STAGES) & 1u;
-      if (PKTMA) {
-        const int pq = it % PK_SLOTS;
-        if (!mbar_wait(smem_u32(&bars->full_pk[pq]), (it / PK_SLOTS) & 1u, abort_flag)) break;
-        const uint32_t* src = reinterpret_cast<const uint32_t*>(sm.pk[pq]);
-        if constexpr (!TRANS) {
-          // a row of the slot is 32 bytes: read it whole with two 16-byte loads (consecutive
-          // lanes are consecutive rows, so narrower loads would pile onto four banks) and
-          // pick this stage's words: 4-bit uses all eight, 3-bit six starting at word 0 or 2
-#pragma unroll
-          for (int k = 0; k < UPT; k += 2) {
-            const uint4 lo = *reinterpret_cast<const uint4*>(src + rowl[k] * 8);
-            const uint4 hi = *reinterpret_cast<const uint4*>(src + rowl[k] * 8 + 4);
-            const uint32_t w8[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-            if constexpr (BITS == 4) {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) { cur[k].w[e] = w8[e]; cur[k + 1].w[e] = w8[4 + e]; }
-            } else {
-              const bool odd = (cur_kb & 1) != 0;
-#pragma unroll
-              for (int e = 0; e < 3; ++e) {
-                cur[k].w[e] = odd ? w8[2 + e] : w8[e];
-                cur[k + 1].w[e] = odd ? w8[5 + e] : w8[3 + e];
-              }
-            }
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < UPT; ++k) {
-            const uint32_t* r = src + rowl[k] * (4 * BITS) + u4 * BITS;
-#pragma unroll
-            for (int e = 0; e < BITS; ++e) cur[k].w[e] = r[e];
-          }
-        }
-      }
       uint32_t o[UPT][16];
 #pragma unroll
       for (int k = 0; k < UPT; ++k) dequant_unit<BITS, FOLD>(cur[k], p.zeros_f != nullptr, o[k]);
-      if (PKTMA) {
-        // every lane has read its codes by then: hand the slot back
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars->empty_pk[it % PK_SLOTS]));
-      }
       if (!mbar_wait(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) break;
 #pragma unroll
       for (int k = 0; k < UPT; ++k) {
@@ -439,7 +350,6 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act,
       mbar_arrive(smem_u32(&bars->full_a[s]));
 #pragma unroll
       for (int k = 0; k < UPT; ++k) cur[k] = nxt[k];
-      cur_kb = next_kb;
     }
   }
 
@@ -920,22 +830,14 @@ int sm_count(int* n) {
   return PEQA_OK;
 }
 
-template <int BITS, bool TRANS, bool FOLD, bool PKTMA>
-int launch_qgemm_k(const CUtensorMap& tmap, const CUtensorMap& tmap_pk, const QGemmParams& p,
-                   int grid, cudaStream_t st) {
-  auto kern = qgemm_kernel<BITS, TRANS, FOLD, PKTMA>;
+template <int BITS, bool TRANS, bool FOLD>
+int launch_qgemm_t(const CUtensorMap& tmap, const QGemmParams& p, int grid, cudaStream_t st) {
+  auto kern = qgemm_kernel<BITS, TRANS, FOLD>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, SMEM_BYTES, done));
-  kern<<<grid, kQgemmThreads, SMEM_BYTES, st>>>(tmap, tmap_pk, p);
+  kern<<<grid, kQgemmThreads, SMEM_BYTES, st>>>(tmap, p);
   PEQA_CUDA(cudaGetLastError());
   return PEQA_OK;
-}
-
-template <int BITS, bool TRANS, bool FOLD>
-int launch_qgemm_t(const CUtensorMap& tmap, const CUtensorMap& tmap_pk, bool pktma,
-                   const QGemmParams& p, int grid, cudaStream_t st) {
-  return pktma ? launch_qgemm_k<BITS, TRANS, FOLD, true>(tmap, tmap_pk, p, grid, st)
-               : launch_qgemm_k<BITS, TRANS, FOLD, false>(tmap, tmap_pk, p, grid, st);
 }
 
 int launch_qgemm(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T,
@@ -968,29 +870,10 @@ int launch_qgemm(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
   const int tiles = p.r_tiles * p.t_tiles;
   const int grid = tiles < sms ? tiles : sms;
   const bool fold = trans || p.G > 1 || zeros_f != nullptr;
-  // Packed codes by TMA need a 16-byte row pitch: always true for 4-bit, K % 128 == 0 for 3-bit.
-  const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;
-  CUtensorMap tmap_pk = tmap;
-  if (pktma) {
-    EncodeTiledFn enc = nullptr;
-    PEQA_TRY(tensor_map_encoder(&enc));
-    cuuint64_t dims[2] = {(cuuint64_t)p.wpr, (cuuint64_t)p.N};
-    cuuint64_t strides[1] = {(cuuint64_t)p.wpr * 4};
-    cuuint32_t box[2] = {trans ? (cuuint32_t)(4 * w->bits) : 8u, trans ? 64u : 128u};
-    cuuint32_t estr[2] = {1, 1};
-    if (enc(&tmap_pk, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint32_t*>(w->qweight), dims,
-            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cuda_fail(cudaErrorInvalidValue);
-  }
-  if (w->bits == 4) {
-    if (trans) return launch_qgemm_t<4, true, true>(tmap, tmap_pk, pktma, p, grid, st);
-    return fold ? launch_qgemm_t<4, false, true>(tmap, tmap_pk, pktma, p, grid, st)
-                : launch_qgemm_t<4, false, false>(tmap, tmap_pk, pktma, p, grid, st);
-  }
-  if (trans) return launch_qgemm_t<3, true, true>(tmap, tmap_pk, pktma, p, grid, st);
-  return fold ? launch_qgemm_t<3, false, true>(tmap, tmap_pk, pktma, p, grid, st)
-              : launch_qgemm_t<3, false, false>(tmap, tmap_pk, pktma, p, grid, st);
+  // only 3-bit rows have such a pitch: K is a multiple of 64
+  if (trans) return launch_qgemm_t<3, true, true>(tmap, p, grid, st);
+  return fold ? launch_qgemm_t<3, false, true>(tmap, p, grid, st)
+              : launch_qgemm_t<3, false, false>(tmap, p, grid, st);
 }
 
 int gcd_int(int a, int b) { return b == 0 ? a : gcd_int(b, a % b); }
