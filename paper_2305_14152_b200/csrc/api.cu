@@ -168,7 +168,7 @@ extern "C" int peqa_qlinear_fwd(const peqa_qweight_t* w, const void* X, int T, v
   PEQA_TRY(check_gemm_shape(w, T));
   if (!aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  return launch_fwd(w, nullptr, g, X, T, Y, as_stream(stream));
+  return launch_fwd(w, nullptr, g, X, T, Y, as_stream(stream), T);
 }
 
 extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const void* dY, int T,
@@ -189,7 +189,7 @@ extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const vo
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream)));
+  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T));
   if (dS) PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream)));
   return PEQA_OK;
 }
@@ -258,12 +258,12 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     if (slots > 0) {
       float* ds_part = static_cast<float*>(L->workspace);
       PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));
-      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));   // before the scales change
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T));   // before the scales change
       PEQA_TRY(launch_ds_channel(&L->w, ds_part, slots, L->dS, apply_adamw ? &adam : nullptr, st));
       continue;
     }
-    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st));
-    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st));
+    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T));
+    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T));
     PEQA_TRY(launch_ds(&L->w, nullptr, g[i], L->X_bf16, L->dY_bf16, T, L->dS, nullptr, apply_adamw ? &adam : nullptr,
                        L->workspace, L->workspace_bytes, st));
   }
@@ -311,7 +311,7 @@ extern "C" int peqa_qlinear_fwd_zf(const peqa_qweight_t* w, const float* zeros_f
   PEQA_TRY(check_gemm_shape(w, T));
   if (!aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  return launch_fwd(w, zeros_f, g, X, T, Y, as_stream(stream));
+  return launch_fwd(w, zeros_f, g, X, T, Y, as_stream(stream), T);
 }
 
 extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f, const void* X,
@@ -334,7 +334,7 @@ extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream)));
+  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T));
   if (dS) PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream)));
   return PEQA_OK;
 }
@@ -440,8 +440,8 @@ int drain_and_fail(HostPipe* hp, cudaStream_t st, int rc) {
 // way to the device (auxiliary stream `in`) while chunk c runs forward and dX on the
 // caller's stream and chunk c-1 returns Y and dX (auxiliary stream `out`); PCIe carries both
 // directions at once.  dS sums over all tokens, so it runs once after the last chunk, then
-// AdamW.  Forward and dX treat tokens independently; chunking them changes at most the order in
-// which a contraction is summed.  With several linears the copies in of the next linear run while the
+// AdamW.  Forward and dX treat tokens independently and a chunk takes the route of the whole call, so
+// chunking does not change a bit of their results.  With several linears the copies in of the next linear run while the
 // kernels of the current one are still busy.
 
 // Host-side checks of one linear of a host-buffer step; nothing is enqueued.
@@ -471,12 +471,14 @@ int enqueue_host_linear(HostPipe* hp, cudaStream_t st, const peqa_layer_host_lin
                         int64_t step) {
   const peqa_qweight_t* w = &L.w;
   const size_t N = w->out_features, K = w->in_features;
-  const size_t G = w->group_size == 0 ? 1 : K / (size_t)w->group_size;
+  const int g = effective_group(w->in_features, w->group_size);
+  const size_t G = K / (size_t)g;
   // chunks of 256 tokens or more, at most kHostChunksMax: short chunks shorten the time before
   // the first kernel can start and after the last one has ended, which is all copy time
   int chunks = (T + 255) / 256;
   if (chunks > kHostChunksMax) chunks = kHostChunksMax;
-  const int per = ((T + chunks - 1) / chunks + 7) & ~7;   // rows per chunk, 16-byte aligned slices
+  const int unit = part_tokens(w, T);
+  const int per = ((T + chunks - 1) / chunks + unit - 1) / unit * unit;   // rows per chunk
   chunks = (T + per - 1) / per;
   const char* hX = static_cast<const char*>(L.h_X);
   const char* hdY = static_cast<const char*>(L.h_dY);
@@ -496,12 +498,10 @@ int enqueue_host_linear(HostPipe* hp, cudaStream_t st, const peqa_layer_host_lin
     PEQA_CUDA(cudaEventRecord(hp->dy_landed[c], hp->in));
     // the forward needs only X: it runs while dY is still on its way
     PEQA_CUDA(cudaStreamWaitEvent(st, hp->x_landed[c], 0));
-    PEQA_TRY(peqa_qlinear_fwd(w, dX_in + t0 * K * 2, (int)tc, dY_out + t0 * N * 2, L.workspace,
-                              L.workspace_bytes, stream));
+    PEQA_TRY(launch_fwd(w, nullptr, g, dX_in + t0 * K * 2, (int)tc, dY_out + t0 * N * 2, st, T));
     PEQA_CUDA(cudaEventRecord(hp->fwd_done[c], st));
     PEQA_CUDA(cudaStreamWaitEvent(st, hp->dy_landed[c], 0));
-    PEQA_TRY(peqa_qlinear_bwd(w, nullptr, ddY + t0 * N * 2, (int)tc, ddX + t0 * K * 2, nullptr,
-                              L.workspace, L.workspace_bytes, stream));
+    PEQA_TRY(launch_dx(w, nullptr, g, ddY + t0 * N * 2, (int)tc, ddX + t0 * K * 2, st, T));
     PEQA_CUDA(cudaEventRecord(hp->dx_done[c], st));
     // Y goes back while dX is still being computed
     PEQA_CUDA(cudaStreamWaitEvent(hp->out, hp->fwd_done[c], 0));

@@ -477,7 +477,7 @@ int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
   // 22016 x 8192 in groups of 128 at 11 tokens 107 / 80, 4096 x 4096 in groups of 128 at 9 tokens
   // 16 / 12; one scale per channel, 16 tokens: 8192 x 22016 107 / 60, 8192 x 8192 31 / 26, but
   // 22016 x 8192 at 9 tokens 56 / 75 -- many rows are this kernel's better side.
-  if (M > 8 && (fold || p.K >= p.N)) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st);
+  if (M > 8 && (fold || p.K >= p.N)) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st, M);
   PEQA_TRY(status_word(st, &p.status));
   // packed matrix as uint32 [N, wpr]; box = 16 words x 128 rows, 64-byte swizzle
   CUtensorMap tmap_q;

@@ -884,16 +884,28 @@ int ds_piece(int g) { return gcd_int(g, 128); }
 
 }  // namespace
 
+int part_tokens(const peqa_qweight_t* w, int T_call) {
+  int unit = 8;     // 16-byte aligned slices
+  for (int trans = 0; trans < 2; ++trans)
+    if (fwd_pair_supported(w) && split_is_faster(w, T_call, trans)) {
+      const int part = split_part_tokens(w, T_call, trans);
+      unit = unit / gcd_int(unit, part) * part;
+    }
+  return unit;
+}
+
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
-               cudaStream_t st) {
-  if (fwd_pair_supported(w) && split_is_faster(w, T, false)) return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st);
+               cudaStream_t st, int T_call) {
+  if (fwd_pair_supported(w) && split_is_faster(w, T_call, false))
+    return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call);
   if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st) {
-  if (dx_pair_supported(w) && split_is_faster(w, T, true)) return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st);
+              cudaStream_t st, int T_call) {
+  if (dx_pair_supported(w) && split_is_faster(w, T_call, true))
+    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call);
   if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }
@@ -917,7 +929,7 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
                   cudaStream_t st) {
   const int g = w->in_features;
-  if (split_is_faster(w, T, false)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st);
+  if (split_is_faster(w, T, false)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T);
   return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st);
 }
 

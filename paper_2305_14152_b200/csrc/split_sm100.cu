@@ -582,8 +582,18 @@ int split_ds_slots(const peqa_qweight_t* w, int T) {
   return plan.t_tiles * ((plan.nt + SM_DUMP_TOK - 1) / SM_DUMP_TOK);
 }
 
+// A part of a call (its tokens from a multiple of this on) gets the clusters it has in the whole call:
+// whole token tiles, and as many as make whole clusters of q tiles.
+int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans) {
+  const int r_tiles = ((trans ? w->in_features : w->out_features) + SM_ROWS - 1) / SM_ROWS;
+  const SplitPlan plan = plan_split(r_tiles, trans ? w->out_features : w->in_features, T_call, sm_count_or(148));
+  int m = 1;
+  while (m * r_tiles % plan.q != 0) ++m;
+  return m * plan.nt;
+}
+
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st) {
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call) {
   SplitParams p;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
@@ -602,11 +612,11 @@ int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
   p.R = trans ? p.K : p.N;
   const int C = trans ? p.N : p.K;
   p.r_tiles = (p.R + SM_ROWS - 1) / SM_ROWS;
-  const SplitPlan plan = plan_split(p.r_tiles, C, T, sm_count_or(148));
+  const SplitPlan plan = plan_split(p.r_tiles, C, T_call, sm_count_or(148));
   p.nt = plan.nt;
   p.q = plan.q;
   p.cshift = plan.cshift;
-  p.tiles = p.r_tiles * plan.t_tiles;
+  p.tiles = p.r_tiles * ((T + plan.nt - 1) / plan.nt);
   p.k_blocks = (C + SM_BK - 1) / SM_BK;
   const int stage_bytes = 2 * (SM_A_BYTES + p.nt * (SM_HALF * 2));
   p.stages = (SM_SMEM_LIMIT - SM_SMEM_FIXED) / stage_bytes;

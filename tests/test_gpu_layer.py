@@ -161,3 +161,29 @@ def test_layer_host_step_rejects_shared_staging_buffers():
     torch.cuda.synchronize()
     for L, b in zip(layers, before):
         assert torch.equal(L.w.scales, b)
+
+
+# whole call / its chunks: CTA-pair kernels / few enough tokens for the cluster-split ones; both cluster-split,
+# with one tile and with three tiles per cluster; a per-channel forward beside a dX
+@pytest.mark.parametrize("N,K,bits,g,T", [(1032, 1088, 4, 32, 2056), (264, 384, 3, 64, 1100), (2056, 1152, 3, 64, 1030),
+                                          (512, 512, 4, 0, 600)])
+def test_host_chunks_take_the_route_of_the_whole_call(N, K, bits, g, T):
+    d = synth.custom(N + T, N, K, T, bits, g, outliers=True, sigma_dy=1e-2)
+    codes, zeros, scales, packed = oracle_layer(d, bits, g)
+
+    def linear():
+        qw = to_qweight(packed, zeros, scales, bits, g, K)
+        return binding.LayerLinear(w=qw, X=bf16_to_dev(d["X"]), dY=bf16_to_dev(d["dY"]),
+                                   Y=torch.empty((T, N), dtype=torch.bfloat16, device="cuda"),
+                                   dX=torch.empty((T, K), dtype=torch.bfloat16, device="cuda"),
+                                   dS=torch.empty_like(qw.scales), m=torch.zeros_like(qw.scales), v=torch.zeros_like(qw.scales),
+                                   workspace=binding.alloc_workspace(binding.OP_BWD, T, qw))
+
+    H, R = _host_linears([linear()], T)[0], linear()
+    binding.layer_train_step_host([H], LR, step=1)
+    binding.layer_train_step([R], LR, step=1)
+    binding.check_status()
+    assert torch.equal(H.h_Y, R.Y.cpu()) and torch.equal(H.h_dX, R.dX.cpu())
+    toks = np.unique(np.concatenate([np.arange(0, T, 61), [T - 1]]))
+    assert_close(H.h_Y.double().numpy()[toks], oracle.fwd(d["X"], packed, zeros, scales, bits, g, tokens=toks), "Y")
+    assert_close(H.h_dX.double().numpy()[toks], oracle.bwd_dx(d["dY"], packed, zeros, scales, K, bits, g, tokens=toks), "dX")
