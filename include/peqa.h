@@ -476,8 +476,8 @@ int peqa_check_status(void* stream);
  * Self-test of the bounded waits (the paper has no counterpart).  Sets, for
  * kernels launched afterwards on the current device, the bound of a single
  * device-side wait to wait_limit_us microseconds (0 restores the default of two
- * seconds) and, when starve_forward is non-zero, makes peqa_qlinear_fwd's
- * CTA-pair kernel announce one byte more than its copies deliver, so that its
+ * seconds) and, when starve_forward is non-zero, makes the kernels of peqa_qlinear_fwd
+ * announce one byte more than their copies deliver, so that the
  * first stage never fills: the kernel must then leave through its time-out path,
  * free its tensor memory and report PEQA_ERR_DEVICE_TIMEOUT through
  * peqa_check_status, leaving the context usable.  Synchronises the device and

@@ -122,8 +122,9 @@ __device__ __forceinline__ void adamw_update(float& s, float gr, float& m, float
 
 // Work items of the CTA-pair kernels (forward, dX).  A tile is 512 tokens x 256 outputs held as
 // two accumulators of 256 tokens.  Tiles are dealt round-robin to the pairs; when the last round
-// would keep at most half of the pairs busy, its tiles are cut into two items of 256 tokens each,
-// so that round takes about half as long.  Items [0, full_items) are whole tiles, the rest are
+// would keep at most half of the pairs busy, its tiles are cut into two items of 256 tokens each.
+// Rebuilding the weights costs the same for one block of tokens as for two, so that round takes 0.8
+// to 0.9 as long (18944 x 8192, one round of 74 tiles: 256 tokens 92 us, 512 tokens 112).  Items [0, full_items) are whole tiles, the rest are
 // halves: item full_items + 2*i + h is half h of tile full_items + i.
 struct PairItems {
   int o_tiles;       // 256-wide tiles along the output dimension
@@ -191,8 +192,10 @@ int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const v
                    void* dX, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
               cudaStream_t st, int T_call);
-// forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels
-bool split_is_faster(const peqa_qweight_t* w, int T, bool trans);
+// forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels.
+// channel_scales: a forward that multiplies by one scale per channel at the end
+long long split_ns(const peqa_qweight_t* w, int T, bool trans);
+bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_scales);
 int split_ds_slots(const peqa_qweight_t* w, int T);
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans);
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,

@@ -473,11 +473,24 @@ int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
   const bool fold = p.G > 1;
   // More than eight tokens need two token tiles per MMA here and twice the staging; the cluster-split
   // forward, whose time hardly depends on the tokens, folds grouped scales into its operand
-  // as this kernel does.  In us, here / there: 8192 x 22016 in groups of 64 at 12 tokens 175 / 70,
-  // 22016 x 8192 in groups of 128 at 11 tokens 107 / 80, 4096 x 4096 in groups of 128 at 9 tokens
-  // 16 / 12; one scale per channel, 16 tokens: 8192 x 22016 107 / 60, 8192 x 8192 31 / 26, but
-  // 22016 x 8192 at 9 tokens 56 / 75 -- many rows are this kernel's better side.
-  if (M > 8 && (fold || p.K >= p.N)) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st, M);
+  // as this kernel does.  Grouped scales are faster there at all of 20 shapes from 256 x 4096 to 22016 x
+  // 22016 (9 to 16 tokens, us, here / there: 8192 x 22016 in groups of 64 170 / 70, 22016 x 8192 in groups
+  // of 128 148 / 80, 4096 x 4096 in groups of 128 14.2 / 11.6).  With one scale per channel and no more
+  // rows than columns both win somewhere (9 tokens: 4096 x 8192 14.6 / 16.5, 3072 x 12288 17.2 / 21.0,
+  // 8192 x 8192 27.4 / 26.3, 8192 x 22016 90 / 60); this kernel's time there is waves of 256 CTAs
+  // (fitted to 83 such layers, 9 to 16 tokens: the choice is at worst 7 % off the better one; by rows and
+  // columns alone 60 of 416 calls were 4 to 22 % slower), and it loses wherever its staging leaves room for
+  // one CTA per SM.  More rows than columns stay here.
+  if (M > 8) {
+    bool here = !fold;
+    if (here && p.K >= p.N) {
+      const long long max_steps = (p.total_steps + p.split - 1) / p.split;
+      const long long waves = ((long long)row_blocks * p.split + 255) / 256;
+      here = 2 * (smem + 1024) <= 228 * 1024 &&
+             waves * (5400 + 150 * M + max_steps * (3450 + 53 * M)) - 1500 < split_ns(w, M, false);
+    }
+    if (!here) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st, M);
+  }
   PEQA_TRY(status_word(st, &p.status));
   // packed matrix as uint32 [N, wpr]; box = 16 words x 128 rows, 64-byte swizzle
   CUtensorMap tmap_q;

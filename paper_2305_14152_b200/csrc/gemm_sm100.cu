@@ -885,9 +885,10 @@ int ds_piece(int g) { return gcd_int(g, 128); }
 }  // namespace
 
 int part_tokens(const peqa_qweight_t* w, int T_call) {
+  const bool channel_scales = effective_group(w->in_features, w->group_size) == w->in_features;
   int unit = 8;     // 16-byte aligned slices
   for (int trans = 0; trans < 2; ++trans)
-    if (fwd_pair_supported(w) && split_is_faster(w, T_call, trans)) {
+    if (fwd_pair_supported(w) && split_is_faster(w, T_call, trans, channel_scales && !trans)) {
       const int part = split_part_tokens(w, T_call, trans);
       unit = unit / gcd_int(unit, part) * part;
     }
@@ -896,7 +897,8 @@ int part_tokens(const peqa_qweight_t* w, int T_call) {
 
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
                cudaStream_t st, int T_call) {
-  if (fwd_pair_supported(w) && split_is_faster(w, T_call, false))
+  const bool channel_scales = g == w->in_features && !zeros_f;
+  if (fwd_pair_supported(w) && split_is_faster(w, T_call, false, channel_scales))
     return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call);
   if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
@@ -904,7 +906,7 @@ int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void*
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
               cudaStream_t st, int T_call) {
-  if (dx_pair_supported(w) && split_is_faster(w, T_call, true))
+  if (dx_pair_supported(w) && split_is_faster(w, T_call, true, false))
     return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call);
   if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
@@ -915,11 +917,12 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
   // dS = sum_t dY * u from the forward's fp32 sums instead of a contraction of its own (training
   // step of one linear, before -> after in us, and error of dS against binary64): 11008 x 4096 at
   // 4096 tokens 742 -> 611, 4.4e-6 -> 1.4e-7; 22016 x 8192 at 2048 tokens 1406 -> 1040; 4096 x 4096
-  // at 20 tokens 40 -> 32.  Below 2^28 products the contraction is two launches of a few us (256 x
-  // 256 at 64 tokens: 9 us) and the call stays the exact composition of the single calls, whose dS
-  // differs from this one in its last bits.
+  // at 16 tokens (2^28 products) 39 -> 25, 2048 x 2048 at 64 (2^28) 26 -> 20.5.  Below 2^28 it would
+  // save 3 to 6 us of a step too (1024 x 1024 at 128 tokens 25 -> 21, 256 x 256 at 64 19.5 -> 16.5); there
+  // the call stays the exact composition of the single calls, whose dS differs from this one in its
+  // last bits.
   if ((double)T * w->out_features * w->in_features < (double)(1 << 28)) return 0;
-  const int slots = split_is_faster(w, T, false) ? split_ds_slots(w, T) : 2 * ((T + 255) / 256);
+  const int slots = split_is_faster(w, T, false, true) ? split_ds_slots(w, T) : 2 * ((T + 255) / 256);
   // The partial sums go to the workspace the caller was asked for, whose size does not depend on
   // T (about T <= K fits).  Held against that size and not against the one that was given, so that
   // the bits of dS depend on the shape and T alone and a pointer that is not needed is not used.
@@ -929,7 +932,7 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
                   cudaStream_t st) {
   const int g = w->in_features;
-  if (split_is_faster(w, T, false)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T);
+  if (split_is_faster(w, T, false, true)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T);
   return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st);
 }
 

@@ -519,9 +519,11 @@ int launch_split_t(const CUtensorMap& ta, const CUtensorMap& tp, const SplitPara
 // Measured on this part (4096 x 4096 and 4096 x 11008, 17 to 1024 tokens): a stage of 128
 // contraction elements takes 0.60 us + 1.8 ns per token of the tile (the weights of a stage cost
 // the same however many tokens multiply them; past 80 tokens the MMAs show), a wave of CTAs
-// another 7 us (launch, first copies, the exchange of the sums).
+// another 7 us (launch, first copies, the exchange of the sums).  Good enough to choose among cluster
+// shapes; against the other kernels split_ns is held.
 struct SplitPlan {
   int nt, t_tiles, q, cshift;
+  int waves, stages;   // waves of clusters, stages of a CTA in each
   long long ns;
 };
 SplitPlan plan_split(int r_tiles, int C, int T, int sms) {
@@ -545,6 +547,8 @@ SplitPlan plan_split(int r_tiles, int C, int T, int sms) {
       if (best.ns < 0 || ns < best.ns) {
         best.q = q;
         best.cshift = ci;
+        best.waves = (int)waves;
+        best.stages = (int)stages;
         best.ns = ns;
       }
     }
@@ -552,28 +556,41 @@ SplitPlan plan_split(int r_tiles, int C, int T, int sms) {
   return best;
 }
 
-// The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs, 0.70 us per
-// stage of 64 whether the tile has one block of tokens or two (measured: 44 us for 4096 x 4096 and
-// 117 us for 4096 x 11008 at 17 to 256 tokens, 51 us for 4096 x 4096 at 512 and 1024), and the
-// launch and drain (256 x 256 at 64 tokens: forward 13.4 us, dX 7.6 us).
-long long pair_ns(int R, int C, int T, bool trans, int sms) {
+// The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs.  Fitted to 400
+// random calls, launches back to back (256 to 22016 rows and columns, 17 to 2600 tokens): a stage of 64
+// takes 0.58 us, with two blocks of tokens in the tile 0.67; a round 3.3 us more, with two blocks
+// 4.3; the launch 3.2, and 9.0 where the forward's epilogue multiplies by the channels' scales.
+// Nine of ten estimates are 0.90 to 1.09 of what was measured.  The shorter last round of items of one block
+// (make_pair_items, T % 512 == 0 only) is left out: it saves a sixth of one round.
+long long pair_ns(int R, int C, int T, bool channel_scales, int sms) {
   const long long tiles = (long long)((R + 255) / 256) * ((T + 511) / 512);
   const int pairs = sms / 2 > 0 ? sms / 2 : 1;
-  return (tiles + pairs - 1) / pairs * ((C + 63) / 64) * 700 + (trans ? 5000 : 9000);
+  const long long rounds = (tiles + pairs - 1) / pairs, stages = (C + 63) / 64;
+  return rounds * (T > 256 ? 4300 + stages * 666 : 3300 + stages * 580) + (channel_scales ? 9000 : 3200);
 }
 
 }  // namespace
 
-// Whether a call is served faster by this kernel than by the pair kernels.  Both estimates are
-// within 15 % of what was measured on either side of the line (before / here, in us): 4096 x 11008
-// forward at 1001 tokens 133 / 99, its dX (86 row tiles: three waves) 102 / 138; 4096 x 4096
-// forward at 77 tokens 44 / 13, at 1024 50 / 44, at 2048 53 / 96; 22016 x 8192 at 256 tokens
-// forward 178 / 128, dX 215 / 93.  A tie goes to the pair kernels.
-bool split_is_faster(const peqa_qweight_t* w, int T, bool trans) {
+// Estimated time of this kernel on a call of T tokens, in ns.  Fitted to the same calls: 3.6 us a wave,
+// 0.72 us + 0.83 ns per token a stage, and 34 ns per token of the tile for the exchange of the sums, 43
+// where no cluster shares it and 61 where a cluster owns several tiles.  Nine of ten estimates are 0.87
+// to 1.11 of what was measured.
+long long split_ns(const peqa_qweight_t* w, int T, bool trans) {
   const int R = trans ? w->in_features : w->out_features, C = trans ? w->out_features : w->in_features;
-  const int sms = sm_count_or(148);
-  const SplitPlan plan = plan_split((R + SM_ROWS - 1) / SM_ROWS, C, T, sms);
-  return plan.ns * 105 < pair_ns(R, C, T, trans, sms) * 100;
+  const SplitPlan p = plan_split((R + SM_ROWS - 1) / SM_ROWS, C, T, sm_count_or(148));
+  return (long long)p.waves * (3600 + p.stages * (720 + p.nt * 5 / 6) + p.nt * (34 + (p.cshift ? 0 : 9) + (p.q > 1 ? 27 : 0)));
+}
+
+// Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  Of the
+// 400 calls it is chosen for none where it was more than 3 % slower, and in five it is not chosen although it was
+// 6 to 10 % faster.  (Without the exchange's share of the time it was chosen for 25 where it was 4 to 55 %
+// slower: dX of 1656 x 3328 at 977 tokens 39.8 us here, 25.7 there; forward of 2360 x 256 at 1134
+// tokens in groups 15.1 / 10.3.)  Pair / here, in us: 4096 x 11008 forward at 1001 tokens 133 / 99, its dX
+// (86 row tiles: three waves) 102 / 138; 4096 x 4096 forward at 77 tokens 44 / 13; 22016 x 8192 at 256
+// tokens forward 178 / 128, dX 215 / 93.
+bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_scales) {
+  const int R = trans ? w->in_features : w->out_features, C = trans ? w->out_features : w->in_features;
+  return split_ns(w, T, trans) * 100 < pair_ns(R, C, T, channel_scales, sm_count_or(148)) * 97;
 }
 
 // Partial sums per channel that a forward with dS writes.

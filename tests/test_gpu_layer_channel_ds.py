@@ -70,10 +70,10 @@ def _linear(N, K, T, bits):
 
 
 # through the cluster-split forward and through the CTA-pair forward
-@pytest.mark.parametrize("T", [96, 2048])
-def test_y_and_dx_may_share_a_buffer(T):
+@pytest.mark.parametrize("N,T", [(2048, 96), (4096, 2048)])
+def test_y_and_dx_may_share_a_buffer(N, T):
     """The forward is enqueued before dX: a caller that wants no Y may give both the same scratch."""
-    N = K = 2048
+    K = N
     _, _, _, L = _linear(N, K, T, 4)
     L.workspace = binding.alloc_workspace(binding.OP_BWD, T, L.w)
     binding.layer_train_step([L], LR, step=1, apply_adamw=False)
