@@ -933,8 +933,8 @@ int x_pitch_for(int steps) {
 // adds its sums up through distributed shared memory.  The estimate, in ns, from timelines of
 // single CTAs: a warp's step of a pair 1600 (3000 with groups inside the step, a third more with
 // two token tiles), 10 per token and step staged, 2500 for the cluster's exchange, 1500 + 400 M per
-// further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 18.5 us, at 22016 x 8192
-// 65 / 46, in groups of 64 at 8192 x 8192 97 / 28.
+// further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at 22016 x 8192
+// 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
 int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;

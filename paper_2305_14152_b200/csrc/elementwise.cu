@@ -308,7 +308,7 @@ quantize_rtn_kernel(const float* __restrict__ W, int N, int K, int g, int cpg_sh
 // of the lanes of a group lane u works out the constants of the u-th (two divisions and a reciprocal,
 // which every lane would otherwise repeat for each of its runs).
 // HBM bound: 22016 x 8192 in groups of 64, 3-bit, 125 us = 6.3 TB/s (131 through the row-wise
-// kernel), 8192 x 22016 135 us (161: a CTA held one row at a time), 8192 x 8192 49 us (52).
+// kernel), 8192 x 22016 125 us (161: a CTA held one row at a time), 8192 x 8192 49 us (52).
 constexpr int kGroupThreads = 256;
 template <int BITS, int LPG>
 __global__ void __launch_bounds__(kGroupThreads, 4)
