@@ -168,7 +168,7 @@ extern "C" int peqa_qlinear_fwd(const peqa_qweight_t* w, const void* X, int T, v
   PEQA_TRY(check_gemm_shape(w, T));
   if (!aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  return launch_fwd(w, nullptr, g, X, T, Y, as_stream(stream), T);
+  return launch_fwd(w, nullptr, g, X, T, Y, as_stream(stream), T, 0);
 }
 
 extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const void* dY, int T,
@@ -189,7 +189,7 @@ extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const vo
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T));
+  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T, 0));
   if (dS) PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream)));
   return PEQA_OK;
 }
@@ -258,12 +258,12 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     if (slots > 0) {
       float* ds_part = static_cast<float*>(L->workspace);
       PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));
-      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T));   // before the scales change
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0));   // before the scales change
       PEQA_TRY(launch_ds_channel(&L->w, ds_part, slots, L->dS, apply_adamw ? &adam : nullptr, st));
       continue;
     }
-    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T));
-    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T));
+    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T, 0));
+    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0));
     PEQA_TRY(launch_ds(&L->w, nullptr, g[i], L->X_bf16, L->dY_bf16, T, L->dS, nullptr, apply_adamw ? &adam : nullptr,
                        L->workspace, L->workspace_bytes, st));
   }
@@ -311,7 +311,7 @@ extern "C" int peqa_qlinear_fwd_zf(const peqa_qweight_t* w, const float* zeros_f
   PEQA_TRY(check_gemm_shape(w, T));
   if (!aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  return launch_fwd(w, zeros_f, g, X, T, Y, as_stream(stream), T);
+  return launch_fwd(w, zeros_f, g, X, T, Y, as_stream(stream), T, 0);
 }
 
 extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f, const void* X,
@@ -334,7 +334,7 @@ extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T));
+  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T, 0));
   if (dS) PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream)));
   return PEQA_OK;
 }
@@ -498,10 +498,10 @@ int enqueue_host_linear(HostPipe* hp, cudaStream_t st, const peqa_layer_host_lin
     PEQA_CUDA(cudaEventRecord(hp->dy_landed[c], hp->in));
     // the forward needs only X: it runs while dY is still on its way
     PEQA_CUDA(cudaStreamWaitEvent(st, hp->x_landed[c], 0));
-    PEQA_TRY(launch_fwd(w, nullptr, g, dX_in + t0 * K * 2, (int)tc, dY_out + t0 * N * 2, st, T));
+    PEQA_TRY(launch_fwd(w, nullptr, g, dX_in + t0 * K * 2, (int)tc, dY_out + t0 * N * 2, st, T, (int)t0));
     PEQA_CUDA(cudaEventRecord(hp->fwd_done[c], st));
     PEQA_CUDA(cudaStreamWaitEvent(st, hp->dy_landed[c], 0));
-    PEQA_TRY(launch_dx(w, nullptr, g, ddY + t0 * N * 2, (int)tc, ddX + t0 * K * 2, st, T));
+    PEQA_TRY(launch_dx(w, nullptr, g, ddY + t0 * N * 2, (int)tc, ddX + t0 * K * 2, st, T, (int)t0));
     PEQA_CUDA(cudaEventRecord(hp->dx_done[c], st));
     // Y goes back while dX is still being computed
     PEQA_CUDA(cudaStreamWaitEvent(hp->out, hp->fwd_done[c], 0));

@@ -168,11 +168,11 @@ __device__ __forceinline__ void pair_item(const PairItems& it, int item, int T, 
 
 // Entry points implemented in the individual translation units.
 // zeros_f != nullptr: real-valued zero-points [N, G] (App. K) replace w->zeros.  A call of T_call tokens may
-// be launched in parts of T tokens, all but the last a multiple of part_tokens(w, T_call): every part
-// takes the route of the whole call and sums in its order, so its results are the same bits.
+// be launched in parts of T tokens from t0 on (X, Y: of the part; t0 a multiple of part_tokens(w, T_call)): every
+// part takes the route of the whole call and sums in its order, so its results are the same bits.
 int part_tokens(const peqa_qweight_t* w, int T_call);
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
-               cudaStream_t st, int T_call);
+               cudaStream_t st, int T_call, int t0);
 // Forward and, from its fp32 sums, the scale gradient of a layer with one scale per channel in two
 // launches: the forward leaves partial sums per channel, launch_ds_channel adds them (and makes the
 // AdamW step).  fwd_ds_slots: rows of N floats that takes, at most ds_workspace_bytes; 0 when the
@@ -191,7 +191,7 @@ bool dx_pair_supported(const peqa_qweight_t* w);
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
                    void* dX, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call);
+              cudaStream_t st, int T_call, int t0);
 // forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels.
 // channel_scales: a forward that multiplies by one scale per channel at the end
 long long split_ns(const peqa_qweight_t* w, int T, bool trans);
@@ -199,7 +199,7 @@ bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_sc
 int split_ds_slots(const peqa_qweight_t* w, int T);
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans);
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call);
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0);
 // adam != nullptr: the AdamW step on (w->scales, m, v) is applied where dS is produced
 struct DsAdam {
   AdamWConsts c;

@@ -489,7 +489,7 @@ int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
       here = 2 * (smem + 1024) <= 228 * 1024 &&
              waves * (5400 + 150 * M + max_steps * (3450 + 53 * M)) - 1500 < split_ns(w, M, false);
     }
-    if (!here) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st, M);
+    if (!here) return launch_split(w, nullptr, g, X, M, Y, false, nullptr, nullptr, st, M, 0);
   }
   PEQA_TRY(status_word(st, &p.status));
   // packed matrix as uint32 [N, wpr]; box = 16 words x 128 rows, 64-byte swizzle

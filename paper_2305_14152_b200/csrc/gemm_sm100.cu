@@ -896,18 +896,18 @@ int part_tokens(const peqa_qweight_t* w, int T_call) {
 }
 
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
-               cudaStream_t st, int T_call) {
+               cudaStream_t st, int T_call, int t0) {
   const bool channel_scales = g == w->in_features && !zeros_f;
   if (fwd_pair_supported(w) && split_is_faster(w, T_call, false, channel_scales))
-    return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call);
+    return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call, t0);
   if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call) {
+              cudaStream_t st, int T_call, int t0) {
   if (dx_pair_supported(w) && split_is_faster(w, T_call, true, false))
-    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call);
+    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call, t0);
   if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }
@@ -932,7 +932,7 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
                   cudaStream_t st) {
   const int g = w->in_features;
-  if (split_is_faster(w, T, false, true)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T);
+  if (split_is_faster(w, T, false, true)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T, 0);
   return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st);
 }
 

@@ -67,7 +67,9 @@ struct SplitParams {
   __nv_bfloat16* out;     // [T, R]
   int N, K, G, g, g_shift, T;
   int R;                  // output features
-  int r_tiles, tiles;     // row tiles, row tiles * token tiles
+  int r_tiles, tiles;     // row tiles, row tiles * token tiles (of the whole call)
+  int tile0, tile1;       // tiles of this launch, see launch_split
+  int first, t_first;     // tile its first cluster begins with, its first token tile
   int k_blocks;
   int nt;                 // tokens per tile, a multiple of 16
   int stages;
@@ -164,14 +166,16 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem_base = bars->tmem_base;
 
-  // ---- this CTA's stages: [lo, hi) of the cluster's list, tile0 first, then the next tile
+  // ---- this CTA's stages: [lo, hi) of the cluster's list, its first tile's, then the next tile's.  The
+  // list is cut as in the whole call; a part of a call leaves out the stages of tiles that are not its own.
   const int csize = 1 << p.cshift;
   const int rank = (int)(blockIdx.x & (csize - 1));
-  const int first_tile = (int)(blockIdx.x >> p.cshift) * p.q;
-  const int q = min(p.q, p.tiles - first_tile);
-  const int L = q * p.k_blocks;
+  const int first_tile = p.first + (int)(blockIdx.x >> p.cshift) * p.q;
+  const int L = min(p.q, p.tiles - first_tile) * p.k_blocks;
   auto range_lo = [&](int r) { return (r * L) >> p.cshift; };
-  const int lo = range_lo(rank), hi = range_lo(rank + 1);
+  const int j_lo = max(0, p.tile0 - first_tile), j_hi = min(p.q, p.tile1 - first_tile);   // its own tiles
+  const int lo = min(max(range_lo(rank), j_lo * p.k_blocks), j_hi * p.k_blocks);
+  const int hi = min(max(range_lo(rank + 1), lo), j_hi * p.k_blocks);
   const int n_it = hi - lo;
   const int j0 = lo / p.k_blocks;                            // first tile of the range
   const int split_at = (j0 + 1) * p.k_blocks - lo;           // local stages of the first tile
@@ -179,7 +183,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   // local stage -> k-block; row and token tile of the segment
   auto kb_of = [&](int it) { return it < split_at ? kb0 + it : it - split_at; };
   auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
-  auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles) * p.nt; };
+  auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles - p.t_first) * p.nt; };
 
   if (warp == 0) {
     // ------------------------------------------------ activation TMA (one lane)
@@ -398,10 +402,10 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     cluster_sync_all();
     if (worker) {
       const int toks = min(tok_pass, p.nt - tp);
-      for (int j = 0; j < q; ++j) {
+      for (int j = j_lo; j < j_hi; ++j) {
         const int tile = first_tile + j;
         const int r0 = (tile % p.r_tiles) * SM_ROWS + rank * rows_per;
-        const int t0 = (tile / p.r_tiles) * p.nt + tp;
+        const int t0 = (tile / p.r_tiles - p.t_first) * p.nt + tp;
         // contributors: the CTAs whose ranges meet [j * k_blocks, (j + 1) * k_blocks)
         const int b0 = j * p.k_blocks, b1 = b0 + p.k_blocks;
         uint32_t from = 0, second = 0;     // contributing ranks; those that hold it as second segment
@@ -409,7 +413,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         for (int r = 0; r < 8; ++r) {
           const int rl = range_lo(r), rh = range_lo(r + 1);
           if (r < csize && rl < b1 && rh > b0 && rh > rl) from |= 1u << r;
-          if (rl < b0) second |= 1u << r;
+          if (rl < b0 && j > j_lo) second |= 1u << r;
         }
         float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);   // vec_per divides kSplitWorkers: a thread keeps its rows
         for (int idx = wtid; idx < toks * vec_per; idx += kSplitWorkers) {
@@ -496,7 +500,7 @@ int launch_split_t(const CUtensorMap& ta, const CUtensorMap& tp, const SplitPara
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, SM_SMEM_LIMIT, done));
   cudaLaunchConfig_t cfg = {};
-  const int clusters = (p.tiles + p.q - 1) / p.q;
+  const int clusters = (p.tile1 - p.first + p.q - 1) / p.q;
   cfg.gridDim = dim3(clusters << p.cshift, 1, 1);
   cfg.blockDim = dim3(kSplitThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
@@ -599,18 +603,16 @@ int split_ds_slots(const peqa_qweight_t* w, int T) {
   return plan.t_tiles * ((plan.nt + SM_DUMP_TOK - 1) / SM_DUMP_TOK);
 }
 
-// A part of a call (its tokens from a multiple of this on) gets the clusters it has in the whole call:
-// whole token tiles, and as many as make whole clusters of q tiles.
+// A part of a call begins at a multiple of this: whole token tiles.
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans) {
   const int r_tiles = ((trans ? w->in_features : w->out_features) + SM_ROWS - 1) / SM_ROWS;
-  const SplitPlan plan = plan_split(r_tiles, trans ? w->out_features : w->in_features, T_call, sm_count_or(148));
-  int m = 1;
-  while (m * r_tiles % plan.q != 0) ++m;
-  return m * plan.nt;
+  return plan_split(r_tiles, trans ? w->out_features : w->in_features, T_call, sm_count_or(148)).nt;
 }
 
+// The T tokens from t0 on of a call of T_call tokens (act, out: of the part).  Plan and cut are those of the
+// whole call, so a token's sums are added in the same order in whichever part it comes.
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call) {
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0) {
   SplitParams p;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
@@ -633,7 +635,11 @@ int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
   p.nt = plan.nt;
   p.q = plan.q;
   p.cshift = plan.cshift;
-  p.tiles = p.r_tiles * ((T + plan.nt - 1) / plan.nt);
+  p.tiles = p.r_tiles * plan.t_tiles;
+  p.tile0 = p.r_tiles * (t0 / plan.nt);
+  p.tile1 = p.r_tiles * ((t0 + T + plan.nt - 1) / plan.nt);
+  p.first = p.tile0 / p.q * p.q;
+  p.t_first = t0 / plan.nt;
   p.k_blocks = (C + SM_BK - 1) / SM_BK;
   const int stage_bytes = 2 * (SM_A_BYTES + p.nt * (SM_HALF * 2));
   p.stages = (SM_SMEM_LIMIT - SM_SMEM_FIXED) / stage_bytes;
