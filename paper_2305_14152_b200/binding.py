@@ -1,9 +1,13 @@
-"""ctypes binding of libpeqa_b200.so: argument marshalling only.
+"""Binding of libpeqa_b200.so: argument marshalling only.
 
 Every function has the name of the C entry point it calls (see include/peqa.h)
 minus the ``peqa_`` prefix.  torch provides device memory and the current
 stream; all arithmetic runs in the library's CUDA kernels.  There is no CPU
 fallback: a missing library or a non-zero status raises.
+
+The calls a program makes once per layer and step (forward, decode, layer step,
+AdamW) are marshalled by the extension module ``_native`` (csrc/pybinding.cpp), the
+others through ctypes.
 """
 from __future__ import annotations
 
@@ -16,6 +20,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpeqa_b200.so")
 _lib = None
+_native = None
 
 OP_FWD, OP_BWD, OP_DECODE, OP_BWD_DS_FROM_Y, OP_BWD_DSDZ = 0, 1, 2, 3, 4
 
@@ -124,6 +129,17 @@ def lib() -> ctypes.CDLL:
             getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
+
+
+def _load_native():
+    """The extension module that marshals the frequent calls; never falls back."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _native as module
+        module.bind_error(PeqaError)
+        _native = module
+    return _native
 
 
 def _check(status: int, where: str) -> None:
@@ -237,15 +253,7 @@ def _ws(ws):
 
 
 def qlinear_fwd(w: QWeight, X: torch.Tensor, Y: torch.Tensor | None = None, workspace=None):
-    _dev(X, torch.bfloat16, "X")
-    T = X.shape[0]
-    if Y is None:
-        Y = X.new_empty((T, w.N))
-    cs = w.c_struct()
-    wp, wb = _ws(workspace)
-    _check(lib().peqa_qlinear_fwd(ctypes.byref(cs), X.data_ptr(), T, Y.data_ptr(), wp, wb,
-                                  _stream()), "peqa_qlinear_fwd")
-    return Y
+    return (_native or _load_native()).qlinear_fwd(w, X, Y, workspace)
 
 
 def qlinear_bwd(w: QWeight, X, dY: torch.Tensor, dX=None, dS=None, workspace=None,
@@ -267,25 +275,11 @@ def qlinear_bwd(w: QWeight, X, dY: torch.Tensor, dX=None, dS=None, workspace=Non
 
 
 def qlinear_decode(w: QWeight, X: torch.Tensor, Y: torch.Tensor | None = None, workspace=None):
-    _dev(X, torch.bfloat16, "X")
-    M = X.shape[0]
-    if Y is None:
-        Y = X.new_empty((M, w.N))
-    if workspace is None:
-        workspace = alloc_workspace(OP_DECODE, M, w)
-    cs = w.c_struct()
-    wp, wb = _ws(workspace)
-    _check(lib().peqa_qlinear_decode(ctypes.byref(cs), X.data_ptr(), M, Y.data_ptr(), wp, wb,
-                                     _stream()), "peqa_qlinear_decode")
-    return Y
+    return (_native or _load_native()).qlinear_decode(w, X, Y, workspace)
 
 
 def scale_adamw(scales, dS, m, v, lr, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, step=1):
-    for t, n in ((scales, "scales"), (dS, "dS"), (m, "m"), (v, "v")):
-        _dev(t, torch.float32, n)
-    _check(lib().peqa_scale_adamw(scales.data_ptr(), dS.data_ptr(), m.data_ptr(), v.data_ptr(),
-                                  scales.numel(), lr, beta1, beta2, eps, weight_decay, step,
-                                  _stream()), "peqa_scale_adamw")
+    (_native or _load_native()).scale_adamw(scales, dS, m, v, lr, beta1, beta2, eps, weight_decay, step)
 
 
 def train_step_host(w: QWeight, h_X, h_dY, h_Y, h_dX, h_dS, d_X, d_dY, d_Y, d_dX, d_dS, d_m, d_v,
@@ -358,24 +352,7 @@ def layer_train_step(linears, lr: float = 0.0, beta1=0.9, beta2=0.999, eps=1e-8,
                      apply_adamw=True) -> None:
     """Forward, dX and dS (and, with apply_adamw, the AdamW step on the scales) of every linear of
     `linears` in one library call."""
-    arr = (_LayerLinear * len(linears))()
-    T = linears[0].dY.shape[0]
-    for a, L in zip(arr, linears):
-        _dev(L.X, torch.bfloat16, "X")
-        _dev(L.dY, torch.bfloat16, "dY")
-        _dev(L.Y, torch.bfloat16, "Y")
-        _dev(L.dX, torch.bfloat16, "dX")
-        _dev(L.dS, torch.float32, "dS")
-        if L.dY.shape[0] != T or L.X.shape[0] != T:
-            raise ValueError("all linears of a layer step take the same number of tokens")
-        wp, wb = _ws(L.workspace)
-        a.w = L.w.c_struct()
-        a.X, a.dY, a.Y, a.dX, a.dS = (L.X.data_ptr(), L.dY.data_ptr(), L.Y.data_ptr(), L.dX.data_ptr(),
-                                      L.dS.data_ptr())
-        a.m, a.v = _ptr(L.m), _ptr(L.v)
-        a.workspace, a.workspace_bytes = wp, wb
-    _check(lib().peqa_layer_train_step(arr, len(linears), T, 1 if apply_adamw else 0, lr, beta1, beta2, eps,
-                                       weight_decay, step, _stream()), "peqa_layer_train_step")
+    (_native or _load_native()).layer_train_step(linears, apply_adamw, lr, beta1, beta2, eps, weight_decay, step)
 
 
 @dataclass
@@ -518,21 +495,7 @@ def qlinear_decode_prepared(w: QWeight, prepared: torch.Tensor, X: torch.Tensor,
                             scale_table=None, task_ids=None):
     """Decode from the prepared weights; with scale_table [n_tasks, N, G] and task_ids [M] every
     token uses the scales of its own task."""
-    _dev(prepared, torch.int32, "prepared")
-    _dev(X, torch.bfloat16, "X")
-    M = X.shape[0]
-    if Y is None:
-        Y = X.new_empty((M, w.N))
-    n_tasks = 0
-    if task_ids is not None:
-        _dev(scale_table, torch.float32, "scale_table")
-        _dev(task_ids, torch.int32, "task_ids")
-        n_tasks = scale_table.shape[0]
-    cs = w.c_struct()
-    _check(lib().peqa_qlinear_decode_prepared(ctypes.byref(cs), prepared.data_ptr(), X.data_ptr(), M,
-                                              Y.data_ptr(), _ptr(scale_table), n_tasks, _ptr(task_ids),
-                                              _stream()), "peqa_qlinear_decode_prepared")
-    return Y
+    return (_native or _load_native()).qlinear_decode_prepared(w, prepared, X, Y, scale_table, task_ids)
 
 
 def probe_read(buf: torch.Tensor, sink: torch.Tensor) -> None:
@@ -543,15 +506,7 @@ def probe_read(buf: torch.Tensor, sink: torch.Tensor) -> None:
 
 def qlinear_fwd_zf(w: QWeight, zeros_f: torch.Tensor, X: torch.Tensor, Y=None):
     """Forward with real-valued zero-points zeros_f fp32 [N, G] (App. K)."""
-    _dev(zeros_f, torch.float32, "zeros_f")
-    _dev(X, torch.bfloat16, "X")
-    T = X.shape[0]
-    if Y is None:
-        Y = X.new_empty((T, w.N))
-    cs = w.c_struct()
-    _check(lib().peqa_qlinear_fwd_zf(ctypes.byref(cs), zeros_f.data_ptr(), X.data_ptr(), T, Y.data_ptr(),
-                                     _stream()), "peqa_qlinear_fwd_zf")
-    return Y
+    return (_native or _load_native()).qlinear_fwd_zf(w, zeros_f, X, Y)
 
 
 def qlinear_bwd_zf(w: QWeight, zeros_f: torch.Tensor, X, dY: torch.Tensor, need_dx=True, need_grads=True,
@@ -573,11 +528,7 @@ def qlinear_bwd_zf(w: QWeight, zeros_f: torch.Tensor, X, dY: torch.Tensor, need_
 
 
 def zero_adamw(zeros_f, dZ, m, v, lr, beta1=0.9, beta2=0.999, eps=1e-8, weight_decay=0.0, step=1):
-    for t, n in ((zeros_f, "zeros_f"), (dZ, "dZ"), (m, "m"), (v, "v")):
-        _dev(t, torch.float32, n)
-    _check(lib().peqa_zero_adamw(zeros_f.data_ptr(), dZ.data_ptr(), m.data_ptr(), v.data_ptr(),
-                                 zeros_f.numel(), lr, beta1, beta2, eps, weight_decay, step, _stream()),
-           "peqa_zero_adamw")
+    (_native or _load_native()).zero_adamw(zeros_f, dZ, m, v, lr, beta1, beta2, eps, weight_decay, step)
 
 
 def selftest_configure(wait_limit_us: int = 0, starve_forward: bool = False) -> None:

@@ -5,11 +5,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpeqa_b200.so")
+NATIVE_SRC = os.path.join(CSRC, "pybinding.cpp")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -31,6 +34,24 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _build_native(verbose: bool) -> None:
+    """The extension module that marshals the frequent calls (binding.py)."""
+    import torch
+    base = os.path.dirname(os.path.abspath(torch.__file__))
+    libs = os.path.join(base, "lib")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-I", os.path.join(ROOT, "include"), "-I", os.path.join(base, "include"),
+           "-I", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           "-I", sysconfig.get_paths()["include"], "-I", "/usr/local/cuda/include",
+           NATIVE_SRC, "-o", NATIVE, "-L", libs, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+           "-L", HERE, "-lpeqa_b200", "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + libs]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+    if res.returncode != 0:
+        raise RuntimeError("building _native.so failed")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or _stale():
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -40,6 +61,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(res.stdout + res.stderr)
         if res.returncode != 0:
             raise RuntimeError("nvcc failed building libpeqa_b200.so")
+    header = os.path.join(ROOT, "include", "peqa.h")
+    if force or not os.path.exists(NATIVE) or \
+            os.path.getmtime(NATIVE) < max(os.path.getmtime(NATIVE_SRC), os.path.getmtime(header)):
+        _build_native(verbose)
     return LIB
 
 
