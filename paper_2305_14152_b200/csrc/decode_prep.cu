@@ -8,11 +8,8 @@
 //   * everything one warp needs for one step (8 rows x 512 columns) is one
 //     contiguous block that a single bulk copy moves into shared memory, in the
 //     order the lanes read it (16 bytes per lane and read, no bank conflicts);
-//   * the sixteen contraction slots of one warp-level MMA are sixteen columns of
-//     one 32-column run, so they share a quantization group and the scale and
-//     zero-point can be applied per group to the accumulator;
-//   * the two codes one logic operation extracts as a bf16 pair are the codes of
-//     two ADJACENT columns, so the activations are used in their natural order.
+//   * the contraction slots of a warp-level MMA are columns of one quantization
+//     group, so the scale and zero-point can be applied per group to the accumulator.
 //
 // Layout.  rg = row / 8, r = row % 8, step t = column / 512 (T = ceil(K / 512)
 // steps; columns beyond K hold zero codes), C = bits.  Block (rg, t) is C*512
@@ -37,10 +34,18 @@
 // through a private ring in shared memory: lane 0 issues one bulk copy per slot
 // (one or two steps of a pair: 3 to 8 KiB of contiguous memory; streaming reads
 // on this part want few, large copies and well over 100 KiB in flight per SM)
-// and all lanes wait on the slot's mbarrier.  Codes reach the tensor core as the biased integers
-// (bias + q) they are after one logic operation; the bias terms come off the sum
-// step by step or group by group, the zero-point's with the group (or the row):
-//   y += s * (acc - z * sum_j x_j - sum_j bias_j x_j).
+// and all lanes wait on the slot's mbarrier.  The zero-point's term comes off the sums with the
+// group (or the row):
+//   y += s * (acc - z * sum_j x_j).
+//
+// Operands.  The integer pipe is what a step of 16 rows x 512 columns is made of, so codes go to the
+// tensor core as the fp16 subnormals q * 2^(o - 24) that a code in the low bits of a half-word is
+// after one AND (f16_pair in dequant.cuh): 21 integer operations for 32 three-bit codes and 20 for
+// four-bit ones, where bf16 operands with an exponent put in took 26 and 28 and left a bias to take off every
+// sum.  The activations are brought to the range of fp16 by a power of two per token, which is
+// exact, and lose the 2^o.  Seven linears of a LLaMA-65B layer in groups of 64, one token, 163.9 ->
+// 150.4 us; of a LLaMA-7B layer in groups of 128, seven tokens of several tasks, 94.3 -> 85.1; one scale per
+// channel, where the main loop is the smaller part, 16 tokens 230.9 -> 227.3, one token unchanged.
 // When a warp's range crosses into the next pair it parks its sums in shared
 // memory; at the end the parked sums of each pair are added in warp order, so
 // results do not depend on timing.  What that final pass needs per token, row and
@@ -58,6 +63,7 @@
 // therefore read before earlier work in the stream is known to be complete:
 // they must be final when the call is made.
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 #include "dequant.cuh"
@@ -106,13 +112,23 @@ struct PrepParams {
   int* status;
 };
 
+// d += a * b, or d = a * b when FRESH
+template <bool FRESH>
 __device__ __forceinline__ void pmma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                            uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-      "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  if constexpr (FRESH) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+  } else {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  }
 }
 
 // Contiguous bulk copy global -> shared memory; its bytes are credited to `bar`.  Both
@@ -200,9 +216,9 @@ struct StepRegs {
   uint4 b[BITS];
 };
 
-// MMAs 2*MM and 2*MM + 1 of string S: run 4*S + MM of the step, whose eight columns of this
-// lane are one 16-byte word of activations per token.
-template <int BITS, int NT, bool HAS_B, int MM>
+// Pairs 4*MM .. 4*MM + 3 of a string, whose eight activations are one 16-byte word per token: two MMAs.
+// FRESH: the first of a quantization group.
+template <int BITS, int NT, bool HAS_B, int MM, bool FRESH>
 __device__ __forceinline__ void run_mma2(const uint32_t (&wa)[BITS], const uint32_t (&wb)[BITS],
                                          const uint8_t* x0, const uint8_t* x1,
                                          float (&acc)[NT][4], float (&acc2)[NT][4]) {
@@ -210,29 +226,46 @@ __device__ __forceinline__ void run_mma2(const uint32_t (&wa)[BITS], const uint3
   uint4 xb = make_uint4(0u, 0u, 0u, 0u);
   if (NT == 2) xb = *reinterpret_cast<const uint4*>(x1 + MM * 64);
   uint32_t f0[4], f1[4];
-  dq::mma_pairs_stream<BITS, 2 * MM>(wa, f0[0], f0[2]);
-  dq::mma_pairs_stream<BITS, 2 * MM + 1>(wa, f1[0], f1[2]);
+  f0[0] = dq::f16_pair<BITS, 4 * MM>(wa);
+  f0[2] = dq::f16_pair<BITS, 4 * MM + 1>(wa);
+  f1[0] = dq::f16_pair<BITS, 4 * MM + 2>(wa);
+  f1[2] = dq::f16_pair<BITS, 4 * MM + 3>(wa);
   f0[1] = f0[3] = f1[1] = f1[3] = 0u;
   if (HAS_B) {
-    dq::mma_pairs_stream<BITS, 2 * MM>(wb, f0[1], f0[3]);
-    dq::mma_pairs_stream<BITS, 2 * MM + 1>(wb, f1[1], f1[3]);
+    f0[1] = dq::f16_pair<BITS, 4 * MM>(wb);
+    f0[3] = dq::f16_pair<BITS, 4 * MM + 1>(wb);
+    f1[1] = dq::f16_pair<BITS, 4 * MM + 2>(wb);
+    f1[3] = dq::f16_pair<BITS, 4 * MM + 3>(wb);
   }
-  // the two MMAs of a run go to different accumulators, so that consecutive MMAs of a warp do
+  // the two MMAs go to different accumulators, so that consecutive MMAs of a warp do
   // not wait for one another (a single chain of 32 dependent MMAs per step cost 5 % of the
   // kernel); the halves are added when the sums are taken off
-  pmma_16816(acc[0], f0, xa.x, xa.y);
-  pmma_16816(acc2[0], f1, xa.z, xa.w);
+  pmma_16816<FRESH>(acc[0], f0, xa.x, xa.y);
+  pmma_16816<false>(acc2[0], f1, xa.z, xa.w);
   if (NT == 2) {
-    pmma_16816(acc[1], f0, xb.x, xb.y);
-    pmma_16816(acc2[1], f1, xb.z, xb.w);
+    pmma_16816<FRESH>(acc[1], f0, xb.x, xb.y);
+    pmma_16816<false>(acc2[1], f1, xb.z, xb.w);
   }
 }
 
-// Bias the code of string column cs (0..31) carries when it reaches the tensor core.
-template <int BITS>
-__host__ __device__ constexpr float column_bias(int cs) {
-  if (BITS == 4) return 128.0f;
-  return dq::stream_alt(3, cs >> 1) ? ((cs & 1) ? 16.0f : 64.0f) : ((cs & 1) ? 128.0f : 8.0f);
+// Eight activations (pairs 4*MM .. 4*MM + 3 of a string) in the order and the scale the codes want them:
+// v holds the sixteen of the string's half in their natural order, multiplied by the token's factor;
+// unit[o] = 2^-o takes out what the code's place in its fp16 multiplies in.
+template <int BITS, int MM>
+__device__ __forceinline__ uint4 x_pairs(const float (&v)[16]) {
+  uint32_t out[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    constexpr int half0 = (MM >> 1) * 16;
+    const int j = 4 * MM + e;
+    const int lo = dq::string_column(BITS, dq::f16_lo_bit(BITS, j)) - half0;
+    const int hi = dq::string_column(BITS, dq::f16_hi_bit(BITS, j)) - half0;
+    const float a = v[lo] * (1.0f / (float)(1 << dq::f16_lo_o(BITS, j)));
+    const float b = v[hi] * (1.0f / (float)(1 << dq::f16_hi_o(BITS, j)));
+    const __half2 h = __floats2half2_rn(a, b);
+    out[e] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return make_uint4(out[0], out[1], out[2], out[3]);
 }
 
 // GSH: quantization groups of 32 << GSH columns (1: 64, 2: 128, 3: 256), or 0: one group
@@ -255,6 +288,7 @@ decode_prep_kernel(const PrepParams p) {
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base + kPBarBytes);   // [0] flag, [1] limit
   int* wbound = const_cast<int*>(abort_flag) + 8;                            // [warps + 1] bounds of the chunk
   float* tsum = reinterpret_cast<float*>(wbound + kPWarps + 2);              // [16] sum of a token's x (not GROUPED)
+  float* tinv = tsum + 16;                                                   // [16] factor of a token's sums, see stage
   const int toks = (p.M + 1) & ~1;                                           // tokens kept of a tile
   // pitch of a row's tokens in the per-output tables: toks rounded up to 2 mod 4, so that the
   // sixteen rows a warp reads for one token fall into sixteen different banks
@@ -267,11 +301,10 @@ decode_prep_kernel(const PrepParams p) {
   float* part = reinterpret_cast<float*>(rowzs + (size_t)p.pairs_per_cta * 16);       // [warps][2][16][tp]
   float* ywhole = part + (size_t)kPWarps * 2 * 16 * tp;                      // [pairs][16][tp]
   float* yacc = ywhole + (size_t)p.pairs_per_cta * 16 * tp;                  // [pairs][16][tp] (several chunks)
-  float* sums = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * 16 * tp : 0);
-  // sums, GROUPED: [groups of the chunk][TOKP][2] = (sum x, sum bias*x) per group and token;
-  // else [steps of the chunk][TOKP] minus the sum of bias * x, then [16 warps] shares of a token's sum of x
-  const size_t sum_floats = GROUPED ? (size_t)p.spc * GPS * TOKP * 2 : (size_t)p.spc * TOKP + kPWarps;
-  float* xshare = sums + (size_t)p.spc * TOKP;                           // (not GROUPED)
+  float* xshare = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * 16 * tp : 0);     // [warps] shares of a token's sum of x
+  uint32_t* xmax = reinterpret_cast<uint32_t*>(xshare + kPWarps);        // [warps] largest |x| of a warp's share (bf16 bits)
+  float* sums = xshare + 2 * kPWarps;                                    // GROUPED: [groups of the chunk][TOKP] sum of x
+  const size_t sum_floats = GROUPED ? (size_t)p.spc * GPS * TOKP : 0;
   uint8_t* xs = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(sums + sum_floats) + 127) & ~static_cast<uintptr_t>(127));
   uint8_t* ring = xs + (((size_t)p.M * p.x_pitch + 127) & ~static_cast<size_t>(127));
@@ -430,29 +463,11 @@ decode_prep_kernel(const PrepParams p) {
     const int col0 = (t_lo + ch * p.spc) * kStepCols;              // first column of the chunk
     const int ccols = min(p.K - col0, spc_c * kStepCols);          // real columns in it
     if (ch > 0) __syncthreads();                                   // the previous chunk is no longer read
-    // ---- stage X[:, chunk] (columns beyond K read as zero) and take, per token, the sum of x
-    // and the sum of bias * x: per group (a thread stages and sums whole groups), or over the
-    // pieces this thread staged itself, added up per warp (the warps' shares are added in
-    // warp order when the rows are finished)
-    const int pieces = spc_c * (kStepCols / 8);                    // 16-byte pieces per token
-    // bias of the two columns in word e of a piece whose run in the step is run % 4 == rq
-    auto piece_sums = [&](const uint8_t* ptr, int rq, float& sx, float& sb) {
-      const uint4 v = *reinterpret_cast<const uint4*>(ptr);
-      const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float lo = __uint_as_float(wv[e] << 16), hi = __uint_as_float(wv[e] & 0xFFFF0000u);
-        sx += lo + hi;
-        float b0 = 128.0f, b1 = 128.0f;
-        if (BITS == 3) {
-          const bool alt = (dq::stream_alt_mask3() >> (4 * rq + e)) & 1u;
-          b0 = alt ? 64.0f : 8.0f;
-          b1 = alt ? 16.0f : 128.0f;
-        }
-        sb = fmaf(b0, lo, sb);
-        sb = fmaf(b1, hi, sb);
-      }
-    };
+    // ---- stage X[:, chunk] (columns beyond K read as zero): copied as it is, then turned in place into
+    // the fp16 operands that meet the codes (x_pairs), with the sums of x per token or per group.  A
+    // token's activations are first multiplied by a power of two that brings the largest of them to
+    // [2^15, 2^16): what is then below the normal fp16 numbers is less than 2^-29 of the largest, so fp16
+    // holds all that a fp32 sum with the largest in it would.  tinv undoes the factor and the 2^-24 of the codes.
     auto stage_piece = [&](int m, int pc) {
       uint8_t* dst = xs + (size_t)m * p.x_pitch + pc * 16;
       if (pc * 8 < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)m * p.K + col0 + pc * 8);
@@ -470,70 +485,103 @@ decode_prep_kernel(const PrepParams p) {
     };
     uint32_t z_own = 0u;
     float s_own = 0.0f;
-    if (GROUPED) {
-      const int ngr = spc_c * GPS;
-      constexpr int gpieces = RUNS_PER_GROUP * 4;                  // 16-byte pieces per group
-      for (int idx = threadIdx.x; idx < ngr * p.M; idx += kPThreads) {
-        const int gi = idx / p.M, m = idx - gi * p.M;
-        for (int pc = 0; pc < gpieces; ++pc) stage_piece(m, gi * gpieces + pc);
-      }
-      if (ch == 0 && lane == 0)
-        for (int s = 1; s < p.slots; ++s) issue_next();
-      if (warp == kPWarps - 1) share_bounds(spc_c);                          // while the activations are on their way
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      for (int idx = threadIdx.x; idx < ngr * p.M; idx += kPThreads) {
-        const int gi = idx / p.M, m = idx - gi * p.M;
-        const uint8_t* row = xs + (size_t)m * p.x_pitch + (size_t)gi * gpieces * 16;
-        float sx = 0.0f, sb = 0.0f;
-        for (int pc = 0; pc < gpieces; ++pc)
-          piece_sums(row + pc * 16, (gi * RUNS_PER_GROUP + (pc >> 2)) & 3, sx, sb);
-        sums[((size_t)gi * TOKP + m) * 2] = sx;
-        sums[((size_t)gi * TOKP + m) * 2 + 1] = sb;
-      }
-    } else {
-      // A token belongs to 16 / Mp warps (Mp: M rounded up to a power of two); a warp copies
-      // every (16 / Mp)-th step of its token and sums what it copied itself, so
-      // it needs no other warp's copies.  run % 4 of a lane's pieces is fixed.
-      int mp = 1;
-      while (mp < p.M) mp <<= 1;
-      const int wpt = kPWarps / mp;                                // warps per token
-      const int tok = warp / wpt, sub = warp - tok * wpt;
+    // A token belongs to 16 / Mp warps (Mp: M rounded up to a power of two); a warp copies and turns
+    // every (16 / Mp)-th step of its token, two at a time: lane 16 * j + 4 * s + c4 owns what string s
+    // of the j-th of them meets in lanes c4 of the MMAs, so it needs no other thread's copies.
+    int mp = 1;
+    while (mp < p.M) mp <<= 1;
+    const int wpt = kPWarps / mp;                                  // warps per token
+    const int tok = warp / wpt, sub = warp - tok * wpt;
+    uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + ((lane >> 2) & 3) * 256 + c4 * 16;
+    const int st0 = sub + (lane >> 4) * wpt;
+    if (tok < p.M)
+      for (int st = st0; st < spc_c; st += 2 * wpt)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) stage_piece(tok, st * 64 + ((lane >> 2) & 3) * 16 + r * 4 + c4);
+    if (ch == 0 && lane == 0)
+      for (int s = 1; s < p.slots; ++s) issue_next();
+    if (warp == kPWarps - 1) share_bounds(spc_c);                            // while the activations are on their way
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    {
+      uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
       if (tok < p.M)
-        for (int st = sub; st < spc_c; st += wpt) {
-          stage_piece(tok, st * 64 + lane);
-          stage_piece(tok, st * 64 + 32 + lane);
-        }
-      if (ch == 0 && lane == 0)
-        for (int s = 1; s < p.slots; ++s) issue_next();
-      if (warp == kPWarps - 1) share_bounds(spc_c);                          // while the activations are on their way
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncwarp();
-      if (tok < p.M) {
-        float sx = 0.0f;
-        const uint8_t* row = xs + (size_t)tok * p.x_pitch;
-        // steps by fours; the four sums fold into one register on the way down the lanes: 6
-        // shuffles instead of 20, lane 8 * j ends with the j-th
-        for (int st = sub; st < spc_c; st += 4 * wpt) {
-          float sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int st = st0; st < spc_c; st += 2 * wpt)
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (st + j * wpt < spc_c) {
-              piece_sums(row + ((st + j * wpt) * 64 + lane) * 16, (lane >> 2) & 3, sx, sb[j]);
-              piece_sums(row + ((st + j * wpt) * 64 + 32 + lane) * 16, (lane >> 2) & 3, sx, sb[j]);
+          for (int r = 0; r < 4; ++r) {
+            const uint4 v = *reinterpret_cast<const uint4*>(own + st * 1024 + r * 64);
+            mx = __vmaxu2(__vmaxu2(mx, v.x & 0x7FFF7FFFu), v.y & 0x7FFF7FFFu);
+            mx = __vmaxu2(__vmaxu2(mx, v.z & 0x7FFF7FFFu), v.w & 0x7FFF7FFFu);
+          }
+      mx = __reduce_max_sync(0xffffffffu, max(mx & 0xFFFFu, mx >> 16));
+      if (lane == 0) xmax[warp] = mx;
+    }
+    __syncthreads();
+    if (tok < p.M) {
+      uint32_t mx = 0u;
+      for (int w = 0; w < wpt; ++w) mx = max(mx, xmax[tok * wpt + w]);
+      // factor 2^k, its exponent field: 15 - (E - 127) + 127 with E the largest one's, a finite number for all E
+      const int kf = min(269 - (int)(mx >> 7), 253);
+      const float up = __uint_as_float((uint32_t)kf << 23);        // 2^k, k = kf - 127 in [-113, 126]
+      float sx = 0.0f;                                             // this lane's share of the token's sum (times 2^k)
+      for (int sb = sub; sb < spc_c; sb += 2 * wpt) {
+        const int st = sb + (lane >> 4) * wpt;
+        const bool live = st < spc_c;
+        float hsum[2] = {0.0f, 0.0f};                              // of the string's first and second half
+        if (live) {
+          uint8_t* at = own + st * 1024;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float v[16];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const uint4 raw = *reinterpret_cast<const uint4*>(at + (2 * h + q) * 64);
+              const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
+                v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
+              }
             }
-          const bool u16 = lane & 16, u8 = lane & 8;
-          const float t0 = (u16 ? sb[2] : sb[0]) + __shfl_xor_sync(0xffffffffu, u16 ? sb[0] : sb[2], 16);
-          const float t1 = (u16 ? sb[3] : sb[1]) + __shfl_xor_sync(0xffffffffu, u16 ? sb[1] : sb[3], 16);
-          float t = (u8 ? t1 : t0) + __shfl_xor_sync(0xffffffffu, u8 ? t0 : t1, 8);
+            float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-          for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-          const int mine = st + (lane >> 3) * wpt;
-          if ((lane & 7) == 0 && mine < spc_c) sums[mine * TOKP + tok] = -t;
+            for (int e = 0; e < 16; ++e) t[e & 3] += v[e];
+            hsum[h] = (t[0] + t[1]) + (t[2] + t[3]);
+            if (h == 0) {
+              *reinterpret_cast<uint4*>(at) = x_pairs<BITS, 0>(v);
+              *reinterpret_cast<uint4*>(at + 64) = x_pairs<BITS, 1>(v);
+            } else {
+              *reinterpret_cast<uint4*>(at + 128) = x_pairs<BITS, 2>(v);
+              *reinterpret_cast<uint4*>(at + 192) = x_pairs<BITS, 3>(v);
+            }
+          }
         }
+        if (!GROUPED) {
+          sx += hsum[0] + hsum[1];
+        } else {
+          // a group of 64 columns is half a string of the four lanes c4, 128 a string, 256 two strings;
+          // in the units of the accumulators: 2^-24 for the codes
+          if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+#pragma unroll
+          for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
+            float t = hsum[h];
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
+            const int str = (lane >> 2) & 3;
+            const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
+            if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
+              sums[(size_t)(st * GPS + gi) * TOKP + tok] = t * 5.9604644775390625e-8f;
+          }
+        }
+      }
+      if (!GROUPED) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        if (lane == 0) xshare[warp] = sx;
+        // 2^-k: its exponent field is 254 - kf, and 2^-126 (a normal number) at the least
+        if (lane == 0) xshare[warp] = sx * __uint_as_float((uint32_t)(254 - kf) << 23);
       }
+      // what is left of 2^(24 - k) after 2^12, which is applied first
+      if (sub == 0 && lane == 0) tinv[tok] = __uint_as_float((uint32_t)(266 - kf) << 23);
     }
     __syncthreads();
 
@@ -555,13 +603,16 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         const int tk = nt * 8 + c4 * 2;
-        const float* v = GROUPED ? yv[nt] : acc[nt];
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
         if (tk < toks) {
-          *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0], v[1]);
-          *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2], v[3]);
+          const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
+          *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0] * f.x, v[1] * f.y);
+          *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2] * f.x, v[3] * f.y);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = yv[nt][e] = 0.0f;
+        for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
       }
     };
     const uint8_t* xl = xs + (size_t)(r8 < p.M ? r8 : 0) * p.x_pitch + c4 * 16;
@@ -622,37 +673,32 @@ decode_prep_kernel(const PrepParams p) {
             load_groups<TG>(tab + (size_t)rowb * p.G, p.G - gstep0, has_b, p.G, gsb[e]);
           }
         }
-        // group gi of the step is complete: take z * sum x + sum bias * x off and scale
-        auto flush = [&](int gi) {
+        // group gi of the step begins: one of its two accumulators starts at -z * sum x ...
+        auto begin = [&](int gi) {
           const int q = gi % TG;
-          const float za = (float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
-          const float zb = (float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+          const float za = -(float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+          const float zb = -(float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
-            const float4 sv = *reinterpret_cast<const float4*>(sums + ((size_t)(tl * GPS + gi) * TOKP + nt * 8 + c4 * 2) * 2);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float sx = e ? sv.z : sv.x, sbx = e ? sv.w : sv.y;
-              const float sa = gsa[e % NS][q], sb = gsb[e % NS][q];
-              yv[nt][e] = fmaf(sa, (acc[nt][e] - fmaf(za, sx, sbx)) + acc2[nt][e], yv[nt][e]);
-              yv[nt][2 + e] = fmaf(sb, (acc[nt][2 + e] - fmaf(zb, sx, sbx)) + acc2[nt][2 + e], yv[nt][2 + e]);
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = 0.0f;
+            const float2 sx = *reinterpret_cast<const float2*>(sums + (size_t)(tl * GPS + gi) * TOKP + nt * 8 + c4 * 2);
+            acc2[nt][0] = za * sx.x;
+            acc2[nt][1] = za * sx.y;
+            acc2[nt][2] = zb * sx.x;
+            acc2[nt][3] = zb * sx.y;
           }
         };
-
-        if (!GROUPED) {
-          // one of the two accumulators of a step starts at minus the step's bias terms, so that what
-          // is carried from step to step is the small sum of q * x: carried along with the bias (up
-          // to 128 per column) it would lose bits of the result
+        // ... and ends: scale
+        auto flush = [&](int gi) {
+          const int q = gi % TG;
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const float2 b = *reinterpret_cast<const float2*>(sums + (size_t)tl * TOKP + nt * 8 + c4 * 2);
-            acc2[nt][0] = acc2[nt][2] = b.x;
-            acc2[nt][1] = acc2[nt][3] = b.y;
-          }
-        }
+          for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              yv[nt][e] = fmaf(gsa[e % NS][q], acc[nt][e] + acc2[nt][e], yv[nt][e]);
+              yv[nt][2 + e] = fmaf(gsb[e % NS][q], acc[nt][2 + e] + acc2[nt][2 + e], yv[nt][2 + e]);
+            }
+        };
+
         const uint32_t* fa = reinterpret_cast<const uint32_t*>(w.a);
         const uint32_t* fb = reinterpret_cast<const uint32_t*>(w.b);
         const uint8_t* x0 = xl + (size_t)tl * (kStepCols * 2);
@@ -667,28 +713,38 @@ decode_prep_kernel(const PrepParams p) {
           }
           const uint8_t* xs0 = x0 + s * 256;
           const uint8_t* xs1 = x1 + s * 256;
-          if (has_b) {
-            run_mma2<BITS, NT, true, 0>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, true, 1>(wa, wb, xs0, xs1, acc, acc2);
-            if (GROUPED && RUNS_PER_GROUP == 2) flush(2 * s);
-            run_mma2<BITS, NT, true, 2>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, true, 3>(wa, wb, xs0, xs1, acc, acc2);
-          } else {
-            run_mma2<BITS, NT, false, 0>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, false, 1>(wa, wb, xs0, xs1, acc, acc2);
-            if (GROUPED && RUNS_PER_GROUP == 2) flush(2 * s);
-            run_mma2<BITS, NT, false, 2>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, false, 3>(wa, wb, xs0, xs1, acc, acc2);
+          constexpr bool kHalf = GROUPED && RUNS_PER_GROUP == 2;     // a group is half a string
+          if (GROUPED && RUNS_PER_GROUP <= 4) begin(kHalf ? 2 * s : s);
+          if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) begin(s >> 1);
+          constexpr bool kFresh = GROUPED && RUNS_PER_GROUP <= 4;
+          if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
           }
-          if (GROUPED && RUNS_PER_GROUP == 2) flush(2 * s + 1);
+          if (has_b) {
+            run_mma2<BITS, NT, true, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, true, 1, false>(wa, wb, xs0, xs1, acc, acc2);
+            if (kHalf) {
+              flush(2 * s);
+              begin(2 * s + 1);
+            }
+            run_mma2<BITS, NT, true, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, true, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+          } else {
+            run_mma2<BITS, NT, false, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, false, 1, false>(wa, wb, xs0, xs1, acc, acc2);
+            if (kHalf) {
+              flush(2 * s);
+              begin(2 * s + 1);
+            }
+            run_mma2<BITS, NT, false, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, false, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+          }
+          if (kHalf) flush(2 * s + 1);
           if (GROUPED && RUNS_PER_GROUP == 4) flush(s);
           if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1)) flush(s >> 1);
-        }
-        if (!GROUPED) {
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[nt][e] += acc2[nt][e];
         }
         if (j + 1 == nsteps) {
           // Every lane has read its part of the slot: it can be refilled.  Behind the step's MMAs, where
@@ -708,8 +764,6 @@ decode_prep_kernel(const PrepParams p) {
     if (cur_pair >= 0) park();
     if (!GROUPED) {
       if (warp == kPWarps - 1) {                       // the tokens' sums of x from their warps' shares
-        int mp = 1;
-        while (mp < p.M) mp <<= 1;
         float t = lane < kPWarps ? xshare[lane] : 0.0f;
         for (int o = kPWarps / mp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (lane < kPWarps && (lane & (kPWarps / mp - 1)) == 0) tsum[lane / (kPWarps / mp)] = t;
@@ -965,7 +1019,7 @@ int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
         size_t b = 128 + kPHeadBytes + (kPWarps * 2 + c.pairs) * sums;
         if (spc < Tl) b += c.pairs * sums;
         b += (size_t)((c.pairs + 3) & ~3) * 4 + (size_t)c.pairs * 16 * 8;
-        b += ((size_t)spc * (grouped ? 2 * gps : 1) * TOKP + kPWarps) * 4 + 128;
+        b += ((grouped ? (size_t)spc * gps * TOKP : 0) + 2 * kPWarps) * 4 + 128;
         b += (((size_t)M * x_pitch_for(spc)) + 127) / 128 * 128;
         b += (size_t)kPWarps * slots * sps * step_bytes;
         return b;

@@ -262,5 +262,74 @@ __device__ __forceinline__ void mma_pairs_stream(const uint32_t (&w)[BITS], uint
   }
 }
 
+// ---------------------------------------------------------------------------
+// fp16 operands without a bias (the prepared decode).  A code in the ten mantissa bits of an fp16 whose
+// exponent bits are zero is the subnormal q * 2^(o - 24), o being its lowest bit: the tensor core takes
+// it exactly, so one logic operation per pair is all there is, no exponent to put in and no bias to take
+// off the sums.  Three-bit codes fit at o = 0..7, four-bit codes at 0..6, in either half of a window, so
+// a shift serves up to three pairs: 16 logic operations and 5 shifts for 32 three-bit codes, 16 and 4 for
+// four-bit ones (the bf16 pairs above: 16 and 10, 16 and 12).  The factor 2^o is taken out of the
+// activation the code meets, which is exact.
+// A string's pairs 0..7 hold its columns 0..15 and pairs 8..15 its columns 16..31, so that two runs of
+// 32 columns of the matrix make eight pairs of every lane.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int f16_lo_bit(int bits, int j) {
+  constexpr int lo3[16] = {0, 3, 6, 9, 12, 15, 36, 39, 42, 45, 54, 66, 69, 72, 75, 78};
+  return bits == 3 ? lo3[j] : 32 * (j / 4) + 4 * (j % 4);
+}
+__host__ __device__ constexpr int f16_hi_bit(int bits, int j) {
+  constexpr int hi3[16] = {18, 21, 24, 27, 30, 33, 48, 51, 57, 60, 63, 81, 84, 87, 90, 93};
+  return bits == 3 ? hi3[j] : f16_lo_bit(4, j) + 16;
+}
+// first bit of the pair's 32-bit window of the string
+__host__ __device__ constexpr int f16_window(int bits, int j) {
+  constexpr int win3[16] = {0, 0, 4, 4, 10, 10, 32, 32, 38, 38, 47, 64, 64, 71, 71, 71};
+  return bits == 3 ? win3[j] : 32 * (j / 4) + 8 * (j % 4 / 2);
+}
+// places of the pair's codes in their fp16: the codes count 2^o
+__host__ __device__ constexpr int f16_lo_o(int bits, int j) { return f16_lo_bit(bits, j) - f16_window(bits, j); }
+__host__ __device__ constexpr int f16_hi_o(int bits, int j) { return f16_hi_bit(bits, j) - f16_window(bits, j) - 16; }
+// a window that reaches into the next word needs a funnel shift; the same for all pairs of a window, so
+// that they share it
+__host__ __device__ constexpr bool f16_funnel(int bits, int j) {
+  for (int k = 0; k < 16; ++k)
+    if (f16_window(bits, k) == f16_window(bits, j) &&
+        f16_hi_bit(bits, k) + bits > 32 * (f16_window(bits, j) / 32 + 1))
+      return true;
+  return false;
+}
+// string column (0..31) whose code lies at this bit of the string
+__host__ __device__ constexpr int string_column(int bits, int bit) {
+  for (int k = 0; k < 16; ++k) {
+    if (bits * stream_lo(bits, k) == bit) return 2 * k;
+    if (bits * stream_hi(bits, k) == bit) return 2 * k + 1;
+  }
+  return -1;
+}
+__host__ __device__ constexpr bool f16_pairs_ok(int bits) {
+  uint32_t seen = 0u;
+  for (int j = 0; j < 16; ++j) {
+    const int lo = string_column(bits, f16_lo_bit(bits, j)), hi = string_column(bits, f16_hi_bit(bits, j));
+    if (lo < 0 || hi < 0 || lo / 16 != j / 8 || hi / 16 != j / 8) return false;
+    if (f16_lo_o(bits, j) < 0 || f16_lo_o(bits, j) + bits > 10) return false;
+    if (f16_hi_o(bits, j) < 0 || f16_hi_o(bits, j) + bits > 10) return false;
+    seen |= 1u << lo | 1u << hi;
+  }
+  return seen == 0xFFFFFFFFu;
+}
+static_assert(f16_pairs_ok(3) && f16_pairs_ok(4), "every column once, its code inside the mantissa");
+
+// Pair J of a string as two fp16 subnormals.
+template <int BITS, int J>
+__device__ __forceinline__ uint32_t f16_pair(const uint32_t (&w)[BITS]) {
+  constexpr int start = f16_window(BITS, J), a = start / 32, sh = start % 32;
+  constexpr uint32_t m = (1u << BITS) - 1u;
+  constexpr uint32_t mask = m << f16_lo_o(BITS, J) | m << (16 + f16_hi_o(BITS, J));
+  uint32_t x;
+  if constexpr (f16_funnel(BITS, J)) x = __funnelshift_r(w[a], w[a + 1], sh);
+  else x = w[a] >> sh;
+  return x & mask;
+}
+
 }  // namespace dq
 }  // namespace peqa
