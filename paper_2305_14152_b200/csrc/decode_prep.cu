@@ -56,6 +56,13 @@
 // Activations are staged in shared memory, all of K when they fit, otherwise in
 // chunks of steps with the per-output sums carried in shared memory.
 //
+// Canonical rows (CANON).  Where no second copy of the weights is kept the same kernel streams the packed matrix
+// itself: a step is 16 rows x 512 columns all the same, copied row by row with 16-byte asynchronous
+// copies by all lanes, and since the order of a contraction is free a lane takes 32 columns in a
+// row where the prepared order gives it eight of each of four runs.  The copies wait for the preceding
+// kernel, which may have written the matrix; before that its codes are only asked for in L2.  LLaMA-7B layer in groups
+// of 128, three sequences: 103.6 us through decode_stream_kernel, 81.7 here.
+//
 // Launch overlap.  The kernel is launched with programmatic stream
 // serialization: it lets the next kernel in the stream start as soon as SMs
 // free up, requests its own first weights at once, and only then waits for the
@@ -91,7 +98,7 @@ constexpr int kPHeadBytes = (kPBarBytes + 32 + (kPWarps + 1) * 4 + 4 + 16 * 8 + 
 __host__ __device__ inline int tok_pitch(int toks) { return toks + ((6 - (toks & 3)) & 3); }
 
 struct PrepParams {
-  const uint8_t* P;         // prepared weights
+  const uint8_t* P;         // prepared or canonical weights
   const uint8_t* zeros;     // [N, G]
   const float* scales;      // [N, G] or table [n_tasks, N, G]
   const __nv_bfloat16* X;   // [M, K]
@@ -108,6 +115,7 @@ struct PrepParams {
   int sps;                  // steps per slot (1 or 2)
   int x_pitch;              // bytes between staged token rows
   int pairs_per_cta;
+  int row_bytes;            // of the canonical matrix
   int cshift;               // log2 of the CTAs that share a range of rows, each with a slice of K
   int* status;
 };
@@ -158,6 +166,12 @@ __device__ __forceinline__ uint4 ring_load(uint32_t addr) {
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "r"(addr)
                : "memory");
+  return v;
+}
+
+__device__ __forceinline__ uint32_t ring_load1(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
 
@@ -248,31 +262,39 @@ __device__ __forceinline__ void run_mma2(const uint32_t (&wa)[BITS], const uint3
   }
 }
 
-// Eight activations (pairs 4*MM .. 4*MM + 3 of a string) in the order and the scale the codes want them:
-// v holds the sixteen of the string's half in their natural order, multiplied by the token's factor;
-// unit[o] = 2^-o takes out what the code's place in its fp16 multiplies in.
-template <int BITS, int MM>
-__device__ __forceinline__ uint4 x_pairs(const float (&v)[16]) {
+// The eight activations that meet pairs 4*MM .. 4*MM + 3 of a string, in that order and without the factors
+// 2^o of the codes' places.  v: the string's 32 activations, multiplied by the token's factor, in the order
+// of its columns (prepared: dq::string_column; canonical: the code at bit b is column b / BITS).
+template <int BITS, bool CANON, int MM>
+__device__ __forceinline__ uint4 x_pairs(const float (&v)[32]) {
   uint32_t out[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    constexpr int half0 = (MM >> 1) * 16;
     const int j = 4 * MM + e;
-    const int lo = dq::string_column(BITS, dq::f16_lo_bit(BITS, j)) - half0;
-    const int hi = dq::string_column(BITS, dq::f16_hi_bit(BITS, j)) - half0;
-    const float a = v[lo] * (1.0f / (float)(1 << dq::f16_lo_o(BITS, j)));
-    const float b = v[hi] * (1.0f / (float)(1 << dq::f16_hi_o(BITS, j)));
-    const __half2 h = __floats2half2_rn(a, b);
+    const int lo = CANON ? dq::f16_lo_bit(BITS, j) / BITS : dq::string_column(BITS, dq::f16_lo_bit(BITS, j));
+    const int hi = CANON ? dq::f16_hi_bit(BITS, j) / BITS : dq::string_column(BITS, dq::f16_hi_bit(BITS, j));
+    const __half2 h = __floats2half2_rn(v[lo] * (1.0f / (float)(1 << dq::f16_lo_o(BITS, j))),
+                                        v[hi] * (1.0f / (float)(1 << dq::f16_hi_o(BITS, j))));
     out[e] = *reinterpret_cast<const uint32_t*>(&h);
   }
   return make_uint4(out[0], out[1], out[2], out[3]);
 }
 
+// A step of canonical rows in the ring.  Three-bit rows of 192 bytes at a pitch of 208: the 32 words that
+// the lanes of a warp read at once (rows r8, columns c4) fall into different banks.  Four-bit rows of 256
+// bytes, chunk c of row r at c ^ 4 * (r & 1), so that the 16-byte reads of two rows do not meet.
+template <int BITS>
+struct CanonRow {
+  static constexpr int chunks = 4 * BITS;                    // 16-byte chunks of 512 codes
+  static constexpr int pitch = BITS == 3 ? 208 : 256;
+};
+
 // GSH: quantization groups of 32 << GSH columns (1: 64, 2: 128, 3: 256), or 0: one group
 // per row or groups that are multiples of 512 columns (the sums of a whole staged chunk of
 // steps are taken off at once, which needs the chunk to lie inside one group).
 // TASKS: grouped scales with a table per task (NT = 1 only).
-template <int BITS, int NT, int GSH, bool TASKS>
+// CANON: the weights are the canonical packed matrix.
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON>
 __global__ void __launch_bounds__(kPThreads, 1)
 decode_prep_kernel(const PrepParams p) {
   constexpr int C = BITS;                            // 16-byte chunks per lane, step and group
@@ -325,7 +347,8 @@ decode_prep_kernel(const PrepParams p) {
   const int trail = rest & 1;
   const int F = rest >> 1;                           // full pairs
   const int npairs = lead + F + trail;
-  const int slot_bytes = 2 * BLK * p.sps;
+  using Row = CanonRow<BITS>;
+  const int slot_bytes = CANON ? 16 * Row::pitch : 2 * BLK * p.sps;
 
   // the next kernel of the stream may be scheduled as SMs free up
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -335,7 +358,7 @@ decode_prep_kernel(const PrepParams p) {
     abort_flag[1] = p.status[4];
   }
   if (lane == 0) {
-    for (int s = 0; s < p.slots; ++s) mbar_init(smem_u32(&bars[warp * kPMaxSlots + s]), 1);
+    for (int s = 0; s < p.slots; ++s) mbar_init(smem_u32(&bars[warp * kPMaxSlots + s]), CANON ? 32 : 1);
     fence_mbar_init();
   }
   __syncwarp();
@@ -361,7 +384,7 @@ decode_prep_kernel(const PrepParams p) {
   auto pair_full = [&](int lp) { return lp >= lead && lp < lead + F; };
   // first row group of local pair lp (the only one of a half pair)
   auto pair_rg = [&](int lp) { return lp == 0 ? rg0 : 2 * (P0 + lp); };
-  // ---- ring: issue cursor (only lane 0 uses it)
+  // ---- ring: issue cursor (canonical: the lanes copy together; prepared: only lane 0 uses it)
   const uint32_t ring_w = smem_u32(ring) + (uint32_t)warp * (uint32_t)(p.slots * slot_bytes);
   const uint32_t bar_w = smem_u32(&bars[warp * kPMaxSlots]);
   int i_ch = 0, i_lin = 0, i_hi = 0, i_spc = 1;
@@ -386,6 +409,21 @@ decode_prep_kernel(const PrepParams p) {
     const int slot = i_slot;
     const uint32_t bar = bar_w + slot * 8;
     const uint32_t dst = ring_w + slot * slot_bytes;
+    if constexpr (CANON) {
+      // the rows' pieces of the step, 16 bytes per lane and copy; what lies beyond a row's end is not copied
+      // (its places meet activations that are zero)
+      const uint32_t off = (uint32_t)t * (Row::chunks * 16);
+      const uint8_t* src = p.P + (size_t)rg * 8 * p.row_bytes + off;
+      const int rows = pair_full(lp) ? 16 : 8;
+#pragma unroll
+      for (int q = 0; q < Row::chunks / 2; ++q) {
+        const int idx = q * 32 + lane, r = idx / Row::chunks, c = idx - r * Row::chunks;
+        if (r < rows && off + 16u * c < (uint32_t)p.row_bytes)
+          cp_async_16(dst + r * Row::pitch + 16 * (BITS == 4 ? c ^ ((r & 1) << 2) : c),
+                      src + (size_t)r * p.row_bytes + 16 * c);
+      }
+      cp_async_mbar_arrive_noinc(bar);
+    } else {
     // block (rg, t) lies at (((rg >> 1) * T + t) * 2 + (rg & 1)) * BLK
     const uint8_t* src = p.P + ((((size_t)(rg >> 1) * p.T + t) * 2 + (rg & 1)) * BLK);
     if (pair_full(lp)) {
@@ -395,6 +433,7 @@ decode_prep_kernel(const PrepParams p) {
       mbar_arrive_expect_tx(bar, n * BLK);
       bulk_load(dst, src, BLK, bar);
       if (n == 2) bulk_load(dst + 2 * BLK, src + 2 * BLK, BLK, bar);
+    }
     }
     i_slot = i_slot + 1 == p.slots ? 0 : i_slot + 1;
     i_lin += n;
@@ -434,7 +473,15 @@ decode_prep_kernel(const PrepParams p) {
   // One slot per warp is requested while the preceding kernel drains; the others follow the
   // activation requests of the first chunk, which would otherwise queue behind a full ring of
   // weights on their way into this SM (the CTAs that start last wait longest for them).
-  if (lane == 0) {
+  // The canonical matrix may be the result of the preceding kernel, so its codes are only asked for in L2,
+  // which a late write of them updates.
+  if (CANON) {
+    const uint32_t lo = (uint32_t)t_lo * (Row::chunks * 16);
+    const uint32_t hi = min((uint32_t)p.row_bytes, (uint32_t)(t_lo + n_t) * (Row::chunks * 16));
+    for (int r = (int)threadIdx.x; r < (rg_end - rg0) * 8; r += kPThreads)
+      prefetch_l2(p.P + ((size_t)rg0 * 8 + r) * p.row_bytes + lo, hi - lo);
+    issue_seek();
+  } else if (lane == 0) {
     issue_seek();
     issue_next();
   }
@@ -468,11 +515,6 @@ decode_prep_kernel(const PrepParams p) {
     // token's activations are first multiplied by a power of two that brings the largest of them to
     // [2^15, 2^16): what is then below the normal fp16 numbers is less than 2^-29 of the largest, so fp16
     // holds all that a fp32 sum with the largest in it would.  tinv undoes the factor and the 2^-24 of the codes.
-    auto stage_piece = [&](int m, int pc) {
-      uint8_t* dst = xs + (size_t)m * p.x_pitch + pc * 16;
-      if (pc * 8 < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)m * p.K + col0 + pc * 8);
-      else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
-    };
     // zero-point and scale of a row, for the final sums (a table per task: scales are looked up there)
     auto row_zs = [&](int r, uint32_t& z, float& sc) {
       z = 0u;
@@ -492,16 +534,24 @@ decode_prep_kernel(const PrepParams p) {
     while (mp < p.M) mp <<= 1;
     const int wpt = kPWarps / mp;                                  // warps per token
     const int tok = warp / wpt, sub = warp - tok * wpt;
-    uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + ((lane >> 2) & 3) * 256 + c4 * 16;
+    const int str = (lane >> 2) & 3;                               // the lane's string of a step
+    uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + str * 256 + c4 * 16;
     const int st0 = sub + (lane >> 4) * wpt;
     if (tok < p.M)
       for (int st = st0; st < spc_c; st += 2 * wpt)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) stage_piece(tok, st * 64 + ((lane >> 2) & 3) * 16 + r * 4 + c4);
-    if (ch == 0 && lane == 0)
-      for (int s = 1; s < p.slots; ++s) issue_next();
+        for (int r = 0; r < 4; ++r) {
+          // the string's columns by eights: one in each of its four runs, or 32 in a row
+          const int col = st * kStepCols + str * 128 + (CANON ? c4 * 32 + r * 8 : r * 32 + c4 * 8);
+          uint8_t* dst = own + st * 1024 + r * 64;
+          if (col < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)tok * p.K + col0 + col);
+          else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+        }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (ch == 0 && (CANON || lane == 0))
+      for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
     if (warp == kPWarps - 1) share_bounds(spc_c);                            // while the activations are on their way
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");           // (the ring's copies belong to no group)
     {
       uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
       if (tok < p.M)
@@ -529,31 +579,25 @@ decode_prep_kernel(const PrepParams p) {
         float hsum[2] = {0.0f, 0.0f};                              // of the string's first and second half
         if (live) {
           uint8_t* at = own + st * 1024;
+          float v[32];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            float v[16];
+          for (int q = 0; q < 4; ++q) {
+            const uint4 raw = *reinterpret_cast<const uint4*>(at + q * 64);
+            const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
+            float t0 = 0.0f, t1 = 0.0f;
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const uint4 raw = *reinterpret_cast<const uint4*>(at + (2 * h + q) * 64);
-              const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
-                v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
-              }
+            for (int e = 0; e < 4; ++e) {
+              v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
+              v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
+              t0 += v[q * 8 + 2 * e];
+              t1 += v[q * 8 + 2 * e + 1];
             }
-            float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int e = 0; e < 16; ++e) t[e & 3] += v[e];
-            hsum[h] = (t[0] + t[1]) + (t[2] + t[3]);
-            if (h == 0) {
-              *reinterpret_cast<uint4*>(at) = x_pairs<BITS, 0>(v);
-              *reinterpret_cast<uint4*>(at + 64) = x_pairs<BITS, 1>(v);
-            } else {
-              *reinterpret_cast<uint4*>(at + 128) = x_pairs<BITS, 2>(v);
-              *reinterpret_cast<uint4*>(at + 192) = x_pairs<BITS, 3>(v);
-            }
+            hsum[q >> 1] += t0 + t1;
           }
+          *reinterpret_cast<uint4*>(at) = x_pairs<BITS, CANON, 0>(v);
+          *reinterpret_cast<uint4*>(at + 64) = x_pairs<BITS, CANON, 1>(v);
+          *reinterpret_cast<uint4*>(at + 128) = x_pairs<BITS, CANON, 2>(v);
+          *reinterpret_cast<uint4*>(at + 192) = x_pairs<BITS, CANON, 3>(v);
         }
         if (!GROUPED) {
           sx += hsum[0] + hsum[1];
@@ -567,7 +611,6 @@ decode_prep_kernel(const PrepParams p) {
             t += __shfl_xor_sync(0xffffffffu, t, 1);
             t += __shfl_xor_sync(0xffffffffu, t, 2);
             if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
-            const int str = (lane >> 2) & 3;
             const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
             if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
               sums[(size_t)(st * GPS + gi) * TOKP + tok] = t * 5.9604644775390625e-8f;
@@ -643,15 +686,34 @@ decode_prep_kernel(const PrepParams p) {
         const bool has_b = pair_full(lp);
         StepRegs<BITS> w;
         {
-          const uint32_t sp = ring_w + (uint32_t)(slot * slot_bytes + j * 2 * BLK + lane * 16);
+          const uint32_t sp = ring_w + (uint32_t)(slot * slot_bytes);
+          if constexpr (CANON && BITS == 4) {
 #pragma unroll
-          for (int c = 0; c < C; ++c) w.a[c] = ring_load(sp + c * 512);
-          if (has_b) {
+            for (int c = 0; c < 4; ++c) {
+              const uint32_t at = sp + r8 * Row::pitch + (((4 * c + c4) ^ ((r8 & 1) << 2)) << 4);
+              w.a[c] = ring_load(at);
+              w.b[c] = has_b ? ring_load(at + 8 * Row::pitch) : make_uint4(0u, 0u, 0u, 0u);
+            }
+          } else if constexpr (CANON) {
+            uint32_t* wa = reinterpret_cast<uint32_t*>(w.a);
+            uint32_t* wb = reinterpret_cast<uint32_t*>(w.b);
 #pragma unroll
-            for (int c = 0; c < C; ++c) w.b[c] = ring_load(sp + (C + c) * 512);
+            for (int c = 0; c < 12; ++c) {
+              const uint32_t at = sp + r8 * Row::pitch + (c / 3) * 48 + c4 * 12 + (c % 3) * 4;
+              wa[c] = ring_load1(at);
+              wb[c] = has_b ? ring_load1(at + 8 * Row::pitch) : 0u;
+            }
           } else {
+            const uint32_t at = sp + (uint32_t)(j * 2 * BLK + lane * 16);
 #pragma unroll
-            for (int c = 0; c < C; ++c) w.b[c] = make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 0; c < C; ++c) w.a[c] = ring_load(at + c * 512);
+            if (has_b) {
+#pragma unroll
+              for (int c = 0; c < C; ++c) w.b[c] = ring_load(at + (C + c) * 512);
+            } else {
+#pragma unroll
+              for (int c = 0; c < C; ++c) w.b[c] = make_uint4(0u, 0u, 0u, 0u);
+            }
           }
         }
 
@@ -750,9 +812,14 @@ decode_prep_kernel(const PrepParams p) {
           // Every lane has read its part of the slot: it can be refilled.  Behind the step's MMAs, where
           // the fence finds the reads done; right behind the reads it waits for them (LLaMA-65B layer in
           // groups of 64, one token: 166 us there, 164 here).
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) issue_next();
+          if constexpr (CANON) {
+            __syncwarp();               // these copies go through the proxy of the reads
+            issue_next();
+          } else {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) issue_next();
+          }
         }
         ++lin;
         if (++tl == spc_c) {
@@ -989,12 +1056,12 @@ int x_pitch_for(int steps) {
 // two token tiles), 10 per token and step staged, 2500 for the cluster's exchange, 1500 + 400 M per
 // further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at 22016 x 8192
 // 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
-int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
+int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
   const int NT = M <= 8 ? 1 : 2, TOKP = 8 * NT;
   const int tp = tok_pitch((M + 1) & ~1);
-  const int step_bytes = 2 * bits * 512;
+  const int step_bytes = canon ? 16 * (bits == 3 ? CanonRow<3>::pitch : CanonRow<4>::pitch) : 2 * bits * 512;
   const bool grouped = gcols < kStepCols;
   const int gps = grouped ? kStepCols / gcols : 0;
   // a chunk must lie inside one quantization group unless the groups are applied per step
@@ -1028,7 +1095,7 @@ int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
       const int shapes[4][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}};   // {slots, steps per slot}
       // all of the CTA's K staged at once, with the best ring that fits ...
       if (grouped || one_group) {
-        for (int i = 0; i < 4 && c.spc == 0; ++i)
+        for (int i = canon ? 1 : 0; i < 4 && c.spc == 0; ++i)
           if (need(Tl, shapes[i][0], shapes[i][1]) <= (size_t)kPSmemLimit) {
             c.spc = Tl;
             c.slots = shapes[i][0];
@@ -1059,9 +1126,9 @@ int plan_prep(int N, int K, int M, int bits, int gcols, PrepPlan* plan) {
   return plan->ns < 0 ? PEQA_ERR_TOO_LARGE : PEQA_OK;
 }
 
-template <int BITS, int NT, int GSH, bool TASKS>
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON>
 int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS>;
+  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS, CANON>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, kPSmemLimit, done));
   cudaLaunchConfig_t cfg = {};
@@ -1082,21 +1149,26 @@ int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
   return PEQA_OK;
 }
 
-template <int BITS, int NT, bool TASKS>
+template <int BITS, int NT, bool TASKS, bool CANON>
 int launch_prep_g(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
   switch (gsh) {
-    case 1: return launch_prep_t<BITS, NT, 1, TASKS>(p, grid, smem, st);
-    case 2: return launch_prep_t<BITS, NT, 2, TASKS>(p, grid, smem, st);
-    case 3: return launch_prep_t<BITS, NT, 3, TASKS>(p, grid, smem, st);
-    default: return launch_prep_t<BITS, NT, 0, false>(p, grid, smem, st);   // tasks: looked up per row
+    case 1:
+      if constexpr (!CANON) return launch_prep_t<BITS, NT, 1, TASKS, CANON>(p, grid, smem, st);
+      return PEQA_ERR_BAD_SHAPE;
+    case 2: return launch_prep_t<BITS, NT, 2, TASKS, CANON>(p, grid, smem, st);
+    case 3: return launch_prep_t<BITS, NT, 3, TASKS, CANON>(p, grid, smem, st);
+    default: return launch_prep_t<BITS, NT, 0, false, CANON>(p, grid, smem, st);   // tasks: looked up per row
   }
 }
 
 template <int BITS>
-int launch_prep_b(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
-  if (p.M > 8) return launch_prep_g<BITS, 2, false>(p, gsh, grid, smem, st);
-  return p.task_ids ? launch_prep_g<BITS, 1, true>(p, gsh, grid, smem, st)
-                    : launch_prep_g<BITS, 1, false>(p, gsh, grid, smem, st);
+int launch_prep_b(const PrepParams& p, bool canon, int gsh, int grid, size_t smem, cudaStream_t st) {
+  if (canon)
+    return p.M > 8 ? launch_prep_g<BITS, 2, false, true>(p, gsh, grid, smem, st)
+                   : launch_prep_g<BITS, 1, false, true>(p, gsh, grid, smem, st);
+  if (p.M > 8) return launch_prep_g<BITS, 2, false, false>(p, gsh, grid, smem, st);
+  return p.task_ids ? launch_prep_g<BITS, 1, true, false>(p, gsh, grid, smem, st)
+                    : launch_prep_g<BITS, 1, false, false>(p, gsh, grid, smem, st);
 }
 
 int check_prep_layer(const peqa_qweight_t* w) {
@@ -1112,7 +1184,72 @@ bool prep_group_supported(int K, int g) {
   return g == K || g % kStepCols == 0 || g == 64 || g == 128 || g == 256;
 }
 
+// One launch, or two of at most eight tokens each, over prepared or canonical weights.
+int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, const void* X, int M, void* Y,
+               const float* scale_table, int n_tasks, const int32_t* task_ids, cudaStream_t st) {
+  PrepPlan plan;
+  bool two = false;
+  if (M > 8) {
+    PrepPlan half;
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, canon, &half));
+    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, &plan) != PEQA_OK ||
+          2 * half.ns < plan.ns;
+  } else {
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, &plan));
+  }
+  if (two) {
+    // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
+    // table per task (the scales of four tokens per lane do not fit in registers), where all tokens
+    // at once would be worked through in more chunks or waves, and where their parked sums leave no
+    // room in shared memory (from about 42000 rows on for 16 tokens, 68000 for 12, 113000 for 9).
+    const int h = (M + 1) / 2;
+    const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
+    PEQA_TRY(run_decode(w, weights, canon, g, X, h, Y, scale_table, n_tasks, task_ids, st));
+    return run_decode(w, weights, canon, g, static_cast<const char*>(X) + (size_t)h * K * 2, M - h,
+                      static_cast<char*>(Y) + (size_t)h * N * 2, scale_table, n_tasks,
+                      task_ids ? task_ids + h : nullptr, st);
+  }
+  PrepParams p;
+  p.P = static_cast<const uint8_t*>(weights);
+  p.zeros = w->zeros;
+  p.scales = task_ids ? scale_table : w->scales;
+  p.X = static_cast<const __nv_bfloat16*>(X);
+  p.Y = static_cast<__nv_bfloat16*>(Y);
+  p.task_ids = task_ids;
+  p.n_tasks = n_tasks;
+  p.N = w->out_features;
+  p.K = w->in_features;
+  p.G = p.K / g;
+  p.M = M;
+  p.rgs = p.N / 8;
+  p.rg_per_cta = plan.rg_per_cta;
+  p.T = plan.T;
+  p.spc = plan.spc;
+  p.nchunks = plan.nchunks;
+  p.slots = plan.slots;
+  p.sps = plan.sps;
+  p.x_pitch = plan.x_pitch;
+  p.pairs_per_cta = plan.pairs;
+  p.cshift = plan.cshift;
+  p.row_bytes = p.K / 8 * w->bits;
+  PEQA_TRY(status_word(st, &p.status));
+  const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
+  return w->bits == 3 ? launch_prep_b<3>(p, canon, gsh, plan.grid, plan.smem, st)
+                      : launch_prep_b<4>(p, canon, gsh, plan.grid, plan.smem, st);
+}
+
 }  // namespace
+
+bool decode_rows_supported(const peqa_qweight_t* w, int g, int M) {
+  PrepPlan plan;
+  return w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == 128 || g == 256) &&
+         plan_prep(w->out_features, w->in_features, M > 8 ? (M + 1) / 2 : M, w->bits, g, true, &plan) == PEQA_OK;
+}
+
+int launch_decode_rows(const peqa_qweight_t* w, int g, const void* X, int M, void* Y, const float* scale_table,
+                       int n_tasks, const int32_t* task_ids, cudaStream_t st) {
+  return run_decode(w, w->qweight, true, g, X, M, Y, scale_table, n_tasks, task_ids, st);
+}
 
 }  // namespace peqa
 
@@ -1174,53 +1311,5 @@ extern "C" int peqa_qlinear_decode_prepared(const peqa_qweight_t* w, const uint3
   }
   if (!aligned16(prepared) || !aligned16(X) || !aligned16(Y)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
-  PrepPlan plan;
-  bool two = false;
-  if (M > 8) {
-    PrepPlan half;
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, &half));
-    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan) != PEQA_OK ||
-          2 * half.ns < plan.ns;
-  } else {
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, &plan));
-  }
-  if (two) {
-    // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
-    // table per task (the scales of four tokens per lane do not fit in registers), where all tokens
-    // at once would be worked through in more chunks or waves, and where their parked sums leave no
-    // room in shared memory (from about 42000 rows on for 16 tokens, 68000 for 12, 113000 for 9).
-    const int h = (M + 1) / 2;
-    const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
-    PEQA_TRY(peqa_qlinear_decode_prepared(w, prepared, X, h, Y, scale_table, n_tasks, task_ids, stream));
-    return peqa_qlinear_decode_prepared(w, prepared, static_cast<const char*>(X) + (size_t)h * K * 2, M - h,
-                                        static_cast<char*>(Y) + (size_t)h * N * 2, scale_table, n_tasks,
-                                        task_ids ? task_ids + h : nullptr, stream);
-  }
-  PrepParams p;
-  p.P = reinterpret_cast<const uint8_t*>(prepared);
-  p.zeros = w->zeros;
-  p.scales = task_ids ? scale_table : w->scales;
-  p.X = static_cast<const __nv_bfloat16*>(X);
-  p.Y = static_cast<__nv_bfloat16*>(Y);
-  p.task_ids = task_ids;
-  p.n_tasks = n_tasks;
-  p.N = w->out_features;
-  p.K = w->in_features;
-  p.G = p.K / g;
-  p.M = M;
-  p.rgs = p.N / 8;
-  p.rg_per_cta = plan.rg_per_cta;
-  p.T = plan.T;
-  p.spc = plan.spc;
-  p.nchunks = plan.nchunks;
-  p.slots = plan.slots;
-  p.sps = plan.sps;
-  p.x_pitch = plan.x_pitch;
-  p.pairs_per_cta = plan.pairs;
-  p.cshift = plan.cshift;
-  cudaStream_t st = as_stream(stream);
-  PEQA_TRY(status_word(st, &p.status));
-  const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
-  return w->bits == 3 ? launch_prep_b<3>(p, gsh, plan.grid, plan.smem, st)
-                      : launch_prep_b<4>(p, gsh, plan.grid, plan.smem, st);
+  return run_decode(w, prepared, false, g, X, M, Y, scale_table, n_tasks, task_ids, as_stream(stream));
 }

@@ -1,0 +1,63 @@
+"""GPU parity of the decode that streams the canonical rows through the kernel of the prepared decode, and of
+the fp16 operands both are made of: a row group alone, half pairs, rows that end inside a step, groups that
+are a string, two strings, a step and more; tokens of any magnitude in one batch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2305_14152_b200 import binding, synth
+from gpu_util import assert_close, bf16_to_dev, dev_to_f64, oracle_layer, to_qweight
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,K,bits,g", [(8, 128, 3, 0), (8, 128, 4, 128), (200, 1408, 3, 128), (200, 1408, 4, 0),
+                                        (1032, 1280, 3, 256), (2056, 8192, 4, 512), (264, 22016, 3, 0), (4104, 4224, 4, 128)])
+def test_canonical_rows(N, K, bits, g):
+    d = synth.custom(N + K, N, K, 16, bits, g, outliers=True)
+    codes, zeros, scales, packed = oracle_layer(d, bits, g)
+    qw = to_qweight(packed, zeros, scales, bits, g, K)
+    ref = oracle.fwd(d["X"], packed, zeros, scales, bits, g)
+    for M in (1, 2, 5, 8, 9, 16):
+        guard = torch.full((M * N + 512,), 7.0, dtype=torch.bfloat16, device="cuda")
+        Y = guard[256:256 + M * N].view(M, N)
+        X = bf16_to_dev(d["X"][:M])
+        binding.qlinear_decode(qw, X, Y)
+        again = binding.qlinear_decode(qw, X)
+        binding.check_status()
+        assert torch.all(guard[:256] == 7.0) and torch.all(guard[-256:] == 7.0), "wrote outside its output"
+        assert torch.equal(Y, again)
+        assert_close(dev_to_f64(Y), ref[:M], f"M={M}")
+
+
+@pytest.mark.parametrize("bits,g", [(3, 0), (4, 0), (3, 64), (4, 128), (3, 256)])
+def test_tokens_of_any_magnitude(bits, g):
+    """A token is brought to the range of fp16 by a power of two of its own, so its result is as exact at 2^-90
+    as at 2^90 and with one element 2^12 times the others; a token of zeros gives zeros, one with an infinity or
+    a NaN nothing finite, and neither touches its neighbours."""
+    N, K, M = 264, 1536, 8
+    d = synth.custom(5 + bits + g, N, K, M, bits, g, outliers=True)
+    codes, zeros, scales, packed = oracle_layer(d, bits, g)
+    qw = to_qweight(packed, zeros, scales, bits, g, K)
+    prep = binding.decode_prepare(qw)
+    X = synth.bf16_bits_to_f32(d["X"]).astype(np.float32)
+    X[1] *= 2.0 ** -90
+    X[2] *= 2.0 ** 90
+    X[3, 700] = 4096.0
+    X[4] = 0.0
+    X[5, 3] = np.inf
+    X[6, 1500] = np.nan
+    Xb = synth.f32_to_bf16_bits(X)
+    torch.cuda.synchronize()
+    out = [binding.qlinear_decode_prepared(qw, prep, bf16_to_dev(Xb))]
+    if g != 64:
+        out.append(binding.qlinear_decode(qw, bf16_to_dev(Xb)))
+    binding.check_status()
+    ref = oracle.fwd(Xb[[0, 1, 2, 3, 7]], packed, zeros, scales, bits, g)
+    for Y in out:
+        got = dev_to_f64(Y)
+        for i, m in enumerate((0, 1, 2, 3, 7)):
+            assert_close(got[m] / np.abs(ref[i]).max(), ref[i] / np.abs(ref[i]).max(), f"token {m}")
+        assert np.all(got[4] == 0.0)
+        assert not np.any(np.isfinite(got[5])) and not np.any(np.isfinite(got[6]))
