@@ -368,6 +368,8 @@ extern "C" int peqa_qlinear_decode_multitask(const peqa_qweight_t* w, const floa
   if (!aligned16(X) || !aligned16(Y) || !aligned16(scale_table)) return PEQA_ERR_ALIGNMENT;
   PEQA_TRY(check_arch());
   if (!decode_stream_supported(w, g, M)) return PEQA_ERR_BAD_SHAPE;
+  if (decode_rows_are_faster(w, g, M))
+    return launch_decode_rows(w, g, X, M, Y, scale_table, n_tasks, task_ids, as_stream(stream));
   return launch_decode_stream(w, g, X, M, Y, scale_table, n_tasks, task_ids, as_stream(stream));
 }
 

@@ -430,13 +430,23 @@ int launch_decode_t(const CUtensorMap& tmap_q, const DecodeParams& p, int row_bl
 
 size_t decode_workspace_bytes(const peqa_qweight_t*, int, int) { return 0; }
 
+// Up to eight tokens, 45 shapes from 272 to 22016 rows and columns (us, decode_stream_kernel or, where its activations
+// do not fit, decode_kernel / the kernel of the prepared decode).  Groups of 128 or 256 columns: faster there at
+// all of 17, 664 x 768 6.5 / 6.1, 11008 x 4096 17.5 / 13.4, 848 x 19328 29.5 / 11.7.  One scale per channel: the streaming
+// kernel's set-up is 1 us shorter, so it keeps what it does in one block of 32 rows per CTA and few steps
+// of K (1872 x 512 4.8 / 6.2, 3768 x 1664 4.8 / 6.6, 4096 x 4096 6.5 / 7.2); more rows or columns are slower there
+// (11152 x 256 8.5 / 6.8, 15240 x 640 10.0 / 7.9, 1520 x 11136 10.9 / 8.1, 21784 x 21632 133 / 78; worst 8192 x 8192 12.7 / 12.9).
+bool decode_rows_are_faster(const peqa_qweight_t* w, int g, int M) {
+  if (M > 8 || !decode_rows_supported(w, g, M)) return false;
+  if (g != w->in_features || !decode_stream_supported(w, g, M)) return true;
+  const int sms = sm_count_or(148);
+  return (w->out_features / 8 + sms - 1) / sms > 4 || w->in_features > 5120;
+}
+
 int launch_decode(const peqa_qweight_t* w, int g, const void* X, int M, void* Y,
                   void* workspace, size_t workspace_bytes, cudaStream_t st) {
   (void)workspace; (void)workspace_bytes;
-  // Groups of 128 or 256 columns, up to eight tokens: 3 to 60 % faster through the kernel of the prepared decode at
-  // 16 of 17 shapes from 472 x 1920 to 15664 x 2176 (us, here / there: 664 x 768 6.5 / 6.1, 11008 x 4096 17.2 / 13.7,
-  // 848 x 19328 29.5 / 11.7).
-  if (M <= 8 && decode_rows_supported(w, g, M)) return launch_decode_rows(w, g, X, M, Y, nullptr, 0, nullptr, st);
+  if (decode_rows_are_faster(w, g, M)) return launch_decode_rows(w, g, X, M, Y, nullptr, 0, nullptr, st);
   if (decode_stream_supported(w, g, M)) return launch_decode_stream(w, g, X, M, Y, nullptr, 1, nullptr, st);
   DecodeParams p;
   p.qw = w->qweight;

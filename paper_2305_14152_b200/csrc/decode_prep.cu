@@ -56,6 +56,15 @@
 // Activations are staged in shared memory, all of K when they fit, otherwise in
 // chunks of steps with the per-output sums carried in shared memory.
 //
+// One or two tokens (I8).  Of the eight token columns of an fp16 MMA one or two would be used.  Integer MMAs cover
+// twice the contraction, so the activations go in as whole numbers: a step's 512 are scaled by a power
+// of two of their own to at most 2^30 and cut into four signed base-256 digits, which fill the eight
+// columns for two tokens; the codes are unsigned bytes, eight integer operations for 32 four-bit codes
+// and 14 (groups of 64: 18) for three-bit ones (i8_string).  Sums of products are exact until a group (or a
+// step) is scaled, and what the 30 bits do not hold is less than fp32 sums lose.  A step of a warp takes
+// about 1200 cycles instead of 2100 (groups of 64: 2200 / 3000).  One token, us, fp16 / here: 22016 x 8192 in
+// groups of 64 28.8 / 25.0, 8192 x 8192 14.6 / 12.6, 11008 x 4096 9.5 / 7.7, 4096 x 4096 6.2 / 5.6, 256 x 256 5.0 / 4.1.
+//
 // Canonical rows (CANON).  Where no second copy of the weights is kept the same kernel streams the packed matrix
 // itself: a step is 16 rows x 512 columns all the same, copied row by row with 16-byte asynchronous
 // copies by all lanes, and since the order of a contraction is free a lane takes 32 columns in a
@@ -90,8 +99,9 @@ constexpr int kPThreads = kPWarps * 32;
 constexpr int kPSmemLimit = 227 * 1024;
 constexpr int kPMaxSlots = 4;
 constexpr int kStepCols = 512;
+constexpr int kI8Units = 64;                                      // most (token, step)s of the integer kernel
 constexpr int kPBarBytes = kPWarps * kPMaxSlots * 8;              // the warps' mbarriers
-// + abort flag, wait limit, the bounds of the warps' steps and, per token, the sums of x and bias * x
+// + abort flag, wait limit, the bounds of the warps' steps and, per token, the sum of x and the factor of its sums
 constexpr int kPHeadBytes = (kPBarBytes + 32 + (kPWarps + 1) * 4 + 4 + 16 * 8 + 127) / 128 * 128;
 
 // Pitch (floats) of a row's tokens in the per-output tables of shared memory.
@@ -223,6 +233,52 @@ __device__ __forceinline__ void load_zero_bytes(const uint8_t* src, int left, bo
   }
 }
 
+// d += a * b, or d = a * b when FRESH: unsigned codes, signed digits of the activations.
+template <bool FRESH>
+__device__ __forceinline__ void imma_16832(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                           uint32_t b0, uint32_t b1) {
+  if constexpr (FRESH) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(0));
+  } else {
+    asm volatile(
+        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+  }
+}
+
+// The activations that meet registers 2*JP*2 .. 2*JP*2 + 3 of a string (two MMAs), as signed base-256 digits:
+// out[d] is the 16 bytes of digit d.  v: the string's 32 activations times the token's factor 2^k.
+template <int BITS, bool CANON, bool HALF, int JP>
+__device__ __forceinline__ void x_digits(const float (&v)[32], uint4 (&out)[4]) {
+  uint32_t word[4][4];                             // [register][digit]
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t x[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = 4 * JP + q;
+      const int col = dq::position_column(BITS, CANON, dq::i8_pos(BITS, HALF, r, b));
+      // digits in [-128, 127]: 128 is added to the three lower bytes, with carries, and taken off each
+      const int xi = __float2int_rn(v[col] * (1.0f / (float)(1 << dq::i8_o(BITS, HALF, r, b))));
+      x[b] = ((uint32_t)xi + 0x00808080u) ^ 0x00808080u;
+    }
+    const uint32_t t0 = dq::prmt(x[0], x[1], 0x5140u), t1 = dq::prmt(x[2], x[3], 0x5140u);
+    const uint32_t t2 = dq::prmt(x[0], x[1], 0x7362u), t3 = dq::prmt(x[2], x[3], 0x7362u);
+    word[q][0] = dq::prmt(t0, t1, 0x5410u);
+    word[q][1] = dq::prmt(t0, t1, 0x7632u);
+    word[q][2] = dq::prmt(t2, t3, 0x5410u);
+    word[q][3] = dq::prmt(t2, t3, 0x7632u);
+  }
+#pragma unroll
+  for (int d = 0; d < 4; ++d) out[d] = make_uint4(word[0][d], word[1][d], word[2][d], word[3][d]);
+}
+
 // One lane's weights of one step: row r of the pair's two groups.
 template <int BITS>
 struct StepRegs {
@@ -294,7 +350,11 @@ struct CanonRow {
 // steps are taken off at once, which needs the chunk to lie inside one group).
 // TASKS: grouped scales with a table per task (NT = 1 only).
 // CANON: the weights are the canonical packed matrix.
-template <int BITS, int NT, int GSH, bool TASKS, bool CANON>
+// I8 (one or two tokens, NT = 1, all of K staged at once): integer MMAs.  A token's activations are whole
+// numbers of up to 31 bits times a power of two, cut into four signed digits, and the MMA's eight columns
+// are two tokens x four digits, which fp16 operands would leave idle.  An MMA covers twice the columns,
+// the codes are cheaper to take out (i8_string), and the sums of a group are exact.
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8>
 __global__ void __launch_bounds__(kPThreads, 1)
 decode_prep_kernel(const PrepParams p) {
   constexpr int C = BITS;                            // 16-byte chunks per lane, step and group
@@ -325,11 +385,15 @@ decode_prep_kernel(const PrepParams p) {
   float* yacc = ywhole + (size_t)p.pairs_per_cta * 16 * tp;                  // [pairs][16][tp] (several chunks)
   float* xshare = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * 16 * tp : 0);     // [warps] shares of a token's sum of x
   uint32_t* xmax = reinterpret_cast<uint32_t*>(xshare + kPWarps);        // [warps] largest |x| of a warp's share (bf16 bits)
-  float* sums = xshare + 2 * kPWarps;                                    // GROUPED: [groups of the chunk][TOKP] sum of x
+  // I8, in their place: [steps of the tokens] sum of x and factor of the sums
+  float* xsum = xshare;
+  float* xinv = xshare + kI8Units;
+  float* sums = xshare + (I8 ? 2 * kI8Units : 2 * kPWarps);              // GROUPED: [groups of the chunk][TOKP] sum of x
   const size_t sum_floats = GROUPED ? (size_t)p.spc * GPS * TOKP : 0;
   uint8_t* xs = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(sums + sum_floats) + 127) & ~static_cast<uintptr_t>(127));
-  uint8_t* ring = xs + (((size_t)p.M * p.x_pitch + 127) & ~static_cast<size_t>(127));
+  // I8: a row of x_pitch bytes per token and digit
+  uint8_t* ring = xs + (((size_t)p.M * (I8 ? 4 : 1) * p.x_pitch + 127) & ~static_cast<size_t>(127));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r8 = lane >> 2, c4 = lane & 3;
@@ -480,11 +544,19 @@ decode_prep_kernel(const PrepParams p) {
     const uint32_t hi = min((uint32_t)p.row_bytes, (uint32_t)(t_lo + n_t) * (Row::chunks * 16));
     for (int r = (int)threadIdx.x; r < (rg_end - rg0) * 8; r += kPThreads)
       prefetch_l2(p.P + ((size_t)rg0 * 8 + r) * p.row_bytes + lo, hi - lo);
-    issue_seek();
-  } else if (lane == 0) {
-    issue_seek();
-    issue_next();
   }
+  // What does not depend on the preceding kernel is worked out before the wait for it: where this warp's steps of
+  // the first chunk lie (the chunks after it look theirs up), and the tables of the final pass.
+  issue_seek();
+  const int lo_first = i_ch == 0 ? i_lin : 0, hi_first = i_ch == 0 ? i_hi : 0;
+  const int lp_first = i_ch == 0 ? i_lp : 0, tl_first = i_ch == 0 ? i_tl : 0;
+  const int last_first = hi_first > lo_first ? (hi_first - 1) / i_spc : -1;
+  if (warp == kPWarps - 1) share_bounds(spc_of(0));
+  if (!CANON && lane == 0) issue_next();
+  // I8: sixteen lanes take a step of a token, a lane half of what one of its strings becomes (the half is
+  // the warp's); the first of them
+  const int u_first = (int)(threadIdx.x >> 4) & 15;
+  const int tok_first = I8 && u_first >= n_t ? 1 : 0;
 
   // everything below reads X or writes Y: the preceding kernel must have completed
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -530,60 +602,55 @@ decode_prep_kernel(const PrepParams p) {
     // A token belongs to 16 / Mp warps (Mp: M rounded up to a power of two); a warp copies and turns
     // every (16 / Mp)-th step of its token, two at a time: lane 16 * j + 4 * s + c4 owns what string s
     // of the j-th of them meets in lanes c4 of the MMAs, so it needs no other thread's copies.
-    int mp = 1;
+    int mp = 1;                                                    // (fp16) M rounded up to a power of two
     while (mp < p.M) mp <<= 1;
-    const int wpt = kPWarps / mp;                                  // warps per token
-    const int tok = warp / wpt, sub = warp - tok * wpt;
-    const int str = (lane >> 2) & 3;                               // the lane's string of a step
-    uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + str * 256 + c4 * 16;
-    const int st0 = sub + (lane >> 4) * wpt;
-    if (tok < p.M)
-      for (int st = st0; st < spc_c; st += 2 * wpt)
+    if constexpr (I8) {
+      // Two turns of loads at a time, the digits of both behind them.  A step has a factor of its own, so no
+      // thread waits for another's activations.
+      const int str = (lane >> 2) & 3, units = p.M * spc_c;
+      const bool upper = warp >= kPWarps / 2;                      // which half of the string's registers
+      const __nv_bfloat16* xcol = p.X + col0 + str * 128 + (CANON ? c4 * 32 : c4 * 8);
+      for (int u0 = 0; u0 < units; u0 += 32) {
+        uint4 raw[2][4];
+        int tok[2], st[2];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          // the string's columns by eights: one in each of its four runs, or 32 in a row
-          const int col = st * kStepCols + str * 128 + (CANON ? c4 * 32 + r * 8 : r * 32 + c4 * 8);
-          uint8_t* dst = own + st * 1024 + r * 64;
-          if (col < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)tok * p.K + col0 + col);
-          else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    if (ch == 0 && (CANON || lane == 0))
-      for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
-    if (warp == kPWarps - 1) share_bounds(spc_c);                            // while the activations are on their way
-    asm volatile("cp.async.wait_group 0;" ::: "memory");           // (the ring's copies belong to no group)
-    {
-      uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
-      if (tok < p.M)
-        for (int st = st0; st < spc_c; st += 2 * wpt)
+        for (int i = 0; i < 2; ++i) {
+          const int u = u0 + u_first + i * 16;                     // (token, step), token-major; two tokens at most
+          tok[i] = u0 + i == 0 ? tok_first : u >= spc_c ? 1 : 0;
+          st[i] = u - (tok[i] ? spc_c : 0);
+          if (u >= units) tok[i] = -1;
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
-            const uint4 v = *reinterpret_cast<const uint4*>(own + st * 1024 + r * 64);
+            raw[i][r] = make_uint4(0u, 0u, 0u, 0u);
+            const int col = st[i] * kStepCols + (CANON ? r * 8 : r * 32);
+            if (tok[i] >= 0 && col + str * 128 + (CANON ? c4 * 32 : c4 * 8) < ccols)
+              raw[i][r] = __ldg(reinterpret_cast<const uint4*>(xcol + (size_t)tok[i] * p.K + col));
+          }
+        }
+        if (u0 == 0 && (CANON || lane == 0))
+          for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (u0 + i * 16 >= units) break;                         // (the same for all)
+          const bool live = tok[i] >= 0;
+          uint32_t mx = 0u;                                        // two largest |x|, as bf16 bits
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const uint4 v = raw[i][r];
             mx = __vmaxu2(__vmaxu2(mx, v.x & 0x7FFF7FFFu), v.y & 0x7FFF7FFFu);
             mx = __vmaxu2(__vmaxu2(mx, v.z & 0x7FFF7FFFu), v.w & 0x7FFF7FFFu);
           }
-      mx = __reduce_max_sync(0xffffffffu, max(mx & 0xFFFFu, mx >> 16));
-      if (lane == 0) xmax[warp] = mx;
-    }
-    __syncthreads();
-    if (tok < p.M) {
-      uint32_t mx = 0u;
-      for (int w = 0; w < wpt; ++w) mx = max(mx, xmax[tok * wpt + w]);
-      // factor 2^k, its exponent field: 15 - (E - 127) + 127 with E the largest one's, a finite number for all E
-      const int kf = min(269 - (int)(mx >> 7), 253);
-      const float up = __uint_as_float((uint32_t)kf << 23);        // 2^k, k = kf - 127 in [-113, 126]
-      float sx = 0.0f;                                             // this lane's share of the token's sum (times 2^k)
-      for (int sb = sub; sb < spc_c; sb += 2 * wpt) {
-        const int st = sb + (lane >> 4) * wpt;
-        const bool live = st < spc_c;
-        float hsum[2] = {0.0f, 0.0f};                              // of the string's first and second half
-        if (live) {
-          uint8_t* at = own + st * 1024;
+          mx = max(mx & 0xFFFFu, mx >> 16);
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          // |x| 2^k < 2^30 (2^-k a fp32 number: k <= 149), 2^k in two factors where it is not one
+          const int k = min(156 - (int)(mx >> 7), 149);
+          const float up = __uint_as_float((uint32_t)(min(k, 126) + 127) << 23);
           float v[32];
+          float hsum[2] = {0.0f, 0.0f};                            // of the string's first and second half
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint4 raw = *reinterpret_cast<const uint4*>(at + q * 64);
-            const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
+            const uint32_t wv[4] = {raw[i][q].x, raw[i][q].y, raw[i][q].z, raw[i][q].w};
             float t0 = 0.0f, t1 = 0.0f;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -594,47 +661,166 @@ decode_prep_kernel(const PrepParams p) {
             }
             hsum[q >> 1] += t0 + t1;
           }
-          *reinterpret_cast<uint4*>(at) = x_pairs<BITS, CANON, 0>(v);
-          *reinterpret_cast<uint4*>(at + 64) = x_pairs<BITS, CANON, 1>(v);
-          *reinterpret_cast<uint4*>(at + 128) = x_pairs<BITS, CANON, 2>(v);
-          *reinterpret_cast<uint4*>(at + 192) = x_pairs<BITS, CANON, 3>(v);
-        }
-        if (!GROUPED) {
-          sx += hsum[0] + hsum[1];
-        } else {
-          // a group of 64 columns is half a string of the four lanes c4, 128 a string, 256 two strings;
-          // in the units of the accumulators: 2^-24 for the codes
-          if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+          if (k > 126) {
+            const float up2 = __uint_as_float((uint32_t)(k - 126 + 127) << 23);
 #pragma unroll
-          for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
-            float t = hsum[h];
-            t += __shfl_xor_sync(0xffffffffu, t, 1);
-            t += __shfl_xor_sync(0xffffffffu, t, 2);
-            if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
-            const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
-            if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
-              sums[(size_t)(st * GPS + gi) * TOKP + tok] = t * 5.9604644775390625e-8f;
+            for (int e = 0; e < 32; ++e) v[e] *= up2;
+            hsum[0] *= up2;
+            hsum[1] *= up2;
+          }
+          if (live) {
+            uint8_t* at = xs + (size_t)tok[i] * 4 * p.x_pitch + st[i] * kStepCols + str * 128 + c4 * 16;
+            uint4 dig[4];
+            if (upper) {
+              x_digits<BITS, CANON, GSH == 1, 1>(v, dig);
+              at += 64;
+            } else {
+              x_digits<BITS, CANON, GSH == 1, 0>(v, dig);
+            }
+#pragma unroll
+            for (int d = 0; d < 4; ++d) *reinterpret_cast<uint4*>(at + d * p.x_pitch) = dig[d];
+          }
+          if (upper) continue;                                     // (the warp) the sums are the other half's
+          // 2^-k; an infinity or a NaN among the activations makes it a NaN, and with it the token
+          const float inv = mx >= 0x7F80u ? __uint_as_float(0x7FC00000u)
+                                          : __uint_as_float(k <= 126 ? (uint32_t)(127 - k) << 23 : 1u << (149 - k));
+          const int u = u0 + u_first + i * 16;
+          if (live && (lane & 15) == 0) xinv[u] = inv;
+          if (!GROUPED) {
+            float t = hsum[0] + hsum[1];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (live && (lane & 15) == 0) xsum[u] = t * inv;
+          } else {
+            if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+#pragma unroll
+            for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
+              float t = hsum[h];
+              t += __shfl_xor_sync(0xffffffffu, t, 1);
+              t += __shfl_xor_sync(0xffffffffu, t, 2);
+              if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
+              const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
+              // in the units of the upper two digits' sums
+              if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
+                sums[(size_t)(st[i] * GPS + gi) * TOKP + tok[i]] = t * (1.0f / 65536.0f);
+            }
           }
         }
       }
-      if (!GROUPED) {
+    } else {
+      const int wpt = kPWarps / mp;                                  // warps per token
+      const int tok = warp / wpt, sub = warp - tok * wpt;
+      const int str = (lane >> 2) & 3;                               // the lane's string of a step
+      uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + str * 256 + c4 * 16;
+      const int st0 = sub + (lane >> 4) * wpt;
+      if (tok < p.M)
+        for (int st = st0; st < spc_c; st += 2 * wpt)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        // 2^-k: its exponent field is 254 - kf, and 2^-126 (a normal number) at the least
-        if (lane == 0) xshare[warp] = sx * __uint_as_float((uint32_t)(254 - kf) << 23);
+          for (int r = 0; r < 4; ++r) {
+            // the string's columns by eights: one in each of its four runs, or 32 in a row
+            const int col = st * kStepCols + str * 128 + (CANON ? c4 * 32 + r * 8 : r * 32 + c4 * 8);
+            uint8_t* dst = own + st * 1024 + r * 64;
+            if (col < ccols) cp_async_16(smem_u32(dst), p.X + (size_t)tok * p.K + col0 + col);
+            else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+          }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (ch == 0 && (CANON || lane == 0))
+        for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
+      if (ch > 0 && warp == kPWarps - 1) share_bounds(spc_c);                  // while the activations are on their way
+      asm volatile("cp.async.wait_group 0;" ::: "memory");           // (the ring's copies belong to no group)
+      {
+        uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
+        if (tok < p.M)
+          for (int st = st0; st < spc_c; st += 2 * wpt)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const uint4 v = *reinterpret_cast<const uint4*>(own + st * 1024 + r * 64);
+              mx = __vmaxu2(__vmaxu2(mx, v.x & 0x7FFF7FFFu), v.y & 0x7FFF7FFFu);
+              mx = __vmaxu2(__vmaxu2(mx, v.z & 0x7FFF7FFFu), v.w & 0x7FFF7FFFu);
+            }
+        mx = __reduce_max_sync(0xffffffffu, max(mx & 0xFFFFu, mx >> 16));
+        if (lane == 0) xmax[warp] = mx;
       }
-      // what is left of 2^(24 - k) after 2^12, which is applied first
-      if (sub == 0 && lane == 0) tinv[tok] = __uint_as_float((uint32_t)(266 - kf) << 23);
+      __syncthreads();
+      if (tok < p.M) {
+        uint32_t mx = 0u;
+        for (int w = 0; w < wpt; ++w) mx = max(mx, xmax[tok * wpt + w]);
+        // factor 2^k, its exponent field: 15 - (E - 127) + 127 with E the largest one's, a finite number for all E
+        const int kf = min(269 - (int)(mx >> 7), 253);
+        const float up = __uint_as_float((uint32_t)kf << 23);        // 2^k, k = kf - 127 in [-113, 126]
+        float sx = 0.0f;                                             // this lane's share of the token's sum (times 2^k)
+        for (int sb = sub; sb < spc_c; sb += 2 * wpt) {
+          const int st = sb + (lane >> 4) * wpt;
+          const bool live = st < spc_c;
+          float hsum[2] = {0.0f, 0.0f};                              // of the string's first and second half
+          if (live) {
+            uint8_t* at = own + st * 1024;
+            float v[32];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint4 raw = *reinterpret_cast<const uint4*>(at + q * 64);
+              const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
+              float t0 = 0.0f, t1 = 0.0f;
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
+                v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
+                t0 += v[q * 8 + 2 * e];
+                t1 += v[q * 8 + 2 * e + 1];
+              }
+              hsum[q >> 1] += t0 + t1;
+            }
+            *reinterpret_cast<uint4*>(at) = x_pairs<BITS, CANON, 0>(v);
+            *reinterpret_cast<uint4*>(at + 64) = x_pairs<BITS, CANON, 1>(v);
+            *reinterpret_cast<uint4*>(at + 128) = x_pairs<BITS, CANON, 2>(v);
+            *reinterpret_cast<uint4*>(at + 192) = x_pairs<BITS, CANON, 3>(v);
+          }
+          if (!GROUPED) {
+            sx += hsum[0] + hsum[1];
+          } else {
+            // a group of 64 columns is half a string of the four lanes c4, 128 a string, 256 two strings;
+            // in the units of the accumulators: 2^-24 for the codes
+            if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+#pragma unroll
+            for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
+              float t = hsum[h];
+              t += __shfl_xor_sync(0xffffffffu, t, 1);
+              t += __shfl_xor_sync(0xffffffffu, t, 2);
+              if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
+              const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
+              if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
+                sums[(size_t)(st * GPS + gi) * TOKP + tok] = t * 5.9604644775390625e-8f;
+            }
+          }
+        }
+        if (!GROUPED) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
+          // 2^-k: its exponent field is 254 - kf, and 2^-126 (a normal number) at the least
+          if (lane == 0) xshare[warp] = sx * __uint_as_float((uint32_t)(254 - kf) << 23);
+        }
+        // what is left of 2^(24 - k) after 2^12, which is applied first
+        if (sub == 0 && lane == 0) tinv[tok] = __uint_as_float((uint32_t)(266 - kf) << 23);
+      }
     }
     __syncthreads();
 
     // a row per thread is fetched now and put down after the main loop, so that nothing waits for it
     if (!GROUPED) row_zs((int)threadIdx.x, z_own, s_own);
     // ---- this warp's steps of the chunk
-    const int lo = wbound[warp], hi = wbound[warp + 1];
-    const int first_pair = lo / spc_c, last_pair = hi > lo ? (hi - 1) / spc_c : -1;
+    int lo = lo_first, hi = hi_first, first_pair = lp_first, last_pair = last_first, tl = tl_first;
+    if (!I8 && ch > 0) {
+      lo = wbound[warp];
+      hi = wbound[warp + 1];
+      first_pair = lo / spc_c;
+      last_pair = hi > lo ? (hi - 1) / spc_c : -1;
+      tl = lo - first_pair * spc_c;
+    }
     int cur_pair = -1;
+    // I8: yv[0][0] and yv[0][1] are this lane's share of its two rows (rows r8 and r8 + 8), token c4 / 2, of the
+    // lower (c4 even) or upper two digits
     float acc[NT][4], acc2[NT][4], yv[NT][4];
+    const float zfac = (c4 & 1) ? -1.0f : 0.0f;
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -643,22 +829,33 @@ decode_prep_kernel(const PrepParams p) {
       float* mine = cur_pair == first_pair  ? part + (size_t)(warp * 2) * 16 * tp
                     : cur_pair == last_pair ? part + (size_t)(warp * 2 + 1) * 16 * tp
                                             : ywhole + (size_t)cur_pair * 16 * tp;
+      if constexpr (I8) {
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int tk = nt * 8 + c4 * 2;
-        float v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
-        if (tk < toks) {
-          const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
-          *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0] * f.x, v[1] * f.y);
-          *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2] * f.x, v[3] * f.y);
+        for (int e = 0; e < 2; ++e) {
+          float v = (c4 & 1) ? yv[0][e] * 65536.0f : yv[0][e];
+          v += __shfl_xor_sync(0xffffffffu, v, 1);
+          if ((c4 & 1) == 0) mine[(r8 + 8 * e) * tp + (c4 >> 1)] = v;
+          yv[0][e] = 0.0f;
         }
+      } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
+        for (int nt = 0; nt < NT; ++nt) {
+          const int tk = nt * 8 + c4 * 2;
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
+          if (tk < toks) {
+            const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
+            *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0] * f.x, v[1] * f.y);
+            *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2] * f.x, v[3] * f.y);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
+        }
       }
     };
-    const uint8_t* xl = xs + (size_t)(r8 < p.M ? r8 : 0) * p.x_pitch + c4 * 16;
+    // I8: this lane's column of the MMAs is digit r8 % 4 of token r8 / 4
+    const uint8_t* xl = xs + (size_t)(I8 ? (p.M > 1 ? r8 : r8 & 3) : r8 < p.M ? r8 : 0) * p.x_pitch + c4 * 16;
     const uint8_t* xh = xs + (size_t)(r8 + 8 < p.M ? r8 + 8 : 0) * p.x_pitch + c4 * 16;
 
     // tasks of this lane's two tokens (grouped scales with a table per task)
@@ -666,10 +863,11 @@ decode_prep_kernel(const PrepParams p) {
     if (TASKS) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)
-        if (c4 * 2 + e < p.M) task_of[e] = min(max(__ldg(p.task_ids + c4 * 2 + e), 0), p.n_tasks - 1);
+        if ((I8 ? c4 >> 1 : c4 * 2 + e) < p.M)
+          task_of[e] = min(max(__ldg(p.task_ids + (I8 ? c4 >> 1 : c4 * 2 + e)), 0), p.n_tasks - 1);
     }
     int lin = lo;
-    int lp = lo / spc_c, tl = lo - lp * spc_c;
+    int lp = first_pair;
     while (ok && lin < hi) {
       const int nsteps = (p.sps == 2 && lin + 1 < hi && tl + 1 < spc_c) ? 2 : 1;
       const int slot = c_slot;
@@ -722,7 +920,7 @@ decode_prep_kernel(const PrepParams p) {
         // where a group ends, their latency was on the path of every group
         const int rowa = pair_rg(lp) * 8 + r8, rowb = rowa + 8;
         const int gstep0 = (t_lo + ch * p.spc + tl) * GPS;         // first group of the step
-        constexpr int TG = GROUPED ? GPS : 1, NS = TASKS ? 2 : 1;
+        constexpr int TG = GROUPED ? GPS : 1, NS = TASKS && !I8 ? 2 : 1;
         float gsa[NS][TG], gsb[NS][TG];
         uint32_t gza[(TG + 3) / 4], gzb[(TG + 3) / 4];             // four zero-points to a word
         if (GROUPED) {
@@ -735,78 +933,139 @@ decode_prep_kernel(const PrepParams p) {
             load_groups<TG>(tab + (size_t)rowb * p.G, p.G - gstep0, has_b, p.G, gsb[e]);
           }
         }
-        // group gi of the step begins: one of its two accumulators starts at -z * sum x ...
-        auto begin = [&](int gi) {
-          const int q = gi % TG;
-          const float za = -(float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
-          const float zb = -(float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+        if constexpr (I8) {
+          // per string (a lane's 32 columns) four MMAs; a group is half a string (two MMAs), a string or two
+          const uint32_t* fa = reinterpret_cast<const uint32_t*>(w.a);
+          const uint32_t* fb = reinterpret_cast<const uint32_t*>(w.b);
+          const uint8_t* x0 = xl + (size_t)tl * kStepCols;
+          int d0[4], d1[4];
+          float ys[2] = {0.0f, 0.0f};              // of the step, in units of 2^-k
+          // rows r8 (d[0], d[1]: the lower and the higher of two digits) and r8 + 8; exact in 32 bits for 256 columns
+          auto value = [&](const int (&d)[4], int e) { return (float)(d[2 * e] + d[2 * e + 1] * 256); };
+          auto flush = [&](int gi, const int (&d)[4]) {
+            const int q = gi % TG;
+            const float sx = sums[(size_t)(tl * GPS + gi) * TOKP + (c4 >> 1)] * zfac;
+            const float za = (float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+            const float zb = (float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+            ys[0] = fmaf(gsa[0][q], fmaf(za, sx, value(d, 0)), ys[0]);
+            ys[1] = fmaf(gsb[0][q], fmaf(zb, sx, value(d, 1)), ys[1]);
+          };
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const float2 sx = *reinterpret_cast<const float2*>(sums + (size_t)(tl * GPS + gi) * TOKP + nt * 8 + c4 * 2);
-            acc2[nt][0] = za * sx.x;
-            acc2[nt][1] = za * sx.y;
-            acc2[nt][2] = zb * sx.x;
-            acc2[nt][3] = zb * sx.y;
-          }
-        };
-        // ... and ends: scale
-        auto flush = [&](int gi) {
-          const int q = gi % TG;
+          for (int s = 0; s < 4; ++s) {
+            uint32_t wa[BITS], wb[BITS], ra[8], rb[8];
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              yv[nt][e] = fmaf(gsa[e % NS][q], acc[nt][e] + acc2[nt][e], yv[nt][e]);
-              yv[nt][2 + e] = fmaf(gsb[e % NS][q], acc[nt][2 + e] + acc2[nt][2 + e], yv[nt][2 + e]);
+            for (int e = 0; e < BITS; ++e) {
+              wa[e] = fa[s * BITS + e];
+              wb[e] = fb[s * BITS + e];
             }
-        };
-
-        const uint32_t* fa = reinterpret_cast<const uint32_t*>(w.a);
-        const uint32_t* fb = reinterpret_cast<const uint32_t*>(w.b);
-        const uint8_t* x0 = xl + (size_t)tl * (kStepCols * 2);
-        const uint8_t* x1 = xh + (size_t)tl * (kStepCols * 2);
+            dq::i8_string<BITS, GSH == 1>(wa, ra);
+            dq::i8_string<BITS, GSH == 1>(wb, rb);
+            const uint4 xa = *reinterpret_cast<const uint4*>(x0 + s * 128);
+            const uint4 xb = *reinterpret_cast<const uint4*>(x0 + s * 128 + 64);
+            constexpr bool kHalf = GSH == 1;
+            const bool fresh = GSH == 1 || GSH == 2 || s == 0 || (GSH == 3 && (s & 1) == 0);
+            // two chains of MMAs, so that they do not wait for one another; half a string (kHalf): a chain each
+            if (fresh) {
+              imma_16832<true>(d0, ra[0], rb[0], ra[1], rb[1], xa.x, xa.y);
+              imma_16832<true>(d1, ra[4], rb[4], ra[5], rb[5], xb.x, xb.y);
+            } else {
+              imma_16832<false>(d0, ra[0], rb[0], ra[1], rb[1], xa.x, xa.y);
+              imma_16832<false>(d1, ra[4], rb[4], ra[5], rb[5], xb.x, xb.y);
+            }
+            imma_16832<false>(d0, ra[2], rb[2], ra[3], rb[3], xa.z, xa.w);
+            imma_16832<false>(d1, ra[6], rb[6], ra[7], rb[7], xb.z, xb.w);
+            if (kHalf) {
+              flush(2 * s, d0);
+              flush(2 * s + 1, d1);
+            } else if (GROUPED && (RUNS_PER_GROUP == 4 || (s & 1))) {
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          uint32_t wa[BITS], wb[BITS];
-#pragma unroll
-          for (int e = 0; e < BITS; ++e) {
-            wa[e] = fa[s * BITS + e];
-            wb[e] = fb[s * BITS + e];
+              for (int e = 0; e < 4; ++e) d0[e] += d1[e];
+              flush(RUNS_PER_GROUP == 4 ? s : s >> 1, d0);
+            }
           }
-          const uint8_t* xs0 = x0 + s * 256;
-          const uint8_t* xs1 = x1 + s * 256;
-          constexpr bool kHalf = GROUPED && RUNS_PER_GROUP == 2;     // a group is half a string
-          if (GROUPED && RUNS_PER_GROUP <= 4) begin(kHalf ? 2 * s : s);
-          if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) begin(s >> 1);
-          constexpr bool kFresh = GROUPED && RUNS_PER_GROUP <= 4;
-          if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) {
+          if (!GROUPED) {
+            // a step's sums of one digit are below 2^24: exact as fp32, each chain's
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              ys[e] = fmaf(256.0f, (float)(d0[2 * e + 1] + d1[2 * e + 1]), (float)(d0[2 * e] + d1[2 * e]));
+          }
+          const float inv = xinv[(p.M > 1 && c4 >= 2 ? spc_c : 0) + tl];
+          yv[0][0] = fmaf(ys[0], inv, yv[0][0]);
+          yv[0][1] = fmaf(ys[1], inv, yv[0][1]);
+        } else {
+          // group gi of the step begins: one of its two accumulators starts at -z * sum x ...
+          auto begin = [&](int gi) {
+            const int q = gi % TG;
+            const float za = -(float)((gza[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+            const float zb = -(float)((gzb[q >> 2] >> (8 * (q & 3))) & 0xFFu);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+              const float2 sx = *reinterpret_cast<const float2*>(sums + (size_t)(tl * GPS + gi) * TOKP + nt * 8 + c4 * 2);
+              acc2[nt][0] = za * sx.x;
+              acc2[nt][1] = za * sx.y;
+              acc2[nt][2] = zb * sx.x;
+              acc2[nt][3] = zb * sx.y;
+            }
+          };
+          // ... and ends: scale
+          auto flush = [&](int gi) {
+            const int q = gi % TG;
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-              for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
-          }
-          if (has_b) {
-            run_mma2<BITS, NT, true, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, true, 1, false>(wa, wb, xs0, xs1, acc, acc2);
-            if (kHalf) {
-              flush(2 * s);
-              begin(2 * s + 1);
+              for (int e = 0; e < 2; ++e) {
+                yv[nt][e] = fmaf(gsa[e % NS][q], acc[nt][e] + acc2[nt][e], yv[nt][e]);
+                yv[nt][2 + e] = fmaf(gsb[e % NS][q], acc[nt][2 + e] + acc2[nt][2 + e], yv[nt][2 + e]);
+              }
+          };
+
+          const uint32_t* fa = reinterpret_cast<const uint32_t*>(w.a);
+          const uint32_t* fb = reinterpret_cast<const uint32_t*>(w.b);
+          const uint8_t* x0 = xl + (size_t)tl * (kStepCols * 2);
+          const uint8_t* x1 = xh + (size_t)tl * (kStepCols * 2);
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            uint32_t wa[BITS], wb[BITS];
+#pragma unroll
+            for (int e = 0; e < BITS; ++e) {
+              wa[e] = fa[s * BITS + e];
+              wb[e] = fb[s * BITS + e];
             }
-            run_mma2<BITS, NT, true, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, true, 3, false>(wa, wb, xs0, xs1, acc, acc2);
-          } else {
-            run_mma2<BITS, NT, false, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, false, 1, false>(wa, wb, xs0, xs1, acc, acc2);
-            if (kHalf) {
-              flush(2 * s);
-              begin(2 * s + 1);
+            const uint8_t* xs0 = x0 + s * 256;
+            const uint8_t* xs1 = x1 + s * 256;
+            constexpr bool kHalf = GROUPED && RUNS_PER_GROUP == 2;     // a group is half a string
+            if (GROUPED && RUNS_PER_GROUP <= 4) begin(kHalf ? 2 * s : s);
+            if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) begin(s >> 1);
+            constexpr bool kFresh = GROUPED && RUNS_PER_GROUP <= 4;
+            if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1) == 0) {
+#pragma unroll
+              for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
             }
-            run_mma2<BITS, NT, false, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
-            run_mma2<BITS, NT, false, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+            if (has_b) {
+              run_mma2<BITS, NT, true, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
+              run_mma2<BITS, NT, true, 1, false>(wa, wb, xs0, xs1, acc, acc2);
+              if (kHalf) {
+                flush(2 * s);
+                begin(2 * s + 1);
+              }
+              run_mma2<BITS, NT, true, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
+              run_mma2<BITS, NT, true, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+            } else {
+              run_mma2<BITS, NT, false, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
+              run_mma2<BITS, NT, false, 1, false>(wa, wb, xs0, xs1, acc, acc2);
+              if (kHalf) {
+                flush(2 * s);
+                begin(2 * s + 1);
+              }
+              run_mma2<BITS, NT, false, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
+              run_mma2<BITS, NT, false, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+            }
+            if (kHalf) flush(2 * s + 1);
+            if (GROUPED && RUNS_PER_GROUP == 4) flush(s);
+            if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1)) flush(s >> 1);
           }
-          if (kHalf) flush(2 * s + 1);
-          if (GROUPED && RUNS_PER_GROUP == 4) flush(s);
-          if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1)) flush(s >> 1);
         }
         if (j + 1 == nsteps) {
           // Every lane has read its part of the slot: it can be refilled.  Behind the step's MMAs, where
@@ -831,9 +1090,18 @@ decode_prep_kernel(const PrepParams p) {
     if (cur_pair >= 0) park();
     if (!GROUPED) {
       if (warp == kPWarps - 1) {                       // the tokens' sums of x from their warps' shares
-        float t = lane < kPWarps ? xshare[lane] : 0.0f;
-        for (int o = kPWarps / mp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane < kPWarps && (lane & (kPWarps / mp - 1)) == 0) tsum[lane / (kPWarps / mp)] = t;
+        if constexpr (I8) {
+          for (int m = 0; m < p.M; ++m) {
+            float t = 0.0f;
+            for (int st = lane; st < spc_c; st += 32) t += xsum[m * spc_c + st];
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) tsum[m] = t;
+          }
+        } else {
+          float t = lane < kPWarps ? xshare[lane] : 0.0f;
+          for (int o = kPWarps / mp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          if (lane < kPWarps && (lane & (kPWarps / mp - 1)) == 0) tsum[lane / (kPWarps / mp)] = t;
+        }
       }
       if (threadIdx.x < npairs * 16) rowzs[threadIdx.x] = make_float2((float)z_own, s_own);
       for (int r = threadIdx.x + kPThreads; r < npairs * 16; r += kPThreads) {
@@ -1035,6 +1303,7 @@ __global__ void prep_layout_kernel(const uint32_t* __restrict__ src, uint32_t* _
 
 struct PrepPlan {
   int rg_per_cta, grid, T, spc, nchunks, slots, sps, x_pitch, pairs, cshift;
+  bool i8;
   size_t smem;
   long long ns;      // estimated time
 };
@@ -1056,7 +1325,10 @@ int x_pitch_for(int steps) {
 // two token tiles), 10 per token and step staged, 2500 for the cluster's exchange, 1500 + 400 M per
 // further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at 22016 x 8192
 // 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
-int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* plan) {
+//
+// i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
+// staged at once, at most two steps to a half-warp.
+int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
   const int NT = M <= 8 ? 1 : 2, TOKP = 8 * NT;
@@ -1069,6 +1341,7 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* pl
   const bool one_group = gcols >= K;
   // clusters of 1, 2, 4, 8 CTAs that run at once (the larger ones leave SMs of a GPC idle)
   const int active[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
+  auto pitch_for = [&](int spc) { return i8 ? spc * kStepCols + 64 : x_pitch_for(spc); };    // i8: of a digit
   plan->ns = -1;
   for (int ci = 0; ci < 4; ++ci)
     for (int waves = 1; waves <= (ci ? 2 : 1); ++waves) {
@@ -1086,15 +1359,15 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* pl
         size_t b = 128 + kPHeadBytes + (kPWarps * 2 + c.pairs) * sums;
         if (spc < Tl) b += c.pairs * sums;
         b += (size_t)((c.pairs + 3) & ~3) * 4 + (size_t)c.pairs * 16 * 8;
-        b += ((grouped ? (size_t)spc * gps * TOKP : 0) + 2 * kPWarps) * 4 + 128;
-        b += (((size_t)M * x_pitch_for(spc)) + 127) / 128 * 128;
+        b += ((grouped ? (size_t)spc * gps * TOKP : 0) + (i8 ? 2 * kI8Units : 2 * kPWarps)) * 4 + 128;
+        b += (((size_t)M * (i8 ? 4 : 1) * pitch_for(spc)) + 127) / 128 * 128;
         b += (size_t)kPWarps * slots * sps * step_bytes;
         return b;
       };
       // ring shapes in order of preference: bytes in flight first, larger copies on a tie
       const int shapes[4][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}};   // {slots, steps per slot}
       // all of the CTA's K staged at once, with the best ring that fits ...
-      if (grouped || one_group) {
+      if ((grouped || one_group) && (!i8 || M * Tl <= kI8Units)) {
         for (int i = canon ? 1 : 0; i < 4 && c.spc == 0; ++i)
           if (need(Tl, shapes[i][0], shapes[i][1]) <= (size_t)kPSmemLimit) {
             c.spc = Tl;
@@ -1103,7 +1376,7 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* pl
           }
       }
       // ... else (one CTA per range) the largest chunk of steps beside a ring of two single steps
-      if (c.spc == 0 && ci == 0) {
+      if (c.spc == 0 && ci == 0 && !i8) {
         for (int spc = c.T; spc >= 1 && c.spc == 0; --spc) {
           if (!grouped && !one_group && (steps_per_group % spc) != 0) continue;
           if (need(spc, 2, 1) <= (size_t)kPSmemLimit) {
@@ -1115,10 +1388,11 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* pl
       }
       if (c.spc == 0) continue;
       c.nchunks = (Tl + c.spc - 1) / c.spc;
-      c.x_pitch = x_pitch_for(c.spc);
+      c.x_pitch = pitch_for(c.spc);
+      c.i8 = i8;
       c.smem = need(c.spc, c.slots, c.sps);
       const long long steps = ((long long)c.rg_per_cta * Tl + 1) / 2;
-      const long long per_step = (grouped ? 3000 : 1600) * (NT == 2 ? 13 : 10) / 10;
+      const long long per_step = i8 ? (grouped ? 1900 : 1000) : (grouped ? 3000 : 1600) * (NT == 2 ? 13 : 10) / 10;
       c.ns = waves * ((steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * 10 + 4000 + (ci ? 2500 : 0) +
                       (c.nchunks - 1) * (1500 + 400 * M)) + (waves - 1) * 10000;
       if (plan->ns < 0 || c.ns < plan->ns) *plan = c;
@@ -1126,9 +1400,9 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, PrepPlan* pl
   return plan->ns < 0 ? PEQA_ERR_TOO_LARGE : PEQA_OK;
 }
 
-template <int BITS, int NT, int GSH, bool TASKS, bool CANON>
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8>
 int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS, CANON>;
+  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS, CANON, I8>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, kPSmemLimit, done));
   cudaLaunchConfig_t cfg = {};
@@ -1149,26 +1423,28 @@ int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
   return PEQA_OK;
 }
 
-template <int BITS, int NT, bool TASKS, bool CANON>
+template <int BITS, int NT, bool TASKS, bool CANON, bool I8>
 int launch_prep_g(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
   switch (gsh) {
     case 1:
-      if constexpr (!CANON) return launch_prep_t<BITS, NT, 1, TASKS, CANON>(p, grid, smem, st);
+      if constexpr (!CANON) return launch_prep_t<BITS, NT, 1, TASKS, CANON, I8>(p, grid, smem, st);
       return PEQA_ERR_BAD_SHAPE;
-    case 2: return launch_prep_t<BITS, NT, 2, TASKS, CANON>(p, grid, smem, st);
-    case 3: return launch_prep_t<BITS, NT, 3, TASKS, CANON>(p, grid, smem, st);
-    default: return launch_prep_t<BITS, NT, 0, false, CANON>(p, grid, smem, st);   // tasks: looked up per row
+    case 2: return launch_prep_t<BITS, NT, 2, TASKS, CANON, I8>(p, grid, smem, st);
+    case 3: return launch_prep_t<BITS, NT, 3, TASKS, CANON, I8>(p, grid, smem, st);
+    default: return launch_prep_t<BITS, NT, 0, false, CANON, I8>(p, grid, smem, st);   // tasks: looked up per row
   }
 }
 
-template <int BITS>
-int launch_prep_b(const PrepParams& p, bool canon, int gsh, int grid, size_t smem, cudaStream_t st) {
-  if (canon)
-    return p.M > 8 ? launch_prep_g<BITS, 2, false, true>(p, gsh, grid, smem, st)
-                   : launch_prep_g<BITS, 1, false, true>(p, gsh, grid, smem, st);
-  if (p.M > 8) return launch_prep_g<BITS, 2, false, false>(p, gsh, grid, smem, st);
-  return p.task_ids ? launch_prep_g<BITS, 1, true, false>(p, gsh, grid, smem, st)
-                    : launch_prep_g<BITS, 1, false, false>(p, gsh, grid, smem, st);
+template <int BITS, bool CANON>
+int launch_prep_b(const PrepParams& p, bool i8, int gsh, int grid, size_t smem, cudaStream_t st) {
+  if (p.M > 8) return launch_prep_g<BITS, 2, false, CANON, false>(p, gsh, grid, smem, st);
+  if constexpr (!CANON) {
+    if (p.task_ids)
+      return i8 ? launch_prep_g<BITS, 1, true, false, true>(p, gsh, grid, smem, st)
+                : launch_prep_g<BITS, 1, true, false, false>(p, gsh, grid, smem, st);
+  }
+  return i8 ? launch_prep_g<BITS, 1, false, CANON, true>(p, gsh, grid, smem, st)
+            : launch_prep_g<BITS, 1, false, CANON, false>(p, gsh, grid, smem, st);
 }
 
 int check_prep_layer(const peqa_qweight_t* w) {
@@ -1191,11 +1467,11 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
   bool two = false;
   if (M > 8) {
     PrepPlan half;
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, canon, &half));
-    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, &plan) != PEQA_OK ||
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, canon, false, &half));
+    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, false, &plan) != PEQA_OK ||
           2 * half.ns < plan.ns;
-  } else {
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, &plan));
+  } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, true, &plan) != PEQA_OK) {
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, false, &plan));
   }
   if (two) {
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
@@ -1234,16 +1510,19 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
   p.row_bytes = p.K / 8 * w->bits;
   PEQA_TRY(status_word(st, &p.status));
   const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
-  return w->bits == 3 ? launch_prep_b<3>(p, canon, gsh, plan.grid, plan.smem, st)
-                      : launch_prep_b<4>(p, canon, gsh, plan.grid, plan.smem, st);
+  if (canon)
+    return w->bits == 3 ? launch_prep_b<3, true>(p, plan.i8, gsh, plan.grid, plan.smem, st)
+                        : launch_prep_b<4, true>(p, plan.i8, gsh, plan.grid, plan.smem, st);
+  return w->bits == 3 ? launch_prep_b<3, false>(p, plan.i8, gsh, plan.grid, plan.smem, st)
+                      : launch_prep_b<4, false>(p, plan.i8, gsh, plan.grid, plan.smem, st);
 }
 
 }  // namespace
 
 bool decode_rows_supported(const peqa_qweight_t* w, int g, int M) {
   PrepPlan plan;
-  return w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == 128 || g == 256) &&
-         plan_prep(w->out_features, w->in_features, M > 8 ? (M + 1) / 2 : M, w->bits, g, true, &plan) == PEQA_OK;
+  return w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == w->in_features || g == 128 || g == 256) &&
+         plan_prep(w->out_features, w->in_features, M > 8 ? (M + 1) / 2 : M, w->bits, g, true, false, &plan) == PEQA_OK;
 }
 
 int launch_decode_rows(const peqa_qweight_t* w, int g, const void* X, int M, void* Y, const float* scale_table,

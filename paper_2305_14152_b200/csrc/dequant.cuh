@@ -331,5 +331,81 @@ __device__ __forceinline__ uint32_t f16_pair(const uint32_t (&w)[BITS]) {
   return x & mask;
 }
 
+// ---------------------------------------------------------------------------
+// Codes as unsigned bytes, for integer MMAs.  A code inside a byte of a word of the string, at bit o of it,
+// is q * 2^o, so one AND makes four operands: 4-bit strings are eight ANDs for 32 codes, without a shift.
+// Of a 3-bit string's 32 codes 24 lie inside a byte (six ANDs); the eight that straddle two are
+// gathered into two words (two shifts and two logic operations each).  The factor 2^o is taken out of the
+// activation the code meets.  Register r (0..7) of a string, byte b, holds the code at position
+// i8_pos, times 2^i8_o; registers 2j and 2j + 1 are one MMA's.  HALF: registers 0..3 hold the
+// string's columns 0..15 and 4..7 its columns 16..31 (four byte permutations more for 3-bit strings).
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int i8_pos(int bits, bool half, int r, int b) {
+  if (bits == 4) return 8 * (r / 2) + 2 * b + (r & 1);
+  constexpr int plain[8][4] = {{0, 3, 6, 8},     {1, 4, 7, 9},     {11, 14, 16, 19}, {12, 15, 17, 20},
+                               {22, 24, 27, 30}, {23, 25, 28, 31}, {2, 5, 13, 10},   {18, 21, 29, 26}};
+  constexpr int halves[8][4] = {{0, 3, 6, 8},     {1, 4, 7, 9},     {11, 2, 16, 5},   {12, 13, 17, 10},
+                                {22, 24, 27, 30}, {23, 25, 28, 31}, {14, 18, 19, 21}, {15, 29, 20, 26}};
+  return half ? halves[r][b] : plain[r][b];
+}
+__host__ __device__ constexpr int i8_o(int bits, bool half, int r, int b) {
+  const int p = i8_pos(bits, half, r, b);
+  if (bits == 4) return 4 * (p & 1);
+  switch (p) {                                     // the gathered ones
+    case 2: case 10: case 13: case 18: case 26: case 29: return 0;
+    case 5: case 21: return 1;
+    default: return 3 * p % 8;
+  }
+}
+// string column of the code at position p
+__host__ __device__ constexpr int position_column(int bits, bool canon, int p) {
+  return canon ? p : string_column(bits, bits * p);
+}
+__host__ __device__ constexpr bool i8_ok(int bits, bool half) {
+  uint32_t seen = 0u;
+  for (int r = 0; r < 8; ++r)
+    for (int b = 0; b < 4; ++b) {
+      const int p = i8_pos(bits, half, r, b);
+      if (i8_o(bits, half, r, b) + bits > 8) return false;
+      if (half && string_column(bits, bits * p) / 16 != r / 4) return false;
+      seen |= 1u << p;
+    }
+  return seen == 0xFFFFFFFFu;
+}
+static_assert(i8_ok(3, false) && i8_ok(3, true) && i8_ok(4, false) && i8_ok(4, true), "every code once, inside its byte");
+
+template <int BITS, bool HALF>
+__device__ __forceinline__ void i8_string(const uint32_t (&w)[BITS], uint32_t (&r)[8]) {
+  if constexpr (BITS == 4) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      r[2 * j] = w[j] & 0x0F0F0F0Fu;
+      r[2 * j + 1] = w[j] & 0xF0F0F0F0u;
+    }
+  } else {
+    r[0] = w[0] & 0x071C0E07u;
+    r[1] = w[0] & 0x38E07038u;
+    const uint32_t l1 = w[1] & 0x0E071C0Eu, h1 = w[1] & 0x7038E070u;
+    // positions 2, 5, 10 (bits 6, 15, 30) and 13 (bit 39); 18, 21, 26 (54, 63, 78) and 29 (87)
+    const uint32_t s1 = lop3_and_or(w[1] << 9, 0x00070000u, __funnelshift_r(w[0], w[1], 6) & 0x07000E07u);
+    const uint32_t s2 = lop3_and_or(w[2] >> 7, 0x00070000u, __funnelshift_r(w[1], w[2], 22) & 0x07000E07u);
+    if constexpr (HALF) {
+      r[2] = prmt(l1, s1, 0x5240u);
+      r[3] = prmt(h1, s1, 0x7260u);
+      r[4] = w[2] & 0x1C0E071Cu;
+      r[5] = w[2] & 0xE07038E0u;
+      r[6] = prmt(l1, s2, 0x5341u);
+      r[7] = prmt(h1, s2, 0x7361u);
+    } else {
+      r[2] = l1;
+      r[3] = h1;
+      r[4] = w[2] & 0x1C0E071Cu;
+      r[5] = w[2] & 0xE07038E0u;
+      r[6] = s1;
+      r[7] = s2;
+    }
+  }
+}
+
 }  // namespace dq
 }  // namespace peqa
