@@ -48,8 +48,7 @@ constexpr int X_GROUPS = 4;
 constexpr int kDxThreads = 896;  // warps: 0 act TMA, 1 MMA, 2 TMEM alloc, 3 code TMA, 4-11 epilogue, 12-27 dequant
 
 struct DxBarriers {
-  uint64_t full_act[XSTAGES];   // leader: dY bytes of both CTAs landed
-  uint64_t full_w[XSTAGES];     // leader: weight halves of both CTAs written
+  uint64_t full[XSTAGES];       // leader: both CTAs' dY landed and weight halves written
   uint64_t empty[XSTAGES];      // each CTA: MMAs that read the stage completed
   uint64_t pk_full[XQ_SLOTS];   // each CTA: packed codes landed
   uint64_t pk_empty[XQ_SLOTS];  // each CTA: the owning group has read the slot
@@ -94,8 +93,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
-      mbar_init(smem_u32(&bars->full_act[s]), 1);
-      mbar_init(smem_u32(&bars->full_w[s]), 8);           // 4 warps of one group in each CTA
+      mbar_init(smem_u32(&bars->full[s]), 1 + 8);         // the dY copies, 4 warps of one group in each CTA
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
     for (int q = 0; q < XQ_SLOTS; ++q) {
@@ -142,8 +140,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
           const int s = it % XSTAGES;
           const uint32_t ph = (it / XSTAGES) & 1u;
           if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
-          if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full_act[s]), 2 * blocks * XBLK_BYTES);
-          const uint32_t bar = mapa_shared(smem_u32(&bars->full_act[s]), 0);
+          if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full[s]), 2 * blocks * XBLK_BYTES);
+          const uint32_t bar = mapa_shared(smem_u32(&bars->full[s]), 0);
           tma_load_2d_pair(smem_u32(base + s * XSTAGE_BYTES), &tmap_dy, bar, kb * XK, t0);
           if (blocks == 2)
             tma_load_2d_pair(smem_u32(base + s * XSTAGE_BYTES + XBLK_BYTES), &tmap_dy, bar, kb * XK, t0 + 256);
@@ -172,8 +170,18 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   } else if (warp == 1) {
     // ------------------------------------------ MMA issuer (leader CTA, one lane)
     if (leader && lane == 0) {
+      // One thread issues everything and a tensor core holds little more than the MMA it works on, so
+      // what this thread does between the last MMA of a stage and the first of the next is a gap in the
+      // tensor pipe.  Weights and activations share a barrier, the next stage's is asked for before the
+      // last MMA of this one (its answer takes about 100 cycles, an MMA 128), and descriptors are
+      // advanced by additions (the address field counts 16-byte units).
       constexpr uint32_t idesc = idesc_bf16_f32(256, 256, 0, 1);
-      uint32_t it = 0;
+      const uint32_t a0 = smem_u32(base);
+      const uint64_t adesc0 = smem_desc_sw128(a0, 16, 1024);
+      const uint64_t bdesc0 = smem_desc_sw128(a0 + XA_BYTES, 64 * 128, 1024);
+      const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
+      uint32_t s = 0, ph = 0;
+      bool ready = false;
       int local = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
@@ -181,23 +189,28 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
         pair_item(p.items, tile, p.T, j_tile, tt0, blocks);
         if (!mbar_wait_cluster(smem_u32(&bars->acc_empty), (uint32_t)(local & 1) ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int s = it % XSTAGES;
-          const uint32_t ph = (it / XSTAGES) & 1u;
-          if (!mbar_wait_cluster(smem_u32(&bars->full_w[s]), ph, abort_flag) ||
-              !mbar_wait_cluster(smem_u32(&bars->full_act[s]), ph, abort_flag)) { ok = false; break; }
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          if (!ready && !mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(base + s * XSTAGE_BYTES);
-          const uint32_t b_addr = a_addr + XA_BYTES;
-          for (int m = 0; m < blocks; ++m) {
-#pragma unroll
-            for (int k = 0; k < XK / 16; ++k) {
-              const uint64_t adesc = smem_desc_sw128(a_addr + m * XBLK_BYTES + k * 32, 16, 1024);
-              const uint64_t bdesc = smem_desc_sw128(b_addr + k * (16 * 128), 64 * 128, 1024);
-              mma_bf16_ss_pair(tmem_base + m * 256, adesc, bdesc, idesc, (kb | k) != 0 ? 1u : 0u);
-            }
+          const uint64_t adesc = adesc0 + s * (XSTAGE_BYTES >> 4), bdesc = bdesc0 + s * (XSTAGE_BYTES >> 4);
+          const uint32_t at = s;
+          if (++s == XSTAGES) {
+            s = 0;
+            ph ^= 1u;
           }
-          mma_commit_pair(smem_u32(&bars->empty[s]), 3);
+          if (blocks == 2) {
+#pragma unroll
+            for (int k = 0; k < XK / 16; ++k)
+              mma_bf16_ss_pair(tmem_base, adesc + k * (32 / 16), bdesc + k * (16 * 128 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          const uint64_t alast = blocks == 2 ? adesc + (XBLK_BYTES >> 4) : adesc;
+          const uint32_t dlast = blocks == 2 ? tmem_base + 256 : tmem_base;
+#pragma unroll
+          for (int k = 0; k < XK / 16; ++k) {
+            if (k == XK / 16 - 1) ready = mbar_test_cluster(full0 + s * 8, ph);
+            mma_bf16_ss_pair(dlast, alast + k * (32 / 16), bdesc + k * (16 * 128 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          mma_commit_pair(empty0 + at * 8, 3);
         }
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full), 3);
       }
@@ -277,7 +290,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
     const int swz = row_a & 7;
     const uint32_t off_a = (uint32_t)((u4 >> 1) * (64 * 128) + row_a * 128);
     const uint32_t off_b = (uint32_t)((u4 >> 1) * (64 * 128) + row_b * 128);
-    const uint32_t full_w_leader0 = mapa_shared(smem_u32(&bars->full_w[0]), 0);
+    const uint32_t full_leader0 = mapa_shared(smem_u32(&bars->full[0]), 0);
     const uint32_t total_it = (uint32_t)my_tiles * (uint32_t)p.k_blocks;
     int pf_tile = pair, pf_kb = grp;
     while (pf_kb >= p.k_blocks) { pf_kb -= p.k_blocks; pf_tile += n_pairs; }
@@ -362,7 +375,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       // make the tile visible to the tensor cores of both CTAs, then tell the leader
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster_release(full_w_leader0 + s * 8);
+      if (lane == 0) mbar_arrive_cluster_release(full_leader0 + s * 8);
       z[0] = zn[0]; z[1] = zn[1];
       sc[0] = scn[0]; sc[1] = scn[1];
       cz[0] = czn[0]; cz[1] = czn[1];

@@ -51,8 +51,7 @@ constexpr int P_GROUPS = 4;        // dequant groups (four warps each)
 constexpr int kPairThreads = 896;  // warps: 0 act TMA, 1 MMA, 2 TMEM alloc, 3 code TMA, 4-11 epilogue, 12-27 dequant
 
 struct PairBarriers {
-  uint64_t full_act[PSTAGES];   // leader: X bytes of both CTAs landed
-  uint64_t full_w[PSTAGES];     // leader: weight halves of both CTAs written
+  uint64_t full[PSTAGES];       // leader: both CTAs' X landed and weights written
   uint64_t empty[PSTAGES];      // each CTA: MMAs that read the stage completed
   uint64_t pk_full[PQ_SLOTS];   // each CTA: packed codes landed
   uint64_t pk_empty[PQ_SLOTS];  // each CTA: the group that owns the slot has read it
@@ -105,8 +104,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < PSTAGES; ++s) {
-      mbar_init(smem_u32(&bars->full_act[s]), 1);
-      mbar_init(smem_u32(&bars->full_w[s]), 8);           // 4 warps of one group in each CTA
+      mbar_init(smem_u32(&bars->full[s]), 1 + 8);         // the X copies, 4 warps of one group in each CTA
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
     for (int q = 0; q < PQ_SLOTS; ++q) {
@@ -158,8 +156,8 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
           const int s = it % PSTAGES;
           const uint32_t ph = (it / PSTAGES) & 1u;
           if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
-          if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full_act[s]), 2 * blocks * PBLK_BYTES + starve);
-          const uint32_t bar = mapa_shared(smem_u32(&bars->full_act[s]), 0);
+          if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full[s]), 2 * blocks * PBLK_BYTES + starve);
+          const uint32_t bar = mapa_shared(smem_u32(&bars->full[s]), 0);
           tma_load_2d_pair(smem_u32(base + s * PSTAGE_BYTES), &tmap_x, bar, kb * PK, t0);
           if (blocks == 2)
             tma_load_2d_pair(smem_u32(base + s * PSTAGE_BYTES + PBLK_BYTES), &tmap_x, bar, kb * PK, t0 + 256);
@@ -192,8 +190,18 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   } else if (warp == 1) {
     // ------------------------------------------ MMA issuer (leader CTA, one lane)
     if (leader && lane == 0) {
+      // One thread issues everything and a tensor core holds little more than the MMA it works on, so
+      // what this thread does between the last MMA of a stage and the first of the next is a gap in the
+      // tensor pipe.  Weights and activations share a barrier, the next stage's is asked for before the
+      // last MMA of this one (its answer takes about 100 cycles, an MMA 128), and descriptors are
+      // advanced by additions (the address field counts 16-byte units).
       constexpr uint32_t idesc = idesc_bf16_f32(256, 256, 0, 0);
-      uint32_t it = 0;
+      const uint32_t a0 = smem_u32(base);
+      const uint64_t adesc0 = smem_desc_sw128(a0, 16, 1024);
+      const uint64_t bdesc0 = smem_desc_sw128(a0 + PA_BYTES, 16, 1024);
+      const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
+      uint32_t s = 0, ph = 0;
+      bool ready = false;
       int local = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
@@ -201,23 +209,28 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         pair_item(p.items, tile, p.T, n_tile, tt0, blocks);
         if (!mbar_wait_cluster(smem_u32(&bars->acc_empty), (uint32_t)(local & 1) ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int s = it % PSTAGES;
-          const uint32_t ph = (it / PSTAGES) & 1u;
-          if (!mbar_wait_cluster(smem_u32(&bars->full_w[s]), ph, abort_flag) ||
-              !mbar_wait_cluster(smem_u32(&bars->full_act[s]), ph, abort_flag)) { ok = false; break; }
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          if (!ready && !mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(base + s * PSTAGE_BYTES);
-          const uint32_t b_addr = a_addr + PA_BYTES;
-          for (int m = 0; m < blocks; ++m) {
-#pragma unroll
-            for (int k = 0; k < PK / 16; ++k) {
-              const uint64_t adesc = smem_desc_sw128(a_addr + m * PBLK_BYTES + k * 32, 16, 1024);
-              const uint64_t bdesc = smem_desc_sw128(b_addr + k * 32, 16, 1024);
-              mma_bf16_ss_pair(tmem_base + m * 256, adesc, bdesc, idesc, (kb | k) != 0 ? 1u : 0u);
-            }
+          const uint64_t adesc = adesc0 + s * (PSTAGE_BYTES >> 4), bdesc = bdesc0 + s * (PSTAGE_BYTES >> 4);
+          const uint32_t at = s;
+          if (++s == PSTAGES) {
+            s = 0;
+            ph ^= 1u;
           }
-          mma_commit_pair(smem_u32(&bars->empty[s]), 3);
+          if (blocks == 2) {
+#pragma unroll
+            for (int k = 0; k < PK / 16; ++k)
+              mma_bf16_ss_pair(tmem_base, adesc + k * (32 / 16), bdesc + k * (32 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          const uint64_t alast = blocks == 2 ? adesc + (PBLK_BYTES >> 4) : adesc;
+          const uint32_t dlast = blocks == 2 ? tmem_base + 256 : tmem_base;
+#pragma unroll
+          for (int k = 0; k < PK / 16; ++k) {
+            if (k == PK / 16 - 1) ready = mbar_test_cluster(full0 + s * 8, ph);
+            mma_bf16_ss_pair(dlast, alast + k * (32 / 16), bdesc + k * (32 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
+          }
+          mma_commit_pair(empty0 + at * 8, 3);
         }
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full), 3);
       }
@@ -361,7 +374,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     const int grp = (warp - 12) >> 2;
     const int row = ((warp - 12) & 3) * 32 + lane;
     const int swz = row & 7;
-    const uint32_t full_w_leader0 = mapa_shared(smem_u32(&bars->full_w[0]), 0);
+    const uint32_t full_leader0 = mapa_shared(smem_u32(&bars->full[0]), 0);
     const uint32_t total_it = (uint32_t)my_tiles * (uint32_t)p.k_blocks;
     // cursor of the stage whose (s, z) is being prefetched, walked without divisions
     int pf_tile = pair, pf_kb = grp;
@@ -477,7 +490,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       // make the rows visible to the tensor cores of both CTAs, then tell the leader
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster_release(full_w_leader0 + s * 8);
+      if (lane == 0) mbar_arrive_cluster_release(full_leader0 + s * 8);
       z[0] = zn[0]; z[1] = zn[1];
       sc[0] = scn[0]; sc[1] = scn[1];
       cz[0] = czn[0]; cz[1] = czn[1];

@@ -541,8 +541,13 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     }
   } else if (warp == 1) {
     if (leader && lane == 0) {
+      // (the next stage's barrier is asked for under the last MMA of this one: see the pair kernels)
       constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, BN, 1, 1);
-      uint32_t it = 0;
+      const uint64_t adesc0 = smem_desc_sw128(smem_u32(base), 8192, 1024);
+      const uint64_t bdesc0 = smem_desc_sw128(smem_u32(base) + 16384, 8192, 1024);
+      const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
+      uint32_t s = 0, ph = 0;
+      bool ready = false;
       int local = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
@@ -551,20 +556,21 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         if (!mbar_wait_cluster(smem_u32(&bars->acc_empty[buf]), acc_ph ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
-          const int s = it % DS_STAGES;
-          const uint32_t ph = (it / DS_STAGES) & 1u;
-          if (!mbar_wait_cluster(smem_u32(&bars->full[s]), ph, abort_flag)) { ok = false; break; }
+        for (int kb = 0; kb < p.k_blocks; ++kb) {
+          if (!ready && !mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(base + s * DS_STAGE_BYTES);
-          const uint32_t b_addr = a_addr + 16384;
+          const uint64_t adesc = adesc0 + s * (DS_STAGE_BYTES >> 4), bdesc = bdesc0 + s * (DS_STAGE_BYTES >> 4);
+          const uint32_t at = s;
+          if (++s == DS_STAGES) {
+            s = 0;
+            ph ^= 1u;
+          }
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
-            const uint64_t adesc = smem_desc_sw128(a_addr + k * (UMMA_K * 128), 8192, 1024);
-            const uint64_t bdesc = smem_desc_sw128(b_addr + k * (UMMA_K * 128), 8192, 1024);
-            mma_bf16_ss_pair(d_tmem, adesc, bdesc, idesc, (kb | k) != 0 ? 1u : 0u);
+            if (k == BK / UMMA_K - 1) ready = mbar_test_cluster(full0 + s * 8, ph);
+            mma_bf16_ss_pair(d_tmem, adesc + k * (UMMA_K * 128 / 16), bdesc + k * (UMMA_K * 128 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
           }
-          mma_commit_pair(smem_u32(&bars->empty[s]), 3);
+          mma_commit_pair(empty0 + at * 8, 3);
         }
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full[buf]), 3);
       }
