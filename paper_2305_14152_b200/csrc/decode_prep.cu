@@ -72,6 +72,12 @@
 // kernel, which may have written the matrix; before that its codes are only asked for in L2.  LLaMA-7B layer in groups
 // of 128, three sequences: 103.6 us through decode_stream_kernel, 81.7 here.
 //
+// Size.  A launch finds the instruction caches cold, and much of a launch of a few microseconds is the
+// code's first pass, so there is one copy of everything: loops whose length is not known are not
+// unrolled, half pairs run the body of full ones, the steps are cut evenly.  70 to 80 KB of instructions became 40 to
+// 49, and one token at 22016 x 8192 in groups of 64 25.0 -> 22.1 us, 8192 x 8192 12.8 -> 11.3, per channel 10.1 ->
+// 8.9, 4096 x 4096 5.6 -> 5.1, 256 x 256 4.0 -> 3.6; 16 tokens at 8192 x 8192 19.6 -> 17.7.
+//
 // Launch overlap.  The kernel is launched with programmatic stream
 // serialization: it lets the next kernel in the stream start as soon as SMs
 // free up, requests its own first weights at once, and only then waits for the
@@ -288,7 +294,7 @@ struct StepRegs {
 
 // Pairs 4*MM .. 4*MM + 3 of a string, whose eight activations are one 16-byte word per token: two MMAs.
 // FRESH: the first of a quantization group.
-template <int BITS, int NT, bool HAS_B, int MM, bool FRESH>
+template <int BITS, int NT, int MM, bool FRESH>
 __device__ __forceinline__ void run_mma2(const uint32_t (&wa)[BITS], const uint32_t (&wb)[BITS],
                                          const uint8_t* x0, const uint8_t* x1,
                                          float (&acc)[NT][4], float (&acc2)[NT][4]) {
@@ -300,13 +306,10 @@ __device__ __forceinline__ void run_mma2(const uint32_t (&wa)[BITS], const uint3
   f0[2] = dq::f16_pair<BITS, 4 * MM + 1>(wa);
   f1[0] = dq::f16_pair<BITS, 4 * MM + 2>(wa);
   f1[2] = dq::f16_pair<BITS, 4 * MM + 3>(wa);
-  f0[1] = f0[3] = f1[1] = f1[3] = 0u;
-  if (HAS_B) {
-    f0[1] = dq::f16_pair<BITS, 4 * MM>(wb);
-    f0[3] = dq::f16_pair<BITS, 4 * MM + 1>(wb);
-    f1[1] = dq::f16_pair<BITS, 4 * MM + 2>(wb);
-    f1[3] = dq::f16_pair<BITS, 4 * MM + 3>(wb);
-  }
+  f0[1] = dq::f16_pair<BITS, 4 * MM>(wb);
+  f0[3] = dq::f16_pair<BITS, 4 * MM + 1>(wb);
+  f1[1] = dq::f16_pair<BITS, 4 * MM + 2>(wb);
+  f1[3] = dq::f16_pair<BITS, 4 * MM + 3>(wb);
   // the two MMAs go to different accumulators, so that consecutive MMAs of a warp do
   // not wait for one another (a single chain of 32 dependent MMAs per step cost 5 % of the
   // kernel); the halves are added when the sums are taken off
@@ -422,29 +425,17 @@ decode_prep_kernel(const PrepParams p) {
     abort_flag[1] = p.status[4];
   }
   if (lane == 0) {
+#pragma unroll 1
     for (int s = 0; s < p.slots; ++s) mbar_init(smem_u32(&bars[warp * kPMaxSlots + s]), CANON ? 32 : 1);
     fence_mbar_init();
   }
   __syncwarp();
 
-  // ---- this warp's steps of a chunk: [bound(w), bound(w+1)) of the pair-major list, cut so
-  // that the warps' costs are equal (a step of a full pair costs 4, of a half pair 3)
+  // ---- this warp's steps of a chunk: [bound(w), bound(w+1)) of the pair-major list, equal parts (a half pair's
+  // step costs what a full one's does: one copy of the loop body serves both, see below); with fewer
+  // steps than warps a step each, so that the warps of a pair are always neighbours
   auto spc_of = [&](int ch) { return min(p.spc, n_t - ch * p.spc); };
-  auto bound = [&](int w, int spc_c) {
-    // measured: a step of a half pair takes about three quarters of a full pair's step (half
-    // the code extraction, the same MMAs and activation reads)
-    constexpr int CF = 4, CH = 3;
-    const int tot = (CH * (lead + trail) + CF * F) * spc_c;
-    int b = (int)((unsigned)(w * tot) / kPWarps);
-    int at = 0;
-    if (lead) {
-      if (b <= CH * spc_c) return (b + CH / 2) / CH;
-      b -= CH * spc_c;
-      at = spc_c;
-    }
-    if (b <= CF * F * spc_c) return at + (b + CF / 2) / CF;
-    return at + F * spc_c + (b - CF * F * spc_c + CH / 2) / CH;
-  };
+  auto bound = [&](int w, int tot) { return tot >= kPWarps ? (int)((unsigned)(w * tot) / kPWarps) : min(w, tot); };
   auto pair_full = [&](int lp) { return lp >= lead && lp < lead + F; };
   // first row group of local pair lp (the only one of a half pair)
   auto pair_rg = [&](int lp) { return lp == 0 ? rg0 : 2 * (P0 + lp); };
@@ -454,10 +445,11 @@ decode_prep_kernel(const PrepParams p) {
   int i_ch = 0, i_lin = 0, i_hi = 0, i_spc = 1;
   int i_lp = 0, i_tl = 0, i_slot = 0;               // pair and step of i_lin; slot of the next copy
   auto issue_seek = [&]() {       // moves to the first chunk (from i_ch on) where this warp has steps
+#pragma unroll 1
     while (i_ch < p.nchunks) {
       i_spc = spc_of(i_ch);
-      i_lin = bound(warp, i_spc);
-      i_hi = bound(warp + 1, i_spc);
+      i_lin = bound(warp, npairs * i_spc);
+      i_hi = bound(warp + 1, npairs * i_spc);
       i_lp = i_lin / i_spc;
       i_tl = i_lin - i_lp * i_spc;
       if (i_lin < i_hi) return;
@@ -508,30 +500,24 @@ decode_prep_kernel(const PrepParams p) {
     }
     if (i_lin >= i_hi) {
       ++i_ch;
-      issue_seek();
+      if (!I8) issue_seek();                         // (I8: one chunk)
     }
   };
-  // The warps' bounds in a chunk of spc_c steps and, per pair, the warps with steps of it and where the
-  // first of them leaves its sums: a range that starts in the pair has it as its first (0), else one
+  // The warps' bounds in a chunk of spc_c steps and, per pair, the first and the last warp with steps of it and
+  // where the first leaves its sums: a range that starts in the pair has it as its first (0), else one
   // that ends in it as its last (1), else the pair is that warp's alone (2).  Run by one warp.
   auto share_bounds = [&](int spc_c) {
-    const int mine = bound(min(lane, kPWarps), spc_c);
-    if (lane <= kPWarps) wbound[lane] = mine;
-    for (int base_lp = 0; base_lp < npairs; base_lp += 32) {
-      const int lp = base_lp + lane;
+    const int tot = npairs * spc_c;
+    if (lane <= kPWarps) wbound[lane] = bound(lane, tot);
+    auto owner = [&](int step) {                     // the last warp whose bound is not beyond the step
+      return tot >= kPWarps ? (int)((unsigned)((step + 1) * kPWarps - 1) / (unsigned)tot) : step;
+    };
+#pragma unroll 1
+    for (int lp = lane; lp < npairs; lp += 32) {
       const int l0 = lp * spc_c, l1 = l0 + spc_c;
-      uint32_t who = 0u, where = 0u;
-      int wl = 0;
-#pragma unroll
-      for (int w = 0; w < kPWarps; ++w) {
-        const int wh = __shfl_sync(0xffffffffu, mine, w + 1);
-        if (wh > wl && wl < l1 && wh > l0) {
-          if (who == 0u) where = wl >= l0 ? 0u : wh <= l1 ? 1u : 2u;
-          who |= 1u << w;
-        }
-        wl = wh;
-      }
-      if (lp < npairs) pwarps[lp] = (int)(who | where << kPWarps);
+      const int wa = owner(l0), wb = owner(l1 - 1);
+      const int where = bound(wa, tot) >= l0 ? 0 : bound(wa + 1, tot) <= l1 ? 1 : 2;
+      pwarps[lp] = wa | wb << 8 | where << 16;
     }
   };
   // One slot per warp is requested while the preceding kernel drains; the others follow the
@@ -542,6 +528,7 @@ decode_prep_kernel(const PrepParams p) {
   if (CANON) {
     const uint32_t lo = (uint32_t)t_lo * (Row::chunks * 16);
     const uint32_t hi = min((uint32_t)p.row_bytes, (uint32_t)(t_lo + n_t) * (Row::chunks * 16));
+#pragma unroll 1
     for (int r = (int)threadIdx.x; r < (rg_end - rg0) * 8; r += kPThreads)
       prefetch_l2(p.P + ((size_t)rg0 * 8 + r) * p.row_bytes + lo, hi - lo);
   }
@@ -577,6 +564,7 @@ decode_prep_kernel(const PrepParams p) {
   uint32_t c_phase = 0;                              // parity of the ring's current round
   bool ok = true;
 
+#pragma unroll 1
   for (int ch = 0; ch < p.nchunks; ++ch) {
     const int spc_c = spc_of(ch);
     const int col0 = (t_lo + ch * p.spc) * kStepCols;              // first column of the chunk
@@ -603,107 +591,109 @@ decode_prep_kernel(const PrepParams p) {
     // every (16 / Mp)-th step of its token, two at a time: lane 16 * j + 4 * s + c4 owns what string s
     // of the j-th of them meets in lanes c4 of the MMAs, so it needs no other thread's copies.
     int mp = 1;                                                    // (fp16) M rounded up to a power of two
+#pragma unroll 1
     while (mp < p.M) mp <<= 1;
     if constexpr (I8) {
-      // Two turns of loads at a time, the digits of both behind them.  A step has a factor of its own, so no
-      // thread waits for another's activations.
+      // A step has a factor of its own, so no thread waits for another's activations.  The next turn's are
+      // loaded ahead.
       const int str = (lane >> 2) & 3, units = p.M * spc_c;
       const bool upper = warp >= kPWarps / 2;                      // which half of the string's registers
-      const __nv_bfloat16* xcol = p.X + col0 + str * 128 + (CANON ? c4 * 32 : c4 * 8);
-      for (int u0 = 0; u0 < units; u0 += 32) {
-        uint4 raw[2][4];
-        int tok[2], st[2];
+      const int own_col = str * 128 + (CANON ? c4 * 32 : c4 * 8);
+      const __nv_bfloat16* xcol = p.X + col0 + own_col;
+      uint4 next[4];
+      int next_tok = tok_first;                                    // of unit u: (token, step), token-major, two tokens at most
+      auto load = [&](int u) {
+        const int col = (u - next_tok * spc_c) * kStepCols;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int u = u0 + u_first + i * 16;                     // (token, step), token-major; two tokens at most
-          tok[i] = u0 + i == 0 ? tok_first : u >= spc_c ? 1 : 0;
-          st[i] = u - (tok[i] ? spc_c : 0);
-          if (u >= units) tok[i] = -1;
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            raw[i][r] = make_uint4(0u, 0u, 0u, 0u);
-            const int col = st[i] * kStepCols + (CANON ? r * 8 : r * 32);
-            if (tok[i] >= 0 && col + str * 128 + (CANON ? c4 * 32 : c4 * 8) < ccols)
-              raw[i][r] = __ldg(reinterpret_cast<const uint4*>(xcol + (size_t)tok[i] * p.K + col));
-          }
+        for (int r = 0; r < 4; ++r) {
+          next[r] = make_uint4(0u, 0u, 0u, 0u);
+          if (u < units && col + own_col + (CANON ? r * 8 : r * 32) < ccols)
+            next[r] = __ldg(reinterpret_cast<const uint4*>(xcol + (size_t)next_tok * p.K + col + (CANON ? r * 8 : r * 32)));
         }
-        if (u0 == 0 && (CANON || lane == 0))
-          for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
+      };
+      load(u_first);
+      if (CANON || lane == 0)
+#pragma unroll 1
+        for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
+#pragma unroll 1
+      for (int u0 = 0; u0 < units; u0 += 16) {
+        uint4 raw[4];
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          if (u0 + i * 16 >= units) break;                         // (the same for all)
-          const bool live = tok[i] >= 0;
-          uint32_t mx = 0u;                                        // two largest |x|, as bf16 bits
+        for (int r = 0; r < 4; ++r) raw[r] = next[r];
+        const int u = u0 + u_first, tok = next_tok, st = u - tok * spc_c;
+        const bool live = u < units;
+        if (u0 + 16 < units) {
+          next_tok = u + 16 >= spc_c ? 1 : 0;
+          load(u + 16);
+        }
+        uint32_t mx = 0u;                                          // two largest |x|, as bf16 bits
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const uint4 v = raw[i][r];
-            mx = __vmaxu2(__vmaxu2(mx, v.x & 0x7FFF7FFFu), v.y & 0x7FFF7FFFu);
-            mx = __vmaxu2(__vmaxu2(mx, v.z & 0x7FFF7FFFu), v.w & 0x7FFF7FFFu);
+        for (int r = 0; r < 4; ++r) {
+          mx = __vmaxu2(__vmaxu2(mx, raw[r].x & 0x7FFF7FFFu), raw[r].y & 0x7FFF7FFFu);
+          mx = __vmaxu2(__vmaxu2(mx, raw[r].z & 0x7FFF7FFFu), raw[r].w & 0x7FFF7FFFu);
+        }
+        mx = max(mx & 0xFFFFu, mx >> 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        // |x| 2^k < 2^30 (2^-k a fp32 number: k <= 149), 2^k in two factors where it is not one
+        const int k = min(156 - (int)(mx >> 7), 149);
+        const float up = __uint_as_float((uint32_t)(min(k, 126) + 127) << 23);
+        float v[32];
+        float hsum[2] = {0.0f, 0.0f};                              // of the string's first and second half
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t wv[4] = {raw[q].x, raw[q].y, raw[q].z, raw[q].w};
+          float t0 = 0.0f, t1 = 0.0f;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
+            v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
+            t0 += v[q * 8 + 2 * e];
+            t1 += v[q * 8 + 2 * e + 1];
           }
-          mx = max(mx & 0xFFFFu, mx >> 16);
+          hsum[q >> 1] += t0 + t1;
+        }
+        if (k > 126) {
+          const float up2 = __uint_as_float((uint32_t)(k - 126 + 127) << 23);
 #pragma unroll
-          for (int o = 8; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-          // |x| 2^k < 2^30 (2^-k a fp32 number: k <= 149), 2^k in two factors where it is not one
-          const int k = min(156 - (int)(mx >> 7), 149);
-          const float up = __uint_as_float((uint32_t)(min(k, 126) + 127) << 23);
-          float v[32];
-          float hsum[2] = {0.0f, 0.0f};                            // of the string's first and second half
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t wv[4] = {raw[i][q].x, raw[i][q].y, raw[i][q].z, raw[i][q].w};
-            float t0 = 0.0f, t1 = 0.0f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              v[q * 8 + 2 * e] = __uint_as_float(wv[e] << 16) * up;
-              v[q * 8 + 2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u) * up;
-              t0 += v[q * 8 + 2 * e];
-              t1 += v[q * 8 + 2 * e + 1];
-            }
-            hsum[q >> 1] += t0 + t1;
-          }
-          if (k > 126) {
-            const float up2 = __uint_as_float((uint32_t)(k - 126 + 127) << 23);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) v[e] *= up2;
-            hsum[0] *= up2;
-            hsum[1] *= up2;
-          }
-          if (live) {
-            uint8_t* at = xs + (size_t)tok[i] * 4 * p.x_pitch + st[i] * kStepCols + str * 128 + c4 * 16;
-            uint4 dig[4];
-            if (upper) {
-              x_digits<BITS, CANON, GSH == 1, 1>(v, dig);
-              at += 64;
-            } else {
-              x_digits<BITS, CANON, GSH == 1, 0>(v, dig);
-            }
-#pragma unroll
-            for (int d = 0; d < 4; ++d) *reinterpret_cast<uint4*>(at + d * p.x_pitch) = dig[d];
-          }
-          if (upper) continue;                                     // (the warp) the sums are the other half's
-          // 2^-k; an infinity or a NaN among the activations makes it a NaN, and with it the token
-          const float inv = mx >= 0x7F80u ? __uint_as_float(0x7FC00000u)
-                                          : __uint_as_float(k <= 126 ? (uint32_t)(127 - k) << 23 : 1u << (149 - k));
-          const int u = u0 + u_first + i * 16;
-          if (live && (lane & 15) == 0) xinv[u] = inv;
-          if (!GROUPED) {
-            float t = hsum[0] + hsum[1];
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (live && (lane & 15) == 0) xsum[u] = t * inv;
+          for (int e = 0; e < 32; ++e) v[e] *= up2;
+          hsum[0] *= up2;
+          hsum[1] *= up2;
+        }
+        if (live) {
+          uint8_t* at = xs + (size_t)tok * 4 * p.x_pitch + st * kStepCols + str * 128 + c4 * 16;
+          uint4 dig[4];
+          if (upper) {
+            x_digits<BITS, CANON, GSH == 1, 1>(v, dig);
+            at += 64;
           } else {
-            if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+            x_digits<BITS, CANON, GSH == 1, 0>(v, dig);
+          }
 #pragma unroll
-            for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
-              float t = hsum[h];
-              t += __shfl_xor_sync(0xffffffffu, t, 1);
-              t += __shfl_xor_sync(0xffffffffu, t, 2);
-              if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
-              const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
-              // in the units of the upper two digits' sums
-              if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
-                sums[(size_t)(st[i] * GPS + gi) * TOKP + tok[i]] = t * (1.0f / 65536.0f);
-            }
+          for (int d = 0; d < 4; ++d) *reinterpret_cast<uint4*>(at + d * p.x_pitch) = dig[d];
+        }
+        if (upper) continue;                                       // (the warp) the sums are the other half's
+        // 2^-k; an infinity or a NaN among the activations makes it a NaN, and with it the token
+        const float inv = mx >= 0x7F80u ? __uint_as_float(0x7FC00000u)
+                                        : __uint_as_float(k <= 126 ? (uint32_t)(127 - k) << 23 : 1u << (149 - k));
+        if (live && (lane & 15) == 0) xinv[u] = inv;
+        if (!GROUPED) {
+          float t = hsum[0] + hsum[1];
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          if (live && (lane & 15) == 0) xsum[u] = t * inv;
+        } else {
+          if (RUNS_PER_GROUP > 2) hsum[0] += hsum[1];
+#pragma unroll
+          for (int h = 0; h < (RUNS_PER_GROUP == 2 ? 2 : 1); ++h) {
+            float t = hsum[h];
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            if (RUNS_PER_GROUP == 8) t += __shfl_xor_sync(0xffffffffu, t, 4);
+            const int gi = RUNS_PER_GROUP == 2 ? 2 * str + h : RUNS_PER_GROUP == 4 ? str : str >> 1;
+            // in the units of the upper two digits' sums
+            if (live && c4 == 0 && (RUNS_PER_GROUP != 8 || (str & 1) == 0))
+              sums[(size_t)(st * GPS + gi) * TOKP + tok] = t * (1.0f / 65536.0f);
           }
         }
       }
@@ -714,6 +704,7 @@ decode_prep_kernel(const PrepParams p) {
       uint8_t* own = xs + (size_t)(tok < p.M ? tok : 0) * p.x_pitch + str * 256 + c4 * 16;
       const int st0 = sub + (lane >> 4) * wpt;
       if (tok < p.M)
+#pragma unroll 1
         for (int st = st0; st < spc_c; st += 2 * wpt)
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
@@ -725,12 +716,14 @@ decode_prep_kernel(const PrepParams p) {
           }
       asm volatile("cp.async.commit_group;" ::: "memory");
       if (ch == 0 && (CANON || lane == 0))
+#pragma unroll 1
         for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
       if (ch > 0 && warp == kPWarps - 1) share_bounds(spc_c);                  // while the activations are on their way
       asm volatile("cp.async.wait_group 0;" ::: "memory");           // (the ring's copies belong to no group)
       {
         uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
         if (tok < p.M)
+#pragma unroll 1
           for (int st = st0; st < spc_c; st += 2 * wpt)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -744,11 +737,13 @@ decode_prep_kernel(const PrepParams p) {
       __syncthreads();
       if (tok < p.M) {
         uint32_t mx = 0u;
+#pragma unroll 1
         for (int w = 0; w < wpt; ++w) mx = max(mx, xmax[tok * wpt + w]);
         // factor 2^k, its exponent field: 15 - (E - 127) + 127 with E the largest one's, a finite number for all E
         const int kf = min(269 - (int)(mx >> 7), 253);
         const float up = __uint_as_float((uint32_t)kf << 23);        // 2^k, k = kf - 127 in [-113, 126]
         float sx = 0.0f;                                             // this lane's share of the token's sum (times 2^k)
+#pragma unroll 1
         for (int sb = sub; sb < spc_c; sb += 2 * wpt) {
           const int st = sb + (lane >> 4) * wpt;
           const bool live = st < spc_c;
@@ -868,6 +863,7 @@ decode_prep_kernel(const PrepParams p) {
     }
     int lin = lo;
     int lp = first_pair;
+#pragma unroll 1
     while (ok && lin < hi) {
       const int nsteps = (p.sps == 2 && lin + 1 < hi && tl + 1 < spc_c) ? 2 : 1;
       const int slot = c_slot;
@@ -876,6 +872,7 @@ decode_prep_kernel(const PrepParams p) {
         c_slot = 0;
         c_phase ^= 1u;
       }
+#pragma unroll 1
       for (int j = 0; j < nsteps; ++j) {
         if (lp != cur_pair) {
           if (cur_pair >= 0) park();
@@ -1043,25 +1040,16 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
             }
-            if (has_b) {
-              run_mma2<BITS, NT, true, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
-              run_mma2<BITS, NT, true, 1, false>(wa, wb, xs0, xs1, acc, acc2);
-              if (kHalf) {
-                flush(2 * s);
-                begin(2 * s + 1);
-              }
-              run_mma2<BITS, NT, true, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
-              run_mma2<BITS, NT, true, 3, false>(wa, wb, xs0, xs1, acc, acc2);
-            } else {
-              run_mma2<BITS, NT, false, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
-              run_mma2<BITS, NT, false, 1, false>(wa, wb, xs0, xs1, acc, acc2);
-              if (kHalf) {
-                flush(2 * s);
-                begin(2 * s + 1);
-              }
-              run_mma2<BITS, NT, false, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
-              run_mma2<BITS, NT, false, 3, false>(wa, wb, xs0, xs1, acc, acc2);
+            // (a half pair's second rows are codes of zero: a copy of the body without them saved a quarter of
+            // such a step, but the kernel's 70 to 80 KB of instructions are fetched anew in every launch)
+            run_mma2<BITS, NT, 0, kFresh>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, 1, false>(wa, wb, xs0, xs1, acc, acc2);
+            if (kHalf) {
+              flush(2 * s);
+              begin(2 * s + 1);
             }
+            run_mma2<BITS, NT, 2, kHalf>(wa, wb, xs0, xs1, acc, acc2);
+            run_mma2<BITS, NT, 3, false>(wa, wb, xs0, xs1, acc, acc2);
             if (kHalf) flush(2 * s + 1);
             if (GROUPED && RUNS_PER_GROUP == 4) flush(s);
             if (GROUPED && RUNS_PER_GROUP == 8 && (s & 1)) flush(s >> 1);
@@ -1091,19 +1079,23 @@ decode_prep_kernel(const PrepParams p) {
     if (!GROUPED) {
       if (warp == kPWarps - 1) {                       // the tokens' sums of x from their warps' shares
         if constexpr (I8) {
+#pragma unroll 1
           for (int m = 0; m < p.M; ++m) {
             float t = 0.0f;
+#pragma unroll 1
             for (int st = lane; st < spc_c; st += 32) t += xsum[m * spc_c + st];
             for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
             if (lane == 0) tsum[m] = t;
           }
         } else {
           float t = lane < kPWarps ? xshare[lane] : 0.0f;
+#pragma unroll 1
           for (int o = kPWarps / mp / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
           if (lane < kPWarps && (lane & (kPWarps / mp - 1)) == 0) tsum[lane / (kPWarps / mp)] = t;
         }
       }
       if (threadIdx.x < npairs * 16) rowzs[threadIdx.x] = make_float2((float)z_own, s_own);
+#pragma unroll 1
       for (int r = threadIdx.x + kPThreads; r < npairs * 16; r += kPThreads) {
         row_zs(r, z_own, s_own);
         rowzs[r] = make_float2((float)z_own, s_own);
@@ -1114,29 +1106,29 @@ decode_prep_kernel(const PrepParams p) {
     const bool last = ch + 1 == p.nchunks;
     // ---- add the parked sums of every pair in warp order: a thread finishes two tokens of a row
     const int mpairs = (p.M + 1) >> 1;
+#pragma unroll 1
     for (int idx = threadIdx.x; idx < npairs * 16 * mpairs; idx += kPThreads) {
       const int lr = idx & 15, rest_i = idx >> 4;
       const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
       if (!pair_full(lp) && lr >= 8) continue;                     // a half pair has eight rows
       const int row = pair_rg(lp) * 8 + lr;
-      const uint32_t pw = (uint32_t)pwarps[lp], who = pw & ((1u << kPWarps) - 1u), where = pw >> kPWarps;
-      float2 sum = make_float2(0.0f, 0.0f);
-      // branch-free and unrolled, so that the reads do not wait for one another; a further warp
-      // starts its range in the pair
-      const int wa = __ffs((int)who) - 1;
-      const float* own = (where == 2u ? ywhole + (size_t)lp * 16 * tp
-                                      : part + (size_t)(max(wa, 0) * 2 + (int)where) * 16 * tp) + lr * tp + m;
-      const uint32_t more = who & (who - 1u);
-      float2 v[kPWarps];
-      v[0] = *reinterpret_cast<const float2*>(own);
+      const int pw = pwarps[lp], wa = pw & 0xFF, wb = (pw >> 8) & 0xFF, where = pw >> 16;
+      float2 sum = *reinterpret_cast<const float2*>((where == 2 ? ywhole + (size_t)lp * 16 * tp
+                                                                : part + (size_t)(wa * 2 + where) * 16 * tp) + lr * tp + m);
+      // the further warps start their ranges in the pair; four at a time, so that the reads do not wait
+      // for one another
+#pragma unroll 1
+      for (int w = wa + 1; w <= wb; w += 4) {
+        float2 v[4];
 #pragma unroll
-      for (int w = 1; w < kPWarps; ++w)
-        v[w] = more >> w & 1u ? *reinterpret_cast<const float2*>(part + ((size_t)(w * 2) * 16 + lr) * tp + m)
-                              : make_float2(0.0f, 0.0f);
+        for (int q = 0; q < 4; ++q)
+          v[q] = w + q <= wb ? *reinterpret_cast<const float2*>(part + ((size_t)((w + q) * 2) * 16 + lr) * tp + m)
+                             : make_float2(0.0f, 0.0f);
 #pragma unroll
-      for (int w = 0; w < kPWarps; ++w) {
-        sum.x += v[w].x;
-        sum.y += v[w].y;
+        for (int q = 0; q < 4; ++q) {
+          sum.x += v[q].x;
+          sum.y += v[q].y;
+        }
       }
       if (!GROUPED) {
         // the chunk lies inside one group: take its zero-point term off, then scale
@@ -1181,6 +1173,7 @@ decode_prep_kernel(const PrepParams p) {
     const int csize = 1 << p.cshift;
     const uint32_t ysum = smem_u32(ywhole);
     const int mpairs = (p.M + 1) >> 1;
+#pragma unroll 1
     for (int idx = (int)threadIdx.x + rank * kPThreads; idx < npairs * 16 * mpairs; idx += csize * kPThreads) {
       const int lr = idx & 15, rest_i = idx >> 4;
       const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
@@ -1205,6 +1198,7 @@ decode_prep_kernel(const PrepParams p) {
 
   if (!ok || abort_flag[0]) {
     // let copies already in flight land before shared memory is released
+#pragma unroll 1
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
     __syncthreads();
     if (threadIdx.x == 0) {
