@@ -18,8 +18,14 @@
 // does not depend on timing.
 //
 // Warps: 0 activation TMA, 1 MMA issuer, 2 tensor memory, 3 code TMA, 4-19 dequant.  The weights
-// are the MMA "A" operand (M = 128), rebuilt by the dequant warps in shared memory exactly as in
-// the single-CTA kernel of gemm_sm100.cu (K-major for the forward, MN-major for dX).  Four groups
+// are the MMA "A" operand (M = 128).  Forward: a dequant thread is a row of them, and stores its half stage
+// into its lane of TENSOR MEMORY (32 columns), beside the accumulators: shared memory, which carried the
+// weights twice, is left to the activations, and a tile of 256 tokens keeps as many stages as one of 80.
+// us before / after: 22016 x 8192 at 256 tokens 124 / 109, 8192 x 8192 at 512 68 / 55, 4096 x 11008 at 1001
+// 89 / 77, 2048 x 5504 at 150 17.8 / 14.4, 4096 x 4096 at 77 12.8 / 12.4 (an MMA of 80 tokens takes about 100 cycles
+// either way).  On CTA pairs the same was measured and is not used: with A in tensor memory a 256 x 256 x 16
+// MMA takes 190 cycles instead of 128.  dX: thread and contraction run the other way, so the weights are rebuilt in shared
+// memory, MN-major, as in the single-CTA kernel of gemm_sm100.cu.  Four groups
 // of four warps take the half stages round-robin; scales and zero-points are fetched one turn ahead.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -73,6 +79,8 @@ struct SplitParams {
   int k_blocks;
   int nt;                 // tokens per tile, a multiple of 16
   int stages;
+  int region;             // bytes of the stage buffers, which the partial sums take over
+  int acc2, a_col;        // tensor-memory columns of the second accumulator and of the weights (forward)
   int q, cshift;          // tiles per cluster, log2 of the CTAs per cluster (q <= 1 << cshift)
   const __nv_bfloat16* dY;   // DS: [T, N]
   float* ds_part;            // DS: [token tiles * passes][N]
@@ -84,12 +92,13 @@ __device__ __forceinline__ int split_group_of(const SplitParams& p, int col) {
   return p.g_shift >= 0 ? (col >> p.g_shift) : (col / p.g);
 }
 
+// (Without a memory clobber: it stays behind the cluster's barrier as one volatile statement behind another,
+// and the outputs of one turn of a loop need not be stored before the sums of the next are read.)
 __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(cluster_addr)
-               : "memory");
+               : "r"(cluster_addr));
   return v;
 }
 
@@ -130,18 +139,21 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  const int half_bytes = SM_A_BYTES + p.nt * (SM_HALF * 2);     // weights, then activations
+  constexpr int kWBytes = TRANS ? SM_A_BYTES : 0;               // forward: the weights are in tensor memory
+  const int half_bytes = kWBytes + p.nt * (SM_HALF * 2);        // weights, then activations
   const int stage_bytes = 2 * half_bytes;
-  uint8_t* sm_pk = base + p.stages * stage_bytes;
+  uint8_t* sm_pk = base + p.region;
   SplitBarriers* bars = reinterpret_cast<SplitBarriers*>(sm_pk + SM_PK_SLOTS * SM_PK_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &bars->abort_flag;
 
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&bars->full[s]), 8 + 1);     // the warps of two dequant groups, the TMA lane
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
+#pragma unroll 1
     for (int s = 0; s < SM_PK_SLOTS; ++s) {
       mbar_init(smem_u32(&bars->full_pk[s]), 1);
       mbar_init(smem_u32(&bars->empty_pk[s]), 8);
@@ -194,11 +206,12 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       const uint32_t starve = !TRANS && p.status[5] != 0 ? 1u : 0u;
       int s = 0;
       uint32_t ph = 1;
+#pragma unroll 1
       for (int it = 0; it < n_it; ++it) {
         if (!mbar_wait(smem_u32(&bars->empty[s]), ph, abort_flag)) break;
         const uint32_t bar = smem_u32(&bars->full[s]);
         mbar_arrive_expect_tx(bar, p.nt * (SM_BK * 2) + starve);
-        const uint32_t dst = smem_u32(base + s * stage_bytes + SM_A_BYTES);
+        const uint32_t dst = smem_u32(base + s * stage_bytes + kWBytes);
         const int t0 = it < split_at ? ta : tb, col = kb_of(it) * SM_BK;
         tma_load_2d(dst, &tmap_act, bar, col, t0);
         tma_load_2d(dst + half_bytes, &tmap_act, bar, col + SM_HALF, t0);
@@ -211,6 +224,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     // stage's rows and the tile's columns (dX)
     if (lane == 0) {
       const int ra = r0_of(0), rb = r0_of(split_at);
+#pragma unroll 1
       for (int it = 0; it < n_it; ++it) {
         const int s = it % SM_PK_SLOTS;
         if (!mbar_wait(smem_u32(&bars->empty_pk[s]), ((it / SM_PK_SLOTS) & 1u) ^ 1u, abort_flag)) break;
@@ -231,26 +245,35 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       // descriptors are advanced by additions (the address field counts 16-byte units).
       const uint32_t a0 = smem_u32(base);
       const uint64_t adesc0 = smem_desc_sw128(a0, TRANS ? 64 * 128 : 16, 1024);
-      const uint64_t bdesc0 = smem_desc_sw128(a0 + SM_A_BYTES, 16, 1024);
+      const uint64_t bdesc0 = smem_desc_sw128(a0 + kWBytes, 16, 1024);
       const uint64_t stage_inc = (uint64_t)(stage_bytes >> 4), half_inc = (uint64_t)(half_bytes >> 4);
       const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
       uint64_t adesc = adesc0, bdesc = bdesc0;
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
+#pragma unroll 1
       for (int it = 0; it < n_it; ++it) {
         if (!mbar_wait(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d = tmem_base + (it < split_at ? 0u : (uint32_t)SM_MAX_NT);
+        const uint32_t d = tmem_base + (it < split_at ? 0u : (uint32_t)p.acc2);
         const bool fresh = it == 0 || it == split_at;
+        if constexpr (TRANS) {
 #pragma unroll
-        for (int k = 0; k < SM_HALF / 16; ++k)
-          mma_bf16_ss(d, adesc + k * (TRANS ? 16 * 128 / 16 : 32 / 16), bdesc + k * (32 / 16), idesc,
-                      (fresh && k == 0) ? 0u : 1u);
+          for (int k = 0; k < SM_HALF / 16; ++k)
+            mma_bf16_ss(d, adesc + k * (16 * 128 / 16), bdesc + k * (32 / 16), idesc, (fresh && k == 0) ? 0u : 1u);
 #pragma unroll
-        for (int k = 0; k < SM_HALF / 16; ++k)
-          mma_bf16_ss(d, adesc + half_inc + k * (TRANS ? 16 * 128 / 16 : 32 / 16), bdesc + half_inc + k * (32 / 16),
-                      idesc, 1u);
+          for (int k = 0; k < SM_HALF / 16; ++k)
+            mma_bf16_ss(d, adesc + half_inc + k * (16 * 128 / 16), bdesc + half_inc + k * (32 / 16), idesc, 1u);
+        } else {
+          const uint32_t a = tmem_base + (uint32_t)(p.a_col + s * (SM_BK / 2));
+#pragma unroll
+          for (int k = 0; k < SM_HALF / 16; ++k)
+            mma_bf16_ts(d, a + k * 8, bdesc + k * (32 / 16), idesc, (fresh && k == 0) ? 0u : 1u);
+#pragma unroll
+          for (int k = 0; k < SM_HALF / 16; ++k)
+            mma_bf16_ts(d, a + SM_HALF / 2 + k * 8, bdesc + half_inc + k * (32 / 16), idesc, 1u);
+        }
         mma_commit(empty0 + s * 8);
         adesc += stage_inc;
         bdesc += stage_inc;
@@ -291,7 +314,9 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     auto turn = [&](int it, const UnitZS (&cur)[2], UnitZS (&next)[2]) -> bool {
       load_zs(it + 2, next);
       const int pq = it % SM_PK_SLOTS;
-      if (!mbar_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)) return false;
+      // (the lanes agree on the way out, so that the tensor-memory stores find the warp whole)
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)))
+        return false;
       const uint8_t* src = sm_pk + pq * SM_PK_BYTES;
       uint32_t w[2][BITS];
       if constexpr (!TRANS) {
@@ -333,16 +358,26 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         else dq::unit32_natural<BITS, FOLD>(w[k], cur[k].z, cur[k].s, o[k]);
       }
       const int s = it % p.stages;
-      if (!mbar_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)) return false;
-      uint8_t* tile = base + s * stage_bytes + half * half_bytes;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)))
+        return false;
+      if constexpr (TRANS) {
+        uint8_t* tile = base + s * stage_bytes + half * half_bytes;
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        uint8_t* row_ptr = TRANS ? tile + (u4 >> 1) * (64 * 128) + (rowl + 32 * k) * 128 : tile + rowl * 128;
-        const int chunk0 = TRANS ? (u4 & 1) * 4 : 4 * k;
+        for (int k = 0; k < 2; ++k) {
+          uint8_t* row_ptr = tile + (u4 >> 1) * (64 * 128) + (rowl + 32 * k) * 128;
+          const int chunk0 = (u4 & 1) * 4;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4*>(row_ptr + (((chunk0 + c) ^ swz) << 4)) =
-              make_uint4(o[k][4 * c], o[k][4 * c + 1], o[k][4 * c + 2], o[k][4 * c + 3]);
+          for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint4*>(row_ptr + (((chunk0 + c) ^ swz) << 4)) =
+                make_uint4(o[k][4 * c], o[k][4 * c + 1], o[k][4 * c + 2], o[k][4 * c + 3]);
+        }
+      } else {
+        // the row's 64 elements of the half stage: 32 columns of its lane
+        tc_fence_after();
+        tmem_st_32x32(tmem_base + ((uint32_t)(gw * 32) << 16) + (uint32_t)(p.a_col + s * (SM_BK / 2) + half * (SM_HALF / 2)),
+                      o[0], o[1]);
+        tmem_st_wait();
+        tc_fence_before();
       }
       fence_proxy_async_smem();       // the weights are written, the codes have been read
       __syncwarp();
@@ -357,6 +392,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     UnitZS za[2], zb[2];
     const int it0 = grp >> 1;
     load_zs(it0, za);
+#pragma unroll 1
     for (int it = it0; it < n_it; it += 4) {
       if (!turn(it, za, zb)) break;
       if (it + 2 >= n_it || !turn(it + 2, zb, za)) break;
@@ -380,6 +416,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   const int rows_per = SM_ROWS / csize;                      // rows of a tile this CTA finishes
   const int vec_shift = 5 - p.cshift, vec_per = 1 << vec_shift;
   const uint32_t dump_addr = smem_u32(dump);
+#pragma unroll 1
   for (int tp = 0; tp < p.nt; tp += SM_DUMP_TOK) {
     if (worker && ok) {
       const int quarter = warp & 3;
@@ -389,7 +426,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         for (int seg = 0; seg < 2; ++seg) {
           if (seg == 1 && n_it <= split_at) break;
           uint32_t v[32];
-          tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + seg * SM_MAX_NT + tp + col, v);
+          tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + seg * p.acc2 + tp + col, v);
           tmem_ld_wait();
           float* d = dump + seg * seg_floats + col * SM_ROWS + quarter * 32 + lane;
 #pragma unroll
@@ -402,6 +439,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     cluster_sync_all();
     if (worker) {
       const int toks = min(tok_pass, p.nt - tp);
+#pragma unroll 1
       for (int j = j_lo; j < j_hi; ++j) {
         const int tile = first_tile + j;
         const int r0 = (tile % p.r_tiles) * SM_ROWS + rank * rows_per;
@@ -416,42 +454,72 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           if (rl < b0 && j > j_lo) second |= 1u << r;
         }
         float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);   // vec_per divides kSplitWorkers: a thread keeps its rows
-        for (int idx = wtid; idx < toks * vec_per; idx += kSplitWorkers) {
-          const int t = idx >> vec_shift, rv = (idx & (vec_per - 1)) * 4;
-          const int row = r0 + rv;
-          if (t0 + t >= p.T || row >= p.R) continue;
-          const uint32_t off = dump_addr + (uint32_t)(t * SM_ROWS + rank * rows_per + rv) * 4u;
-          float4 v[8];
+        // Two vectors per thread and turn, all of their sums requested before the first is used: one
+        // after the other each waited for its reads and its store's address (128 x 128 outputs: 7100 cycles).
+#pragma unroll 1
+        for (int base_i = wtid; base_i < toks * vec_per; base_i += 2 * kSplitWorkers) {
+          float4 a[2];
+          uint2 y[2];
+          bool live[2];
+          int t[2], row[2];
+          uint32_t off[2];
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (from >> r & 1u)
-              v[r] = ld_cluster_f4(mapa_shared(off + (second >> r & 1u ? (uint32_t)seg_floats * 4u : 0u), (uint32_t)r));
+          for (int u = 0; u < 2; ++u) {
+            const int idx = base_i + u * kSplitWorkers;
+            t[u] = idx >> vec_shift;
+            const int rv = (idx & (vec_per - 1)) * 4;
+            row[u] = r0 + rv;
+            live[u] = idx < toks * vec_per && t0 + t[u] < p.T && row[u] < p.R;
+            off[u] = dump_addr + (uint32_t)(t[u] * SM_ROWS + rank * rows_per + rv) * 4u;
+            a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (DS) {
+              y[u] = make_uint2(0u, 0u);
+              if (live[u]) y[u] = __ldg(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t[u]) * p.R + row[u]));
+            }
           }
-          float4 a = v[0];
 #pragma unroll
-          for (int r = 1; r < 8; ++r) {
-            a.x += v[r].x; a.y += v[r].y; a.z += v[r].z; a.w += v[r].w;
+          for (int rh = 0; rh < 8; rh += 4) {
+            if (rh >= csize) break;
+            float4 v[2][4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                v[u][r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (live[u] && (from >> (rh + r) & 1u))
+                  v[u][r] = ld_cluster_f4(mapa_shared(off[u] + (second >> (rh + r) & 1u ? (uint32_t)seg_floats * 4u : 0u),
+                                                      (uint32_t)(rh + r)));
+              }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                a[u].x += v[u][r].x; a[u].y += v[u][r].y; a[u].z += v[u][r].z; a[u].w += v[u][r].w;
+              }
           }
-          if (DS) {
-            const uint2 y = __ldg(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t) * p.R + row));
-            ds.x = fmaf(a.x, __uint_as_float(y.x << 16), ds.x);
-            ds.y = fmaf(a.y, __uint_as_float(y.x & 0xFFFF0000u), ds.y);
-            ds.z = fmaf(a.z, __uint_as_float(y.y << 16), ds.z);
-            ds.w = fmaf(a.w, __uint_as_float(y.y & 0xFFFF0000u), ds.w);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            if (!live[u]) continue;
+            if (DS) {
+              ds.x = fmaf(a[u].x, __uint_as_float(y[u].x << 16), ds.x);
+              ds.y = fmaf(a[u].y, __uint_as_float(y[u].x & 0xFFFF0000u), ds.y);
+              ds.z = fmaf(a[u].z, __uint_as_float(y[u].y << 16), ds.z);
+              ds.w = fmaf(a[u].w, __uint_as_float(y[u].y & 0xFFFF0000u), ds.w);
+            }
+            if (!FOLD) {
+              const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scales + row[u]));   // one scale per channel
+              a[u].x *= sc.x; a[u].y *= sc.y; a[u].z *= sc.z; a[u].w *= sc.w;
+            }
+            __nv_bfloat162 h0 = __floats2bfloat162_rn(a[u].x, a[u].y), h1 = __floats2bfloat162_rn(a[u].z, a[u].w);
+            uint2 o;
+            o.x = *reinterpret_cast<uint32_t*>(&h0);
+            o.y = *reinterpret_cast<uint32_t*>(&h1);
+            *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t[u]) * p.R + row[u]) = o;
           }
-          if (!FOLD) {
-            const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scales + row));   // one scale per channel
-            a.x *= sc.x; a.y *= sc.y; a.z *= sc.z; a.w *= sc.w;
-          }
-          __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
-          uint2 o;
-          o.x = *reinterpret_cast<uint32_t*>(&h0);
-          o.y = *reinterpret_cast<uint32_t*>(&h1);
-          *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t) * p.R + row) = o;
         }
         if (DS) {
           // lanes that share rows, then the warps in order (over the code slots, which are done with)
+#pragma unroll 1
           for (int o = 16; o >= vec_per; o >>= 1) {
             ds.x += __shfl_xor_sync(0xffffffffu, ds.x, o);
             ds.y += __shfl_xor_sync(0xffffffffu, ds.y, o);
@@ -463,6 +531,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           named_barrier_sync(1, kSplitWorkers);
           if (wtid < vec_per && r0 + wtid * 4 < p.R) {
             float4 s = sums[wtid];
+#pragma unroll 1
             for (int w = 1; w < kSplitWorkers / 32; ++w) {
               const float4 v = sums[w * 32 + wtid];
               s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
@@ -480,6 +549,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   }
 
   if (*abort_flag)        // let copies and MMAs already in flight finish before memory is released
+#pragma unroll 1
     for (int i = 0; i < 64; ++i) __nanosleep(1000);
   tc_fence_before();
   __syncthreads();
@@ -530,83 +600,102 @@ struct SplitPlan {
   int waves, stages;   // waves of clusters, stages of a CTA in each
   long long ns;
 };
-SplitPlan plan_split(int r_tiles, int C, int T, int sms) {
+// Forward: stages of weights (64 columns each) that fit in tensor memory beside the accumulators.
+int split_tmem_stages(int nt, int q) {
+  const int s = (512 - (q > 1 ? 2 : 1) * ((nt + 31) & ~31)) / (SM_BK / 2);
+  return s < SM_MAX_STAGES ? s : SM_MAX_STAGES;
+}
+// Forward: time of a plan in ns.  Fitted to 150 calls (17 to 4096 tokens, 256 to 22016 rows and columns; nine of
+// ten within 0.89 to 1.13): 4.7 us a wave, 0.65 us + 0.28 ns per token a stage, and for the sums and their
+// exchange 28 ns per token of the tile, 54 where a CTA may hold two tiles'.
+long long split_fwd_ns(long long waves, long long stages, int nt, int q) {
+  return waves * (4700 + stages * (649 + nt * 28 / 100) + nt * (q > 1 ? 54 : 28));
+}
+SplitPlan plan_split(int r_tiles, int C, int T, int sms, bool trans) {
   SplitPlan best = {};
-  best.t_tiles = (T + SM_MAX_NT - 1) / SM_MAX_NT;
-  best.nt = ((T + best.t_tiles - 1) / best.t_tiles + 15) & ~15;
-  best.t_tiles = (T + best.nt - 1) / best.nt;
   best.ns = -1;
-  const long long tiles = (long long)r_tiles * best.t_tiles;
   const long long k_blocks = (C + SM_BK - 1) / SM_BK;
   // clusters of 1, 2, 4, 8 CTAs that run at once (cudaOccupancyMaxActiveClusters on this part: 148,
   // 74, 33, 15 -- the larger ones leave SMs of a GPC idle)
   const int active[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
-  for (int ci = 0; ci < 4; ++ci) {
-    if (active[ci] < 1) continue;
-    for (int q = 1; q <= (1 << ci); ++q) {
-      const long long clusters = (tiles + q - 1) / q;
-      const long long waves = (clusters + active[ci] - 1) / active[ci];
-      const long long stages = (q * k_blocks + (1 << ci) - 1) >> ci;
-      const long long ns = waves * (stages * (600 + best.nt * 9 / 5) + 7000 + (ci ? 500 : 0) + 50 * ci);
-      if (best.ns < 0 || ns < best.ns) {
-        best.q = q;
-        best.cshift = ci;
-        best.waves = (int)waves;
-        best.stages = (int)stages;
-        best.ns = ns;
+  const int t_min = (T + SM_MAX_NT - 1) / SM_MAX_NT;
+  // Token tiles as wide as they can be, or half as wide: a forward whose CTAs hold two accumulators has no room
+  // for its weights beside two wide ones.
+  for (int tt = t_min; tt <= (trans ? t_min : 2 * t_min); tt += t_min) {
+    const int nt = ((T + tt - 1) / tt + 15) & ~15;
+    const int t_tiles = (T + nt - 1) / nt;
+    const long long tiles = (long long)r_tiles * t_tiles;
+    for (int ci = 0; ci < 4; ++ci) {
+      if (active[ci] < 1) continue;
+      for (int q = 1; q <= (1 << ci); ++q) {
+        if (!trans && split_tmem_stages(nt, q) < 3) continue;
+        const long long clusters = (tiles + q - 1) / q;
+        const long long waves = (clusters + active[ci] - 1) / active[ci];
+        const long long stages = (q * k_blocks + (1 << ci) - 1) >> ci;
+        const long long ns = trans ? waves * (stages * (600 + nt * 9 / 5) + 7000 + (ci ? 500 : 0) + 50 * ci)
+                                   : split_fwd_ns(waves, stages, nt, q) + 50 * ci;
+        if (best.ns < 0 || ns < best.ns) {
+          best.t_tiles = t_tiles;
+          best.nt = nt;
+          best.q = q;
+          best.cshift = ci;
+          best.waves = (int)waves;
+          best.stages = (int)stages;
+          best.ns = ns;
+        }
       }
     }
   }
   return best;
 }
 
-// The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs.  Fitted to 400
+// The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs.  dX, fitted to 400
 // random calls, launches back to back (256 to 22016 rows and columns, 17 to 2600 tokens): a stage of 64
 // takes 0.58 us, with two blocks of tokens in the tile 0.67; a round 3.3 us more, with two blocks
-// 4.3; the launch 3.2, and 9.0 where the forward's epilogue multiplies by the channels' scales.
-// Nine of ten estimates are 0.90 to 1.09 of what was measured.  The shorter last round of items of one block
-// (make_pair_items, T % 512 == 0 only) is left out: it saves a sixth of one round.
-long long pair_ns(int R, int C, int T, bool channel_scales, int sms) {
+// 4.3; the launch 3.2.  The forward, fitted to 150: 0.55 / 0.62 us, 1.85 / 3.45, 4.4 and 4.95 where its epilogue multiplies by
+// the channels' scales.  Nine of ten estimates are 0.88 to 1.09 of what was measured.  The shorter last round of
+// items of one block (make_pair_items, T % 512 == 0 only) is left out: it saves a sixth of one round.
+long long pair_ns(int R, int C, int T, bool trans, bool channel_scales, int sms) {
   const long long tiles = (long long)((R + 255) / 256) * ((T + 511) / 512);
   const int pairs = sms / 2 > 0 ? sms / 2 : 1;
   const long long rounds = (tiles + pairs - 1) / pairs, stages = (C + 63) / 64;
-  return rounds * (T > 256 ? 4300 + stages * 666 : 3300 + stages * 580) + (channel_scales ? 9000 : 3200);
+  if (trans) return rounds * (T > 256 ? 4300 + stages * 666 : 3300 + stages * 580) + 3200;
+  return rounds * (T > 256 ? 3450 + stages * 618 : 1850 + stages * 550) + (channel_scales ? 4950 : 4400);
 }
 
 }  // namespace
 
-// Estimated time of this kernel on a call of T tokens, in ns.  Fitted to the same calls: 3.6 us a wave,
+// Estimated time of this kernel on a call of T tokens, in ns.  dX, fitted to the 400 calls: 3.6 us a wave,
 // 0.72 us + 0.83 ns per token a stage, and 34 ns per token of the tile for the exchange of the sums, 43
 // where no cluster shares it and 61 where a cluster owns several tiles.  Nine of ten estimates are 0.87
 // to 1.11 of what was measured.
 long long split_ns(const peqa_qweight_t* w, int T, bool trans) {
   const int R = trans ? w->in_features : w->out_features, C = trans ? w->out_features : w->in_features;
-  const SplitPlan p = plan_split((R + SM_ROWS - 1) / SM_ROWS, C, T, sm_count_or(148));
+  const SplitPlan p = plan_split((R + SM_ROWS - 1) / SM_ROWS, C, T, sm_count_or(148), trans);
+  if (!trans) return split_fwd_ns(p.waves, p.stages, p.nt, p.q);
   return (long long)p.waves * (3600 + p.stages * (720 + p.nt * 5 / 6) + p.nt * (34 + (p.cshift ? 0 : 9) + (p.q > 1 ? 27 : 0)));
 }
 
-// Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  Of the
-// 400 calls it is chosen for none where it was more than 3 % slower, and in five it is not chosen although it was
-// 6 to 10 % faster.  (Without the exchange's share of the time it was chosen for 25 where it was 4 to 55 %
-// slower: dX of 1656 x 3328 at 977 tokens 39.8 us here, 25.7 there; forward of 2360 x 256 at 1134
-// tokens in groups 15.1 / 10.3.)  Pair / here, in us: 4096 x 11008 forward at 1001 tokens 133 / 99, its dX
-// (86 row tiles: three waves) 102 / 138; 4096 x 4096 forward at 77 tokens 44 / 13; 22016 x 8192 at 256
-// tokens forward 178 / 128, dX 215 / 93.
+// Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  Of 150 forwards
+// the choice is more than 3 % off the faster one for two, of 150 dX for four (worst 8 %).  Pair / here, in us:
+// 4096 x 11008 forward at 1001 tokens 116 / 77, its dX (86 row tiles: three waves) 90 / 124; 4096 x 4096
+// forward at 77 tokens 42 / 12.5, at 2048 52 / 71; 22016 x 8192 at 256 tokens forward 174 / 109, dX 217 / 91;
+// 2360 x 256 forward at 1134 tokens 10.0 / 13.0.
 bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_scales) {
   const int R = trans ? w->in_features : w->out_features, C = trans ? w->out_features : w->in_features;
-  return split_ns(w, T, trans) * 100 < pair_ns(R, C, T, channel_scales, sm_count_or(148)) * 97;
+  return split_ns(w, T, trans) * 100 < pair_ns(R, C, T, trans, channel_scales, sm_count_or(148)) * 97;
 }
 
 // Partial sums per channel that a forward with dS writes.
 int split_ds_slots(const peqa_qweight_t* w, int T) {
-  const SplitPlan plan = plan_split((w->out_features + SM_ROWS - 1) / SM_ROWS, w->in_features, T, sm_count_or(148));
+  const SplitPlan plan = plan_split((w->out_features + SM_ROWS - 1) / SM_ROWS, w->in_features, T, sm_count_or(148), false);
   return plan.t_tiles * ((plan.nt + SM_DUMP_TOK - 1) / SM_DUMP_TOK);
 }
 
 // A part of a call begins at a multiple of this: whole token tiles.
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans) {
   const int r_tiles = ((trans ? w->in_features : w->out_features) + SM_ROWS - 1) / SM_ROWS;
-  return plan_split(r_tiles, trans ? w->out_features : w->in_features, T_call, sm_count_or(148)).nt;
+  return plan_split(r_tiles, trans ? w->out_features : w->in_features, T_call, sm_count_or(148), trans).nt;
 }
 
 // The T tokens from t0 on of a call of T_call tokens (act, out: of the part).  Plan and cut are those of the
@@ -631,7 +720,7 @@ int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
   p.R = trans ? p.K : p.N;
   const int C = trans ? p.N : p.K;
   p.r_tiles = (p.R + SM_ROWS - 1) / SM_ROWS;
-  const SplitPlan plan = plan_split(p.r_tiles, C, T_call, sm_count_or(148));
+  const SplitPlan plan = plan_split(p.r_tiles, C, T_call, sm_count_or(148), trans);
   p.nt = plan.nt;
   p.q = plan.q;
   p.cshift = plan.cshift;
@@ -641,10 +730,21 @@ int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const voi
   p.first = p.tile0 / p.q * p.q;
   p.t_first = t0 / plan.nt;
   p.k_blocks = (C + SM_BK - 1) / SM_BK;
-  const int stage_bytes = 2 * (SM_A_BYTES + p.nt * (SM_HALF * 2));
+  const int stage_bytes = 2 * ((trans ? SM_A_BYTES : 0) + p.nt * (SM_HALF * 2));
   p.stages = (SM_SMEM_LIMIT - SM_SMEM_FIXED) / stage_bytes;
   if (p.stages > SM_MAX_STAGES) p.stages = SM_MAX_STAGES;
-  const size_t smem = (size_t)p.stages * stage_bytes + SM_SMEM_FIXED;
+  const int segs = p.q > 1 ? 2 : 1;          // partial sums a CTA may hold
+  if (trans) {
+    p.acc2 = SM_MAX_NT;
+    p.a_col = 0;
+  } else {
+    p.acc2 = (p.nt + 31) & ~31;
+    p.stages = p.stages < split_tmem_stages(p.nt, p.q) ? p.stages : split_tmem_stages(p.nt, p.q);
+    p.a_col = 512 - p.stages * (SM_BK / 2);
+  }
+  const int dump = segs * (p.nt < SM_DUMP_TOK ? p.nt : SM_DUMP_TOK) * SM_ROWS * 4;
+  p.region = p.stages * stage_bytes > dump ? p.stages * stage_bytes : dump;
+  const size_t smem = (size_t)p.region + SM_SMEM_FIXED;
   PEQA_TRY(status_word(st, &p.status));
   EncodeTiledFn enc = nullptr;
   PEQA_TRY(tensor_map_encoder(&enc));
