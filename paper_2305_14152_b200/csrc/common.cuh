@@ -45,6 +45,23 @@ int allow_smem(Kern kern, int bytes, std::atomic<uint64_t>& done) {
   return PEQA_OK;
 }
 
+// Launches a kernel that begins with griddepcontrol.wait: its blocks stand ready when the kernel before it ends
+// (a training step of one 256 x 256 layer, whose last launch adds up 256 sums: 1 us).
+template <typename... P, typename... A>
+int launch_after(void (*kern)(P...), int blocks, int threads, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+  return PEQA_OK;
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Effective group size (per-channel when 0 or K) or 0 when invalid.

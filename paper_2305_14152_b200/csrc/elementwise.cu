@@ -429,6 +429,7 @@ __global__ void unpack_kernel(const uint32_t* __restrict__ qweight, long long to
 __global__ void adamw_kernel(float* __restrict__ s, const float* __restrict__ grad,
                              float* __restrict__ m, float* __restrict__ v, long long n,
                              const AdamWConsts c) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (; i < n; i += stride) {
@@ -549,10 +550,8 @@ extern "C" int peqa_scale_adamw(float* scales, const float* dS, float* m, float*
   if (numel <= 0 || step < 1) return PEQA_ERR_BAD_SHAPE;
   PEQA_TRY(check_arch());
   const int grid = grid_for(numel, 256);
-  adamw_kernel<<<grid, 256, 0, as_stream(stream)>>>(scales, dS, m, v, (long long)numel,
-                                                   adamw_consts(lr, beta1, beta2, eps, weight_decay, step));
-  PEQA_CUDA(cudaGetLastError());
-  return PEQA_OK;
+  return launch_after(adamw_kernel, grid, 256, as_stream(stream), scales, dS, m, v, (long long)numel,
+                      adamw_consts(lr, beta1, beta2, eps, weight_decay, step));
 }
 
 // App. K's "zero-points only" and "both" modes: the same AdamW step on the real-valued

@@ -743,6 +743,7 @@ __global__ void ds_reduce_zf_kernel(const float* __restrict__ partial_s, const f
                                     float* __restrict__ dS, float* __restrict__ dZ, long long n_out,
                                     int pieces_per_group, const float* __restrict__ zeros_f,
                                     const float* __restrict__ scales, int bits) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_out) return;
   float acc_s = 0.0f, acc_w = 0.0f;
@@ -766,6 +767,7 @@ __global__ void ds_reduce_kernel(const float* __restrict__ partial, float* __res
                                  const float* __restrict__ neg_scales, AdamWConsts adam,
                                  float* __restrict__ adam_s, float* __restrict__ adam_m,
                                  float* __restrict__ adam_v) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_out) return;
   const float* src = partial + e * pieces_per_group;
@@ -1081,20 +1083,14 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
     const long long n_out = (long long)p.N * p.G;
     const int ppg = g / p.piece;
     const int blocks = (int)((n_out + 255) / 256);
-    if (zeros_f) {
-      ds_reduce_zf_kernel<<<blocks, 256, 0, st>>>(p.out, p.out_z, dS, dZ, n_out, ppg, zeros_f, w->scales,
-                                                  w->bits);
-      PEQA_CUDA(cudaGetLastError());
-      return PEQA_OK;
-    }
-    ds_reduce_kernel<<<blocks, 256, 0, st>>>(p.out, dS, n_out, ppg, nullptr, p.adam, p.adam_s,
-                                             p.adam_m, p.adam_v);
-    PEQA_CUDA(cudaGetLastError());
-    if (dZ) {
-      ds_reduce_kernel<<<blocks, 256, 0, st>>>(p.out_z, dZ, n_out, ppg, w->scales, AdamWConsts{},
-                                               nullptr, nullptr, nullptr);
-      PEQA_CUDA(cudaGetLastError());
-    }
+    if (zeros_f)
+      return launch_after(ds_reduce_zf_kernel, blocks, 256, st, p.out, p.out_z, dS, dZ, n_out, ppg, zeros_f, w->scales,
+                          (int)w->bits);
+    PEQA_TRY(launch_after(ds_reduce_kernel, blocks, 256, st, p.out, dS, n_out, ppg, nullptr, p.adam, p.adam_s, p.adam_m,
+                          p.adam_v));
+    if (dZ)
+      PEQA_TRY(launch_after(ds_reduce_kernel, blocks, 256, st, p.out_z, dZ, n_out, ppg, w->scales, AdamWConsts{}, nullptr,
+                            nullptr, nullptr));
   }
   return PEQA_OK;
 }
