@@ -141,7 +141,8 @@ __device__ __forceinline__ void adamw_update(float& s, float gr, float& m, float
 // two accumulators of 256 tokens.  Tiles are dealt round-robin to the pairs; when the last round
 // would keep at most half of the pairs busy, its tiles are cut into two items of 256 tokens each.
 // Rebuilding the weights costs the same for one block of tokens as for two, so that round takes 0.8
-// to 0.9 as long (18944 x 8192, one round of 74 tiles: 256 tokens 92 us, 512 tokens 112).  Items [0, full_items) are whole tiles, the rest are
+// to 0.9 as long (18944 x 8192, one round of 74 tiles: 256 tokens 92 us, 512 tokens 112).  Every tile must have
+// two blocks to cut, the last row of tiles too (T % 512).  Items [0, full_items) are whole tiles, the rest are
 // halves: item full_items + 2*i + h is half h of tile full_items + i.
 struct PairItems {
   int o_tiles;       // 256-wide tiles along the output dimension
@@ -155,7 +156,7 @@ inline PairItems make_pair_items(int o_tiles, int t_tiles, int T, int pairs) {
   it.full_items = tiles;
   it.total_items = tiles;
   const int rem = pairs > 0 ? tiles % pairs : 0;
-  if (T % 512 == 0 && tiles > pairs && rem > 0 && 2 * rem <= pairs) {
+  if ((T % 512 == 0 || T % 512 > 256) && tiles > pairs && rem > 0 && 2 * rem <= pairs) {
     it.full_items = tiles - rem;
     it.total_items = tiles + rem;
   }

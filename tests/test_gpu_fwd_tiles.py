@@ -41,3 +41,25 @@ def test_scale_gradient_of_token_tiles(N, K, T):
     assert_close(dev_to_f64(L.Y)[toks], oracle.fwd(d["X"], packed, zeros, scales, 4, 0, tokens=toks), "Y")
     assert_close(dev_to_f64(L.dX)[toks], oracle.bwd_dx(d["dY"], packed, zeros, scales, K, 4, 0, tokens=toks), "dX")
     assert_close(dev_to_f64(L.dS)[rows], oracle.bwd_ds(d["X"], d["dY"], packed, zeros, 4, 0, rows=rows), "dS")
+
+
+@pytest.mark.parametrize("T", [769, 1001])
+@pytest.mark.parametrize("N,K,g", [(9728, 1024, 0), (1024, 9728, 64)])
+def test_short_last_round_of_ragged_tokens(N, K, g, T):
+    """76 tiles of 512 x 256 on 74 CTA pairs (forward of the first shape, dX of the second): the last two are halved,
+    and the last row of tiles has from one token on in its second half."""
+    d = synth.custom(N + T, N, K, T, 4, g, outliers=True, sigma_dy=1e-2)
+    codes, zeros, scales, packed = oracle_layer(d, 4, g)
+    qw = to_qweight(packed, zeros, scales, 4, g, K)
+    new = lambda c: torch.full((T + 2, c), 7.0, dtype=torch.bfloat16, device="cuda")
+    Y, dX = new(N), new(K)
+    L = binding.LayerLinear(w=qw, X=bf16_to_dev(d["X"]), dY=bf16_to_dev(d["dY"]), Y=Y[1:T + 1], dX=dX[1:T + 1],
+                            dS=torch.empty_like(qw.scales), workspace=binding.alloc_workspace(binding.OP_BWD, T, qw))
+    binding.layer_train_step([L], apply_adamw=False)
+    binding.check_status()
+    for out in (Y, dX):
+        assert torch.all(out[0] == 7.0) and torch.all(out[-1] == 7.0), "wrote outside its output"
+    toks, rows = np.array([0, 255, 256, 511, 512, 767, 768, T - 1]), np.arange(0, N, 997)
+    assert_close(dev_to_f64(L.Y)[toks], oracle.fwd(d["X"], packed, zeros, scales, 4, g, tokens=toks), "Y")
+    assert_close(dev_to_f64(L.dX)[toks], oracle.bwd_dx(d["dY"], packed, zeros, scales, K, 4, g, tokens=toks), "dX")
+    assert_close(dev_to_f64(L.dS)[rows], oracle.bwd_ds(d["X"], d["dY"], packed, zeros, 4, g, rows=rows), "dS")
