@@ -524,14 +524,9 @@ decode_prep_kernel(const PrepParams p) {
   // activation requests of the first chunk, which would otherwise queue behind a full ring of
   // weights on their way into this SM (the CTAs that start last wait longest for them).
   // The canonical matrix may be the result of the preceding kernel, so its codes are only asked for in L2,
-  // which a late write of them updates.
-  if (CANON) {
-    const uint32_t lo = (uint32_t)t_lo * (Row::chunks * 16);
-    const uint32_t hi = min((uint32_t)p.row_bytes, (uint32_t)(t_lo + n_t) * (Row::chunks * 16));
-#pragma unroll 1
-    for (int r = (int)threadIdx.x; r < (rg_end - rg0) * 8; r += kPThreads)
-      prefetch_l2(p.P + ((size_t)rg0 * 8 + r) * p.row_bytes + lo, hi - lo);
-  }
+  // which a late write of them updates: two steps a warp.  All of the CTA's rows at once kept the activations waiting (one scale
+  // per channel, us: 22016 x 8192, two tokens, 22.2 / 18.8, 8192 x 8192, one, 10.3 / 9.6); one step a warp is 2 to 3 %
+  // slower than all in groups of 128 and 256.
   // What does not depend on the preceding kernel is worked out before the wait for it: where this warp's steps of
   // the first chunk lie (the chunks after it look theirs up), and the tables of the final pass.
   issue_seek();
@@ -539,7 +534,15 @@ decode_prep_kernel(const PrepParams p) {
   const int lp_first = i_ch == 0 ? i_lp : 0, tl_first = i_ch == 0 ? i_tl : 0;
   const int last_first = hi_first > lo_first ? (hi_first - 1) / i_spc : -1;
   if (warp == kPWarps - 1) share_bounds(spc_of(0));
-  if (!CANON && lane == 0) issue_next();
+  if (CANON) {
+    // a row's piece of this warp's first two steps per lane
+    const int rg = pair_rg(lp_first);
+    const uint32_t off = (uint32_t)(t_lo + tl_first) * (Row::chunks * 16);
+    if (hi_first > lo_first && lane < (pair_full(lp_first) ? 16 : 8))
+      prefetch_l2(p.P + ((size_t)rg * 8 + lane) * p.row_bytes + off, min((uint32_t)p.row_bytes - off, (uint32_t)Row::chunks * 32));
+  } else if (lane == 0) {
+    issue_next();
+  }
   // I8: sixteen lanes take a step of a token, a lane half of what one of its strings becomes (the half is
   // the warp's); the first of them
   const int u_first = (int)(threadIdx.x >> 4) & 15;
