@@ -198,44 +198,37 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t cluster_addr) {
 }
 
 // Values of a step's quantization groups: the first `left` of TG adjacent entries (those beyond the
-// row's last group read as zero).  G: entries per row; when it is a multiple of TG they are one
-// aligned vector and never partly beyond the row.
-template <int TG>
-__device__ __forceinline__ void load_groups(const float* src, int left, bool row_ok, int G, float (&v)[TG]) {
+// row's last group read as zero).  V: entries come as aligned vectors of V, none of them partly beyond the row.
+// (All forms in one kernel, behind a test of the alignment, were 2 KB more for a launch to fetch.  One token in
+// groups of 64, us: 4096 x 4096 6.0 -> 5.3, 22016 x 8192 22.0 -> 21.3, 4096 x 11008, whose 172 groups a
+// row were single loads, 12.0 -> 9.8; seven of several tasks in groups of 128, 4096 x 11008, 19.4 -> 16.2.)
+template <int TG, int V>
+__device__ __forceinline__ void load_groups(const float* src, int left, bool row_ok, float (&v)[TG]) {
 #pragma unroll
-  for (int q = 0; q < TG; ++q) v[q] = 0.0f;
-  if (!row_ok || left <= 0) return;
-  if (TG >= 2 && (G % TG) == 0 && (reinterpret_cast<uintptr_t>(src) & (TG >= 4 ? 15u : 7u)) == 0) {
-    if constexpr (TG >= 4) {
-#pragma unroll
-      for (int q = 0; q < TG / 4; ++q) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(src) + q);
-        v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
-      }
-    } else if constexpr (TG == 2) {
-      const float2 t = __ldg(reinterpret_cast<const float2*>(src));
-      v[0] = t.x; v[1] = t.y;
+  for (int q = 0; q < TG; q += V) {
+    const bool on = row_ok && q < left;
+    if constexpr (V == 4) {
+      const float4 t = on ? __ldg(reinterpret_cast<const float4*>(src + q)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      v[q] = t.x; v[q + 1] = t.y; v[q + 2] = t.z; v[q + 3] = t.w;
+    } else if constexpr (V == 2) {
+      const float2 t = on ? __ldg(reinterpret_cast<const float2*>(src + q)) : make_float2(0.0f, 0.0f);
+      v[q] = t.x; v[q + 1] = t.y;
+    } else {
+      v[q] = on ? __ldg(src + q) : 0.0f;
     }
-  } else {
-#pragma unroll
-    for (int q = 0; q < TG; ++q)
-      if (q < left) v[q] = __ldg(src + q);
   }
 }
 // The same for zero-points, four to a word.
-template <int TG>
-__device__ __forceinline__ void load_zero_bytes(const uint8_t* src, int left, bool row_ok, int G,
-                                                uint32_t (&v)[(TG + 3) / 4]) {
+template <int TG, int V>
+__device__ __forceinline__ void load_zero_bytes(const uint8_t* src, int left, bool row_ok, uint32_t (&v)[(TG + 3) / 4]) {
 #pragma unroll
   for (int q = 0; q < (TG + 3) / 4; ++q) v[q] = 0u;
-  if (!row_ok || left <= 0) return;
-  if (TG >= 4 && (G % TG) == 0 && (reinterpret_cast<uintptr_t>(src) & 3u) == 0) {
 #pragma unroll
-    for (int q = 0; q < TG / 4; ++q) v[q] = __ldg(reinterpret_cast<const uint32_t*>(src) + q);
-  } else {
-#pragma unroll
-    for (int q = 0; q < TG; ++q)
-      if (q < left) v[q >> 2] |= (uint32_t)__ldg(src + q) << (8 * (q & 3));
+  for (int q = 0; q < TG; q += V) {
+    if (!row_ok || q >= left) continue;
+    if constexpr (V == 4) v[q / 4] = __ldg(reinterpret_cast<const uint32_t*>(src + q));
+    else if constexpr (V == 2) v[q / 4] |= (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(src + q)) << (8 * (q & 3));
+    else v[q / 4] |= (uint32_t)__ldg(src + q) << (8 * (q & 3));
   }
 }
 
@@ -348,6 +341,7 @@ struct CanonRow {
   static constexpr int pitch = BITS == 3 ? 208 : 256;
 };
 
+// V: the groups of a row are aligned vectors of so many, see load_groups.
 // GSH: quantization groups of 32 << GSH columns (1: 64, 2: 128, 3: 256), or 0: one group
 // per row or groups that are multiples of 512 columns (the sums of a whole staged chunk of
 // steps are taken off at once, which needs the chunk to lie inside one group).
@@ -357,7 +351,7 @@ struct CanonRow {
 // numbers of up to 31 bits times a power of two, cut into four signed digits, and the MMA's eight columns
 // are two tokens x four digits, which fp16 operands would leave idle.  An MMA covers twice the columns,
 // the codes are cheaper to take out (i8_string), and the sums of a group are exact.
-template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8>
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8, int V>
 __global__ void __launch_bounds__(kPThreads, 1)
 decode_prep_kernel(const PrepParams p) {
   constexpr int C = BITS;                            // 16-byte chunks per lane, step and group
@@ -924,13 +918,13 @@ decode_prep_kernel(const PrepParams p) {
         float gsa[NS][TG], gsb[NS][TG];
         uint32_t gza[(TG + 3) / 4], gzb[(TG + 3) / 4];             // four zero-points to a word
         if (GROUPED) {
-          load_zero_bytes<TG>(p.zeros + (size_t)rowa * p.G + gstep0, p.G - gstep0, true, p.G, gza);
-          load_zero_bytes<TG>(p.zeros + (size_t)rowb * p.G + gstep0, p.G - gstep0, has_b, p.G, gzb);
+          load_zero_bytes<TG, V>(p.zeros + (size_t)rowa * p.G + gstep0, p.G - gstep0, true, gza);
+          load_zero_bytes<TG, V>(p.zeros + (size_t)rowb * p.G + gstep0, p.G - gstep0, has_b, gzb);
 #pragma unroll
           for (int e = 0; e < NS; ++e) {
             const float* tab = p.scales + (TASKS ? (size_t)task_of[e] * p.N * p.G : 0) + gstep0;
-            load_groups<TG>(tab + (size_t)rowa * p.G, p.G - gstep0, true, p.G, gsa[e]);
-            load_groups<TG>(tab + (size_t)rowb * p.G, p.G - gstep0, has_b, p.G, gsb[e]);
+            load_groups<TG, V>(tab + (size_t)rowa * p.G, p.G - gstep0, true, gsa[e]);
+            load_groups<TG, V>(tab + (size_t)rowb * p.G, p.G - gstep0, has_b, gsb[e]);
           }
         }
         if constexpr (I8) {
@@ -1397,9 +1391,9 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
   return plan->ns < 0 ? PEQA_ERR_TOO_LARGE : PEQA_OK;
 }
 
-template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8>
+template <int BITS, int NT, int GSH, bool TASKS, bool CANON, bool I8, int V>
 int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS, CANON, I8>;
+  auto kern = decode_prep_kernel<BITS, NT, GSH, TASKS, CANON, I8, V>;
   static std::atomic<uint64_t> done{0};
   PEQA_TRY(allow_smem(kern, kPSmemLimit, done));
   cudaLaunchConfig_t cfg = {};
@@ -1422,13 +1416,23 @@ int launch_prep_t(const PrepParams& p, int grid, size_t smem, cudaStream_t st) {
 
 template <int BITS, int NT, bool TASKS, bool CANON, bool I8>
 int launch_prep_g(const PrepParams& p, int gsh, int grid, size_t smem, cudaStream_t st) {
+  // A step holds 8, 4 or 2 groups of a row; vectors of them where every row's groups start on one and are whole ones
+  // (a row of 11008 columns has 172 groups of 64 and 86 of 128).
+  auto in_vectors = [&](int v) {
+    return p.G % v == 0 && reinterpret_cast<uintptr_t>(p.scales) % (4 * v) == 0 && reinterpret_cast<uintptr_t>(p.zeros) % v == 0;
+  };
   switch (gsh) {
     case 1:
-      if constexpr (!CANON) return launch_prep_t<BITS, NT, 1, TASKS, CANON, I8>(p, grid, smem, st);
+      if constexpr (!CANON)
+        return in_vectors(4) ? launch_prep_t<BITS, NT, 1, TASKS, CANON, I8, 4>(p, grid, smem, st)
+                             : launch_prep_t<BITS, NT, 1, TASKS, CANON, I8, 1>(p, grid, smem, st);
       return PEQA_ERR_BAD_SHAPE;
-    case 2: return launch_prep_t<BITS, NT, 2, TASKS, CANON, I8>(p, grid, smem, st);
-    case 3: return launch_prep_t<BITS, NT, 3, TASKS, CANON, I8>(p, grid, smem, st);
-    default: return launch_prep_t<BITS, NT, 0, false, CANON, I8>(p, grid, smem, st);   // tasks: looked up per row
+    case 2:
+      return in_vectors(4)   ? launch_prep_t<BITS, NT, 2, TASKS, CANON, I8, 4>(p, grid, smem, st)
+             : in_vectors(2) ? launch_prep_t<BITS, NT, 2, TASKS, CANON, I8, 2>(p, grid, smem, st)
+                             : launch_prep_t<BITS, NT, 2, TASKS, CANON, I8, 1>(p, grid, smem, st);
+    case 3: return launch_prep_t<BITS, NT, 3, TASKS, CANON, I8, 1>(p, grid, smem, st);   // two groups a step
+    default: return launch_prep_t<BITS, NT, 0, false, CANON, I8, 1>(p, grid, smem, st);   // tasks: looked up per row
   }
 }
 

@@ -64,3 +64,32 @@ def test_tokens_of_any_magnitude(bits, g):
             assert_close(got[m] / np.abs(ref[i]).max(), ref[i] / np.abs(ref[i]).max(), f"token {m}")
         assert np.all(got[4] == 0.0)
         assert not np.any(np.isfinite(got[5])) and not np.any(np.isfinite(got[6]))
+
+
+@pytest.mark.parametrize("K,bits,g", [(128, 3, 64), (640, 4, 64), (768, 3, 64), (1024, 4, 64), (384, 3, 128), (768, 4, 128),
+                                      (1024, 3, 128)])
+def test_scales_and_zero_points_off_a_vector(K, bits, g):
+    """Rows whose groups are aligned vectors are read as such; a scale or zero-point array that starts one element
+    off takes the other kernel, with the same bits."""
+    N, M = 72, 16
+    d = synth.custom(N + K + bits, N, K, M, bits, g, outliers=True)
+    codes, zeros, scales, packed = oracle_layer(d, bits, g)
+    qw = to_qweight(packed, zeros, scales, bits, g, K)
+    prep = binding.decode_prepare(qw)
+    G = K // g
+    s_off = torch.zeros(N * G + 1, dtype=torch.float32, device="cuda")[1:].view(N, G).copy_(qw.scales)
+    z_off = torch.zeros(N * G + 1, dtype=torch.uint8, device="cuda")[1:].view(N, G).copy_(qw.zeros)
+    table = torch.stack([qw.scales, 2 * qw.scales])
+    t_off = torch.zeros(2 * N * G + 1, dtype=torch.float32, device="cuda")[1:].view(2, N, G).copy_(table)
+    ids = (torch.arange(M, device="cuda", dtype=torch.int32) % 2).contiguous()
+    X = bf16_to_dev(d["X"])
+    ref = oracle.fwd(d["X"], packed, zeros, scales, bits, g)
+    for m in (1, 2, 7, 16):
+        Y = binding.qlinear_decode_prepared(qw, prep, X[:m])
+        Yt = binding.qlinear_decode_prepared(qw, prep, X[:m], scale_table=table, task_ids=ids[:m])
+        assert_close(dev_to_f64(Y), ref[:m], f"M={m}")
+        for s, z in ((s_off, qw.zeros), (qw.scales, z_off)):
+            off = binding.QWeight(bits, N, K, g, qw.qweight, z, s)
+            assert torch.equal(binding.qlinear_decode_prepared(off, prep, X[:m]), Y)
+            assert torch.equal(binding.qlinear_decode_prepared(off, prep, X[:m], scale_table=t_off, task_ids=ids[:m]), Yt)
+    binding.check_status()
