@@ -147,6 +147,42 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &bars->abort_flag;
 
+  // ---- this CTA's stages: [lo, hi) of the cluster's list, its first tile's, then the next tile's.  The
+  // list is cut as in the whole call; a part of a call leaves out the stages of tiles that are not its own.
+  const int csize = 1 << p.cshift;
+  const int rank = (int)(blockIdx.x & (csize - 1));
+  const int first_tile = p.first + (int)(blockIdx.x >> p.cshift) * p.q;
+  const int L = min(p.q, p.tiles - first_tile) * p.k_blocks;
+  auto range_lo = [&](int r) { return (r * L) >> p.cshift; };
+  const int j_lo = max(0, p.tile0 - first_tile), j_hi = min(p.q, p.tile1 - first_tile);   // its own tiles
+  const int lo = min(max(range_lo(rank), j_lo * p.k_blocks), j_hi * p.k_blocks);
+  const int hi = min(max(range_lo(rank + 1), lo), j_hi * p.k_blocks);
+  const int n_it = hi - lo;
+  const int j0 = lo / p.k_blocks;                            // first tile of the range
+  const int split_at = (j0 + 1) * p.k_blocks - lo;           // local stages of the first tile
+  const int kb0 = lo - j0 * p.k_blocks;
+  // local stage -> k-block; row and token tile of the segment
+  auto kb_of = [&](int it) { return it < split_at ? kb0 + it : it - split_at; };
+  auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
+  auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles - p.t_first) * p.nt; };
+
+  // Forward: the first codes, scales and zero-points are asked for in L2 at once.  (Nothing is read: the preceding
+  // kernel may still be writing them, and L2 is where it writes.)  us before / after: 256 x 256 at 64 tokens 5.8 / 5.4,
+  // 4096 x 4096 at 77 12.55 / 12.3; dX gained nothing (13.0 / 13.2).
+  if constexpr (!TRANS) {
+    if (n_it > 0 && warp == 3 && lane < min(n_it, SM_PK_SLOTS)) {
+      prefetch_tile_2d(&tmap_pk, kb_of(lane) * (4 * BITS), r0_of(lane));
+    } else if (n_it > 0 && warp >= 4 && warp < 8) {
+      const int i = r0_of(0) + (int)threadIdx.x - 128, col = kb_of(0) * SM_BK;
+      if (i < p.N && col < p.K) {
+        const size_t gi = (size_t)i * p.G + split_group_of(p, col);
+        prefetch_l2(p.scales + gi);
+        if (ZF) prefetch_l2(p.zeros_f + gi);
+        else prefetch_l2(p.zeros + gi);
+      }
+    }
+  }
+
   if (threadIdx.x == 0) {
 #pragma unroll 1
     for (int s = 0; s < p.stages; ++s) {
@@ -177,25 +213,6 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem_base = bars->tmem_base;
-
-  // ---- this CTA's stages: [lo, hi) of the cluster's list, its first tile's, then the next tile's.  The
-  // list is cut as in the whole call; a part of a call leaves out the stages of tiles that are not its own.
-  const int csize = 1 << p.cshift;
-  const int rank = (int)(blockIdx.x & (csize - 1));
-  const int first_tile = p.first + (int)(blockIdx.x >> p.cshift) * p.q;
-  const int L = min(p.q, p.tiles - first_tile) * p.k_blocks;
-  auto range_lo = [&](int r) { return (r * L) >> p.cshift; };
-  const int j_lo = max(0, p.tile0 - first_tile), j_hi = min(p.q, p.tile1 - first_tile);   // its own tiles
-  const int lo = min(max(range_lo(rank), j_lo * p.k_blocks), j_hi * p.k_blocks);
-  const int hi = min(max(range_lo(rank + 1), lo), j_hi * p.k_blocks);
-  const int n_it = hi - lo;
-  const int j0 = lo / p.k_blocks;                            // first tile of the range
-  const int split_at = (j0 + 1) * p.k_blocks - lo;           // local stages of the first tile
-  const int kb0 = lo - j0 * p.k_blocks;
-  // local stage -> k-block; row and token tile of the segment
-  auto kb_of = [&](int it) { return it < split_at ? kb0 + it : it - split_at; };
-  auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
-  auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles - p.t_first) * p.nt; };
 
   if (warp == 0) {
     // ------------------------------------------------ activation TMA (one lane)
@@ -654,7 +671,7 @@ SplitPlan plan_split(int r_tiles, int C, int T, int sms, bool trans) {
 // takes 0.58 us, with two blocks of tokens in the tile 0.67; a round 3.3 us more, with two blocks
 // 4.3; the launch 3.2.  The forward, fitted to 150: 0.55 / 0.62 us, 1.85 / 3.45, 4.4 and 4.95 where its epilogue multiplies by
 // the channels' scales.  Nine of ten estimates are 0.88 to 1.09 of what was measured.  The shorter last round of
-// items of one block (make_pair_items, T % 512 == 0 only) is left out: it saves a sixth of one round.
+// items of one block (make_pair_items) is left out: it saves a sixth of one round.
 long long pair_ns(int R, int C, int T, bool trans, bool channel_scales, int sms) {
   const long long tiles = (long long)((R + 255) / 256) * ((T + 511) / 512);
   const int pairs = sms / 2 > 0 ? sms / 2 : 1;
