@@ -473,15 +473,18 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);   // vec_per divides kSplitWorkers: a thread keeps its rows
         // Two vectors per thread and turn, all of their sums requested before the first is used: one
         // after the other each waited for its reads and its store's address (128 x 128 outputs: 7100 cycles).
+        // dX takes one: half the code for a launch to fetch first
+        // (us, one / two: 8192 x 8192 at 45 tokens 28.2 / 28.9, 2672 x 1856 at 142 13.4 / 14.1).
+        constexpr int U = TRANS ? 1 : 2;
 #pragma unroll 1
-        for (int base_i = wtid; base_i < toks * vec_per; base_i += 2 * kSplitWorkers) {
-          float4 a[2];
-          uint2 y[2];
-          bool live[2];
-          int t[2], row[2];
-          uint32_t off[2];
+        for (int base_i = wtid; base_i < toks * vec_per; base_i += U * kSplitWorkers) {
+          float4 a[U];
+          uint2 y[U];
+          bool live[U];
+          int t[U], row[U];
+          uint32_t off[U];
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
+          for (int u = 0; u < U; ++u) {
             const int idx = base_i + u * kSplitWorkers;
             t[u] = idx >> vec_shift;
             const int rv = (idx & (vec_per - 1)) * 4;
@@ -497,9 +500,9 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
 #pragma unroll
           for (int rh = 0; rh < 8; rh += 4) {
             if (rh >= csize) break;
-            float4 v[2][4];
+            float4 v[U][4];
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < U; ++u)
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
                 v[u][r] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -508,14 +511,14 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
                                                       (uint32_t)(rh + r)));
               }
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < U; ++u)
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
                 a[u].x += v[u][r].x; a[u].y += v[u][r].y; a[u].z += v[u][r].z; a[u].w += v[u][r].w;
               }
           }
 #pragma unroll
-          for (int u = 0; u < 2; ++u) {
+          for (int u = 0; u < U; ++u) {
             if (!live[u]) continue;
             if (DS) {
               ds.x = fmaf(a[u].x, __uint_as_float(y[u].x << 16), ds.x);
