@@ -252,7 +252,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmap_q, const DecodeParams p) 
   for (int st = 0; st < nsteps; ++st) {
     const int col0 = kbeg + st * kStepCols + c4 * 128;   // first column of this lane's chunk
     const int slot = st % kDecSlots;
-    if (!ptx::mbar_wait(ptx::smem_u32(&bars->full[slot]), (st / kDecSlots) & 1u, abort_flag)) break;
+    if (!ptx::warp_wait(ptx::smem_u32(&bars->full[slot]), (st / kDecSlots) & 1u, abort_flag)) break;
     {
       const uint8_t* sb = slots + slot * kStepBytes + row_off0;
 #pragma unroll

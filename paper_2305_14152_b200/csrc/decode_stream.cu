@@ -292,7 +292,6 @@ decode_stream_kernel(const StreamParams p) {
     const uint8_t* xrow0 = xs + (size_t)(g8 < p.M ? g8 : 0) * p.x_pitch;
     const uint8_t* xrow1 = xs + (size_t)(g8 + 8 < p.M ? g8 + 8 : 0) * p.x_pitch;
     const bool vec_zs = GROUPED && p.g == 128 && (p.G & 3) == 0;
-    bool ok = true;
 
     for (int rb = 0; rb < nrb; ++rb) {
       int rows[4];
@@ -349,53 +348,51 @@ decode_stream_kernel(const StreamParams p) {
             }
           }
         }
-        if (ok && !ptx::mbar_wait(ptx::smem_u32(&bars->full[slot]), ((uint32_t)(s / p.slots)) & 1u, abort_flag))
-          ok = false;
-        if (ok) {
-          const uint8_t* sb = ring + (size_t)slot * Geo::slot + g8 * Geo::pitch;
+        // (a lane that gives up goes on with the others, over whatever the slot holds)
+        (void)ptx::mbar_wait(ptx::smem_u32(&bars->full[slot]), ((uint32_t)(s / p.slots)) & 1u, abort_flag);
+        const uint8_t* sb = ring + (size_t)slot * Geo::slot + g8 * Geo::pitch;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint32_t w[4][BITS];
+        for (int j = 0; j < 4; ++j) {
+          uint32_t w[4][BITS];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const uint8_t* src = sb + r * (8 * Geo::pitch) + (4 * j + c4) * (BITS * 4);
-              if constexpr (BITS == 4) {
-                const uint4 v = *reinterpret_cast<const uint4*>(src);
-                w[r][0] = v.x; w[r][1] = v.y; w[r][2] = v.z; w[r][3] = v.w;
-              } else {
-                const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src);
-                w[r][0] = s32[0]; w[r][1] = s32[1]; w[r][2] = s32[2];
-              }
+          for (int r = 0; r < 4; ++r) {
+            const uint8_t* src = sb + r * (8 * Geo::pitch) + (4 * j + c4) * (BITS * 4);
+            if constexpr (BITS == 4) {
+              const uint4 v = *reinterpret_cast<const uint4*>(src);
+              w[r][0] = v.x; w[r][1] = v.y; w[r][2] = v.z; w[r][3] = v.w;
+            } else {
+              const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src);
+              w[r][0] = s32[0]; w[r][1] = s32[1]; w[r][2] = s32[2];
             }
-            const int xo = (ch * 4 + j) * kSBlockBytes + c4 * 64;
-            const uint8_t* x0 = xrow0 + xo;
-            const uint8_t* x1 = xrow1 + xo;
-            unit_mma<BITS, NT, 0, 0>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 0, 1>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 1, 0>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 1, 1>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 2, 0>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 2, 1>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 3, 0>(w, x0, x1, acc);
-            unit_mma<BITS, NT, 3, 1>(w, x0, x1, acc);
-            if (GROUPED) {
-              // close the 128-column block: zero-point term out, scale in
+          }
+          const int xo = (ch * 4 + j) * kSBlockBytes + c4 * 64;
+          const uint8_t* x0 = xrow0 + xo;
+          const uint8_t* x1 = xrow1 + xo;
+          unit_mma<BITS, NT, 0, 0>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 0, 1>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 1, 0>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 1, 1>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 2, 0>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 2, 1>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 3, 0>(w, x0, x1, acc);
+          unit_mma<BITS, NT, 3, 1>(w, x0, x1, acc);
+          if (GROUPED) {
+            // close the 128-column block: zero-point term out, scale in
 #pragma unroll
-              for (int nt = 0; nt < NT; ++nt) {
-                const float4 xt = *reinterpret_cast<const float4*>(
-                    xtab + ((size_t)(ch * 4 + j) * TOKP + nt * 8 + 2 * c4) * 2);   // S0 B0 S1 B1
+            for (int nt = 0; nt < NT; ++nt) {
+              const float4 xt = *reinterpret_cast<const float4*>(
+                  xtab + ((size_t)(ch * 4 + j) * TOKP + nt * 8 + 2 * c4) * 2);   // S0 B0 S1 B1
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+              for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                  for (int q = 0; q < 2; ++q) {      // q = 0: row g8 of the half, q = 1: row g8 + 8
-                    const float z = zq[2 * h + q][j], sc = sq[2 * h + q][j];
-                    const float c0 = fmaf(z, xt.x, xt.y);      // z * S + B, token tk
-                    const float c1 = fmaf(z, xt.z, xt.w);      // token tk + 1
-                    tot[h][nt][2 * q] = fmaf(sc, acc[h][nt][2 * q] - c0, tot[h][nt][2 * q]);
-                    tot[h][nt][2 * q + 1] = fmaf(sc, acc[h][nt][2 * q + 1] - c1, tot[h][nt][2 * q + 1]);
-                    acc[h][nt][2 * q] = 0.0f;
-                    acc[h][nt][2 * q + 1] = 0.0f;
-                  }
+                for (int q = 0; q < 2; ++q) {      // q = 0: row g8 of the half, q = 1: row g8 + 8
+                  const float z = zq[2 * h + q][j], sc = sq[2 * h + q][j];
+                  const float c0 = fmaf(z, xt.x, xt.y);      // z * S + B, token tk
+                  const float c1 = fmaf(z, xt.z, xt.w);      // token tk + 1
+                  tot[h][nt][2 * q] = fmaf(sc, acc[h][nt][2 * q] - c0, tot[h][nt][2 * q]);
+                  tot[h][nt][2 * q + 1] = fmaf(sc, acc[h][nt][2 * q + 1] - c1, tot[h][nt][2 * q + 1]);
+                  acc[h][nt][2 * q] = 0.0f;
+                  acc[h][nt][2 * q + 1] = 0.0f;
                 }
               }
             }

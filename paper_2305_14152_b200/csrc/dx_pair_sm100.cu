@@ -234,7 +234,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       pair_item(p.items, tile, p.T, j_tile, tt0, blocks);
       const int j0 = j_tile * 256;
       const int row0 = tt0 + m * 256 + (int)rank * 128 + quarter * 32;   // first token of this warp
-      if (!mbar_wait_cluster(smem_u32(&bars->acc_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
+      if (!warp_wait_cluster(smem_u32(&bars->acc_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
       tc_fence_after();
       int chunks = m < blocks ? (p.K - j0 + 31) / 32 : 0;                // K is a multiple of 32
       chunks = chunks > 8 ? 8 : chunks;
@@ -334,7 +334,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       if (it + X_GROUPS < total_it) load_zs(zn, scn, czn);
       const int s = it % XSTAGES;
       const int q = it % XQ_SLOTS;
-      if (!mbar_wait(smem_u32(&bars->pk_full[q]), (it / XQ_SLOTS) & 1u, abort_flag)) break;
+      if (!warp_wait(smem_u32(&bars->pk_full[q]), (it / XQ_SLOTS) & 1u, abort_flag)) break;
       uint32_t wa[BITS], wb[BITS];
       {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(sm_q + q * XQ_BYTES) + u4 * BITS;
@@ -363,7 +363,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       fence_proxy_async_smem();                                   // the codes have been read
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // slot free
-      if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ((it / XSTAGES) & 1u) ^ 1u, abort_flag)) break;
+      if (!warp_wait_cluster(smem_u32(&bars->empty[s]), ((it / XSTAGES) & 1u) ^ 1u, abort_flag)) break;
       uint8_t* wbuf = base + s * XSTAGE_BYTES + XA_BYTES;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {

@@ -283,13 +283,12 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       };
       float next_scale = chunk_scale(n0);
       if (DS) load_dy(0);
-      if (!mbar_wait_cluster(smem_u32(&bars->acc_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
-      __syncwarp();
+      if (!warp_wait_cluster(smem_u32(&bars->acc_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
       tc_fence_after();
       int chunks = m < blocks ? (p.N - n0 + 31) / 32 : 0;
       chunks = chunks > 8 ? 8 : chunks;
       // the sums of the last tile must have been read before the staging tiles are written again
-      if (DS && local > 0 && !mbar_wait(smem_u32(&bars->ds_free), (uint32_t)(local - 1) & 1u, abort_flag)) { ok = false; break; }
+      if (DS && local > 0 && !warp_wait(smem_u32(&bars->ds_free), (uint32_t)(local - 1) & 1u, abort_flag)) { ok = false; break; }
 #pragma unroll 1
       for (int cc = 0; cc < chunks; ++cc) {
         const int c0 = n0 + cc * 32;
@@ -378,7 +377,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         for (int k = 0; k < 8; ++k) mine[k * 32 + lane] = ds_sum[k];
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&bars->ds_full));
-        if (!mbar_wait(smem_u32(&bars->ds_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
+        if (!warp_wait(smem_u32(&bars->ds_full), (uint32_t)(local & 1), abort_flag)) { ok = false; break; }
         // thread = channel: the four warps of a token block, in order
         const int ch = (warp - 4) * 32 + lane;
         const float* all = reinterpret_cast<const float*>(sm_e);
@@ -476,7 +475,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       if (it + P_GROUPS < total_it) load_zs(zn, scn, czn);
       const int s = it % PSTAGES;
       const int q = it % PQ_SLOTS;
-      if (!mbar_wait(smem_u32(&bars->pk_full[q]), (it / PQ_SLOTS) & 1u, abort_flag)) break;
+      if (!warp_wait(smem_u32(&bars->pk_full[q]), (it / PQ_SLOTS) & 1u, abort_flag)) break;
       uint32_t w[2][BITS];
       {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(sm_q + q * PQ_BYTES) + row * 8;
@@ -506,7 +505,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       fence_proxy_async_smem();                                   // the codes have been read
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->pk_empty[q]));   // slot free
-      if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ((it / PSTAGES) & 1u) ^ 1u, abort_flag)) break;
+      if (!warp_wait_cluster(smem_u32(&bars->empty[s]), ((it / PSTAGES) & 1u) ^ 1u, abort_flag)) break;
       uint8_t* wrow = base + s * PSTAGE_BYTES + PA_BYTES + row * 128;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {

@@ -254,7 +254,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
       const int t0 = (tile / p.r_tiles) * BN;
       const int buf = local & 1;
       const uint32_t acc_ph = (local >> 1) & 1u;
-      if (!mbar_wait(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
+      if (!warp_wait(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after();
       const int r = r0 + ew * 32 + lane;
       float scale = 1.0f;
@@ -337,7 +337,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
       uint32_t o[UPT][16];
 #pragma unroll
       for (int k = 0; k < UPT; ++k) dequant_unit<BITS, FOLD>(cur[k], p.zeros_f != nullptr, o[k]);
-      if (!mbar_wait(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) break;
+      if (!warp_wait(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) break;
 #pragma unroll
       for (int k = 0; k < UPT; ++k) {
         uint8_t* row_ptr = sm.a[s] + row_off[k];
@@ -636,7 +636,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
       uint32_t w[4][BITS];
       if (PKTMA) {
         const int ps = local & 1;
-        if (!mbar_wait(smem_u32(&bars->pk_full[ps]), acc_ph, abort_flag)) { ok = false; break; }
+        if (!warp_wait(smem_u32(&bars->pk_full[ps]), acc_ph, abort_flag)) { ok = false; break; }
         const uint8_t* src = sm_pk + ps * DS_PK_BYTES;
         const int row = quarter * 32 + lane;
         if constexpr (BITS == 4) {
@@ -663,7 +663,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
             w[cc][q] = row_ok && c0 + cc * 32 < p.K ? __ldg(p.qw + (size_t)i * p.wpr + ((c0 >> 5) + cc) * BITS + q) : 0u;
         }
       }
-      if (!mbar_wait_cluster(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
+      if (!warp_wait_cluster(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after();
       float acc = 0.0f, accz = 0.0f;
       float r[4] = {0.f, 0.f, 0.f, 0.f}, rz[4] = {0.f, 0.f, 0.f, 0.f};

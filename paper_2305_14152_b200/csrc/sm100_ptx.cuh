@@ -79,6 +79,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
   }
 }
 
+// The wait of a whole warp whose lanes go on together (shuffles, tensor-memory accesses, __syncwarp): all of
+// them see the phase, or all of them leave.  Left to itself a lane whose bound has run out would be gone
+// while the others wait for it, without a bound, at the next warp-wide instruction.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
+
 // Orders this thread's earlier accesses to shared memory (generic proxy) before later ones of the
 // async proxy: its writes are then visible to TMA and to the tensor cores' operand reads, and its
 // reads are done when a copy refills what was read.  An mbarrier orders threads, not proxies, so a
@@ -323,6 +330,10 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
       }
     }
   }
+}
+// The same for a whole warp, see warp_wait.
+__device__ __forceinline__ bool warp_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait_cluster(bar, parity, abort_flag)) != 0;
 }
 // 2D tiled load issued by either CTA of a pair; completion bytes are credited
 // to `bar`, a shared::cluster address (normally the leader CTA's barrier).

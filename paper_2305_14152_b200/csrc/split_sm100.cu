@@ -331,9 +331,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     auto turn = [&](int it, const UnitZS (&cur)[2], UnitZS (&next)[2]) -> bool {
       load_zs(it + 2, next);
       const int pq = it % SM_PK_SLOTS;
-      // (the lanes agree on the way out, so that the tensor-memory stores find the warp whole)
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)))
-        return false;
+      if (!warp_wait(smem_u32(&bars->full_pk[pq]), (it / SM_PK_SLOTS) & 1u, abort_flag)) return false;
       const uint8_t* src = sm_pk + pq * SM_PK_BYTES;
       uint32_t w[2][BITS];
       if constexpr (!TRANS) {
@@ -375,8 +373,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
         else dq::unit32_natural<BITS, FOLD>(w[k], cur[k].z, cur[k].s, o[k]);
       }
       const int s = it % p.stages;
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)))
-        return false;
+      if (!warp_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)) return false;
       if constexpr (TRANS) {
         uint8_t* tile = base + s * stage_bytes + half * half_bytes;
 #pragma unroll
@@ -422,7 +419,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   const bool worker = warp >= 4;
   bool ok = n_it > 0;
   if (worker && ok) {
-    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag));
+    ok = warp_wait(smem_u32(&bars->acc_full), 0, abort_flag);
     tc_fence_after();
   }
   __syncwarp();

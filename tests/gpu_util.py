@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests: buffer conversion and the error metrics."""
+import ctypes
+
 import numpy as np
 import torch
 
@@ -30,6 +32,31 @@ def assert_close(got: np.ndarray, ref: np.ndarray, what: str):
     assert rel <= REL_L2_TOL, f"{what}: rel-L2 {rel:.3e} > {REL_L2_TOL}"
     assert mx <= MAX_ABS_TOL * np.abs(ref).max(), f"{what}: max-abs {mx:.3e} vs max|ref| {np.abs(ref).max():.3e}"
     return rel, mx
+
+
+def kernels_of(call):
+    """Names (mangled) of the kernels a call launches, from a captured graph of it.  (The profiler drops events in a
+    process that has run for minutes.)"""
+    call()                                          # what is set up once is not captured
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    cu, at = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph())
+    count, names = ctypes.c_size_t(), []
+    assert cu.cuGraphGetNodes(at, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert cu.cuGraphGetNodes(at, nodes, ctypes.byref(count)) == 0
+    for node in nodes:
+        node, kind = ctypes.c_void_p(node), ctypes.c_int()
+        assert cu.cuGraphNodeGetType(node, ctypes.byref(kind)) == 0
+        if kind.value != 0:                         # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        params, name = (ctypes.c_uint64 * 16)(), ctypes.c_char_p()          # CUDA_KERNEL_NODE_PARAMS: the function first
+        assert cu.cuGraphKernelNodeGetParams_v2(node, params) == 0
+        assert cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(params[0])) == 0
+        names.append(name.value.decode())
+    return names
 
 
 def oracle_layer(d, bits, g):
