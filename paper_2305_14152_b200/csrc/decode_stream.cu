@@ -85,6 +85,7 @@ struct StreamParams {
   int x_blocks;             // 128-column blocks staged per token (4 * nchunks)
   int x_pitch;              // bytes between staged token rows
   int slots;                // ring depth
+  int bars;                 // pairs of barriers, see stream_bars
   // multi-task decode (one scale per channel only): token m uses the scales at
   // scales + clamp(task_ids[m], 0, n_tasks - 1) * N; task_ids == nullptr: one task
   const int32_t* task_ids;
@@ -92,12 +93,22 @@ struct StreamParams {
   int* status;
 };
 
-struct StreamBarriers {
-  uint64_t full[kSMaxSlots];    // the step's row pieces have landed
-  uint64_t empty[kSMaxSlots];   // the warp that owns the step has read it
-  int abort_flag;
-  int wait_limit_us;    // must follow abort_flag (read by the bounded waits)
-};
+// Pairs of barriers for the steps of a CTA: "full", the step's row pieces have landed, and "empty", the warp that
+// owns the step has read it.  Step s has pair s % bars, turn s / bars.  A wait tells a turn from the one
+// before it by parity alone, so a warp that waits for a turn while the turn before the last is still open takes it for
+// done; with a pair per ring slot that happens, since the steps of a 32-row block belong to sixteen
+// warps that do not wait for one another: a warp ran ahead of the slot's previous step wherever a block has more steps than
+// the ring slots (4 bits, 8192 columns, two tokens: 16 steps, 15 slots), read codes that were not there, and
+// the ring lost count.  The block's end is the only point all warps pass together.  With nchunks + max(slots, 4) pairs
+// the step one turn earlier lies in an earlier block for whoever waits: for the warp of step s, s - bars; for the
+// producer of step s, which waits for s - slots to be read and knows s - 4 - slots to be read, s - slots - bars; and
+// a copy that would open the next turn waits for a step of a later block.
+inline int stream_bars(int steps, int nchunks, int slots) {
+  const int n = nchunks + (slots > 4 ? slots : 4);
+  return n < steps ? n : steps;
+}
+// bytes of the pairs, the abort flag and the wait limit
+inline size_t stream_bar_bytes(int bars) { return (size_t)bars * 2 * sizeof(uint64_t) + 2 * sizeof(int); }
 
 __device__ __forceinline__ void smma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                            uint32_t b1) {
@@ -138,8 +149,10 @@ decode_stream_kernel(const StreamParams p) {
   float* xtab = reinterpret_cast<float*>(xs + (((size_t)p.M * p.x_pitch + 15) & ~(size_t)15));
   float* xtot = xtab + (size_t)p.x_blocks * TOKP * 2;      // [TOKP][lo, hi] over all of K
   float* partial = xtot + TOKP * 2;                         // [2][kSWarps][32][TOKP]
-  StreamBarriers* bars = reinterpret_cast<StreamBarriers*>(partial + 2 * kSWarps * 32 * TOKP);
-  volatile int* abort_flag = &bars->abort_flag;
+  uint64_t* full = reinterpret_cast<uint64_t*>(partial + 2 * kSWarps * 32 * TOKP);   // [bars]
+  uint64_t* empty = full + p.bars;                                                    // [bars]
+  // followed by the wait limit (read by the bounded waits)
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + p.bars);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g8 = lane >> 2, c4 = lane & 3;
@@ -153,15 +166,17 @@ decode_stream_kernel(const StreamParams p) {
   // of weight traffic they would wait for microseconds, and everything waits for them.
   const int units = p.x_blocks * 4;                    // 32-column units per token, zero past K
   uint4 xv[kSMaxXLoads];
-  if (threadIdx.x == kSThreads) {
-    for (int q = 0; q < p.slots; ++q) {
-      ptx::mbar_init(ptx::smem_u32(&bars->full[q]), 32);   // one arrival per lane of the issuing warp
-      ptx::mbar_init(ptx::smem_u32(&bars->empty[q]), 1);
+  if (is_producer) {
+    for (int q = (int)threadIdx.x - kSThreads; q < p.bars; q += kSProdThreads) {
+      ptx::mbar_init(ptx::smem_u32(&full[q]), 32);   // one arrival per lane of the issuing warp
+      ptx::mbar_init(ptx::smem_u32(&empty[q]), 1);
     }
-    bars->abort_flag = 0;
-    bars->wait_limit_us = p.status[4];
+    if (threadIdx.x == kSThreads) {
+      abort_flag[0] = 0;
+      abort_flag[1] = p.status[4];
+    }
     ptx::fence_mbar_init();
-  } else if (!is_producer) {
+  } else {
 #pragma unroll
     for (int q = 0; q < kSMaxXLoads / 4; ++q) {
       const int idx = q * kSThreads + threadIdx.x;       // one 32-column unit of one token
@@ -186,12 +201,12 @@ decode_stream_kernel(const StreamParams p) {
     const uint8_t* qbytes = reinterpret_cast<const uint8_t*>(p.qw);
     for (int s = warp - kSWarps; s < total_steps; s += kSProducers) {
       const int rb = s / p.nchunks, ch = s - rb * p.nchunks;
-      const int slot = s % p.slots;
+      const int slot = s < p.slots ? s : s % p.slots;
       if (s >= p.slots) {
         int good = 1;
         if (lane == 0)
-          good = ptx::mbar_wait(ptx::smem_u32(&bars->empty[slot]), (((uint32_t)(s / p.slots)) & 1u) ^ 1u,
-                                abort_flag) ? 1 : 0;
+          good = ptx::mbar_wait(ptx::smem_u32(&empty[(s - p.slots) % p.bars]),
+                                ((uint32_t)((s - p.slots) / p.bars)) & 1u, abort_flag) ? 1 : 0;
         good = __shfl_sync(0xffffffffu, good, 0);
         if (!good) break;
       }
@@ -208,7 +223,7 @@ decode_stream_kernel(const StreamParams p) {
           ptx::cp_async_16(ptx::smem_u32(sdst + row * Geo::pitch + 16 * k),
                            qbytes + (size_t)(rbase + row) * row_bytes + off + 16u * k);
       }
-      ptx::cp_async_mbar_arrive_noinc(ptx::smem_u32(&bars->full[slot]));
+      ptx::cp_async_mbar_arrive_noinc(ptx::smem_u32(&full[s < p.bars ? s : s % p.bars]));
     }
   } else {
     // ------------------------------------------------ stage the activations
@@ -311,7 +326,9 @@ decode_stream_kernel(const StreamParams p) {
 
       for (int ch = warp; ch < p.nchunks; ch += kSWarps) {
         const int s = rb * p.nchunks + ch;
-        const int slot = s % p.slots;
+        // (a CTA of one block uses every slot and barrier once: no divisions)
+        const int slot = s < p.slots ? s : s % p.slots;
+        const int turn = s < p.bars ? 0 : s / p.bars, bar = s - turn * p.bars;
         // zero-points and scales of the step's four 128-column blocks, requested before
         // the wait so that their latency is hidden behind it
         float zq[4][4], sq[4][4];
@@ -349,7 +366,7 @@ decode_stream_kernel(const StreamParams p) {
           }
         }
         // (a lane that gives up goes on with the others, over whatever the slot holds)
-        (void)ptx::mbar_wait(ptx::smem_u32(&bars->full[slot]), ((uint32_t)(s / p.slots)) & 1u, abort_flag);
+        (void)ptx::mbar_wait(ptx::smem_u32(&full[bar]), (uint32_t)turn & 1u, abort_flag);
         const uint8_t* sb = ring + (size_t)slot * Geo::slot + g8 * Geo::pitch;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -400,7 +417,7 @@ decode_stream_kernel(const StreamParams p) {
         }
         // the codes of this step are consumed: hand the slot back
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&bars->empty[slot]));
+        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&empty[bar]));
       }
 
       // ---- this warp's partial sums of the block: [32 rows][TOKP]
@@ -452,7 +469,7 @@ decode_stream_kernel(const StreamParams p) {
 }
 
 struct StreamPlan {
-  int rows_per_cta, grid, nchunks, x_blocks, x_pitch, slots;
+  int rows_per_cta, grid, nchunks, x_blocks, x_pitch, slots, bars;
   size_t smem;
 };
 
@@ -479,16 +496,18 @@ int plan_stream(const peqa_qweight_t* w, int g, int M, StreamPlan* plan) {
   // pitch = blocks*288 + pad with pitch % 128 == 8: consecutive tokens land 2 banks apart
   const int raw = plan->x_blocks * kSBlockBytes;
   plan->x_pitch = raw + ((8 - raw % 128) % 128 + 128) % 128;
+  const int steps = ((plan->rows_per_cta + 31) / 32) * plan->nchunks;
   const size_t fixed = 128 /*alignment*/ + (((size_t)M * plan->x_pitch + 15) & ~(size_t)15) +
                        (size_t)plan->x_blocks * TOKP * 2 * sizeof(float) + (size_t)TOKP * 2 * sizeof(float) +
-                       (size_t)2 * kSWarps * 32 * TOKP * sizeof(float) + sizeof(StreamBarriers) + 16;
+                       (size_t)2 * kSWarps * 32 * TOKP * sizeof(float) +
+                       stream_bar_bytes(stream_bars(steps, plan->nchunks, kSMaxSlots)) + 16;
   const size_t slot = w->bits == 3 ? StreamGeom<3>::slot : StreamGeom<4>::slot;
   if (fixed + 8 * slot > (size_t)kSSmemLimit) return PEQA_OK;   // activations too large to stage
   size_t slots = ((size_t)kSSmemLimit - fixed) / slot;
   if (slots > (size_t)kSMaxSlots) slots = kSMaxSlots;
-  const size_t steps = (size_t)((plan->rows_per_cta + 31) / 32) * plan->nchunks;
-  if (slots > steps) slots = steps;
+  if (slots > (size_t)steps) slots = steps;
   plan->slots = (int)slots;
+  plan->bars = stream_bars(steps, plan->nchunks, plan->slots);
   plan->smem = fixed + slots * slot;
   return PEQA_OK;
 }
@@ -539,6 +558,7 @@ int launch_decode_stream(const peqa_qweight_t* w, int g, const void* X, int M, v
   p.x_blocks = plan.x_blocks;
   p.x_pitch = plan.x_pitch;
   p.slots = plan.slots;
+  p.bars = plan.bars;
   PEQA_TRY(status_word(st, &p.status));
   const bool grouped = p.G > 1;
   const int NT = M <= 8 ? 1 : 2;
