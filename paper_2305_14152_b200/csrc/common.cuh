@@ -47,6 +47,7 @@ int allow_smem(Kern kern, int bytes, std::atomic<uint64_t>& done) {
 
 // Launches a kernel that begins with griddepcontrol.wait: its blocks stand ready when the kernel before it ends
 // (a training step of one 256 x 256 layer, whose last launch adds up 256 sums: 1 us).
+// Its pointer parameters are not __restrict__ (see ld_global in sm100_ptx.cuh).
 template <typename... P, typename... A>
 int launch_after(void (*kern)(P...), int blocks, int threads, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};

@@ -208,13 +208,13 @@ __device__ __forceinline__ void load_groups(const float* src, int left, bool row
   for (int q = 0; q < TG; q += V) {
     const bool on = row_ok && q < left;
     if constexpr (V == 4) {
-      const float4 t = on ? __ldg(reinterpret_cast<const float4*>(src + q)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const float4 t = on ? ld_global(reinterpret_cast<const float4*>(src + q)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       v[q] = t.x; v[q + 1] = t.y; v[q + 2] = t.z; v[q + 3] = t.w;
     } else if constexpr (V == 2) {
-      const float2 t = on ? __ldg(reinterpret_cast<const float2*>(src + q)) : make_float2(0.0f, 0.0f);
+      const float2 t = on ? ld_global(reinterpret_cast<const float2*>(src + q)) : make_float2(0.0f, 0.0f);
       v[q] = t.x; v[q + 1] = t.y;
     } else {
-      v[q] = on ? __ldg(src + q) : 0.0f;
+      v[q] = on ? ld_global(src + q) : 0.0f;
     }
   }
 }
@@ -226,9 +226,9 @@ __device__ __forceinline__ void load_zero_bytes(const uint8_t* src, int left, bo
 #pragma unroll
   for (int q = 0; q < TG; q += V) {
     if (!row_ok || q >= left) continue;
-    if constexpr (V == 4) v[q / 4] = __ldg(reinterpret_cast<const uint32_t*>(src + q));
-    else if constexpr (V == 2) v[q / 4] |= (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(src + q)) << (8 * (q & 3));
-    else v[q / 4] |= (uint32_t)__ldg(src + q) << (8 * (q & 3));
+    if constexpr (V == 4) v[q / 4] = ld_global(reinterpret_cast<const uint32_t*>(src + q));
+    else if constexpr (V == 2) v[q / 4] |= (uint32_t)ld_global(reinterpret_cast<const uint16_t*>(src + q)) << (8 * (q & 3));
+    else v[q / 4] |= (uint32_t)ld_global(src + q) << (8 * (q & 3));
   }
 }
 
@@ -579,8 +579,8 @@ decode_prep_kernel(const PrepParams p) {
       const int lp = r >> 4, lr = r & 15;
       if (r >= npairs * 16 || (!pair_full(lp) && lr >= 8)) return;
       const size_t at = (size_t)(pair_rg(lp) * 8 + lr) * p.G + (p.G == 1 ? 0 : col0 / (p.K / p.G));
-      z = __ldg(p.zeros + at);
-      if (!p.task_ids) sc = __ldg(p.scales + at);
+      z = ld_global(p.zeros + at);
+      if (!p.task_ids) sc = ld_global(p.scales + at);
     };
     uint32_t z_own = 0u;
     float s_own = 0.0f;
@@ -605,7 +605,7 @@ decode_prep_kernel(const PrepParams p) {
         for (int r = 0; r < 4; ++r) {
           next[r] = make_uint4(0u, 0u, 0u, 0u);
           if (u < units && col + own_col + (CANON ? r * 8 : r * 32) < ccols)
-            next[r] = __ldg(reinterpret_cast<const uint4*>(xcol + (size_t)next_tok * p.K + col + (CANON ? r * 8 : r * 32)));
+            next[r] = ld_global(reinterpret_cast<const uint4*>(xcol + (size_t)next_tok * p.K + col + (CANON ? r * 8 : r * 32)));
         }
       };
       load(u_first);
@@ -856,7 +856,7 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll
       for (int e = 0; e < 2; ++e)
         if ((I8 ? c4 >> 1 : c4 * 2 + e) < p.M)
-          task_of[e] = min(max(__ldg(p.task_ids + (I8 ? c4 >> 1 : c4 * 2 + e)), 0), p.n_tasks - 1);
+          task_of[e] = min(max(ld_global(p.task_ids + (I8 ? c4 >> 1 : c4 * 2 + e)), 0), p.n_tasks - 1);
     }
     int lin = lo;
     int lp = first_pair;
@@ -1139,8 +1139,8 @@ decode_prep_kernel(const PrepParams p) {
           const int gg = p.G == 1 ? 0 : col0 / (p.K / p.G);
           const float* tab = p.scales + (size_t)row * p.G + gg;
           const size_t per = (size_t)p.N * p.G;
-          s0 = __ldg(tab + (size_t)min(max(__ldg(p.task_ids + m), 0), p.n_tasks - 1) * per);
-          if (m + 1 < p.M) s1 = __ldg(tab + (size_t)min(max(__ldg(p.task_ids + m + 1), 0), p.n_tasks - 1) * per);
+          s0 = ld_global(tab + (size_t)min(max(ld_global(p.task_ids + m), 0), p.n_tasks - 1) * per);
+          if (m + 1 < p.M) s1 = ld_global(tab + (size_t)min(max(ld_global(p.task_ids + m + 1), 0), p.n_tasks - 1) * per);
         }
         sum.x = fmaf(-zs.x, t0, sum.x) * s0;
         sum.y = fmaf(-zs.x, t1, sum.y) * s1;

@@ -310,13 +310,13 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
         cz[k] = 0.0f;
         if (i < p.N && pf_col < p.K) {
           const size_t gi = (size_t)i * p.G + dx_group_of(p, pf_col);
-          sc[k] = __ldg(p.scales + gi);
+          sc[k] = ld_global(p.scales + gi);
           if (ZF) {
             float delta;
-            dq::split_zero_point<BITS>(__ldg(p.zeros_f + gi), z[k], delta);
+            dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), z[k], delta);
             cz[k] = -delta * sc[k];
           } else {
-            z[k] = __ldg(p.zeros + gi);
+            z[k] = ld_global(p.zeros + gi);
           }
         }
       }

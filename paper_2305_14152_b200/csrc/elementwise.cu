@@ -426,8 +426,8 @@ __global__ void unpack_kernel(const uint32_t* __restrict__ qweight, long long to
 }
 
 // Elementwise AdamW in binary32 (adamw_update in common.cuh).
-__global__ void adamw_kernel(float* __restrict__ s, const float* __restrict__ grad,
-                             float* __restrict__ m, float* __restrict__ v, long long n,
+__global__ void adamw_kernel(float* s, const float* grad,
+                             float* m, float* v, long long n,
                              const AdamWConsts c) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -272,13 +272,13 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       // after the other, by every lane) a chunk took 7000 cycles, 3500 for the scales and 2600 for dY.
       // With dY (DS) a chunk is worked through in two halves of 16 channels, which leaves registers for that.
       constexpr int W = DS ? 16 : 32;              // channels at a time
-      auto chunk_scale = [&](int c) { return !FOLD && c + lane < p.N ? __ldg(p.scales + c + lane) : 0.0f; };
+      auto chunk_scale = [&](int c) { return !FOLD && c + lane < p.N ? ld_global(p.scales + c + lane) : 0.0f; };
       uint4 dy[2];
       auto load_dy = [&](int c) {                  // tokens and channels beyond the matrix count zero
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           dy[q] = make_uint4(0u, 0u, 0u, 0u);
-          if (m < blocks && row0 + lane < p.T && n0 + c + 8 * q < p.N) dy[q] = __ldg(reinterpret_cast<const uint4*>(dy_row + c + 8 * q));
+          if (m < blocks && row0 + lane < p.T && n0 + c + 8 * q < p.N) dy[q] = ld_global(reinterpret_cast<const uint4*>(dy_row + c + 8 * q));
         }
       };
       float next_scale = chunk_scale(n0);
@@ -427,35 +427,35 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         const size_t gi = (size_t)pf_r * p.G + pair_group_of(p, col);
         if (ZF) {
           float delta;
-          sc[0] = __ldg(p.scales + gi);
-          dq::split_zero_point<BITS>(__ldg(p.zeros_f + gi), z[0], delta);
+          sc[0] = ld_global(p.scales + gi);
+          dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), z[0], delta);
           cz[0] = -delta * sc[0];
           z[1] = z[0]; sc[1] = sc[0]; cz[1] = cz[0];
           if (!one_group && col + 32 < p.K) {
             const size_t g1 = (size_t)pf_r * p.G + pair_group_of(p, col + 32);
-            sc[1] = __ldg(p.scales + g1);
-            dq::split_zero_point<BITS>(__ldg(p.zeros_f + g1), z[1], delta);
+            sc[1] = ld_global(p.scales + g1);
+            dq::split_zero_point<BITS>(ld_global(p.zeros_f + g1), z[1], delta);
             cz[1] = -delta * sc[1];
           }
         } else if (one_group) {
-          z[0] = z[1] = __ldg(p.zeros + gi);
-          if (FOLD) sc[0] = sc[1] = __ldg(p.scales + gi);
+          z[0] = z[1] = ld_global(p.zeros + gi);
+          if (FOLD) sc[0] = sc[1] = ld_global(p.scales + gi);
         } else if (pair_load) {
-          const uint32_t z2 = __ldg(reinterpret_cast<const unsigned short*>(p.zeros + gi));
+          const uint32_t z2 = ld_global(reinterpret_cast<const unsigned short*>(p.zeros + gi));
           z[0] = z2 & 0xFFu;
           z[1] = z2 >> 8;
           if (FOLD) {
-            const float2 s2 = __ldg(reinterpret_cast<const float2*>(p.scales + gi));
+            const float2 s2 = ld_global(reinterpret_cast<const float2*>(p.scales + gi));
             sc[0] = s2.x;
             sc[1] = s2.y;
           }
         } else {
-          z[0] = __ldg(p.zeros + gi);
-          if (FOLD) sc[0] = __ldg(p.scales + gi);
+          z[0] = ld_global(p.zeros + gi);
+          if (FOLD) sc[0] = ld_global(p.scales + gi);
           if (col + 32 < p.K) {
             const size_t g1 = (size_t)pf_r * p.G + pair_group_of(p, col + 32);
-            z[1] = __ldg(p.zeros + g1);
-            if (FOLD) sc[1] = __ldg(p.scales + g1);
+            z[1] = ld_global(p.zeros + g1);
+            if (FOLD) sc[1] = ld_global(p.scales + g1);
           }
         }
       }

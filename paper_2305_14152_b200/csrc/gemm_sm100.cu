@@ -128,16 +128,16 @@ __device__ __forceinline__ Unit<BITS> load_unit(const QGemmParams& p, int i, int
   if (i < p.N && col0 < p.K) {
     const uint32_t* src = p.qw + (size_t)i * p.wpr + (col0 >> 5) * BITS;
 #pragma unroll
-    for (int q = 0; q < BITS; ++q) u.w[q] = __ldg(src + q);
+    for (int q = 0; q < BITS; ++q) u.w[q] = ld_global(src + q);
     const size_t gidx = (size_t)i * p.G + group_of(p, col0);
-    u.s = __ldg(p.scales + gidx);
+    u.s = ld_global(p.scales + gidx);
     u.c = 0.0f;
     if (p.zeros_f) {
       float delta;
-      dq::split_zero_point<BITS>(__ldg(p.zeros_f + gidx), u.z, delta);
+      dq::split_zero_point<BITS>(ld_global(p.zeros_f + gidx), u.z, delta);
       u.c = -delta * u.s;
     } else {
-      u.z = __ldg(p.zeros + gidx);
+      u.z = ld_global(p.zeros + gidx);
     }
   } else {
     // Outside the matrix: codes equal to the zero-point dequantise to exactly 0.
@@ -258,7 +258,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
       tc_fence_after();
       const int r = r0 + ew * 32 + lane;
       float scale = 1.0f;
-      if (!FOLD && r < p.R) scale = __ldg(p.scales + r);  // per-channel forward: s[i] applied here
+      if (!FOLD && r < p.R) scale = ld_global(p.scales + r);  // per-channel forward: s[i] applied here
 #pragma unroll 1
       for (int cc = 0; cc < BN / 32; ++cc) {
         const int tc0 = t0 + cc * 32;
@@ -622,9 +622,9 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         zreal[k] = sc[k] = ms[k] = mm[k] = mv[k] = 0.0f;
         if (k < n_pieces) {
           const size_t gi = (size_t)i * p.G + (p.G == 1 ? 0 : (c0 + k * p.piece) / p.g);
-          if (DZ && p.zeros_f) zreal[k] = __ldg(p.zeros_f + gi);
-          else z[k] = __ldg(p.zeros + gi);
-          if (DZ && p.piece == p.g) sc[k] = __ldg(p.scales + gi);
+          if (DZ && p.zeros_f) zreal[k] = ld_global(p.zeros_f + gi);
+          else z[k] = ld_global(p.zeros + gi);
+          if (DZ && p.piece == p.g) sc[k] = ld_global(p.scales + gi);
         }
       }
       if (ADAM) {
@@ -660,7 +660,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         for (int cc = 0; cc < 4; ++cc) {
 #pragma unroll
           for (int q = 0; q < BITS; ++q)
-            w[cc][q] = row_ok && c0 + cc * 32 < p.K ? __ldg(p.qw + (size_t)i * p.wpr + ((c0 >> 5) + cc) * BITS + q) : 0u;
+            w[cc][q] = row_ok && c0 + cc * 32 < p.K ? ld_global(p.qw + (size_t)i * p.wpr + ((c0 >> 5) + cc) * BITS + q) : 0u;
         }
       }
       if (!warp_wait_cluster(smem_u32(&bars->acc_full[buf]), acc_ph, abort_flag)) { ok = false; break; }
@@ -739,10 +739,10 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
 
 // Real-valued zero-point, groups wider than a piece: dS = sum(pieces) - delta * sum(dW pieces)
 // and dZ = -s * sum(dW pieces), pieces added in index order.
-__global__ void ds_reduce_zf_kernel(const float* __restrict__ partial_s, const float* __restrict__ partial_w,
-                                    float* __restrict__ dS, float* __restrict__ dZ, long long n_out,
-                                    int pieces_per_group, const float* __restrict__ zeros_f,
-                                    const float* __restrict__ scales, int bits) {
+__global__ void ds_reduce_zf_kernel(const float* partial_s, const float* partial_w,
+                                    float* dS, float* dZ, long long n_out,
+                                    int pieces_per_group, const float* zeros_f,
+                                    const float* scales, int bits) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_out) return;
@@ -762,11 +762,11 @@ __global__ void ds_reduce_zf_kernel(const float* __restrict__ partial_s, const f
 // dS[i, gi] = sum of the group's partial pieces, in index order (deterministic); with
 // neg_scales the sum is multiplied by -s[i, gi] (the zero-point gradient); with adam_s the
 // AdamW step on scale e follows at once.
-__global__ void ds_reduce_kernel(const float* __restrict__ partial, float* __restrict__ dS,
+__global__ void ds_reduce_kernel(const float* partial, float* dS,
                                  long long n_out, int pieces_per_group,
-                                 const float* __restrict__ neg_scales, AdamWConsts adam,
-                                 float* __restrict__ adam_s, float* __restrict__ adam_m,
-                                 float* __restrict__ adam_v) {
+                                 const float* neg_scales, AdamWConsts adam,
+                                 float* adam_s, float* adam_m,
+                                 float* adam_v) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_out) return;
@@ -785,9 +785,9 @@ __global__ void ds_reduce_kernel(const float* __restrict__ partial, float* __res
 
 // dS[i] = sum over the token blocks' partial sums, in a fixed order (eight interleaved chains, then
 // these in order), and the AdamW step on scale i with adam_s.
-__global__ void ds_channel_kernel(const float* __restrict__ part, float* __restrict__ dS, int N, int slots,
-                                  AdamWConsts adam, float* __restrict__ adam_s, float* __restrict__ adam_m,
-                                  float* __restrict__ adam_v) {
+__global__ void ds_channel_kernel(const float* part, float* dS, int N, int slots,
+                                  AdamWConsts adam, float* adam_s, float* adam_m,
+                                  float* adam_v) {
   // Launched programmatically: its blocks stand ready when the kernel before (dX) ends (LLaMA-7B MLP, 66
   // tokens, 1.5 us a linear).  The next kernel, which reads the scales written here, is not let in early.
   asm volatile("griddepcontrol.wait;" ::: "memory");

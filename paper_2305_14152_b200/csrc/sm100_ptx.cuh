@@ -22,6 +22,62 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+// A read of memory that the kernel before in the stream may have written, in a kernel that is launched
+// programmatically: an ordinary load behind griddepcontrol.wait.  __ldg, and a load through a const __restrict__
+// parameter that the compiler makes one of, are for data that nobody writes for as long as the kernel lives, and
+// such a kernel lives from before its predecessor's last stores.  The compiler may move the load as it may move a
+// __ldg, but not before the wait: its address comes from behind it, from a statement that stays in order.
+template <typename T>
+__device__ __forceinline__ const T* behind_wait(const T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+__device__ __forceinline__ float ld_global(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ float2 ld_global(const float2* p) {
+  float2 v;
+  asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ float4 ld_global(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ uint8_t ld_global(const uint8_t* p) {
+  uint32_t v;
+  asm("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(behind_wait(p)));
+  return (uint8_t)v;
+}
+__device__ __forceinline__ uint16_t ld_global(const uint16_t* p) {
+  uint16_t v;
+  asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
+  uint32_t v;
+  asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ int32_t ld_global(const int32_t* p) {
+  int32_t v;
+  asm("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ uint2 ld_global(const uint2* p) {
+  uint2 v;
+  asm("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(behind_wait(p)));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_global(const uint4* p) {
+  uint4 v;
+  asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(behind_wait(p)));
+  return v;
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

@@ -117,13 +117,13 @@ __device__ __forceinline__ UnitZS split_load_zs(const SplitParams& p, int i, int
   u.c = 0.0f;
   if (i < p.N && col < p.K) {
     const size_t gi = (size_t)i * p.G + split_group_of(p, col);
-    u.s = __ldg(p.scales + gi);
+    u.s = ld_global(p.scales + gi);
     if (ZF) {
       float delta;
-      dq::split_zero_point<BITS>(__ldg(p.zeros_f + gi), u.z, delta);
+      dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), u.z, delta);
       u.c = -delta * u.s;
     } else {
-      u.z = __ldg(p.zeros + gi);
+      u.z = ld_global(p.zeros + gi);
     }
   }
   return u;
@@ -491,7 +491,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
             a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (DS) {
               y[u] = make_uint2(0u, 0u);
-              if (live[u]) y[u] = __ldg(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t[u]) * p.R + row[u]));
+              if (live[u]) y[u] = ld_global(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t[u]) * p.R + row[u]));
             }
           }
 #pragma unroll
@@ -524,7 +524,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
               ds.w = fmaf(a[u].w, __uint_as_float(y[u].y & 0xFFFF0000u), ds.w);
             }
             if (!FOLD) {
-              const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scales + row[u]));   // one scale per channel
+              const float4 sc = ld_global(reinterpret_cast<const float4*>(p.scales + row[u]));   // one scale per channel
               a[u].x *= sc.x; a[u].y *= sc.y; a[u].z *= sc.z; a[u].w *= sc.w;
             }
             __nv_bfloat162 h0 = __floats2bfloat162_rn(a[u].x, a[u].y), h1 = __floats2bfloat162_rn(a[u].z, a[u].w);
