@@ -12,10 +12,13 @@ others through ctypes.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from dataclasses import dataclass
 
 import torch
+
+from .build import native_path
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpeqa_b200.so")
@@ -136,7 +139,13 @@ def _load_native():
     global _native
     if _native is None:
         lib()
-        from . import _native as module
+        path = native_path()
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2305_14152_b200.build` first, with this "
+                               "interpreter and this torch")
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
         module.bind_error(PeqaError)
         _native = module
     return _native

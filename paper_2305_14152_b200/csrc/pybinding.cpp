@@ -55,11 +55,13 @@ const at::Tensor& dev(PyObject* o, at::ScalarType dtype, const char* name) {
 
 void* ptr_or_null(PyObject* o, const char* name) { return o == Py_None ? nullptr : tensor(o, name).data_ptr(); }
 
-int as_int(PyObject* o) {
-  const long v = PyLong_AsLong(o);
-  if (v == -1 && PyErr_Occurred()) fail();
-  return (int)v;
+// Whole numbers as ctypes takes them: whatever has __index__, modulo the width.
+long long as_long(PyObject* o) {
+  const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
+  if (v == ~0ull && PyErr_Occurred()) fail();
+  return (long long)v;
 }
+int as_int(PyObject* o) { return (int)as_long(o); }
 float as_float(PyObject* o) {
   const double v = PyFloat_AsDouble(o);
   if (v == -1.0 && PyErr_Occurred()) fail();
@@ -113,14 +115,25 @@ void arity(Py_ssize_t n, Py_ssize_t want) {
   fail();
 }
 
-// The output: the caller's, or a new tensor beside `like`.
-PyObject* output(PyObject* given, const at::Tensor& like, int64_t rows, int64_t cols, void** data) {
+// The output: the caller's, or a new tensor beside `like` (of its class, if that is not torch's own).
+PyObject* output(PyObject* given, PyObject* like, int64_t rows, int64_t cols, void** data) {
   if (given != Py_None) {
     *data = tensor(given, "Y").data_ptr();
     Py_INCREF(given);
     return given;
   }
-  at::Tensor t = like.new_empty({rows, cols});
+  if (!THPVariable_CheckExact(like)) {
+    PyObject* made = PyObject_CallMethod(like, "new_empty", "((LL))", (long long)rows, (long long)cols);
+    if (!made) fail();
+    if (!THPVariable_Check(made)) {
+      Py_DECREF(made);
+      PyErr_SetString(PyExc_TypeError, "new_empty did not return a tensor");
+      fail();
+    }
+    *data = THPVariable_Unpack(made).data_ptr();
+    return made;
+  }
+  at::Tensor t = THPVariable_Unpack(like).new_empty({rows, cols});
   *data = t.data_ptr();
   return THPVariable_Wrap(std::move(t));
 }
@@ -147,7 +160,7 @@ PyObject* qlinear_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int64_t T = X.size(0);
   const peqa_qweight_t w = weight(a[0]);
   void* y;
-  Ref Y(output(a[2], X, T, w.out_features, &y));
+  Ref Y(output(a[2], a[1], T, w.out_features, &y));
   const Workspace ws(a[3]);
   void *x = X.data_ptr(), *st = stream();
   check(unlocked([&] { return peqa_qlinear_fwd(&w, x, (int)T, y, ws.p, ws.bytes, st); }), "peqa_qlinear_fwd");
@@ -165,7 +178,7 @@ PyObject* qlinear_fwd_zf(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int64_t T = X.size(0);
   const peqa_qweight_t w = weight(a[0]);
   void* y;
-  Ref Y(output(a[3], X, T, w.out_features, &y));
+  Ref Y(output(a[3], a[2], T, w.out_features, &y));
   void *x = X.data_ptr(), *st = stream();
   check(unlocked([&] { return peqa_qlinear_fwd_zf(&w, zf, x, (int)T, y, st); }), "peqa_qlinear_fwd_zf");
   Py_INCREF(Y.p);
@@ -181,7 +194,7 @@ PyObject* qlinear_decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int64_t M = X.size(0);
   const peqa_qweight_t w = weight(a[0]);
   void* y;
-  Ref Y(output(a[2], X, M, w.out_features, &y));
+  Ref Y(output(a[2], a[1], M, w.out_features, &y));
   void *x = X.data_ptr(), *st = stream();
   const Workspace given(a[3]);
   at::Tensor own;
@@ -209,7 +222,7 @@ PyObject* qlinear_decode_prepared(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int64_t M = X.size(0);
   const peqa_qweight_t w = weight(a[0]);
   void* y;
-  Ref Y(output(a[3], X, M, w.out_features, &y));
+  Ref Y(output(a[3], a[2], M, w.out_features, &y));
   const float* table = nullptr;
   const int32_t* ids = nullptr;
   int n_tasks = 0;
@@ -243,8 +256,7 @@ PyObject* adamw(PyObject* const* a, Py_ssize_t n, const char* values, const char
   float* v = static_cast<float*>(dev(a[3], at::kFloat, "v").data_ptr());
   float c[5];
   for (int i = 0; i < 5; ++i) c[i] = as_float(a[4 + i]);
-  const long long step = PyLong_AsLongLong(a[9]);
-  if (step == -1 && PyErr_Occurred()) fail();
+  const long long step = as_long(a[9]);
   void* st = stream();
   check(unlocked([&] { return entry(s, g, m, v, count, c[0], c[1], c[2], c[3], c[4], (int64_t)step, st); }), where);
   Py_RETURN_NONE;
@@ -264,6 +276,10 @@ PyObject* zero_adamw(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* layer_train_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   HANDLE_TH_ERRORS
   arity(n, 8);
+  if (!PySequence_Check(a[0])) {                   // (an iterator would be used up by one look at it)
+    PyErr_SetString(PyExc_TypeError, "linears: expected a sequence of LayerLinear");
+    fail();
+  }
   Ref seq(PySequence_Fast(a[0], "linears: expected a sequence of LayerLinear"));
   const Py_ssize_t count = PySequence_Fast_GET_SIZE(seq.p);
   if (count == 0) {
@@ -301,8 +317,7 @@ PyObject* layer_train_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (apply < 0) fail();
   float c[5];
   for (int i = 0; i < 5; ++i) c[i] = as_float(a[2 + i]);
-  const long long step = PyLong_AsLongLong(a[7]);
-  if (step == -1 && PyErr_Occurred()) fail();
+  const long long step = as_long(a[7]);
   void* st = stream();
   check(unlocked([&] {
           return peqa_layer_train_step(L.data(), (int)count, (int)T, apply, c[0], c[1], c[2], c[3], c[4], (int64_t)step, st);
