@@ -437,7 +437,7 @@ size_t decode_workspace_bytes(const peqa_qweight_t*, int, int) { return 0; }
 // of K (1872 x 512 4.8 / 6.2, 3768 x 1664 4.8 / 6.6, 4096 x 4096 6.5 / 7.2); more rows or columns are slower there
 // (11152 x 256 8.5 / 6.8, 15240 x 640 10.0 / 7.9, 1520 x 11136 10.9 / 8.1, 21784 x 21632 133 / 78; worst 8192 x 8192 12.7 / 12.9).
 bool decode_rows_are_faster(const peqa_qweight_t* w, int g, int M) {
-  if (M > 8 || !decode_rows_supported(w, g, M)) return false;
+  if (!decode_rows_supported(w, g, M)) return false;
   if (g != w->in_features || !decode_stream_supported(w, g, M)) return true;
   const int sms = sm_count_or(148);
   return (w->out_features / 8 + sms - 1) / sms > 4 || w->in_features > 5120;

@@ -1441,8 +1441,8 @@ int launch_prep_g(const PrepParams& p, int gsh, int grid, size_t smem, cudaStrea
 
 template <int BITS, bool CANON>
 int launch_prep_b(const PrepParams& p, bool i8, int gsh, int grid, size_t smem, cudaStream_t st) {
-  if (p.M > 8) return launch_prep_g<BITS, 2, false, CANON, false>(p, gsh, grid, smem, st);
-  if constexpr (!CANON) {
+  if constexpr (!CANON) {                              // (canonical rows: at most eight tokens, see decode_rows_supported)
+    if (p.M > 8) return launch_prep_g<BITS, 2, false, false, false>(p, gsh, grid, smem, st);
     if (p.task_ids)
       return i8 ? launch_prep_g<BITS, 1, true, false, true>(p, gsh, grid, smem, st)
                 : launch_prep_g<BITS, 1, true, false, false>(p, gsh, grid, smem, st);
@@ -1464,15 +1464,15 @@ bool prep_group_supported(int K, int g) {
   return g == K || g % kStepCols == 0 || g == 64 || g == 128 || g == 256;
 }
 
-// One launch, or two of at most eight tokens each, over prepared or canonical weights.
+// One launch over prepared or canonical weights, or (prepared ones) two of at most eight tokens each.
 int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, const void* X, int M, void* Y,
                const float* scale_table, int n_tasks, const int32_t* task_ids, cudaStream_t st) {
   PrepPlan plan;
   bool two = false;
   if (M > 8) {
     PrepPlan half;
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, canon, false, &half));
-    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, false, &plan) != PEQA_OK ||
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, false, false, &half));
+    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, false, false, &plan) != PEQA_OK ||
           2 * half.ns < plan.ns;
   } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, true, &plan) != PEQA_OK) {
     PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, false, &plan));
@@ -1484,8 +1484,8 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
     // room in shared memory (from about 42000 rows on for 16 tokens, 68000 for 12, 113000 for 9).
     const int h = (M + 1) / 2;
     const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
-    PEQA_TRY(run_decode(w, weights, canon, g, X, h, Y, scale_table, n_tasks, task_ids, st));
-    return run_decode(w, weights, canon, g, static_cast<const char*>(X) + (size_t)h * K * 2, M - h,
+    PEQA_TRY(run_decode(w, weights, false, g, X, h, Y, scale_table, n_tasks, task_ids, st));
+    return run_decode(w, weights, false, g, static_cast<const char*>(X) + (size_t)h * K * 2, M - h,
                       static_cast<char*>(Y) + (size_t)h * N * 2, scale_table, n_tasks,
                       task_ids ? task_ids + h : nullptr, st);
   }
@@ -1525,12 +1525,14 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
 
 bool decode_rows_supported(const peqa_qweight_t* w, int g, int M) {
   PrepPlan plan;
-  return w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == w->in_features || g == 128 || g == 256) &&
-         plan_prep(w->out_features, w->in_features, M > 8 ? (M + 1) / 2 : M, w->bits, g, true, false, &plan) == PEQA_OK;
+  return M <= 8 && w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == w->in_features || g == 128 || g == 256) &&
+         plan_prep(w->out_features, w->in_features, M, w->bits, g, true, false, &plan) == PEQA_OK;
 }
 
 int launch_decode_rows(const peqa_qweight_t* w, int g, const void* X, int M, void* Y, const float* scale_table,
                        int n_tasks, const int32_t* task_ids, cudaStream_t st) {
+  // the instances of canonical rows have one token tile, and know a table per task with one scale per channel only
+  if (M > 8 || (task_ids && g != w->in_features)) return PEQA_ERR_BAD_SHAPE;
   return run_decode(w, w->qweight, true, g, X, M, Y, scale_table, n_tasks, task_ids, st);
 }
 
