@@ -430,15 +430,24 @@ int launch_decode_t(const CUtensorMap& tmap_q, const DecodeParams& p, int row_bl
 
 size_t decode_workspace_bytes(const peqa_qweight_t*, int, int) { return 0; }
 
-// Up to eight tokens, 45 shapes from 272 to 22016 rows and columns (us, decode_stream_kernel or, where its activations
-// do not fit, decode_kernel / the kernel of the prepared decode).  Groups of 128 or 256 columns: faster there at
-// all of 17, 664 x 768 6.5 / 6.1, 11008 x 4096 17.5 / 13.4, 848 x 19328 29.5 / 11.7.  One scale per channel: the streaming
-// kernel's set-up is 1 us shorter, so it keeps what it does in one block of 32 rows per CTA and few steps
-// of K (1872 x 512 4.8 / 6.2, 3768 x 1664 4.8 / 6.6, 4096 x 4096 6.5 / 7.2); more rows or columns are slower there
-// (11152 x 256 8.5 / 6.8, 15240 x 640 10.0 / 7.9, 1520 x 11136 10.9 / 8.1, 21784 x 21632 133 / 78; worst 8192 x 8192 12.7 / 12.9).
+// Up to eight tokens, us, the other kernel that would serve the call / the kernel of the prepared decode (rows).
+// Groups of 128 or 256 columns: by rows, faster at 45 of 47 shapes (664 x 768 6.5 / 6.1, 11008 x 4096 17.5 / 13.4, 848 x 19328
+// 29.5 / 11.7; worst 1288 x 256 5.9 / 6.3).  One scale per channel, activations that fit decode_stream_kernel: by rows
+// from 33 rows per CTA or more than 5120 columns on (11152 x 256 8.5 / 6.8, 1520 x 11136 10.9 / 8.1, 21784 x 21632 133 / 78; worst,
+// with three tokens, 8112 x 2176 8.5 / 9.1).  Below, rows win as often as not (4096 x 4096, one token 5.8 / 5.6,
+// three 7.6 / 9.4; 3768 x 1664 4.8 / 6.6; 344 x 3072, eight 9.0 / 6.0) and those calls stay where they were.
+// One scale per channel, activations that do not fit it: decode_kernel, whose clusters of eight CTAs, two CTAs per SM,
+// run at once up to 33 blocks of 128 rows and need no more for many rows than for few.  Three-bit rows take the
+// other kernel about as long as four-bit ones, decode_kernel less, and where its blocks nearly fill the chip it is
+// faster at 28 of 31 such calls (3888 x 19968, seven tokens 17.9 / 20.9, 4096 x 11008, four 12.0 / 13.2, 3048 x 6400, eight 10.2 /
+// 12.1; worst 3064 x 5632, five 10.9 / 9.8), else at 5 of 87 (5352 x 9344, four bits, eight 25.3 / 15.5, 304 x 18688, four 10.5 / 7.2).
 bool decode_rows_are_faster(const peqa_qweight_t* w, int g, int M) {
   if (!decode_rows_supported(w, g, M)) return false;
-  if (g != w->in_features || !decode_stream_supported(w, g, M)) return true;
+  if (g != w->in_features) return true;
+  if (!decode_stream_supported(w, g, M)) {
+    const int blocks = (w->out_features + kRowsPerCta - 1) / kRowsPerCta;
+    return w->bits != 3 || blocks > 33 || blocks <= (M >= 5 ? 20 : 26);
+  }
   const int sms = sm_count_or(148);
   return (w->out_features / 8 + sms - 1) / sms > 4 || w->in_features > 5120;
 }

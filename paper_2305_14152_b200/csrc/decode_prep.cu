@@ -1314,14 +1314,21 @@ int x_pitch_for(int steps) {
 // One CTA per range needs no exchange of sums, but it stages all of its K: from five to eight tokens
 // on, the activations do not fit beside the rings, and working through K in chunks costs a
 // staging, a parking and a reduce per chunk.  A cluster of 2, 4 or 8 CTAs stages a slice each and
-// adds its sums up through distributed shared memory.  The estimate, in ns, from timelines of
-// single CTAs: a warp's step of a pair 1600 (3000 with groups inside the step, a third more with
-// two token tiles), 10 per token and step staged, 2500 for the cluster's exchange, 1500 + 400 M per
-// further chunk, 10000 more for a second wave of clusters.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at 22016 x 8192
-// 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
+// adds its sums up through distributed shared memory.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at
+// 22016 x 8192 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
+//
+// The estimate, in ns, is fitted to 265 calls (1 to 16 tokens, prepared and canonical), each timed with clusters of 1, 2, 4
+// and 8: nine of ten within 0.90 to 1.15, and the shape it picks costs 1.2 % more than the best of
+// the four on average, 17 % at worst.  2300 a launch; a warp's step of a pair 1650 (2350 with groups inside the
+// step, 13 % more with two token tiles; integer kernel 1200 and 1450; canonical rows 350 more); staging a token's step
+// 45, 85 in the integer kernel, 95 from canonical rows, whose order takes the activations in half sectors; 15 per
+// row group and token for the final pass, 12 where a cluster shares it, and 1350 for the cluster's exchange; 4000
+// per further chunk; 10000 more for a second wave of clusters.  (With 10 ns for staging whatever the kernel and 2500 for
+// the exchange, single CTAs staged 50 to 90 token-steps where a cluster would have been faster, 5.6 % on
+// average: 696 x 14720, two tokens 9.1 / 5.4 us, 368 x 8704, four 7.9 / 5.7, canonical 872 x 8832, five 15.6 / 8.0.)
 //
 // i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
-// staged at once, at most two steps to a half-warp.
+// staged at once, at most four steps to a half-warp.
 int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
@@ -1386,9 +1393,11 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       c.i8 = i8;
       c.smem = need(c.spc, c.slots, c.sps);
       const long long steps = ((long long)c.rg_per_cta * Tl + 1) / 2;
-      const long long per_step = i8 ? (grouped ? 1900 : 1000) : (grouped ? 3000 : 1600) * (NT == 2 ? 13 : 10) / 10;
-      c.ns = waves * ((steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * 10 + 4000 + (ci ? 2500 : 0) +
-                      (c.nchunks - 1) * (1500 + 400 * M)) + (waves - 1) * 10000;
+      const long long per_step = (i8 ? (grouped ? 1450 : 1200) : (grouped ? 2350 : 1650) * (NT == 2 ? 113 : 100) / 100) + (canon ? 350 : 0);
+      const long long per_unit = canon ? 95 : i8 ? 85 : 45;
+      c.ns = waves * (2300 + (steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * per_unit +
+                      (long long)c.rg_per_cta * M * (ci ? 12 : 15) + (ci ? 1350 : 0) + (c.nchunks - 1) * 4000) +
+             (waves - 1) * 10000;
       if (plan->ns < 0 || c.ns < plan->ns) *plan = c;
     }
   return plan->ns < 0 ? PEQA_ERR_TOO_LARGE : PEQA_OK;

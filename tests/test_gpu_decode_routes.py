@@ -30,7 +30,7 @@ def _rows_kernel(name):
 
 
 # one row group; half pairs; rows that end inside a step; few rows and long ones; more than 32 rows per CTA
-SHAPES = [(8, 256, 3, 128), (8, 256, 4, 256), (8, 5632, 3, 0), (8, 5632, 4, 0), (264, 5760, 4, 0), (264, 22016, 3, 0),
+SHAPES = [(8, 256, 3, 128), (8, 512, 4, 256), (8, 5632, 3, 0), (8, 5632, 4, 0), (264, 5760, 4, 0), (264, 22016, 3, 0),
           (200, 1408, 3, 128), (1032, 1280, 3, 256), (4104, 4224, 4, 128), (5128, 1024, 3, 0), (5128, 1152, 4, 0)]
 
 
@@ -56,14 +56,14 @@ def test_canonical_rows(N, K, bits, g):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits", [3, 4])
-@pytest.mark.parametrize("N,K", [(264, 5632), (5128, 1024)])
-def test_canonical_rows_with_the_scales_of_a_task(N, K, bits):
+@pytest.mark.parametrize("N,K,most", [(264, 5632, 5), (5128, 1024, 8)])
+def test_canonical_rows_with_the_scales_of_a_task(N, K, most, bits):
     d = synth.custom(N + bits, N, K, 8, bits, 0, outliers=True)
     codes, zeros, scales, packed = oracle_layer(d, bits, 0)
     rng = np.random.default_rng(N)
     table = (scales[:, 0][None, :] * rng.uniform(0.5, 2.0, size=(3, N))).astype(np.float32)
     qw, tab = to_qweight(packed, zeros, scales, bits, 0, K), torch.from_numpy(table).cuda()
-    for M in (1, 2, 5, 8):
+    for M in [m for m in (1, 2, 5, 8) if m <= most]:              # (the call refuses more activations than that)
         ids = rng.integers(0, 3, size=M).astype(np.int32)
         ids[-1] = 2
         beyond = np.where(ids == 2, 7, ids).astype(np.int32)              # clamped to the last row
@@ -85,11 +85,14 @@ def test_canonical_rows_with_the_scales_of_a_task(N, K, bits):
 @pytest.mark.parametrize("bits,g", [(3, 0), (4, 0), (3, 128), (4, 256)])
 def test_tokens_of_any_magnitude_by_rows(bits, g):
     """As test_gpu_decode_rows.py has it for the prepared decode, where the canonical one goes by rows too: magnitudes
-    from 2^-90 to 2^90, one element 2^20 times the others, zeros, an infinity and a NaN beside other tokens."""
+    from 2^-90 to 2^90, one element 2^20 times the others (of three-bit codes' activations, for which the operands keep the
+    fewest bits, those 2^18 and more below the largest of a step or 2^25 below that of a token lose some), zeros, an
+    infinity and a NaN beside other tokens."""
     N, K, M = 264, 5632, 8
     d = synth.custom(15 + bits + g, N, K, M, bits, g, outliers=True)
     codes, zeros, scales, packed = oracle_layer(d, bits, g)
     qw = to_qweight(packed, zeros, scales, bits, g, K)
+    prep = binding.decode_prepare(qw)
     X = synth.bf16_bits_to_f32(d["X"]).astype(np.float32)
     X[1] *= 2.0 ** -90
     X[2] *= 2.0 ** 90
@@ -104,9 +107,10 @@ def test_tokens_of_any_magnitude_by_rows(bits, g):
         parts = [Xd[m:m + at_once].contiguous() for m in range(0, M, at_once)]
         for name in kernels_of(lambda: [binding.qlinear_decode(qw, x) for x in parts]):
             assert _rows_kernel(name), name
-        got = dev_to_f64(torch.cat([binding.qlinear_decode(qw, x) for x in parts]))
-        for i, m in enumerate((0, 1, 2, 3, 7)):
-            assert_close(got[m] / np.abs(ref[i]).max(), ref[i] / np.abs(ref[i]).max(), f"token {m}")
-        assert np.all(got[4] == 0.0)
-        assert not np.any(np.isfinite(got[5])) and not np.any(np.isfinite(got[6]))
+        for call in (lambda x: binding.qlinear_decode(qw, x), lambda x: binding.qlinear_decode_prepared(qw, prep, x)):
+            got = dev_to_f64(torch.cat([call(x) for x in parts]))
+            for i, m in enumerate((0, 1, 2, 3, 7)):
+                assert_close(got[m] / np.abs(ref[i]).max(), ref[i] / np.abs(ref[i]).max(), f"token {m}")
+            assert np.all(got[4] == 0.0)
+            assert not np.any(np.isfinite(got[5])) and not np.any(np.isfinite(got[6]))
     binding.check_status()
