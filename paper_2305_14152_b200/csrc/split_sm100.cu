@@ -468,71 +468,48 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
           if (rl < b0 && j > j_lo) second |= 1u << r;
         }
         float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);   // vec_per divides kSplitWorkers: a thread keeps its rows
-        // Two vectors per thread and turn, all of their sums requested before the first is used: one
-        // after the other each waited for its reads and its store's address (128 x 128 outputs: 7100 cycles).
-        // dX takes one: half the code for a launch to fetch first
-        // (us, one / two: 8192 x 8192 at 45 tokens 28.2 / 28.9, 2672 x 1856 at 142 13.4 / 14.1).
-        constexpr int U = TRANS ? 1 : 2;
+        // One vector per thread and turn, the sums of four CTAs requested before the first is used.  (Two vectors a
+        // turn were twice the code for a launch to fetch, us, one / two: forward 2672 x 1856 at 142 tokens 11.8 / 12.6, 1096 x
+        // 768 at 32 5.7 / 6.0, 2.1 % over 180 forwards; dX 8192 x 8192 at 45 28.2 / 28.9.)
 #pragma unroll 1
-        for (int base_i = wtid; base_i < toks * vec_per; base_i += U * kSplitWorkers) {
-          float4 a[U];
-          uint2 y[U];
-          bool live[U];
-          int t[U], row[U];
-          uint32_t off[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int idx = base_i + u * kSplitWorkers;
-            t[u] = idx >> vec_shift;
-            const int rv = (idx & (vec_per - 1)) * 4;
-            row[u] = r0 + rv;
-            live[u] = idx < toks * vec_per && t0 + t[u] < p.T && row[u] < p.R;
-            off[u] = dump_addr + (uint32_t)(t[u] * SM_ROWS + rank * rows_per + rv) * 4u;
-            a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (DS) {
-              y[u] = make_uint2(0u, 0u);
-              if (live[u]) y[u] = ld_global(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t[u]) * p.R + row[u]));
-            }
-          }
+        for (int idx = wtid; idx < toks * vec_per; idx += kSplitWorkers) {
+          const int t = idx >> vec_shift, rv = (idx & (vec_per - 1)) * 4;
+          const int row = r0 + rv;
+          if (t0 + t >= p.T || row >= p.R) continue;
+          const uint32_t off = dump_addr + (uint32_t)(t * SM_ROWS + rank * rows_per + rv) * 4u;
+          uint2 y = make_uint2(0u, 0u);
+          if (DS) y = ld_global(reinterpret_cast<const uint2*>(p.dY + (size_t)(t0 + t) * p.R + row));
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int rh = 0; rh < 8; rh += 4) {
             if (rh >= csize) break;
-            float4 v[U][4];
+            float4 v[4];
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-              for (int r = 0; r < 4; ++r) {
-                v[u][r] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (live[u] && (from >> (rh + r) & 1u))
-                  v[u][r] = ld_cluster_f4(mapa_shared(off[u] + (second >> (rh + r) & 1u ? (uint32_t)seg_floats * 4u : 0u),
-                                                      (uint32_t)(rh + r)));
-              }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-              for (int r = 0; r < 4; ++r) {
-                a[u].x += v[u][r].x; a[u].y += v[u][r].y; a[u].z += v[u][r].z; a[u].w += v[u][r].w;
-              }
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            if (!live[u]) continue;
-            if (DS) {
-              ds.x = fmaf(a[u].x, __uint_as_float(y[u].x << 16), ds.x);
-              ds.y = fmaf(a[u].y, __uint_as_float(y[u].x & 0xFFFF0000u), ds.y);
-              ds.z = fmaf(a[u].z, __uint_as_float(y[u].y << 16), ds.z);
-              ds.w = fmaf(a[u].w, __uint_as_float(y[u].y & 0xFFFF0000u), ds.w);
+            for (int r = 0; r < 4; ++r) {
+              v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (from >> (rh + r) & 1u)
+                v[r] = ld_cluster_f4(mapa_shared(off + (second >> (rh + r) & 1u ? (uint32_t)seg_floats * 4u : 0u), (uint32_t)(rh + r)));
             }
-            if (!FOLD) {
-              const float4 sc = ld_global(reinterpret_cast<const float4*>(p.scales + row[u]));   // one scale per channel
-              a[u].x *= sc.x; a[u].y *= sc.y; a[u].z *= sc.z; a[u].w *= sc.w;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              a.x += v[r].x; a.y += v[r].y; a.z += v[r].z; a.w += v[r].w;
             }
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(a[u].x, a[u].y), h1 = __floats2bfloat162_rn(a[u].z, a[u].w);
-            uint2 o;
-            o.x = *reinterpret_cast<uint32_t*>(&h0);
-            o.y = *reinterpret_cast<uint32_t*>(&h1);
-            *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t[u]) * p.R + row[u]) = o;
           }
+          if (DS) {
+            ds.x = fmaf(a.x, __uint_as_float(y.x << 16), ds.x);
+            ds.y = fmaf(a.y, __uint_as_float(y.x & 0xFFFF0000u), ds.y);
+            ds.z = fmaf(a.z, __uint_as_float(y.y << 16), ds.z);
+            ds.w = fmaf(a.w, __uint_as_float(y.y & 0xFFFF0000u), ds.w);
+          }
+          if (!FOLD) {
+            const float4 sc = ld_global(reinterpret_cast<const float4*>(p.scales + row));   // one scale per channel
+            a.x *= sc.x; a.y *= sc.y; a.z *= sc.z; a.w *= sc.w;
+          }
+          __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
+          uint2 o;
+          o.x = *reinterpret_cast<uint32_t*>(&h0);
+          o.y = *reinterpret_cast<uint32_t*>(&h1);
+          *reinterpret_cast<uint2*>(p.out + (size_t)(t0 + t) * p.R + row) = o;
         }
         if (DS) {
           // lanes that share rows, then the warps in order (over the code slots, which are done with)
@@ -629,17 +606,23 @@ long long split_fwd_ns(long long waves, long long stages, int nt, int q) {
   return waves * (4700 + stages * (649 + nt * 28 / 100) + nt * (q > 1 ? 54 : 28));
 }
 SplitPlan plan_split(int r_tiles, int C, int T, int sms, bool trans) {
-  SplitPlan best = {};
-  best.ns = -1;
+  SplitPlan plans[2] = {};             // whole and halved token tiles
+  plans[0].ns = plans[1].ns = -1;
   const long long k_blocks = (C + SM_BK - 1) / SM_BK;
   // clusters of 1, 2, 4, 8 CTAs that run at once (cudaOccupancyMaxActiveClusters on this part: 148,
   // 74, 33, 15 -- the larger ones leave SMs of a GPC idle)
   const int active[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
   const int t_min = (T + SM_MAX_NT - 1) / SM_MAX_NT;
   // Token tiles as wide as they can be, or half as wide: a forward whose CTAs hold two accumulators has no room
-  // for its weights beside two wide ones.
-  for (int tt = t_min; tt <= (trans ? t_min : 2 * t_min); tt += t_min) {
+  // for its weights beside two wide ones, and where one round of CTAs leaves SMs idle the halves share the
+  // exchange (us, whole / halved: 1480 x 384 at 183 tokens 10.6 / 7.0, 4216 x 1664 at 173 13.5 / 11.5).  Halves of 16 tokens gain
+  // nothing (six calls, 0.96 to 1.24 of the time: 4728 x 512 at 18 6.1 / 7.5), and at less than 64 the estimate does not tell
+  // 3 % (2136 x 1024 at 85 7.3 / 7.8).
+  for (int halved = 0; halved < (trans ? 1 : 2); ++halved) {
+    const int tt = t_min << halved;
     const int nt = ((T + tt - 1) / tt + 15) & ~15;
+    if (halved && nt < 32) break;
+    SplitPlan& best = plans[halved];
     const int t_tiles = (T + nt - 1) / nt;
     const long long tiles = (long long)r_tiles * t_tiles;
     for (int ci = 0; ci < 4; ++ci) {
@@ -663,7 +646,7 @@ SplitPlan plan_split(int r_tiles, int C, int T, int sms, bool trans) {
       }
     }
   }
-  return best;
+  return plans[1].ns >= 0 && plans[1].ns * (plans[1].nt < 64 ? 103 : 100) < plans[0].ns * 100 ? plans[1] : plans[0];
 }
 
 // The pair kernels on the same call: rounds of 512 x 256 tiles over the pairs of SMs.  dX, fitted to 400
