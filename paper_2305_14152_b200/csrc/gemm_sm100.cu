@@ -737,19 +737,56 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   }
 }
 
+// An output's pieces lie side by side.  A thread that adds up its own reads every line of memory as often as the
+// line has pieces, out of L1; launched programmatically these kernels find their SM laid out for the contraction
+// before them, with next to no L1, so from 25 pieces on a block of 128 threads reads the pieces of 32 outputs row by row
+// into shared memory and its first warp adds them up, in index order all the same.  us, contraction and
+// reduction, a thread each / this: 456 x 9600 at 60 tokens (75 pieces) 17.8 / 11.3, 1128 x 6016 at 56 16.8 / 10.6,
+// 6800 x 13440 at 75 62 / 50; with fewer pieces a thread each is faster (10048 x 1280 at 53 tokens 11.1 / 11.9, 2304 columns
+// 7.2 / 7.7).
+constexpr int kWidePieces = 25, kWideThreads = 128, kWideRows = 32;
+__device__ __forceinline__ float sum_pieces_wide(const float* partial, long long n_out, int pieces) {
+  __shared__ float tile[kWideRows][33];
+  const long long e0 = (long long)blockIdx.x * kWideRows;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float acc = 0.0f;
+  for (int q0 = 0; q0 < pieces; q0 += 32) {
+#pragma unroll
+    for (int k = 0; k < kWideRows / (kWideThreads / 32); ++k) {
+      const int row = warp + k * (kWideThreads / 32);
+      if (e0 + row < n_out && q0 + lane < pieces) tile[row][lane] = partial[(e0 + row) * pieces + q0 + lane];
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const int n = min(32, pieces - q0);
+      for (int q = 0; q < n; ++q) acc += tile[lane][q];     // (of rows beyond the last one: never stored)
+    }
+    __syncthreads();
+  }
+  return acc;
+}
+
 // Real-valued zero-point, groups wider than a piece: dS = sum(pieces) - delta * sum(dW pieces)
-// and dZ = -s * sum(dW pieces), pieces added in index order.
+// and dZ = -s * sum(dW pieces).
+template <bool WIDE>
 __global__ void ds_reduce_zf_kernel(const float* partial_s, const float* partial_w,
                                     float* dS, float* dZ, long long n_out,
                                     int pieces_per_group, const float* zeros_f,
                                     const float* scales, int bits) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n_out) return;
+  long long e = (long long)blockIdx.x * (WIDE ? kWideRows : blockDim.x) + threadIdx.x;
   float acc_s = 0.0f, acc_w = 0.0f;
-  for (int q = 0; q < pieces_per_group; ++q) {
-    acc_s += partial_s[e * pieces_per_group + q];
-    acc_w += partial_w[e * pieces_per_group + q];
+  if constexpr (WIDE) {
+    acc_s = sum_pieces_wide(partial_s, n_out, pieces_per_group);
+    acc_w = sum_pieces_wide(partial_w, n_out, pieces_per_group);
+    if (threadIdx.x >= kWideRows) return;
+  }
+  if (e >= n_out) return;
+  if constexpr (!WIDE) {
+    for (int q = 0; q < pieces_per_group; ++q) {
+      acc_s += partial_s[e * pieces_per_group + q];
+      acc_w += partial_w[e * pieces_per_group + q];
+    }
   }
   uint32_t zi;
   float delta;
@@ -762,17 +799,24 @@ __global__ void ds_reduce_zf_kernel(const float* partial_s, const float* partial
 // dS[i, gi] = sum of the group's partial pieces, in index order (deterministic); with
 // neg_scales the sum is multiplied by -s[i, gi] (the zero-point gradient); with adam_s the
 // AdamW step on scale e follows at once.
+template <bool WIDE>
 __global__ void ds_reduce_kernel(const float* partial, float* dS,
                                  long long n_out, int pieces_per_group,
                                  const float* neg_scales, AdamWConsts adam,
                                  float* adam_s, float* adam_m,
                                  float* adam_v) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n_out) return;
-  const float* src = partial + e * pieces_per_group;
+  long long e = (long long)blockIdx.x * (WIDE ? kWideRows : blockDim.x) + threadIdx.x;
   float acc = 0.0f;
-  for (int q = 0; q < pieces_per_group; ++q) acc += src[q];
+  if constexpr (WIDE) {
+    acc = sum_pieces_wide(partial, n_out, pieces_per_group);
+    if (threadIdx.x >= kWideRows) return;
+  }
+  if (e >= n_out) return;
+  if constexpr (!WIDE) {
+    const float* src = partial + e * pieces_per_group;
+    for (int q = 0; q < pieces_per_group; ++q) acc += src[q];
+  }
   dS[e] = neg_scales ? -neg_scales[e] * acc : acc;
   if (adam_s) {
     float sv = adam_s[e], mv = adam_m[e], vv = adam_v[e];
@@ -1082,15 +1126,17 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   if (!direct) {
     const long long n_out = (long long)p.N * p.G;
     const int ppg = g / p.piece;
-    const int blocks = (int)((n_out + 255) / 256);
+    const bool wide = ppg >= kWidePieces;
+    const int threads = wide ? kWideThreads : 256;
+    const int blocks = (int)((n_out + (wide ? kWideRows : 256) - 1) / (wide ? kWideRows : 256));
     if (zeros_f)
-      return launch_after(ds_reduce_zf_kernel, blocks, 256, st, p.out, p.out_z, dS, dZ, n_out, ppg, zeros_f, w->scales,
-                          (int)w->bits);
-    PEQA_TRY(launch_after(ds_reduce_kernel, blocks, 256, st, p.out, dS, n_out, ppg, nullptr, p.adam, p.adam_s, p.adam_m,
-                          p.adam_v));
+      return launch_after(wide ? ds_reduce_zf_kernel<true> : ds_reduce_zf_kernel<false>, blocks, threads, st, p.out, p.out_z, dS,
+                          dZ, n_out, ppg, zeros_f, w->scales, (int)w->bits);
+    auto reduce = wide ? ds_reduce_kernel<true> : ds_reduce_kernel<false>;
+    PEQA_TRY(launch_after(reduce, blocks, threads, st, p.out, dS, n_out, ppg, nullptr, p.adam, p.adam_s, p.adam_m, p.adam_v));
     if (dZ)
-      PEQA_TRY(launch_after(ds_reduce_kernel, blocks, 256, st, p.out_z, dZ, n_out, ppg, w->scales, AdamWConsts{}, nullptr,
-                            nullptr, nullptr));
+      PEQA_TRY(launch_after(reduce, blocks, threads, st, p.out_z, dZ, n_out, ppg, w->scales, AdamWConsts{}, nullptr, nullptr,
+                            nullptr));
   }
   return PEQA_OK;
 }
