@@ -559,7 +559,6 @@ decode_prep_kernel(const PrepParams p) {
 
   int c_slot = 0;
   uint32_t c_phase = 0;                              // parity of the ring's current round
-  bool ok = true;
 
 #pragma unroll 1
   for (int ch = 0; ch < p.nchunks; ++ch) {
@@ -866,8 +865,7 @@ decode_prep_kernel(const PrepParams p) {
       const int slot = c_slot;
       // A lane whose bound has run out goes on with the others, over whatever the slot holds: nothing behind
       // the wait then misses it.  (A vote of the warp cost up to 4 %: eight tokens of several tasks at 3520 x 512 5.65 / 5.9 us.)
-      ok = mbar_wait(bar_w + slot * 8, c_phase, abort_flag) && ok;
-      if (!ok) i_ch = p.nchunks;                       // nothing more is asked for
+      if (!mbar_wait(bar_w + slot * 8, c_phase, abort_flag)) i_ch = p.nchunks;     // nothing more is asked for
       if (++c_slot == p.slots) {
         c_slot = 0;
         c_phase ^= 1u;
@@ -1196,7 +1194,7 @@ decode_prep_kernel(const PrepParams p) {
     cluster_sync_all();       // the sums are read by the whole cluster until here
   }
 
-  if (!ok || abort_flag[0]) {
+  if (abort_flag[0]) {
     // let copies already in flight land before shared memory is released
 #pragma unroll 1
     for (int i = 0; i < 64; ++i) __nanosleep(1000);

@@ -29,7 +29,7 @@ def _waits(text):
         elif token != ";":
             around = "".join(heads) + text[start:m.start()]
             statement = text[start:text.index(";", m.start()) + 1].strip()
-            noted = re.fullmatch(r"(ok = mbar_wait\(.*\) && ok|\(void\)ptx::mbar_wait\(.*\));", statement, re.S) is not None
+            noted = re.fullmatch(r"(if \(!mbar_wait\(.*\)\) i_ch = p\.nchunks|\(void\)ptx::mbar_wait\(.*\));", statement, re.S) is not None
             yield text.count("\n", 0, m.start()) + 1, token[:-1], "lane == 0" in around, noted
             continue
         start = m.end()
