@@ -189,7 +189,7 @@ int peqa_qlinear_bwd_ds_adamw(const peqa_qweight_t* w, const void* X_bf16, const
  * A large linear with one scale per channel takes its dS from the forward's fp32
  * sums, dS[i] = sum_t dY[t,i] * sum_j X[t,j] (Q[i,j] - z[i]), instead of contracting
  * dY^T X: the same sum in another order, closer to the exact one.  Large means
- * T*N*K >= 2^28; and the partial sums, one row of N floats per 128 tokens, have to fit
+ * T*N*K >= 2^28; and the partial sums, one row of N floats per 128 tokens or narrower tile, have to fit
  * the workspace of the size above, which holds K / 128 rows: T <= K, or a little less
  * where T is not a multiple of 256.  Which way is taken depends on the shape and T
  * alone, not on the workspace given.

@@ -235,8 +235,8 @@ size_t ds_workspace_bytes(const peqa_qweight_t* w, int g, int T);
 size_t ds_from_y_workspace_bytes(const peqa_qweight_t* w, int T);
 int launch_ds_from_y(const peqa_qweight_t* w, const void* dY, const void* Y, int T, float* dS,
                      void* workspace, cudaStream_t st);
-// canonical weights through the kernel of the prepared decode (decode_prep.cu): one scale per channel, groups of
-// 128 or 256 columns
+// canonical weights through the kernel of the prepared decode (decode_prep.cu), up to eight tokens: one scale per
+// channel, groups of 128 or 256 columns
 bool decode_rows_are_faster(const peqa_qweight_t* w, int g, int M);
 bool decode_rows_supported(const peqa_qweight_t* w, int g, int M);
 int launch_decode_rows(const peqa_qweight_t* w, int g, const void* X, int M, void* Y, const float* scale_table,

@@ -42,8 +42,8 @@
 // tensor core as the fp16 subnormals q * 2^(o - 24) that a code in the low bits of a half-word is
 // after one AND (f16_pair in dequant.cuh): 21 integer operations for 32 three-bit codes and 20 for
 // four-bit ones, where bf16 operands with an exponent put in took 26 and 28 and left a bias to take off every
-// sum.  The activations are brought to the range of fp16 by a power of two per token, which is
-// exact, and lose the 2^o.  Seven linears of a LLaMA-65B layer in groups of 64, one token, 163.9 ->
+// sum.  The activations are brought to the range of fp16 by a power of two per token and lose the 2^o: exact for
+// elements down to 2^-25 of the token's largest, smaller ones lose bits (see the staging).  Seven linears of a LLaMA-65B layer in groups of 64, one token, 163.9 ->
 // 150.4 us; of a LLaMA-7B layer in groups of 128, seven tokens of several tasks, 94.3 -> 85.1; one scale per
 // channel, where the main loop is the smaller part, 16 tokens 230.9 -> 227.3, one token unchanged.
 // When a warp's range crosses into the next pair it parks its sums in shared
@@ -60,8 +60,12 @@
 // twice the contraction, so the activations go in as whole numbers: a step's 512 are scaled by a power
 // of two of their own to at most 2^30 and cut into four signed base-256 digits, which fill the eight
 // columns for two tokens; the codes are unsigned bytes, eight integer operations for 32 four-bit codes
-// and 14 (groups of 64: 18) for three-bit ones (i8_string).  Sums of products are exact until a group (or a
-// step) is scaled, and what the 30 bits do not hold is less than fp32 sums lose.  A step of a warp takes
+// and 14 (groups of 64: 18) for three-bit ones (i8_string).  A code at bit o of its byte counts 2^o, which comes off its
+// activation before that is rounded, so 30 - o bits are kept, 25 at the least (o <= 5): an element's rounding error
+// is at most 2^-25 of the step's largest, exact ones are those down to 2^-17 of it.  Sums of products are
+// exact until a group (or a step) is scaled.  The grain is that of the step's largest element, for groups that do
+// not hold it too; an emulation gave smaller errors than biased bf16 operands with outliers of 2^12 to
+// 2^26 times the others.  A step of a warp takes
 // about 1200 cycles instead of 2100 (groups of 64: 2200 / 3000).  One token, us, fp16 / here: 22016 x 8192 in
 // groups of 64 28.8 / 25.0, 8192 x 8192 14.6 / 12.6, 11008 x 4096 9.5 / 7.7, 4096 x 4096 6.2 / 5.6, 256 x 256 5.0 / 4.1.
 //
@@ -70,7 +74,7 @@
 // copies by all lanes, and since the order of a contraction is free a lane takes 32 columns in a
 // row where the prepared order gives it eight of each of four runs.  The copies wait for the preceding
 // kernel, which may have written the matrix; before that its codes are only asked for in L2.  LLaMA-7B layer in groups
-// of 128, three sequences: 103.6 us through decode_stream_kernel, 81.7 here.
+// of 128, three sequences: 103.6 us through decode_stream_kernel, 72.7 here.
 //
 // Size.  A launch finds the instruction caches cold, and much of a launch of a few microseconds is the
 // code's first pass, so there is one copy of everything: loops whose length is not known are not
@@ -569,8 +573,10 @@ decode_prep_kernel(const PrepParams p) {
     // ---- stage X[:, chunk] (columns beyond K read as zero): copied as it is, then turned in place into
     // the fp16 operands that meet the codes (x_pairs), with the sums of x per token or per group.  A
     // token's activations are first multiplied by a power of two that brings the largest of them to
-    // [2^15, 2^16): what is then below the normal fp16 numbers is less than 2^-29 of the largest, so fp16
-    // holds all that a fp32 sum with the largest in it would.  tinv undoes the factor and the 2^-24 of the codes.
+    // [2^15, 2^16), then by 2^-o of the code's place (o <= 7, four bits: 4).  Operands from 2^-14 on are normal numbers, which
+    // hold a bf16; what is below 2^(o - 29) of the token's largest is rounded to a grain of 2^-24, an error of at most
+    // 2^(o - 40) of the largest (bf16's eight bits fit down to 2^(o - 32)).  That is less than a fp32 sum with the largest in it
+    // loses; the sums of groups without it get the same grain.  tinv undoes the factor and the 2^-24 of the codes.
     // zero-point and scale of a row, for the final sums (a table per task: scales are looked up there)
     auto row_zs = [&](int r, uint32_t& z, float& sc) {
       z = 0u;
@@ -715,7 +721,9 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll 1
         for (int s = CANON ? 0 : 1; s < p.slots; ++s) issue_next();
       if (ch > 0 && warp == kPWarps - 1) share_bounds(spc_c);                  // while the activations are on their way
-      asm volatile("cp.async.wait_group 0;" ::: "memory");           // (the ring's copies belong to no group)
+      // (of the ring's copies the first chunk's are in no group yet; canonical ones issued since, while a chunk
+      // was worked through, joined this chunk's group, and its activations wait for them too)
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
       {
         uint32_t mx = 0u;                                            // two largest |x|, as bf16 bits
         if (tok < p.M)

@@ -269,7 +269,7 @@ __device__ __forceinline__ void mma_pairs_stream(const uint32_t (&w)[BITS], uint
 // off the sums.  Three-bit codes fit at o = 0..7, four-bit codes at 0..6, in either half of a window, so
 // a shift serves up to three pairs: 16 logic operations and 5 shifts for 32 three-bit codes, 16 and 4 for
 // four-bit ones (the bf16 pairs above: 16 and 10, 16 and 12).  The factor 2^o is taken out of the
-// activation the code meets, which is exact.
+// activation the code meets, which is exact as long as that stays a normal number.
 // A string's pairs 0..7 hold its columns 0..15 and pairs 8..15 its columns 16..31, so that two runs of
 // 32 columns of the matrix make eight pairs of every lane.
 // ---------------------------------------------------------------------------
@@ -336,7 +336,7 @@ __device__ __forceinline__ uint32_t f16_pair(const uint32_t (&w)[BITS]) {
 // is q * 2^o, so one AND makes four operands: 4-bit strings are eight ANDs for 32 codes, without a shift.
 // Of a 3-bit string's 32 codes 24 lie inside a byte (six ANDs); the eight that straddle two are
 // gathered into two words (two shifts and two logic operations each).  The factor 2^o is taken out of the
-// activation the code meets.  Register r (0..7) of a string, byte b, holds the code at position
+// activation the code meets, which keeps o bits less.  Register r (0..7) of a string, byte b, holds the code at position
 // i8_pos, times 2^i8_o; registers 2j and 2j + 1 are one MMA's.  HALF: registers 0..3 hold the
 // string's columns 0..15 and 4..7 its columns 16..31 (four byte permutations more for 3-bit strings).
 // ---------------------------------------------------------------------------

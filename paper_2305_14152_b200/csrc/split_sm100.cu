@@ -600,7 +600,7 @@ int split_tmem_stages(int nt, int q) {
   return s < SM_MAX_STAGES ? s : SM_MAX_STAGES;
 }
 // Forward: time of a plan in ns.  Fitted to 150 calls (17 to 4096 tokens, 256 to 22016 rows and columns; nine of
-// ten within 0.89 to 1.13): 4.7 us a wave, 0.65 us + 0.28 ns per token a stage, and for the sums and their
+// ten within 0.89 to 1.13, since the exchange takes one vector per thread 0.94 to 1.14): 4.7 us a wave, 0.65 us + 0.28 ns per token a stage, and for the sums and their
 // exchange 28 ns per token of the tile, 54 where a CTA may hold two tiles'.
 long long split_fwd_ns(long long waves, long long stages, int nt, int q) {
   return waves * (4700 + stages * (649 + nt * 28 / 100) + nt * (q > 1 ? 54 : 28));

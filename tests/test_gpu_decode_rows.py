@@ -1,6 +1,7 @@
-"""GPU parity of the decode that streams the canonical rows through the kernel of the prepared decode, and of
-the fp16 operands both are made of: a row group alone, half pairs, rows that end inside a step, groups that
-are a string, two strings, a step and more; tokens of any magnitude in one batch."""
+"""GPU parity of the canonical decode around its dispatch (of these shapes those with groups of 128 and 256 of a row and
+the long rows of one scale go by rows through the kernel of the prepared decode, the others to the streaming kernel and, with
+more than eight tokens, to the cluster kernels; test_gpu_decode_routes.py asserts which) and of the prepared decode's fp16 and
+integer operands: a row group alone, half pairs, rows that end inside a step; tokens of any magnitude in one batch."""
 import numpy as np
 import pytest
 import torch
