@@ -129,7 +129,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------ dY TMA (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
@@ -150,7 +150,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
     }
   } else if (warp == 3) {
     // ------------------------------------------ packed-code TMA (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
@@ -169,7 +169,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------ MMA issuer (leader CTA, one lane)
-    if (leader && lane == 0) {
+    if (leader) if (const uint32_t lane = elect_lane(); lane == 0) {
       // One thread issues everything and a tensor core holds little more than the MMA it works on, so
       // what this thread does between the last MMA of a stage and the first of the next is a gap in the
       // tensor pipe.  Weights and activations share a barrier, the next stage's is asked for before the

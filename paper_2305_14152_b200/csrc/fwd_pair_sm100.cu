@@ -142,7 +142,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------ activation TMA (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       // self-test knob (peqa_selftest_configure): announce one byte more than will arrive, so
@@ -169,7 +169,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     // A box is 128 rows x 8 words holding the stage's 64 columns; for 3-bit codes the 6
     // words start 2 words into the box on odd k-blocks, which keeps the box start
     // 16-byte aligned.
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
@@ -189,7 +189,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------ MMA issuer (leader CTA, one lane)
-    if (leader && lane == 0) {
+    if (leader) if (const uint32_t lane = elect_lane(); lane == 0) {
       // One thread issues everything and a tensor core holds little more than the MMA it works on, so
       // what this thread does between the last MMA of a stage and the first of the next is a gap in the
       // tensor pipe.  Weights and activations share a barrier, the next stage's is asked for before the

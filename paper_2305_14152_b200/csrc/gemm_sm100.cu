@@ -164,7 +164,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
   extern __shared__ uint8_t smem_raw[];
   SmemView sm = carve_smem(smem_raw);
   Barriers* bars = sm.bars;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   volatile int* abort_flag = &bars->abort_flag;
 
   if (threadIdx.x == 0) {
@@ -195,7 +195,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
@@ -212,7 +212,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmap_act, const QGemmParams p) 
     }
   } else if (warp == 1) {
     // ------------------------------------------------- MMA issuer (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, TRANS ? 1 : 0, 0);
       uint32_t it = 0;
       int local = 0;
@@ -473,7 +473,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* sm_pk = base + DS_STAGES * DS_STAGE_BYTES;
   DsBarriers* bars = reinterpret_cast<DsBarriers*>(sm_pk + 2 * DS_PK_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   volatile int* abort_flag = &bars->abort_flag;
@@ -514,7 +514,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   const int n_pairs = gridDim.x >> 1;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       uint32_t it = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
@@ -540,7 +540,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
       }
     }
   } else if (warp == 1) {
-    if (leader && lane == 0) {
+    if (leader) if (const uint32_t lane = elect_lane(); lane == 0) {
       // (the next stage's barrier is asked for under the last MMA of this one: see the pair kernels)
       constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, BN, 1, 1);
       const uint64_t adesc0 = smem_desc_sw128(smem_u32(base), 8192, 1024);
@@ -577,7 +577,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     }
   } else if (warp == 3) {
     // packed codes of this CTA's 128 rows x 256 columns, a tile ahead of the epilogue (one lane)
-    if (PKTMA && lane == 0) {
+    if (PKTMA) if (const uint32_t lane = elect_lane(); lane == 0) {
       int local = 0;
       for (int tile = pair; tile < total_tiles; tile += n_pairs, ++local) {
         int ti, tj;

@@ -234,6 +234,25 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// The warp's index, which the compiler may hold in a uniform register (threadIdx.x >> 5 differs between threads as far
+// as it can tell).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// 0 in one lane of the (converged) warp, 1 in the others.  The operands of an MMA or a tensor copy are uniform
+// registers.  Behind a test of this the compiler knows that a single thread is active and moves them there at
+// once; behind one of threadIdx.x every MMA cost 107 cycles of its issuing thread, whatever its size (128 x 80 x 16: 40
+// cycles with A in tensor memory, 52 in shared memory; 128 x 16 x 16: 13 and 39).
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 0, 1, p;\n\t"
+      "}\n"
+      : "=r"(r));
+  return r;
+}
+
 // D[tmem] (+)= A[smem desc] * B[smem desc]; accumulate != 0 keeps the old D.
 __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                             uint32_t idesc, uint32_t accumulate) {

@@ -144,7 +144,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   const int stage_bytes = 2 * half_bytes;
   uint8_t* sm_pk = base + p.region;
   SplitBarriers* bars = reinterpret_cast<SplitBarriers*>(sm_pk + SM_PK_SLOTS * SM_PK_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   volatile int* abort_flag = &bars->abort_flag;
 
   // ---- this CTA's stages: [lo, hi) of the cluster's list, its first tile's, then the next tile's.  The
@@ -216,7 +216,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
 
   if (warp == 0) {
     // ------------------------------------------------ activation TMA (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       const int ta = t0_of(0), tb = t0_of(split_at);
       // self-test knob (peqa_selftest_configure): announce one byte more than will arrive, so
       // that the stage never fills and the bounded waits have to end the kernel
@@ -239,7 +239,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     // ------------------------------------------ packed-code TMA (one lane)
     // 128 rows x 128 columns of codes: the tile's rows and the stage's columns (forward), or the
     // stage's rows and the tile's columns (dX)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       const int ra = r0_of(0), rb = r0_of(split_at);
 #pragma unroll 1
       for (int it = 0; it < n_it; ++it) {
@@ -255,7 +255,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     }
   } else if (warp == 1) {
     // ------------------------------------------------- MMA issuer (one lane)
-    if (lane == 0) {
+    if (const uint32_t lane = elect_lane(); lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(SM_ROWS, 16, TRANS ? 1 : 0, 0) +
                              ((uint32_t)((p.nt - 16) >> 3) << 17);
       // One thread issues everything, so its instructions per stage are the pace of the kernel:
