@@ -1175,7 +1175,7 @@ decode_prep_kernel(const PrepParams p) {
   // the outputs per CTA
   if (p.cshift) {
     __syncwarp();
-    cluster_sync_all();
+    cluster_sync_shared();
     const int csize = 1 << p.cshift;
     const uint32_t ysum = smem_u32(ywhole);
     const int mpairs = (p.M + 1) >> 1;
@@ -1199,7 +1199,7 @@ decode_prep_kernel(const PrepParams p) {
       if (m + 1 < p.M) y[p.N] = __float2bfloat16_rn(sum.y);
     }
     __syncwarp();
-    cluster_sync_all();       // the sums are read by the whole cluster until here
+    cluster_sync_reads();     // the sums are read by the whole cluster until here
   }
 
   if (abort_flag[0]) {

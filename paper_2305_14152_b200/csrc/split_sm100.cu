@@ -450,7 +450,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       }
     }
     __syncwarp();
-    cluster_sync_all();
+    cluster_sync_shared();
     if (worker) {
       const int toks = min(tok_pass, p.nt - tp);
 #pragma unroll 1
@@ -539,7 +539,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       }
     }
     __syncwarp();
-    cluster_sync_all();   // the buffers are read by the whole cluster until here
+    cluster_sync_reads();   // the buffers are read by the whole cluster until here
   }
 
   if (*abort_flag)        // let copies and MMAs already in flight finish before memory is released
