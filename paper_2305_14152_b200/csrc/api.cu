@@ -153,6 +153,33 @@ extern "C" size_t peqa_workspace_bytes(int op, int T, const peqa_qweight_t* w) {
   }
 }
 
+// Whether contractions of one call may run side by side (`beside` in common.cuh): nothing that one of them writes (`out`; no
+// bytes: unused) is read or written by another.  Called one after the other they may share buffers, and then stay in that order.
+struct Span {
+  const void* at;
+  size_t bytes;
+};
+static size_t act_bytes(int T, int features) { return (size_t)T * features * 2; }
+static size_t scale_bytes(const peqa_qweight_t* w, int G) { return (size_t)w->out_features * G * sizeof(float); }
+static bool independent(const peqa_qweight_t* w, const float* zeros_f, int G, int T, const void* X, const void* dY,
+                        std::initializer_list<Span> out) {
+  const size_t rows = (size_t)w->out_features;
+  const Span in[] = {{X, act_bytes(T, w->in_features)}, {dY, act_bytes(T, w->out_features)},
+                     {w->qweight, rows * w->in_features * w->bits / 8}, {w->scales, scale_bytes(w, G)},
+                     {w->zeros, zeros_f ? 0 : rows * G}, {zeros_f, zeros_f ? scale_bytes(w, G) : 0}};
+  auto meet = [](const Span& a, const Span& b) {
+    const char *pa = static_cast<const char*>(a.at), *pb = static_cast<const char*>(b.at);
+    return a.bytes && b.bytes && pa < pb + b.bytes && pb < pa + a.bytes;
+  };
+  for (const Span* a = out.begin(); a != out.end(); ++a) {
+    for (const Span& b : in)
+      if (meet(*a, b)) return false;
+    for (const Span* b = out.begin(); b != a; ++b)
+      if (meet(*a, *b)) return false;
+  }
+  return true;
+}
+
 static int check_gemm_shape(const peqa_qweight_t* w, int T) {
   if (T <= 0) return PEQA_ERR_BAD_SHAPE;
   if (w->in_features % 64 != 0 || w->out_features % 8 != 0) return PEQA_ERR_BAD_SHAPE;
@@ -190,7 +217,11 @@ extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const vo
     }
   }
   if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T, 0));
-  if (dS) PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream)));
+  if (dS) {
+    const bool beside = dX && independent(w, nullptr, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
+                                                                    {workspace, ds_workspace_bytes(w, g, T)}});
+    PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream), beside));
+  }
   return PEQA_OK;
 }
 
@@ -254,18 +285,23 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     adam.scales = const_cast<float*>(L->w.scales);
     adam.m = L->m;
     adam.v = L->v;
+    const int G = L->w.in_features / g[i];
+    const size_t opt = apply_adamw ? scale_bytes(&L->w, G) : 0;
+    const bool beside = independent(&L->w, nullptr, G, T, L->X_bf16, L->dY_bf16,
+                                    {{L->Y_bf16, act_bytes(T, L->w.out_features)}, {L->dX_bf16, act_bytes(T, L->w.in_features)},
+                                     {L->dS, scale_bytes(&L->w, G)}, {L->m, opt}, {L->v, opt}, {L->workspace, ds_workspace_bytes(&L->w, g[i], T)}});
     const int slots = fwd_ds_slots(&L->w, g[i], T);
     if (slots > 0) {
       float* ds_part = static_cast<float*>(L->workspace);
       PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));
-      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0));   // before the scales change
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, beside));   // before the scales change
       PEQA_TRY(launch_ds_channel(&L->w, ds_part, slots, L->dS, apply_adamw ? &adam : nullptr, st));
       continue;
     }
     PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T, 0));
-    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0));
+    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, beside));
     PEQA_TRY(launch_ds(&L->w, nullptr, g[i], L->X_bf16, L->dY_bf16, T, L->dS, nullptr, apply_adamw ? &adam : nullptr,
-                       L->workspace, L->workspace_bytes, st));
+                       L->workspace, L->workspace_bytes, st, beside));
   }
   return PEQA_OK;
 }
@@ -335,7 +371,11 @@ extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f
     }
   }
   if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T, 0));
-  if (dS) PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream)));
+  if (dS) {
+    const bool beside = dX && independent(w, zeros_f, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
+                                                                    {dZ, scale_bytes(w, G)}, {workspace, dsdz_workspace_bytes(w, g, T)}});
+    PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream), beside));
+  }
   return PEQA_OK;
 }
 

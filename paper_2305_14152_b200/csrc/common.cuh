@@ -207,10 +207,16 @@ bool fwd_pair_supported(const peqa_qweight_t* w);
 int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T,
                     void* Y, const void* dY, float* ds_part, cudaStream_t st);
 bool dx_pair_supported(const peqa_qweight_t* w);
+// beside (dX, dS): launched behind kernels of the same entry point whose results it does not read and whose operands it does
+// not write (but AdamW, which waits for them), a contraction need not wait for them to end and fills the SMs they leave
+// idle.  A kernel that may have another beside it lets that one in only behind its own wait for what came before, so
+// all of that is complete; and one that ran beside another does not end before it, so whoever waits for the last waits for
+// all.  Training step, us, one after the other / side by side: 256 x 256 at 64 tokens 15.2 / 9.8, 1024 x 1024 in groups of 64 at
+// 200 24.3 / 20.1, 4096 x 4096 in groups of 128 at 2048 166 / 153; gradients with real zero-points 4096 x 11008 at 1001 164 / 135.
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
-                   void* dX, cudaStream_t st);
+                   void* dX, bool beside, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call, int t0);
+              cudaStream_t st, int T_call, int t0, bool beside = false);
 // forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels.
 // channel_scales: a forward that multiplies by one scale per channel at the end
 long long split_ns(const peqa_qweight_t* w, int T, bool trans);
@@ -218,7 +224,7 @@ bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_sc
 int split_ds_slots(const peqa_qweight_t* w, int T);
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans);
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0);
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, bool beside = false);
 // adam != nullptr: the AdamW step on (w->scales, m, v) is applied where dS is produced
 struct DsAdam {
   AdamWConsts c;
@@ -229,7 +235,7 @@ struct DsAdam {
 // zeros_f != nullptr needs dZ: dS is then taken with the real-valued zero-point
 int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, const void* dY,
               int T, float* dS, float* dZ, const DsAdam* adam, void* workspace,
-              size_t workspace_bytes, cudaStream_t st);
+              size_t workspace_bytes, cudaStream_t st, bool beside = false);
 size_t dsdz_workspace_bytes(const peqa_qweight_t* w, int g, int T);
 size_t ds_workspace_bytes(const peqa_qweight_t* w, int g, int T);
 size_t ds_from_y_workspace_bytes(const peqa_qweight_t* w, int T);

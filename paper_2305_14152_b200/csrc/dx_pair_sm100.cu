@@ -67,6 +67,7 @@ struct DxParams {
   int N, K, G, g, g_shift, T;
   int j_tiles, t_tiles, k_blocks;   // 256-column tiles, 512-token tiles, 64-row stages over N
   PairItems items;
+  int beside;           // see common.cuh
   int* status;
 };
 
@@ -117,10 +118,10 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   __syncthreads();
   cluster_sync_all();
   tc_fence_after();
-  // Set-up is done.  The next kernel of the stream may begin its own (programmatic launch);
-  // everything below touches memory that the preceding kernel may still be writing.
+  // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
+  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.items.total_items;      // work items: whole tiles, then halves
   const int pair = blockIdx.x >> 1;
@@ -397,6 +398,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
     atomicExch(p.status, (int)PEQA_ERR_DEVICE_TIMEOUT);
     p.status[1] = (int)blockIdx.x;
   }
+  // beside another kernel: this one has not ended before that one has
+  if (p.beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int BITS, bool ZF>
@@ -432,8 +435,9 @@ bool dx_pair_supported(const peqa_qweight_t* w) {
 }
 
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
-                   void* dX, cudaStream_t st) {
+                   void* dX, bool beside, cudaStream_t st) {
   DxParams p;
+  p.beside = beside;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;

@@ -386,6 +386,7 @@ struct DsParams {
   int vec_ok;        // out, out_z, adam_s, adam_m, adam_v are 16-byte aligned
   int i_tiles, j_tiles, k_blocks;
   int band, band_rows;   // tile order: tiles per band and which dimension is banded (see ds_tile)
+  int beside;           // see common.cuh
   int* status;
 };
 
@@ -414,6 +415,7 @@ __device__ __forceinline__ void ds_tile(const DsParams& p, int tile, int& it, in
 // The leader CTA (rank 0) issues every MMA; both CTAs' TMA loads credit the
 // leader's "full" barrier and tcgen05.commit releases the stage in both CTAs.
 constexpr int DS_STAGES = 6;
+constexpr int DS_NEXT = 2;                                               // tiles asked for ahead (dynamic)
 constexpr int DS_STAGE_BYTES = 2 * (BM * BK * 2);                      // A 16 KiB + B half 16 KiB
 constexpr int DS_PK_BYTES = BM * 128;                                    // packed codes of a CTA's 128 x 256 half tile
 constexpr int DS_SMEM_BYTES = DS_STAGES * DS_STAGE_BYTES + 2 * DS_PK_BYTES + 1024 + 512;
@@ -425,6 +427,12 @@ struct DsBarriers {
   uint64_t acc_empty[2];        // leader: both CTAs' epilogues drained the accumulator
   uint64_t pk_full[2];          // each CTA: packed codes of a tile landed
   uint64_t pk_empty[2];         // each CTA: its epilogue warps have read them
+  uint4 response;               // leader: answer to a request for another tile (dynamic)
+  uint64_t wanted;              // leader: one is wanted
+  uint64_t answered;            // leader: the answer has arrived
+  uint64_t next_full[DS_NEXT];  // each CTA: the number of a further tile stands in next_tile
+  uint64_t next_empty[DS_NEXT]; // leader: every role of both CTAs has read it
+  int next_tile[DS_NEXT];       // -1: no more
   uint32_t tmem_base;
   int abort_flag;
   int wait_limit_us;    // must follow abort_flag (read by the bounded waits)
@@ -464,7 +472,11 @@ __device__ __forceinline__ void store_pieces(float* dst, int n, bool vec, const 
 // the wait (gradient and AdamW, before -> after): 22016 x 8192 in groups of 64 at 40 tokens
 // 235 -> 122 us, 4096 x 4096 in groups of 32 at 77 tokens 42 -> 18 us, 4096 x 11008 per channel at
 // 77 tokens 44 -> 31 us; 8192 x 8192 in groups of 64 at 4096 tokens 427 -> 406 us.
-template <int BITS, bool DZ, bool ADAM, bool PKTMA>
+//
+// DYNAMIC (beside another contraction, see common.cuh): the grid has a CTA pair per tile.  Pairs start on the SMs that the other kernel
+// leaves idle, take over tiles that have not been started (cluster launch control), and those that start late find so
+// many fewer left (us, dealt / taken over: dX, dS and dZ of 4096 x 11008 at 1001 tokens 158 / 135).
+template <int BITS, bool DZ, bool ADAM, bool PKTMA, bool DYNAMIC>
 __global__ void __launch_bounds__(kDsThreads, 1)
 ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ CUtensorMap tmap_x,
           const __grid_constant__ CUtensorMap tmap_pk, const DsParams p) {
@@ -489,6 +501,15 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
       mbar_init(smem_u32(&bars->pk_full[b]), 1);
       mbar_init(smem_u32(&bars->pk_empty[b]), 8);
     }
+    if (DYNAMIC) {
+      for (int b = 0; b < DS_NEXT; ++b) {
+        mbar_init(smem_u32(&bars->next_full[b]), 1);
+        // two copying lanes and eight epilogue warps in each CTA, the leader's issuing lane
+        mbar_init(smem_u32(&bars->next_empty[b]), 2 * 10 + 1);
+      }
+      mbar_init(smem_u32(&bars->wanted), 1);
+      mbar_init(smem_u32(&bars->answered), 1);
+    }
     bars->abort_flag = 0;
     bars->wait_limit_us = p.status[4];
     fence_mbar_init();
@@ -504,20 +525,43 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   __syncthreads();
   cluster_sync_all();          // barriers of both CTAs initialised before any remote arrive
   tc_fence_after();
-  // Set-up is done.  The next kernel of the stream may begin its own (programmatic launch);
-  // everything below touches memory that the preceding kernel may still be writing.
+  // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
+  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.i_tiles * p.j_tiles;   // pair tiles (256 x 256)
   const int pair = blockIdx.x >> 1;
   const int n_pairs = gridDim.x >> 1;
+  // The tile behind `tile`, -1 if there is none: dealt round-robin, or (dynamic) the n-th that warp 2 got hold of.  A role
+  // that reads it in one lane hands in that lane (0), a warp that goes on together reads it together.
+  auto dealt = [&](int tile) { return tile + n_pairs < total_tiles ? tile + n_pairs : -1; };
+  auto taken = [&](uint32_t n) { return *reinterpret_cast<volatile int*>(&bars->next_tile[n % DS_NEXT]); };
+  auto release = [&](uint32_t n) { mbar_arrive_cluster_release(mapa_shared(smem_u32(&bars->next_empty[n % DS_NEXT]), 0)); };
+  auto next_of_lane = [&](uint32_t lane, int tile, uint32_t n) {
+    if (!DYNAMIC) return dealt(tile);
+    if (lane == 0) {
+      if (!mbar_wait_cluster(smem_u32(&bars->next_full[n % DS_NEXT]), (n / DS_NEXT) & 1u, abort_flag)) return -1;
+    }
+    const int next = taken(n);
+    release(n);
+    return next;
+  };
+  auto next_of_warp = [&](int tile, uint32_t n) {
+    if (!DYNAMIC) return dealt(tile);
+    if (!warp_wait_cluster(smem_u32(&bars->next_full[n % DS_NEXT]), (n / DS_NEXT) & 1u, abort_flag)) return -1;
+    const int next = taken(n);
+    __syncwarp();
+    if (lane == 0) release(n);
+    return next;
+  };
 
   if (warp == 0) {
     if (const uint32_t lane = elect_lane(); lane == 0) {
-      uint32_t it = 0;
+      uint32_t it = 0, n = 0;
       bool ok = true;
-      for (int tile = pair; ok && tile < total_tiles; tile += n_pairs) {
+      const int ask_at = DYNAMIC ? max(p.k_blocks - 6, 0) : -1;
+      for (int tile = pair; ok && tile >= 0; tile = next_of_lane(lane, tile, n++)) {
         int ti, tj;
         ds_tile(p, tile, ti, tj);
         const int i0 = ti * (2 * BM) + (int)rank * BM;
@@ -528,6 +572,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
           if (!mbar_wait_cluster(smem_u32(&bars->empty[s]), ph ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t bar = mapa_shared(smem_u32(&bars->full[s]), 0);
           if (leader) mbar_arrive_expect_tx(smem_u32(&bars->full[s]), 2 * DS_STAGE_BYTES);
+          if (leader && kb == ask_at) mbar_arrive(smem_u32(&bars->wanted));
           uint8_t* st = base + s * DS_STAGE_BYTES;
           // Each box is 64 contiguous features x 64 tokens = one 8 KiB MN-major chunk.
 #pragma unroll
@@ -550,7 +595,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
       bool ready = false;
       int local = 0;
       bool ok = true;
-      for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
+      for (int tile = pair; ok && tile >= 0; tile = next_of_lane(lane, tile, (uint32_t)local++)) {
         const int buf = local & 1;
         const uint32_t acc_ph = (local >> 1) & 1u;
         if (!mbar_wait_cluster(smem_u32(&bars->acc_empty[buf]), acc_ph ^ 1u, abort_flag)) { ok = false; break; }
@@ -579,7 +624,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     // packed codes of this CTA's 128 rows x 256 columns, a tile ahead of the epilogue (one lane)
     if (PKTMA) if (const uint32_t lane = elect_lane(); lane == 0) {
       int local = 0;
-      for (int tile = pair; tile < total_tiles; tile += n_pairs, ++local) {
+      for (int tile = pair; tile >= 0; tile = next_of_lane(lane, tile, (uint32_t)local++)) {
         int ti, tj;
         ds_tile(p, tile, ti, tj);
         const int ps = local & 1;
@@ -587,6 +632,28 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         const uint32_t bar = smem_u32(&bars->pk_full[ps]);
         mbar_arrive_expect_tx(bar, BM * 32 * BITS);
         tma_load_2d(smem_u32(sm_pk + ps * DS_PK_BYTES), &tmap_pk, bar, tj * (8 * BITS), ti * (2 * BM) + (int)rank * BM);
+      }
+    }
+  } else if (warp == 2) {
+    // DYNAMIC: takes over a tile that no CTA pair has been started for and tells all roles of both CTAs.  Late in the tile
+    // before: what a pair holds is not there for one that becomes idle.
+    if (DYNAMIC && leader) if (const uint32_t lane = elect_lane(); lane == 0) {
+      const uint32_t answered = smem_u32(&bars->answered), response = smem_u32(&bars->response);
+      for (uint32_t n = 0;; ++n) {
+        const uint32_t q = n % DS_NEXT;
+        if (!mbar_wait(smem_u32(&bars->wanted), n & 1u, abort_flag)) break;
+        if (!mbar_wait_cluster(smem_u32(&bars->next_empty[q]), ((n / DS_NEXT) & 1u) ^ 1u, abort_flag)) break;
+        mbar_arrive_expect_tx(answered, 16);
+        launch_try_cancel(response, answered);
+        if (!mbar_wait(answered, n & 1u, abort_flag)) break;
+        uint32_t first_cta;
+        const int tile = launch_cancelled(response, first_cta) ? (int)(first_cta >> 1) : -1;
+        fence_proxy_async_smem();                      // it has been read: the next answer may be written over it
+        bars->next_tile[q] = tile;
+        st_cluster_u32(mapa_shared(smem_u32(&bars->next_tile[q]), 1), (uint32_t)tile);
+        mbar_arrive(smem_u32(&bars->next_full[q]));
+        mbar_arrive_cluster_release_all(mapa_shared(smem_u32(&bars->next_full[q]), 1));
+        if (tile < 0) break;
       }
     }
   } else if (warp >= 4) {
@@ -599,7 +666,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     const uint32_t acc_empty_leader1 = mapa_shared(smem_u32(&bars->acc_empty[1]), 0);
     int local = 0;
     bool ok = true;
-    for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
+    for (int tile = pair; ok && tile >= 0; tile = next_of_warp(tile, (uint32_t)local++)) {
       int ti, tj;
       ds_tile(p, tile, ti, tj);
       const int i0 = ti * (2 * BM) + (int)rank * BM;
@@ -704,6 +771,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (k < n_pieces) adamw_update(ms[k], r[k], mm[k], mv[k], p.adam);
+        // the kernels this one runs beside read the scales
+        if (p.beside && local == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
         store_pieces(p.adam_s + e0, n_pieces, vec, ms);
         store_pieces(p.adam_m + e0, n_pieces, vec, mm);
         store_pieces(p.adam_v + e0, n_pieces, vec, mv);
@@ -735,6 +804,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     atomicExch(p.status, (int)PEQA_ERR_DEVICE_TIMEOUT);
     p.status[1] = (int)blockIdx.x;
   }
+  // beside another kernel: this one has not ended before that one has (any CTA but the running ones may have been taken over)
+  if (p.beside && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // An output's pieces lie side by side.  A thread that adds up its own reads every line of memory as often as the
@@ -960,10 +1031,10 @@ int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void*
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call, int t0) {
+              cudaStream_t st, int T_call, int t0, bool beside) {
   if (dx_pair_supported(w) && split_is_faster(w, T_call, true, false))
-    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call, t0);
-  if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, st);
+    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call, t0, beside);
+  if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, beside, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }
 
@@ -1021,11 +1092,12 @@ size_t dsdz_workspace_bytes(const peqa_qweight_t* w, int g, int T) {
 
 int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, const void* dY,
               int T, float* dS, float* dZ, const DsAdam* adam, void* workspace,
-              size_t workspace_bytes, cudaStream_t st) {
+              size_t workspace_bytes, cudaStream_t st, bool beside) {
   if (adam && dZ) return PEQA_ERR_BAD_SHAPE;   // dZ reads the scales the step would be rewriting
   if (zeros_f && !dZ) return PEQA_ERR_NULL;    // the correction needs the sums dZ is made of
   (void)workspace_bytes;
   DsParams p;
+  p.beside = beside;
   p.qw = w->qweight;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
@@ -1069,7 +1141,11 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   PEQA_TRY(sm_count(&sms));
   const int tiles = p.i_tiles * p.j_tiles;
   const int max_pairs = sms / 2;
-  const int pairs = tiles < max_pairs ? tiles : max_pairs;
+  // With few tokens a tile is short beside what taking it over costs (us, dealt / taken over, training step: 8192 x 8192 in groups of
+  // 64 at 60 tokens 101.5 / 105.6; 4096 x 4096 in groups of 128 at 333 57.5 / 56.5, at 2048 166.6 / 153.1).
+  const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;   // 4-bit: always; 3-bit: K % 128 == 0
+  const bool dynamic = beside && pktma && tiles > max_pairs && p.k_blocks >= 6;
+  const int pairs = tiles < max_pairs || dynamic ? tiles : max_pairs;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs, 1, 1);
   cfg.blockDim = dim3(kDsThreads, 1, 1);
@@ -1085,7 +1161,6 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;   // 4-bit: always; 3-bit: K % 128 == 0
   CUtensorMap tmap_pk = tmap_x;
   if (pktma) {
     EncodeTiledFn enc = nullptr;
@@ -1100,17 +1175,21 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cuda_fail(cudaErrorInvalidValue);
   }
-#define PEQA_DS_LAUNCH_T(B, Z, A, P)                                                                  \
+#define PEQA_DS_LAUNCH_T(B, Z, A, P, D)                                                               \
   do {                                                                                               \
-    auto kern = ds_kernel<B, Z, A, P>;                                                               \
+    auto kern = ds_kernel<B, Z, A, P, D>;                                                            \
     static std::atomic<uint64_t> done{0};                                                            \
     PEQA_TRY(allow_smem(kern, DS_SMEM_BYTES, done));                                                 \
     PEQA_CUDA(cudaLaunchKernelEx(&cfg, kern, tmap_dy, tmap_x, tmap_pk, p));                          \
   } while (0)
 #define PEQA_DS_LAUNCH(B, Z, A)                     \
   do {                                              \
-    if (B == 4 || pktma) PEQA_DS_LAUNCH_T(B, Z, A, true); \
-    else PEQA_DS_LAUNCH_T(B, Z, A, (B == 4));       \
+    if (B == 4 || pktma) {                          \
+      if (dynamic) PEQA_DS_LAUNCH_T(B, Z, A, true, true); \
+      else PEQA_DS_LAUNCH_T(B, Z, A, true, false);  \
+    } else {                                        \
+      PEQA_DS_LAUNCH_T(B, Z, A, (B == 4), false);   \
+    }                                               \
   } while (0)
   if (w->bits == 4) {
     if (dZ) PEQA_DS_LAUNCH(4, true, false);

@@ -361,6 +361,38 @@ __device__ __forceinline__ void mbar_arrive_cluster_release(uint32_t cluster_add
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
                : "memory");
 }
+// Same, with a release of everything, remote shared memory included.
+__device__ __forceinline__ void mbar_arrive_cluster_release_all(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// Cluster launch control: asks for a cluster of this grid that has not been started, which is then not started any more.  The
+// answer (16 bytes of shared memory, 16-byte aligned) is credited to `bar`.  Not to be asked again after a refusal.
+__device__ __forceinline__ void launch_try_cancel(uint32_t response, uint32_t bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(response),
+               "r"(bar)
+               : "memory");
+}
+// The answer: whether there was one, and its first CTA.
+__device__ __forceinline__ bool launch_cancelled(uint32_t response, uint32_t& first_cta) {
+  uint32_t got;
+  asm volatile(
+      "{\n\t"
+      ".reg .pred p;\n\t"
+      ".reg .b128 answer;\n\t"
+      "ld.shared.b128 answer, [%2];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, answer;\n\t"
+      "selp.u32 %1, 1, 0, p;\n\t"
+      "mov.u32 %0, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, answer;\n\t"
+      "}\n"
+      : "=&r"(first_cta), "=&r"(got)
+      : "r"(response)
+      : "memory");
+  return got != 0;
+}
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

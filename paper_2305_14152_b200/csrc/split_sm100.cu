@@ -84,6 +84,7 @@ struct SplitParams {
   int q, cshift;          // tiles per cluster, log2 of the CTAs per cluster (q <= 1 << cshift)
   const __nv_bfloat16* dY;   // DS: [T, N]
   float* ds_part;            // DS: [token tiles * passes][N]
+  int beside;                // see common.cuh
   int* status;
 };
 
@@ -208,10 +209,10 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // Set-up is done.  The next kernel of the stream may begin its own (programmatic launch);
-  // everything below touches memory that the preceding kernel may still be writing.
+  // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
+  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem_base = bars->tmem_base;
 
   if (warp == 0) {
@@ -555,6 +556,8 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     atomicExch(p.status, (int)PEQA_ERR_DEVICE_TIMEOUT);
     p.status[1] = (int)blockIdx.x;
   }
+  // beside another kernel: this one has not ended before that one has
+  if (p.beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int BITS, bool TRANS, bool FOLD, bool ZF, bool DS = false>
@@ -701,8 +704,9 @@ int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans) {
 // The T tokens from t0 on of a call of T_call tokens (act, out: of the part).  Plan and cut are those of the
 // whole call, so a token's sums are added in the same order in whichever part it comes.
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0) {
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, bool beside) {
   SplitParams p;
+  p.beside = beside;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;

@@ -1,0 +1,89 @@
+"""Contractions of one call run side by side where none writes what another reads or writes.  Whatever SMs and tiles they
+get, the results are the bits of the same contractions one after the other; calls whose buffers meet stay in order."""
+import pytest
+import torch
+
+from paper_2305_14152_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(N, K, bits, g, T, seed=5):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    new = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    w = binding.quantize_rtn(new(N, K) * 0.02, bits, g)
+    return w, new(T, K).bfloat16(), (new(T, N) * 1e-2).bfloat16()
+
+
+def _linear(w, X, dY, T):
+    z = lambda: torch.zeros_like(w.scales)
+    return binding.LayerLinear(w=w, X=X, dY=dY, Y=torch.zeros((T, w.N), dtype=torch.bfloat16, device="cuda"),
+                               dX=torch.zeros((T, w.K), dtype=torch.bfloat16, device="cuda"), dS=z(), m=z(), v=z(),
+                               workspace=binding.alloc_workspace(binding.OP_BWD, T, w))
+
+
+def _one_by_one(L, lr, step):
+    """The step's contractions, each alone on the GPU."""
+    out = []
+    for f in (lambda: binding.qlinear_fwd(L.w, L.X, L.Y), lambda: binding.qlinear_bwd(L.w, None, L.dY, dX=L.dX, need_ds=False),
+              lambda: binding.qlinear_bwd_ds_adamw(L.w, L.X, L.dY, L.m, L.v, lr, step=step, dS=L.dS, workspace=L.workspace)):
+        f()
+        torch.cuda.synchronize()
+    return [t.clone() for t in (L.Y, L.dX, L.dS, L.w.scales, L.m, L.v)]
+
+
+# fewer tiles of dS than CTA pairs; as many tiles as are taken over (81 and more, 384 tokens and more), ragged; both
+# kernels for few tokens; codes that need no TMA row pitch
+@pytest.mark.parametrize("N,K,bits,g,T", [(256, 256, 4, 0, 64), (1024, 512, 3, 64, 200), (2304, 2304, 4, 128, 384), (2312, 2432, 3, 64, 401),
+                                          (2560, 2304, 4, 0, 33), (4096, 2048, 3, 128, 1500), (2304, 2368, 3, 64, 512)])
+def test_a_step_side_by_side_is_the_step_one_by_one(N, K, bits, g, T):
+    w, X, dY = _inputs(N, K, bits, g, T)
+    a = _linear(w, X, dY, T)
+    b = _linear(binding.QWeight(bits, N, K, g, w.qweight, w.zeros, w.scales.clone()), X, dY, T)
+    for step in range(1, 7):                           # AdamW moves the scales the next step's contractions read
+        binding.layer_train_step([a], lr=1e-2, step=step)
+        got = [t.clone() for t in (a.Y, a.dX, a.dS, a.w.scales, a.m, a.v)]
+        for x, y in zip(got, _one_by_one(b, 1e-2, step)):
+            assert torch.equal(x, y)
+    binding.check_status()
+
+
+@pytest.mark.parametrize("N,K,bits,g,T", [(2304, 2304, 4, 128, 384), (1024, 512, 3, 64, 200), (4096, 2048, 3, 0, 700)])
+def test_both_gradients_with_real_zero_points(N, K, bits, g, T):
+    w, X, dY = _inputs(N, K, bits, g, T)
+    zf = w.zeros.float() + 0.1
+    alone = [binding.qlinear_bwd_zf(w, zf, None, dY, need_grads=False)[0]]
+    torch.cuda.synchronize()
+    alone += binding.qlinear_bwd_zf(w, zf, X, dY, need_dx=False)[1:]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for x, y in zip(binding.qlinear_bwd_zf(w, zf, X, dY), alone):
+            assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("shared", ["dX is X", "Y is dY", "dS is in the workspace"])
+def test_buffers_that_meet_keep_the_order(shared):
+    N = K = 1024
+    T = 256
+    w, X, dY = _inputs(N, K, 4, 256, T)
+
+    def linear():
+        L = _linear(binding.QWeight(4, N, K, 256, w.qweight, w.zeros, w.scales.clone()), X.clone(), dY.clone(), T)
+        if shared == "dX is X":
+            L.dX = L.X
+        elif shared == "Y is dY":
+            L.Y = L.dY
+        else:                                          # the sums of the first rows' groups come to lie where pieces lay
+            L.dS = L.workspace.view(torch.uint8).view(torch.float32)[:w.scales.numel()].view(w.scales.shape)
+        return L
+
+    a, b = linear(), linear()
+    binding.layer_train_step([a], lr=0.0, apply_adamw=False)
+    for f in (lambda: binding.qlinear_fwd(b.w, b.X, b.Y), lambda: binding.qlinear_bwd(b.w, None, b.dY, dX=b.dX, need_ds=False)):
+        f()
+        torch.cuda.synchronize()
+    for x, y in ((a.Y, b.Y), (a.dX, b.dX)):
+        assert torch.equal(x, y)
+    if shared != "dS is in the workspace":             # (there the reduction reads and writes the same memory)
+        binding.qlinear_bwd(b.w, b.X, b.dY, dS=b.dS, need_dx=False, workspace=b.workspace)
+        assert torch.equal(a.dS, b.dS)
