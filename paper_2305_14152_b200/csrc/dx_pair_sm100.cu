@@ -301,24 +301,18 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       return j_tile * 256 + (int)rank * 128 + 32 * u4;
     };
     int pf_col = item_col(pf_tile);
-    // cz: the constant term -delta * s of a real-valued zero-point (ZF), else unused
-    auto load_zs = [&](uint32_t (&z)[2], float (&sc)[2], float (&cz)[2]) {
+    // Nothing is made of the values here: they are used a turn later, and an operation on one would wait for it.  z: zero-point,
+    // its bits if real-valued (ZF).
+    auto load_zs = [&](uint32_t (&z)[2], float (&sc)[2]) {
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const int i = pf_kb * XK + (k ? row_b : row_a);
         z[k] = 0u;
         sc[k] = 0.0f;
-        cz[k] = 0.0f;
         if (i < p.N && pf_col < p.K) {
           const size_t gi = (size_t)i * p.G + dx_group_of(p, pf_col);
           sc[k] = ld_global(p.scales + gi);
-          if (ZF) {
-            float delta;
-            dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), z[k], delta);
-            cz[k] = -delta * sc[k];
-          } else {
-            z[k] = ld_global(p.zeros + gi);
-          }
+          z[k] = ZF ? __float_as_uint(ld_global(p.zeros_f + gi)) : ld_global(p.zeros + gi);
         }
       }
       pf_kb += X_GROUPS;
@@ -329,10 +323,10 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       }
     };
     uint32_t z[2], zn[2];
-    float sc[2], scn[2], cz[2], czn[2];
-    if ((uint32_t)grp < total_it) load_zs(z, sc, cz);
+    float sc[2], scn[2];
+    if ((uint32_t)grp < total_it) load_zs(z, sc);
     for (uint32_t it = grp; it < total_it; it += X_GROUPS) {
-      if (it + X_GROUPS < total_it) load_zs(zn, scn, czn);
+      if (it + X_GROUPS < total_it) load_zs(zn, scn);
       const int s = it % XSTAGES;
       const int q = it % XQ_SLOTS;
       if (!warp_wait(smem_u32(&bars->pk_full[q]), (it / XQ_SLOTS) & 1u, abort_flag)) break;
@@ -355,8 +349,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       }
       uint32_t oa[16], ob[16];
       if constexpr (ZF) {
-        dq::unit32_affine<BITS>(wa, z[0], sc[0], cz[0], oa);
-        dq::unit32_affine<BITS>(wb, z[1], sc[1], cz[1], ob);
+        dq::unit32_affine<BITS>(wa, z[0], sc[0], oa);
+        dq::unit32_affine<BITS>(wb, z[1], sc[1], ob);
       } else {
         dq::unit32_natural<BITS, true>(wa, z[0], sc[0], oa);
         dq::unit32_natural<BITS, true>(wb, z[1], sc[1], ob);
@@ -379,7 +373,6 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
       if (lane == 0) mbar_arrive_cluster_release(full_leader0 + s * 8);
       z[0] = zn[0]; z[1] = zn[1];
       sc[0] = scn[0]; sc[1] = scn[1];
-      cz[0] = czn[0]; cz[1] = czn[1];
     }
   }
 

@@ -417,44 +417,27 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
     // channel), and one 2-byte / 8-byte load when the groups are 32 columns wide
     const bool one_group = p.G == 1 || (p.g & 63) == 0;
     const bool pair_load = !one_group && p.g == 32 && (p.G & 1) == 0;
-    // cz: the constant term -delta * s of a real-valued zero-point (ZF), else unused
-    auto load_zs = [&](uint32_t (&z)[2], float (&sc)[2], float (&cz)[2]) {
+    // Nothing is made of the values here: they are used a turn later, and an operation on one would wait for it.  z: zero-point,
+    // its bits if real-valued (ZF), both units' with pair_load; a unit that shares the first one's group has none.
+    auto load_zs = [&](uint32_t (&z)[2], float (&sc)[2]) {
       z[0] = z[1] = 0u;
       sc[0] = sc[1] = 0.0f;
-      cz[0] = cz[1] = 0.0f;
       const int col = pf_kb * PK;
       if (pf_r < p.N && col < p.K) {
         const size_t gi = (size_t)pf_r * p.G + pair_group_of(p, col);
-        if (ZF) {
-          float delta;
-          sc[0] = ld_global(p.scales + gi);
-          dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), z[0], delta);
-          cz[0] = -delta * sc[0];
-          z[1] = z[0]; sc[1] = sc[0]; cz[1] = cz[0];
-          if (!one_group && col + 32 < p.K) {
-            const size_t g1 = (size_t)pf_r * p.G + pair_group_of(p, col + 32);
-            sc[1] = ld_global(p.scales + g1);
-            dq::split_zero_point<BITS>(ld_global(p.zeros_f + g1), z[1], delta);
-            cz[1] = -delta * sc[1];
-          }
-        } else if (one_group) {
-          z[0] = z[1] = ld_global(p.zeros + gi);
-          if (FOLD) sc[0] = sc[1] = ld_global(p.scales + gi);
-        } else if (pair_load) {
-          const uint32_t z2 = ld_global(reinterpret_cast<const unsigned short*>(p.zeros + gi));
-          z[0] = z2 & 0xFFu;
-          z[1] = z2 >> 8;
+        if (!ZF && pair_load) {
+          z[0] = ld_global(reinterpret_cast<const unsigned short*>(p.zeros + gi));
           if (FOLD) {
             const float2 s2 = ld_global(reinterpret_cast<const float2*>(p.scales + gi));
             sc[0] = s2.x;
             sc[1] = s2.y;
           }
         } else {
-          z[0] = ld_global(p.zeros + gi);
+          z[0] = ZF ? __float_as_uint(ld_global(p.zeros_f + gi)) : ld_global(p.zeros + gi);
           if (FOLD) sc[0] = ld_global(p.scales + gi);
-          if (col + 32 < p.K) {
+          if (!one_group && col + 32 < p.K) {
             const size_t g1 = (size_t)pf_r * p.G + pair_group_of(p, col + 32);
-            z[1] = ld_global(p.zeros + g1);
+            z[1] = ZF ? __float_as_uint(ld_global(p.zeros_f + g1)) : ld_global(p.zeros + g1);
             if (FOLD) sc[1] = ld_global(p.scales + g1);
           }
         }
@@ -467,12 +450,12 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       }
     };
     uint32_t z[2], zn[2];
-    float sc[2], scn[2], cz[2], czn[2];
+    float sc[2], scn[2];
     int cur_kb = pf_kb;
-    if ((uint32_t)grp < total_it) load_zs(z, sc, cz);
+    if ((uint32_t)grp < total_it) load_zs(z, sc);
     for (uint32_t it = grp; it < total_it; it += P_GROUPS) {
       const int next_kb = pf_kb;
-      if (it + P_GROUPS < total_it) load_zs(zn, scn, czn);
+      if (it + P_GROUPS < total_it) load_zs(zn, scn);
       const int s = it % PSTAGES;
       const int q = it % PQ_SLOTS;
       if (!warp_wait(smem_u32(&bars->pk_full[q]), (it / PQ_SLOTS) & 1u, abort_flag)) break;
@@ -495,12 +478,13 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
         }
       }
       uint32_t o0[16], o1[16];
+      const float s1 = one_group ? sc[0] : sc[1];
       if constexpr (ZF) {
-        dq::unit32_affine<BITS>(w[0], z[0], sc[0], cz[0], o0);
-        dq::unit32_affine<BITS>(w[1], z[1], sc[1], cz[1], o1);
+        dq::unit32_affine<BITS>(w[0], z[0], sc[0], o0);
+        dq::unit32_affine<BITS>(w[1], one_group ? z[0] : z[1], s1, o1);
       } else {
-        dq::unit32_natural<BITS, FOLD>(w[0], z[0], sc[0], o0);
-        dq::unit32_natural<BITS, FOLD>(w[1], z[1], sc[1], o1);
+        dq::unit32_natural<BITS, FOLD>(w[0], pair_load ? z[0] & 0xFFu : z[0], sc[0], o0);
+        dq::unit32_natural<BITS, FOLD>(w[1], one_group ? z[0] : pair_load ? z[0] >> 8 : z[1], s1, o1);
       }
       fence_proxy_async_smem();                                   // the codes have been read
       __syncwarp();
@@ -520,7 +504,6 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
       if (lane == 0) mbar_arrive_cluster_release(full_leader0 + s * 8);
       z[0] = zn[0]; z[1] = zn[1];
       sc[0] = scn[0]; sc[1] = scn[1];
-      cz[0] = czn[0]; cz[1] = czn[1];
       cur_kb = next_kb;
     }
   }

@@ -109,9 +109,8 @@ struct QGemmParams {
 template <int BITS>
 struct Unit {
   uint32_t w[BITS];
-  uint32_t z;
+  uint32_t z;   // the bits of a real-valued zero-point (App. K)
   float s;
-  float c;   // -delta * s of a real-valued zero-point z + delta (App. K), else 0
 };
 
 __device__ __forceinline__ int group_of(const QGemmParams& p, int col) {
@@ -131,19 +130,11 @@ __device__ __forceinline__ Unit<BITS> load_unit(const QGemmParams& p, int i, int
     for (int q = 0; q < BITS; ++q) u.w[q] = ld_global(src + q);
     const size_t gidx = (size_t)i * p.G + group_of(p, col0);
     u.s = ld_global(p.scales + gidx);
-    u.c = 0.0f;
-    if (p.zeros_f) {
-      float delta;
-      dq::split_zero_point<BITS>(ld_global(p.zeros_f + gidx), u.z, delta);
-      u.c = -delta * u.s;
-    } else {
-      u.z = ld_global(p.zeros + gidx);
-    }
+    u.z = p.zeros_f ? __float_as_uint(ld_global(p.zeros_f + gidx)) : ld_global(p.zeros + gidx);
   } else {
     // Outside the matrix: codes equal to the zero-point dequantise to exactly 0.
     u.z = 0u;
     u.s = 0.0f;
-    u.c = 0.0f;
   }
   return u;
 }
@@ -152,7 +143,7 @@ __device__ __forceinline__ Unit<BITS> load_unit(const QGemmParams& p, int i, int
 // launch, only with FOLD) the affine form (q - zi) * s + c.
 template <int BITS, bool FOLD>
 __device__ __forceinline__ void dequant_unit(const Unit<BITS>& u, bool zf, uint32_t (&o)[16]) {
-  if (FOLD && zf) dq::unit32_affine<BITS>(u.w, u.z, u.s, u.c, o);
+  if (FOLD && zf) dq::unit32_affine<BITS>(u.w, u.z, u.s, o);
   else dq::unit32_natural<BITS, FOLD>(u.w, u.z, u.s, o);
 }
 

@@ -47,14 +47,15 @@ __device__ __forceinline__ float4 ld_global(const float4* p) {
   asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(behind_wait(p)));
   return v;
 }
-__device__ __forceinline__ uint8_t ld_global(const uint8_t* p) {
+// (a whole register: cut down to eight bits it would be waited for where it is loaded)
+__device__ __forceinline__ uint32_t ld_global(const uint8_t* p) {
   uint32_t v;
   asm("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(behind_wait(p)));
-  return (uint8_t)v;
+  return v;
 }
-__device__ __forceinline__ uint16_t ld_global(const uint16_t* p) {
-  uint16_t v;
-  asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(behind_wait(p)));
+__device__ __forceinline__ uint32_t ld_global(const uint16_t* p) {
+  uint32_t v;
+  asm("ld.global.u16 %0, [%1];" : "=r"(v) : "l"(behind_wait(p)));
   return v;
 }
 __device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {

@@ -103,29 +103,22 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
   return v;
 }
 
-// Zero-point and scale of one 32-column unit; c: the constant term -delta * s of a real-valued
-// zero-point (ZF).
+// Zero-point (its bits, if real-valued) and scale of one 32-column unit.  Nothing is made of them where they are loaded, a turn
+// ahead of their use: an operation on one would wait for it.
 struct UnitZS {
   uint32_t z;
-  float s, c;
+  float s;
 };
 
-template <int BITS, bool ZF>
+template <bool ZF>
 __device__ __forceinline__ UnitZS split_load_zs(const SplitParams& p, int i, int col) {
   UnitZS u;
   u.z = 0u;
   u.s = 0.0f;       // outside the matrix: code 0, zero-point 0, scale 0
-  u.c = 0.0f;
   if (i < p.N && col < p.K) {
     const size_t gi = (size_t)i * p.G + split_group_of(p, col);
     u.s = ld_global(p.scales + gi);
-    if (ZF) {
-      float delta;
-      dq::split_zero_point<BITS>(ld_global(p.zeros_f + gi), u.z, delta);
-      u.c = -delta * u.s;
-    } else {
-      u.z = ld_global(p.zeros + gi);
-    }
+    u.z = ZF ? __float_as_uint(ld_global(p.zeros_f + gi)) : ld_global(p.zeros + gi);
   }
   return u;
 }
@@ -316,17 +309,17 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     const int rowl = TRANS ? gw * 8 + (lane & 7) : gw * 32 + lane;
     const int swz = rowl & 7;                          // rows of a thread agree modulo 8
     const int ra = r0_of(0), rb = r0_of(split_at);
+    // (forward) the second unit shares the first one's group unless groups are not multiples of 64 columns
+    const bool one_group = !TRANS && (p.G == 1 || (p.g & 63) == 0);
     auto load_zs = [&](int it, UnitZS (&u)[2]) {
-      if (it >= n_it) { u[0] = UnitZS{0u, 0.f, 0.f}; u[1] = u[0]; return; }
+      if (it >= n_it) { u[0] = UnitZS{0u, 0.f}; u[1] = u[0]; return; }
       const int c0 = kb_of(it) * SM_BK + half * SM_HALF, r0 = it < split_at ? ra : rb;
       if (TRANS) {
-        u[0] = split_load_zs<BITS, ZF>(p, c0 + rowl, r0 + 32 * u4);
-        u[1] = split_load_zs<BITS, ZF>(p, c0 + rowl + 32, r0 + 32 * u4);
+        u[0] = split_load_zs<ZF>(p, c0 + rowl, r0 + 32 * u4);
+        u[1] = split_load_zs<ZF>(p, c0 + rowl + 32, r0 + 32 * u4);
       } else {
-        u[0] = split_load_zs<BITS, ZF>(p, r0 + rowl, c0);
-        // the second unit shares the group unless groups are not multiples of 64 columns
-        if (p.G == 1 || (p.g & 63) == 0) u[1] = u[0];
-        else u[1] = split_load_zs<BITS, ZF>(p, r0 + rowl, c0 + 32);
+        u[0] = split_load_zs<ZF>(p, r0 + rowl, c0);
+        if (!one_group) u[1] = split_load_zs<ZF>(p, r0 + rowl, c0 + 32);
       }
     };
     auto turn = [&](int it, const UnitZS (&cur)[2], UnitZS (&next)[2]) -> bool {
@@ -370,8 +363,10 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
       uint32_t o[2][16];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        if constexpr (ZF) dq::unit32_affine<BITS>(w[k], cur[k].z, cur[k].s, cur[k].c, o[k]);
-        else dq::unit32_natural<BITS, FOLD>(w[k], cur[k].z, cur[k].s, o[k]);
+        const uint32_t z = one_group ? cur[0].z : cur[k].z;
+        const float sc = one_group ? cur[0].s : cur[k].s;
+        if constexpr (ZF) dq::unit32_affine<BITS>(w[k], z, sc, o[k]);
+        else dq::unit32_natural<BITS, FOLD>(w[k], z, sc, o[k]);
       }
       const int s = it % p.stages;
       if (!warp_wait(smem_u32(&bars->empty[s]), ((it / p.stages) & 1u) ^ 1u, abort_flag)) return false;
