@@ -107,6 +107,7 @@ using namespace ptx;
 constexpr int kPWarps = PEQA_PREP_WARPS;
 constexpr int kPThreads = kPWarps * 32;
 constexpr int kPSmemLimit = 227 * 1024;
+constexpr int kPSmemL1 = 195 * 1024;                              // what leaves 60 KB of L1 (see plan_prep)
 constexpr int kPMaxSlots = 4;
 constexpr int kStepCols = 512;
 constexpr int kI8Units = 64;                                      // most (token, step)s of the integer kernel
@@ -114,8 +115,15 @@ constexpr int kPBarBytes = kPWarps * kPMaxSlots * 8;              // the warps' 
 // + abort flag, wait limit, the bounds of the warps' steps and, per token, the sum of x and the factor of its sums
 constexpr int kPHeadBytes = (kPBarBytes + 32 + (kPWarps + 1) * 4 + 4 + 16 * 8 + 127) / 128 * 128;
 
-// Pitch (floats) of a row's tokens in the per-output tables of shared memory.
-__host__ __device__ inline int tok_pitch(int toks) { return toks + ((6 - (toks & 3)) & 3); }
+// A pair's sums in shared memory: token by token, the pair's sixteen rows side by side.  Tokens and halves of rows are
+// exchanged so that the lanes of a warp that puts down the result of an MMA (rows r8, tokens 2 * c4) meet different banks.
+__host__ __device__ inline int pair_sums(int M) { return ((M + 1) & ~1) * 16; }
+__device__ __forceinline__ int sum_at(int token, int row) {
+  return (token ^ ((token >> 2) & 1)) * 16 + (row ^ ((token << 2) & 8));
+}
+// n / d = __umulhi(n, quotient_magic(d)) for n * d < 2^32; 0 stands for d = 1.
+__host__ __device__ inline uint32_t quotient_magic(int d) { return d > 1 ? 0xFFFFFFFFu / (uint32_t)d + 1u : 0u; }
+__device__ __forceinline__ int quotient(int n, uint32_t magic) { return magic ? (int)__umulhi((uint32_t)n, magic) : n; }
 
 struct PrepParams {
   const uint8_t* P;         // prepared or canonical weights
@@ -137,6 +145,7 @@ struct PrepParams {
   int pairs_per_cta;
   int row_bytes;            // of the canonical matrix
   int cshift;               // log2 of the CTAs that share a range of rows, each with a slice of K
+  uint32_t m_magic[2];      // quotient_magic of M and of (M + 1) / 2
   int* status;
 };
 
@@ -195,9 +204,9 @@ __device__ __forceinline__ uint32_t ring_load1(uint32_t addr) {
   return v;
 }
 
-__device__ __forceinline__ float2 ld_cluster_f2(uint32_t cluster_addr) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr) : "memory");
+__device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr));
   return v;
 }
 
@@ -372,19 +381,16 @@ decode_prep_kernel(const PrepParams p) {
   int* wbound = const_cast<int*>(abort_flag) + 8;                            // [warps + 1] bounds of the chunk
   float* tsum = reinterpret_cast<float*>(wbound + kPWarps + 2);              // [16] sum of a token's x (not GROUPED)
   float* tinv = tsum + 16;                                                   // [16] factor of a token's sums, see stage
-  const int toks = (p.M + 1) & ~1;                                           // tokens kept of a tile
-  // pitch of a row's tokens in the per-output tables: toks rounded up to 2 mod 4, so that the
-  // sixteen rows a warp reads for one token fall into sixteen different banks
-  const int tp = tok_pitch(toks);
-  // a warp's range meets other warps' only in its first and its last pair: those sums are parked per
-  // warp, a pair in between is one warp's alone
+  const int pair_floats = pair_sums(p.M);
+  // the warp that has a pair's first step leaves its sums in the pair's place, a warp whose range begins inside a pair (its
+  // first) leaves them in its own
   // per pair: see share_bounds; per row: zero-point and scale
   int* pwarps = reinterpret_cast<int*>(base + kPHeadBytes);                  // [pairs]
   float2* rowzs = reinterpret_cast<float2*>(pwarps + ((p.pairs_per_cta + 3) & ~3));   // [pairs][16]
-  float* part = reinterpret_cast<float*>(rowzs + (size_t)p.pairs_per_cta * 16);       // [warps][2][16][tp]
-  float* ywhole = part + (size_t)kPWarps * 2 * 16 * tp;                      // [pairs][16][tp]
-  float* yacc = ywhole + (size_t)p.pairs_per_cta * 16 * tp;                  // [pairs][16][tp] (several chunks)
-  float* xshare = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * 16 * tp : 0);     // [warps] shares of a token's sum of x
+  float* part = reinterpret_cast<float*>(rowzs + (size_t)p.pairs_per_cta * 16);       // [warps][pair_floats]
+  float* ywhole = part + (size_t)kPWarps * pair_floats;                      // [pairs][pair_floats]
+  float* yacc = ywhole + (size_t)p.pairs_per_cta * pair_floats;              // [pairs][pair_floats] (several chunks)
+  float* xshare = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * pair_floats : 0); // [warps] shares of a token's sum of x
   uint32_t* xmax = reinterpret_cast<uint32_t*>(xshare + kPWarps);        // [warps] largest |x| of a warp's share (bf16 bits)
   // I8, in their place: [steps of the tokens] sum of x and factor of the sums
   float* xsum = xshare;
@@ -501,9 +507,7 @@ decode_prep_kernel(const PrepParams p) {
       if (!I8) issue_seek();                         // (I8: one chunk)
     }
   };
-  // The warps' bounds in a chunk of spc_c steps and, per pair, the first and the last warp with steps of it and
-  // where the first leaves its sums: a range that starts in the pair has it as its first (0), else one
-  // that ends in it as its last (1), else the pair is that warp's alone (2).  Run by one warp.
+  // The warps' bounds in a chunk of spc_c steps and, per pair, the first and the last warp with steps of it.  Run by one warp.
   auto share_bounds = [&](int spc_c) {
     const int tot = npairs * spc_c;
     if (lane <= kPWarps) wbound[lane] = bound(lane, tot);
@@ -513,9 +517,7 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll 1
     for (int lp = lane; lp < npairs; lp += 32) {
       const int l0 = lp * spc_c, l1 = l0 + spc_c;
-      const int wa = owner(l0), wb = owner(l1 - 1);
-      const int where = bound(wa, tot) >= l0 ? 0 : bound(wa + 1, tot) <= l1 ? 1 : 2;
-      pwarps[lp] = wa | wb << 8 | where << 16;
+      pwarps[lp] = owner(l0) | owner(l1 - 1) << 8;
     }
   };
   // One slot per warp is requested while the preceding kernel drains; the others follow the
@@ -816,6 +818,7 @@ decode_prep_kernel(const PrepParams p) {
       tl = lo - first_pair * spc_c;
     }
     int cur_pair = -1;
+    const int own_first = tl == 0 ? -1 : first_pair;               // begins inside it
     // I8: yv[0][0] and yv[0][1] are this lane's share of its two rows (rows r8 and r8 + 8), token c4 / 2, of the
     // lower (c4 even) or upper two digits
     float acc[NT][4], acc2[NT][4], yv[NT][4];
@@ -825,15 +828,13 @@ decode_prep_kernel(const PrepParams p) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
     auto park = [&]() {
-      float* mine = cur_pair == first_pair  ? part + (size_t)(warp * 2) * 16 * tp
-                    : cur_pair == last_pair ? part + (size_t)(warp * 2 + 1) * 16 * tp
-                                            : ywhole + (size_t)cur_pair * 16 * tp;
+      float* mine = cur_pair == own_first ? part + (size_t)warp * pair_floats : ywhole + (size_t)cur_pair * pair_floats;
       if constexpr (I8) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           float v = (c4 & 1) ? yv[0][e] * 65536.0f : yv[0][e];
           v += __shfl_xor_sync(0xffffffffu, v, 1);
-          if ((c4 & 1) == 0) mine[(r8 + 8 * e) * tp + (c4 >> 1)] = v;
+          if ((c4 & 1) == 0 && (c4 >> 1) < p.M) mine[sum_at(c4 >> 1, r8 + 8 * e)] = v;
           yv[0][e] = 0.0f;
         }
       } else {
@@ -843,10 +844,13 @@ decode_prep_kernel(const PrepParams p) {
           float v[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
-          if (tk < toks) {
+          if (tk < p.M) {
             const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
-            *reinterpret_cast<float2*>(mine + r8 * tp + tk) = make_float2(v[0] * f.x, v[1] * f.y);
-            *reinterpret_cast<float2*>(mine + (r8 + 8) * tp + tk) = make_float2(v[2] * f.x, v[3] * f.y);
+            const int at = nt * 128 + sum_at(c4 * 2, r8);          // the other row and token differ in bits 3 and 4
+            mine[at] = v[0] * f.x;
+            mine[at ^ 8] = v[2] * f.x;
+            mine[at ^ 16] = v[1] * f.y;
+            mine[at ^ 24] = v[3] * f.y;
           }
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
@@ -1114,26 +1118,27 @@ decode_prep_kernel(const PrepParams p) {
     const int mpairs = (p.M + 1) >> 1;
 #pragma unroll 1
     for (int idx = threadIdx.x; idx < npairs * 16 * mpairs; idx += kPThreads) {
-      const int lr = idx & 15, rest_i = idx >> 4;
-      const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
+      const int lr = idx & 15, lp = quotient(idx >> 4, p.m_magic[1]), m = ((idx >> 4) - lp * mpairs) * 2;
       if (!pair_full(lp) && lr >= 8) continue;                     // a half pair has eight rows
       const int row = pair_rg(lp) * 8 + lr;
-      const int pw = pwarps[lp], wa = pw & 0xFF, wb = (pw >> 8) & 0xFF, where = pw >> 16;
-      float2 sum = *reinterpret_cast<const float2*>((where == 2 ? ywhole + (size_t)lp * 16 * tp
-                                                                : part + (size_t)(wa * 2 + where) * 16 * tp) + lr * tp + m);
-      // the further warps start their ranges in the pair; four at a time, so that the reads do not wait
-      // for one another
+      const int pw = pwarps[lp], wa = pw & 0xFF, wb = pw >> 8;
+      const int at0 = sum_at(m, lr), at1 = sum_at(m + 1, lr);
+      float* mine = ywhole + (size_t)lp * pair_floats;
+      float sum[2] = {mine[at0], mine[at1]};
+      // four at a time, so that the reads do not wait for one another
 #pragma unroll 1
       for (int w = wa + 1; w <= wb; w += 4) {
-        float2 v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          v[q] = w + q <= wb ? *reinterpret_cast<const float2*>(part + ((size_t)((w + q) * 2) * 16 + lr) * tp + m)
-                             : make_float2(0.0f, 0.0f);
+        float v[4][2];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          sum.x += v[q].x;
-          sum.y += v[q].y;
+          const float* from = part + (size_t)(w + q) * pair_floats;
+          v[q][0] = w + q <= wb ? from[at0] : 0.0f;
+          v[q][1] = w + q <= wb ? from[at1] : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          sum[0] += v[q][0];
+          sum[1] += v[q][1];
         }
       }
       if (!GROUPED) {
@@ -1148,55 +1153,53 @@ decode_prep_kernel(const PrepParams p) {
           s0 = ld_global(tab + (size_t)min(max(ld_global(p.task_ids + m), 0), p.n_tasks - 1) * per);
           if (m + 1 < p.M) s1 = ld_global(tab + (size_t)min(max(ld_global(p.task_ids + m + 1), 0), p.n_tasks - 1) * per);
         }
-        sum.x = fmaf(-zs.x, t0, sum.x) * s0;
-        sum.y = fmaf(-zs.x, t1, sum.y) * s1;
+        sum[0] = fmaf(-zs.x, t0, sum[0]) * s0;
+        sum[1] = fmaf(-zs.x, t1, sum[1]) * s1;
       }
       if (p.nchunks > 1) {
-        float2* ya = reinterpret_cast<float2*>(yacc + ((size_t)lp * 16 + lr) * tp + m);
+        float* ya = yacc + (size_t)lp * pair_floats;
         if (ch > 0) {
-          sum.x += ya->x;
-          sum.y += ya->y;
+          sum[0] += ya[at0];
+          sum[1] += ya[at1];
         }
         if (!last) {
-          *ya = sum;
+          ya[at0] = sum[0];
+          ya[at1] = sum[1];
           continue;
         }
       } else if (p.cshift) {
-        // the pair's place in ywhole: read above by this thread alone
-        *reinterpret_cast<float2*>(ywhole + ((size_t)lp * 16 + lr) * tp + m) = sum;
+        mine[at0] = sum[0];                                        // read above by this thread alone
+        mine[at1] = sum[1];
         continue;
       }
-      p.Y[(size_t)m * p.N + row] = __float2bfloat16_rn(sum.x);
-      if (m + 1 < p.M) p.Y[(size_t)(m + 1) * p.N + row] = __float2bfloat16_rn(sum.y);
+      p.Y[(size_t)m * p.N + row] = __float2bfloat16_rn(sum[0]);
+      if (m + 1 < p.M) p.Y[(size_t)(m + 1) * p.N + row] = __float2bfloat16_rn(sum[1]);
     }
   }
 
-  // ---- the cluster's CTAs hold the sums over their slices of K: added in rank order, a share of
-  // the outputs per CTA
+  // ---- the cluster's CTAs hold the sums over their slices of K: added in rank order, a share of the outputs per
+  // CTA.  A warp reads the sixteen rows of two tokens, two runs of 64 bytes, from each: with a row's tokens side by side a warp's
+  // reads fell into 32 pieces, and the pass took 2900 cycles for 256 rows of 16 tokens.
   if (p.cshift) {
     __syncwarp();
     cluster_sync_shared();
     const int csize = 1 << p.cshift;
     const uint32_t ysum = smem_u32(ywhole);
-    const int mpairs = (p.M + 1) >> 1;
 #pragma unroll 1
-    for (int idx = (int)threadIdx.x + rank * kPThreads; idx < npairs * 16 * mpairs; idx += csize * kPThreads) {
-      const int lr = idx & 15, rest_i = idx >> 4;
-      const int lp = rest_i / mpairs, m = (rest_i - lp * mpairs) * 2;
+    for (int idx = (int)threadIdx.x + rank * kPThreads; idx < npairs * 16 * p.M; idx += csize * kPThreads) {
+      const int lr = idx & 15, lp = quotient(idx >> 4, p.m_magic[0]), m = (idx >> 4) - lp * p.M;
       if (!pair_full(lp) && lr >= 8) continue;
-      const uint32_t at = ysum + (uint32_t)(((lp * 16 + lr) * tp + m) * 4);
-      float2 v[8];
+      const uint32_t at = ysum + (uint32_t)((lp * pair_floats + sum_at(m, lr)) * 4);
+      float sum = 0.0f;
+#pragma unroll 1
+      for (int rh = 0; rh < csize; rh += 4) {
+        float v[4];
 #pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = r < csize ? ld_cluster_f2(mapa_shared(at, (uint32_t)r)) : make_float2(0.f, 0.f);
-      float2 sum = v[0];
+        for (int r = 0; r < 4; ++r) v[r] = rh + r < csize ? ld_cluster_f32(mapa_shared(at, (uint32_t)(rh + r))) : 0.0f;
 #pragma unroll
-      for (int r = 1; r < 8; ++r) {
-        sum.x += v[r].x;
-        sum.y += v[r].y;
+        for (int r = 0; r < 4; ++r) sum += v[r];
       }
-      __nv_bfloat16* y = p.Y + (size_t)m * p.N + pair_rg(lp) * 8 + lr;
-      y[0] = __float2bfloat16_rn(sum.x);
-      if (m + 1 < p.M) y[p.N] = __float2bfloat16_rn(sum.y);
+      p.Y[(size_t)m * p.N + pair_rg(lp) * 8 + lr] = __float2bfloat16_rn(sum);
     }
     __syncwarp();
     cluster_sync_reads();     // the sums are read by the whole cluster until here
@@ -1323,15 +1326,15 @@ int x_pitch_for(int steps) {
 // adds its sums up through distributed shared memory.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at
 // 22016 x 8192 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
 //
-// The estimate, in ns, is fitted to 265 calls (1 to 16 tokens, prepared and canonical), each timed with clusters of 1, 2, 4
-// and 8: nine of ten within 0.90 to 1.15, and the shape it picks costs 1.2 % more than the best of
-// the four on average, 17 % at worst.  2300 a launch; a warp's step of a pair 1650 (2350 with groups inside the
-// step, 13 % more with two token tiles; integer kernel 1200 and 1450; canonical rows 350 more); staging a token's step
-// 45, 85 in the integer kernel, 95 from canonical rows, whose order takes the activations in half sectors; 15 per
-// row group and token for the final pass, 12 where a cluster shares it, and 1350 for the cluster's exchange; 4000
-// per further chunk; 10000 more for a second wave of clusters.  (With 10 ns for staging whatever the kernel and 2500 for
-// the exchange, single CTAs staged 50 to 90 token-steps where a cluster would have been faster, 5.6 % on
-// average: 696 x 14720, two tokens 9.1 / 5.4 us, 368 x 8704, four 7.9 / 5.7, canonical 872 x 8832, five 15.6 / 8.0.)
+// The estimate, in ns, is fitted to 350 timings (116 random calls, 1 to 16 tokens, prepared and canonical, each with clusters of 1, 2, 4
+// and 8 where these fit): the shape it picks costs 0.9 % more than the best of the four on average, 12 % at worst.  2330 a
+// launch; a warp's step of a pair 1720 (2440 with groups inside the step, 23 % more with two token tiles; integer kernel
+// 1220 and 1700; canonical rows 385 more); staging a token's step 26, 40 in the integer kernel, 83 from canonical rows, whose
+// order takes the activations in half sectors; 8.5 per row group and token for the final pass, 5.5 where a cluster shares
+// it, and 390 for the cluster's exchange, 110 more for each doubling; 2260 per further chunk; 10000 more for a second wave of
+// clusters.  (With 1350 and 12 for the exchange, what it took before its barriers and reads were cut down, it picked single CTAs
+// where clusters are faster, us: 4096 x 4096 in groups of 128, eight tokens of several tasks 7.9 / 7.4, 2064 x 5760, three tokens
+// 6.1 / 5.6.)
 //
 // i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
 // staged at once, at most four steps to a half-warp.
@@ -1339,7 +1342,6 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
   const int NT = M <= 8 ? 1 : 2, TOKP = 8 * NT;
-  const int tp = tok_pitch((M + 1) & ~1);
   const int step_bytes = canon ? 16 * (bits == 3 ? CanonRow<3>::pitch : CanonRow<4>::pitch) : 2 * bits * 512;
   const bool grouped = gcols < kStepCols;
   const int gps = grouped ? kStepCols / gcols : 0;
@@ -1362,8 +1364,8 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       // a range that starts and ends at an odd row group holds the most pairs
       c.pairs = c.rg_per_cta / 2 + 1;
       auto need = [&](int spc, int slots, int sps) -> size_t {
-        const size_t sums = (size_t)16 * tp * 4;                      // one pair's
-        size_t b = 128 + kPHeadBytes + (kPWarps * 2 + c.pairs) * sums;
+        const size_t sums = (size_t)pair_sums(M) * 4;                 // one pair's
+        size_t b = 128 + kPHeadBytes + (kPWarps + c.pairs) * sums;
         if (spc < Tl) b += c.pairs * sums;
         b += (size_t)((c.pairs + 3) & ~3) * 4 + (size_t)c.pairs * 16 * 8;
         b += ((grouped ? (size_t)spc * gps * TOKP : 0) + (i8 ? 2 * kI8Units : 2 * kPWarps)) * 4 + 128;
@@ -1373,14 +1375,20 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       };
       // ring shapes in order of preference: bytes in flight first, larger copies on a tie
       const int shapes[4][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}};   // {slots, steps per slot}
-      // all of the CTA's K staged at once, with the best ring that fits ...
+      // all of the CTA's K staged at once, with the best ring that fits, groups inside the step: that fits and leaves L1 the 28 KB
+      // more that shared memory takes from 195 KB on.  A row's scales are read a vector a step and found there again (us, all /
+      // this: eight tokens of several tasks, 8192 x 8192 in groups of 64 24.4 / 21.0, seven, 4096 x 11008 in groups of
+      // 128 17.5 / 14.5; one token, 8192 x 22016 in groups of 64 23.3 / 22.2) ...
       if ((grouped || one_group) && (!i8 || M * Tl <= kI8Units)) {
-        for (int i = canon ? 1 : 0; i < 4 && c.spc == 0; ++i)
-          if (need(Tl, shapes[i][0], shapes[i][1]) <= (size_t)kPSmemLimit) {
+        for (int i = grouped ? 0 : 4; i < 8 && c.spc == 0; ++i) {
+          const int slots = shapes[i & 3][0], sps = shapes[i & 3][1];
+          if (canon && sps > 1) continue;
+          if (need(Tl, slots, sps) <= (size_t)(i < 4 ? kPSmemL1 : kPSmemLimit)) {
             c.spc = Tl;
-            c.slots = shapes[i][0];
-            c.sps = shapes[i][1];
+            c.slots = slots;
+            c.sps = sps;
           }
+        }
       }
       // ... else (one CTA per range) the largest chunk of steps beside a ring of two single steps
       if (c.spc == 0 && ci == 0 && !i8) {
@@ -1399,10 +1407,10 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       c.i8 = i8;
       c.smem = need(c.spc, c.slots, c.sps);
       const long long steps = ((long long)c.rg_per_cta * Tl + 1) / 2;
-      const long long per_step = (i8 ? (grouped ? 1450 : 1200) : (grouped ? 2350 : 1650) * (NT == 2 ? 113 : 100) / 100) + (canon ? 350 : 0);
-      const long long per_unit = canon ? 95 : i8 ? 85 : 45;
-      c.ns = waves * (2300 + (steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * per_unit +
-                      (long long)c.rg_per_cta * M * (ci ? 12 : 15) + (ci ? 1350 : 0) + (c.nchunks - 1) * 4000) +
+      const long long per_step = (i8 ? (grouped ? 1700 : 1220) : (grouped ? 2440 : 1720) * (NT == 2 ? 123 : 100) / 100) + (canon ? 385 : 0);
+      const long long per_unit = canon ? 83 : i8 ? 40 : 26;
+      c.ns = waves * (2330 + (steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * per_unit +
+                      (long long)c.rg_per_cta * M * (ci ? 55 : 85) / 10 + (ci ? 280 + 110 * ci : 0) + (c.nchunks - 1) * 2260) +
              (waves - 1) * 10000;
       if (plan->ns < 0 || c.ns < plan->ns) *plan = c;
     }
@@ -1496,7 +1504,7 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
     // table per task (the scales of four tokens per lane do not fit in registers), where all tokens
     // at once would be worked through in more chunks or waves, and where their parked sums leave no
-    // room in shared memory (from about 42000 rows on for 16 tokens, 68000 for 12, 113000 for 9).
+    // room in shared memory (from about 105000 rows on for 16 tokens, 150000 for 12, 186000 for 9).
     const int h = (M + 1) / 2;
     const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
     PEQA_TRY(run_decode(w, weights, false, g, X, h, Y, scale_table, n_tasks, task_ids, st));
@@ -1527,6 +1535,8 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
   p.pairs_per_cta = plan.pairs;
   p.cshift = plan.cshift;
   p.row_bytes = p.K / 8 * w->bits;
+  p.m_magic[0] = quotient_magic(M);
+  p.m_magic[1] = quotient_magic((M + 1) / 2);
   PEQA_TRY(status_word(st, &p.status));
   const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
   if (canon)
