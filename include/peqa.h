@@ -173,7 +173,8 @@ int peqa_qlinear_bwd_ds_adamw(const peqa_qweight_t* w, const void* X_bf16, const
  * when apply_adamw is non-zero, App. A's AdamW step on its scales where dS becomes
  * final (the calls peqa_qlinear_fwd, peqa_qlinear_bwd (dX only) and
  * peqa_qlinear_bwd_ds_adamw would make, enqueued back to back with every
- * argument of every linear checked before the first launch).  A transformer
+ * argument of every linear checked before the first launch; those of one linear
+ * run side by side where none writes what another reads or writes).  A transformer
  * layer's quantized projections -- q, k, v, o, gate, up, down -- are such a list.
  * Each linear has its own activations X [T, K_i], upstream gradient dY [T, N_i]
  * and outputs Y [T, N_i], dX [T, K_i], dS [N_i, G_i] (overwritten); composing the

@@ -47,7 +47,7 @@
 // 150.4 us; of a LLaMA-7B layer in groups of 128, seven tokens of several tasks, 94.3 -> 85.1; one scale per
 // channel, where the main loop is the smaller part, 16 tokens 230.9 -> 227.3, one token unchanged.
 // When a warp's range crosses into the next pair it parks its sums in shared
-// memory; at the end the parked sums of each pair are added in warp order, so
+// memory, in the pair's place or, if its range begins inside the pair, in its own; at the end the parked sums of each pair are added in warp order, so
 // results do not depend on timing.  What that final pass needs per token, row and
 // pair (sums of x, zero-point and scale, contributing warps) lies ready in tables
 // by then: looked up per output it took twice as long as the main loop (12,000

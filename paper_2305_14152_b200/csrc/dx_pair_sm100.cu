@@ -171,18 +171,15 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   } else if (warp == 1) {
     // ------------------------------------------ MMA issuer (leader CTA, one lane)
     if (leader) if (const uint32_t lane = elect_lane(); lane == 0) {
-      // One thread issues everything and a tensor core holds little more than the MMA it works on, so
-      // what this thread does between the last MMA of a stage and the first of the next is a gap in the
-      // tensor pipe.  Weights and activations share a barrier, the next stage's is asked for before the
-      // last MMA of this one (its answer takes about 100 cycles, an MMA 128), and descriptors are
-      // advanced by additions (the address field counts 16-byte units).
+      // One thread issues everything, the MMAs of a stage in a few cycles each (see elect_lane), so the tensor pipe has work
+      // while this thread waits for the next stage.  Weights and activations share a barrier, and descriptors are advanced
+      // by additions (the address field counts 16-byte units).
       constexpr uint32_t idesc = idesc_bf16_f32(256, 256, 0, 1);
       const uint32_t a0 = smem_u32(base);
       const uint64_t adesc0 = smem_desc_sw128(a0, 16, 1024);
       const uint64_t bdesc0 = smem_desc_sw128(a0 + XA_BYTES, 64 * 128, 1024);
       const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
       uint32_t s = 0, ph = 0;
-      bool ready = false;
       int local = 0;
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += n_pairs, ++local) {
@@ -191,7 +188,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
         if (!mbar_wait_cluster(smem_u32(&bars->acc_empty), (uint32_t)(local & 1) ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after();
         for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!ready && !mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint64_t adesc = adesc0 + s * (XSTAGE_BYTES >> 4), bdesc = bdesc0 + s * (XSTAGE_BYTES >> 4);
           const uint32_t at = s;
@@ -207,10 +204,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
           const uint64_t alast = blocks == 2 ? adesc + (XBLK_BYTES >> 4) : adesc;
           const uint32_t dlast = blocks == 2 ? tmem_base + 256 : tmem_base;
 #pragma unroll
-          for (int k = 0; k < XK / 16; ++k) {
-            if (k == XK / 16 - 1) ready = mbar_test_cluster(full0 + s * 8, ph);
+          for (int k = 0; k < XK / 16; ++k)
             mma_bf16_ss_pair(dlast, alast + k * (32 / 16), bdesc + k * (16 * 128 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
-          }
           mma_commit_pair(empty0 + at * 8, 3);
         }
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full), 3);

@@ -577,13 +577,11 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     }
   } else if (warp == 1) {
     if (leader) if (const uint32_t lane = elect_lane(); lane == 0) {
-      // (the next stage's barrier is asked for under the last MMA of this one: see the pair kernels)
       constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, BN, 1, 1);
       const uint64_t adesc0 = smem_desc_sw128(smem_u32(base), 8192, 1024);
       const uint64_t bdesc0 = smem_desc_sw128(smem_u32(base) + 16384, 8192, 1024);
       const uint32_t full0 = smem_u32(&bars->full[0]), empty0 = smem_u32(&bars->empty[0]);
       uint32_t s = 0, ph = 0;
-      bool ready = false;
       int local = 0;
       bool ok = true;
       for (int tile = pair; ok && tile >= 0; tile = next_of_lane(lane, tile, (uint32_t)local++)) {
@@ -593,7 +591,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * BN;
         for (int kb = 0; kb < p.k_blocks; ++kb) {
-          if (!ready && !mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_cluster(full0 + s * 8, ph, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint64_t adesc = adesc0 + s * (DS_STAGE_BYTES >> 4), bdesc = bdesc0 + s * (DS_STAGE_BYTES >> 4);
           const uint32_t at = s;
@@ -602,10 +600,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
             ph ^= 1u;
           }
 #pragma unroll
-          for (int k = 0; k < BK / UMMA_K; ++k) {
-            if (k == BK / UMMA_K - 1) ready = mbar_test_cluster(full0 + s * 8, ph);
+          for (int k = 0; k < BK / UMMA_K; ++k)
             mma_bf16_ss_pair(d_tmem, adesc + k * (UMMA_K * 128 / 16), bdesc + k * (UMMA_K * 128 / 16), idesc, (kb | k) != 0 ? 1u : 0u);
-          }
           mma_commit_pair(empty0 + at * 8, 3);
         }
         if (ok) mma_commit_pair(smem_u32(&bars->acc_full[buf]), 3);

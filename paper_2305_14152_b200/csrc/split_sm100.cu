@@ -22,9 +22,8 @@
 // into its lane of TENSOR MEMORY (32 columns), beside the accumulators: shared memory, which carried the
 // weights twice, is left to the activations, and a tile of 256 tokens keeps as many stages as one of 80.
 // us before / after: 22016 x 8192 at 256 tokens 124 / 109, 8192 x 8192 at 512 68 / 55, 4096 x 11008 at 1001
-// 89 / 77, 2048 x 5504 at 150 17.8 / 14.4, 4096 x 4096 at 77 12.8 / 12.4 (an MMA of 80 tokens takes about 100 cycles
-// either way).  On CTA pairs the same was measured and is not used: with A in tensor memory a 256 x 256 x 16
-// MMA takes 190 cycles instead of 128.  dX: thread and contraction run the other way, so the weights are rebuilt in shared
+// 89 / 77, 2048 x 5504 at 150 17.8 / 14.4, 4096 x 4096 at 77 12.8 / 12.4 (an MMA of 80 tokens takes 40 cycles so, 52 with A in
+// shared memory, behind an elected lane).  dX: thread and contraction run the other way, so the weights are rebuilt in shared
 // memory, MN-major, as in the single-CTA kernel of gemm_sm100.cu.  Four groups
 // of four warps take the half stages round-robin; scales and zero-points are fetched one turn ahead.
 #include <cuda.h>
@@ -252,8 +251,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     if (const uint32_t lane = elect_lane(); lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(SM_ROWS, 16, TRANS ? 1 : 0, 0) +
                              ((uint32_t)((p.nt - 16) >> 3) << 17);
-      // One thread issues everything, so its instructions per stage are the pace of the kernel:
-      // descriptors are advanced by additions (the address field counts 16-byte units).
+      // Descriptors are advanced by additions (the address field counts 16-byte units).
       const uint32_t a0 = smem_u32(base);
       const uint64_t adesc0 = smem_desc_sw128(a0, TRANS ? 64 * 128 : 16, 1024);
       const uint64_t bdesc0 = smem_desc_sw128(a0 + kWBytes, 16, 1024);
@@ -674,6 +672,9 @@ long long split_ns(const peqa_qweight_t* w, int T, bool trans) {
   return (long long)p.waves * (3600 + p.stages * (720 + p.nt * 5 / 6) + p.nt * (34 + (p.cshift ? 0 : 9) + (p.q > 1 ? 27 : 0)));
 }
 
+// The estimates were fitted before MMAs were issued by an elected lane and weights published by a restricted release; both
+// kernels are a tenth faster since.  Over 140 random calls (40 to 2600 tokens) the choice still costs 0.3 % on average, dX 7560 x 14848 in
+// groups of 64 at 254 tokens the most (us, pair / here 67 / 89); over 60 (17 to 300) the cluster shapes cost 0.3 %.
 // Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  Of 150 forwards
 // the choice is more than 3 % off the faster one for two, of 150 dX for four (worst 8 %).  Pair / here, in us:
 // 4096 x 11008 forward at 1001 tokens 116 / 77, its dX (86 row tiles: three waves) 90 / 124; 4096 x 4096
