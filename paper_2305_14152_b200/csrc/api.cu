@@ -1,5 +1,6 @@
 // C-ABI entry points that only validate and dispatch, plus the library's
 // small amount of per-device state (architecture check, status word).
+#include <initializer_list>
 #include <mutex>
 
 #include "common.cuh"
