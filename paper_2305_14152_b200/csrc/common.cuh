@@ -210,9 +210,10 @@ bool dx_pair_supported(const peqa_qweight_t* w);
 // beside (dX, dS): launched behind kernels of the same entry point whose results it does not read and whose operands it does
 // not write (but AdamW, which waits for them), a contraction need not wait for them to end and fills the SMs they leave
 // idle.  A kernel that may have another beside it lets that one in only behind its own wait for what came before, so
-// all of that is complete; and one that ran beside another does not end before it, so whoever waits for the last waits for
-// all.  Training step, us, one after the other / side by side: 256 x 256 at 64 tokens 15.2 / 9.8, 1024 x 1024 in groups of 64 at
-// 200 24.3 / 20.1, 4096 x 4096 in groups of 128 at 2048 166 / 153; gradients with real zero-points 4096 x 11008 at 1001 164 / 135.
+// all of that is complete, and hands on that it is visible (let_next_in, begin_beside in sm100_ptx.cuh); and one that ran beside another does not
+// end before it, so whoever waits for the last waits for all.  Training step, us, one after the other / side by side: 256 x 256
+// at 64 tokens 15.2 / 10.5, 1024 x 1024 in groups of 64 at 200 24.3 / 20.2, 4096 x 4096 in groups of 128 at 2048 166 / 153; gradients
+// with real zero-points 4096 x 11008 at 1001 164 / 135.
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
                    void* dX, bool beside, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,

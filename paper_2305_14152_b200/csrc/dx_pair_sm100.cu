@@ -92,6 +92,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   const bool leader = rank == 0;
   volatile int* abort_flag = &bars->abort_flag;
 
+  begin_beside(p.beside);
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
       mbar_init(smem_u32(&bars->full[s]), 1 + 8);         // the dY copies, 4 warps of one group in each CTA
@@ -119,9 +120,9 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   cluster_sync_all();
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
-  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  // launched beside it (common.cuh).
   if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_in(p.beside);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.items.total_items;      // work items: whole tiles, then halves
   const int pair = blockIdx.x >> 1;

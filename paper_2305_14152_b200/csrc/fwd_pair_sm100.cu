@@ -130,10 +130,9 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   __syncthreads();
   cluster_sync_all();
   tc_fence_after();
-  // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing.  The next kernel of
-  // the stream is let in behind the wait, see `beside` in common.cuh.
+  // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_in(false);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.items.total_items;      // work items: whole tiles, then halves
   const int pair = blockIdx.x >> 1;

@@ -480,6 +480,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   volatile int* abort_flag = &bars->abort_flag;
+  begin_beside(p.beside);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < DS_STAGES; ++s) {
@@ -517,9 +518,9 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   cluster_sync_all();          // barriers of both CTAs initialised before any remote arrive
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
-  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  // launched beside it (common.cuh).
   if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_in(p.beside);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.i_tiles * p.j_tiles;   // pair tiles (256 x 256)
   const int pair = blockIdx.x >> 1;

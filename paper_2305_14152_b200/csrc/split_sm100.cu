@@ -159,6 +159,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
   auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles - p.t_first) * p.nt; };
 
+  begin_beside(p.beside);
   // Forward: the first codes, scales and zero-points are asked for in L2 at once.  (Nothing is read: the preceding
   // kernel may still be writing them, and L2 is where it writes.)  us before / after: 256 x 256 at 64 tokens 5.8 / 5.4,
   // 4096 x 4096 at 77 12.55 / 12.3; dX gained nothing (13.0 / 13.2).
@@ -202,9 +203,9 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   __syncthreads();
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
-  // launched beside it (common.cuh).  The next kernel of the stream is let in behind the wait.
+  // launched beside it (common.cuh).
   if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_in(p.beside);
   const uint32_t tmem_base = bars->tmem_base;
 
   if (warp == 0) {

@@ -61,6 +61,77 @@ def test_both_gradients_with_real_zero_points(N, K, bits, g, T):
             assert torch.equal(x, y)
 
 
+# both kernels for dX; AdamW in the kernel of dS (groups up to 128), in its reduction and, from 2^28 products on, in the pass
+# that adds the forward's sums (one scale per channel); dS by tiles that are taken over
+@pytest.mark.parametrize("N,bits,g,T", [(256, 4, 0, 64), (512, 4, 32, 40), (1024, 4, 64, 1500), (1024, 3, 256, 333), (2304, 4, 128, 400), (2048, 4, 0, 77),
+                                        (2048, 3, 0, 1500)])
+def test_steps_follow_one_another(N, bits, g, T):
+    """Each linear's Y and dX are the next one's X and dY, and AdamW moves the scales that the next step reads: nothing lies between
+    the calls that would make up for a read that comes early or finds an old value."""
+    depth, steps = 3, 6
+    gen = torch.Generator(device="cuda").manual_seed(N + T)
+    new = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    ws = [binding.quantize_rtn(new(N, N) / N ** 0.5, bits, g) for _ in range(depth)]
+    X, dY = new(T, N).bfloat16(), new(T, N).bfloat16()
+    first = [w.scales.clone() for w in ws]
+    m, v = ([torch.zeros_like(w.scales) for w in ws] for _ in range(2))
+    work = [binding.alloc_workspace(binding.OP_BWD, T, w) for w in ws]
+    act = lambda: torch.zeros((T, N), dtype=torch.bfloat16, device="cuda")
+
+    def outputs():
+        lists = []
+        for _ in range(steps):
+            x, dy, linears = X, dY, []
+            for i, w in enumerate(ws):
+                linears.append(binding.LayerLinear(w=w, X=x, dY=dy, Y=act(), dX=act(), dS=torch.zeros_like(w.scales), m=m[i], v=v[i], workspace=work[i]))
+                x, dy = linears[-1].Y, linears[-1].dX
+            lists.append(linears)
+        return lists
+
+    def reset():
+        for i, w in enumerate(ws):
+            w.scales.copy_(first[i])
+            m[i].zero_()
+            v[i].zero_()
+        torch.cuda.synchronize()
+
+    def all_steps(lists):
+        for step, linears in enumerate(lists, 1):
+            binding.layer_train_step(linears, lr=1e-3, step=step)
+
+    def results(lists):
+        torch.cuda.synchronize()
+        binding.check_status()
+        return [t.clone() for linears in lists for L in linears for t in (L.Y, L.dX, L.dS)] + [t.clone() for t in [w.scales for w in ws] + m + v]
+
+    apart = outputs()
+    reset()
+    for step, linears in enumerate(apart, 1):
+        for L in linears:
+            alone = binding.qlinear_fwd(L.w, L.X), binding.qlinear_bwd(L.w, None, L.dY, need_ds=False)[0]
+            torch.cuda.synchronize()
+            binding.layer_train_step([L], lr=1e-3, step=step)
+            torch.cuda.synchronize()
+            assert torch.equal(L.Y, alone[0]) and torch.equal(L.dX, alone[1])
+    expected = results(apart)
+    assert all(torch.isfinite(t).all() for t in expected) and not torch.equal(first[0], ws[0].scales)
+
+    together = outputs()
+    reset()
+    all_steps(together)
+    for a, b in zip(results(together), expected):
+        assert torch.equal(a, b)
+
+    captured, graph = outputs(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        all_steps(captured)
+    for _ in range(3):
+        reset()
+        graph.replay()
+        for a, b in zip(results(captured), expected):
+            assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("shared", ["dX is X", "Y is dY", "dS is in the workspace"])
 def test_buffers_that_meet_keep_the_order(shared):
     N = K = 1024
