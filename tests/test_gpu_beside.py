@@ -1,5 +1,7 @@
 """Contractions of one call run side by side where none writes what another reads or writes.  Whatever SMs and tiles they
 get, the results are the bits of the same contractions one after the other; calls whose buffers meet stay in order."""
+import ctypes
+
 import pytest
 import torch
 
@@ -132,29 +134,47 @@ def test_steps_follow_one_another(N, bits, g, T):
             assert torch.equal(a, b)
 
 
-@pytest.mark.parametrize("shared", ["dX is X", "Y is dY", "dS is in the workspace"])
+@pytest.mark.parametrize("shared", ["dX is X", "Y is dY", "workspace is dX", "dS is dX", "m is dX"])
 def test_buffers_that_meet_keep_the_order(shared):
+    """What the contractions one after the other leave: a later one's results, or sums under way, where an earlier one's lay."""
     N = K = 1024
     T = 256
-    w, X, dY = _inputs(N, K, 4, 256, T)
+    g = 128 if shared in ("dS is dX", "m is dX") else 256          # 128: dS and AdamW in the contraction itself
+    w, X, dY = _inputs(N, K, 4, g, T)
 
     def linear():
-        L = _linear(binding.QWeight(4, N, K, 256, w.qweight, w.zeros, w.scales.clone()), X.clone(), dY.clone(), T)
+        L = _linear(binding.QWeight(4, N, K, g, w.qweight, w.zeros, w.scales.clone()), X.clone(), dY.clone(), T)
+        as_scales = lambda t: t.view(torch.float32).view(-1)[:w.scales.numel()].view(w.scales.shape)
         if shared == "dX is X":
             L.dX = L.X
         elif shared == "Y is dY":
             L.Y = L.dY
-        else:                                          # the sums of the first rows' groups come to lie where pieces lay
-            L.dS = L.workspace.view(torch.uint8).view(torch.float32)[:w.scales.numel()].view(w.scales.shape)
+        elif shared == "workspace is dX":
+            L.workspace = L.dX.view(torch.uint8).view(-1)
+        elif shared == "dS is dX":
+            L.dS = as_scales(L.dX)
+        else:
+            L.m = as_scales(L.dX)
         return L
 
     a, b = linear(), linear()
-    binding.layer_train_step([a], lr=0.0, apply_adamw=False)
-    for f in (lambda: binding.qlinear_fwd(b.w, b.X, b.Y), lambda: binding.qlinear_bwd(b.w, None, b.dY, dX=b.dX, need_ds=False)):
-        f()
-        torch.cuda.synchronize()
-    for x, y in ((a.Y, b.Y), (a.dX, b.dX)):
-        assert torch.equal(x, y)
-    if shared != "dS is in the workspace":             # (there the reduction reads and writes the same memory)
-        binding.qlinear_bwd(b.w, b.X, b.dY, dS=b.dS, need_dx=False, workspace=b.workspace)
-        assert torch.equal(a.dS, b.dS)
+    binding.layer_train_step([a], lr=1e-2, step=1)
+    _one_by_one(b, 1e-2, 1)
+    for x, y in ((a.Y, b.Y), (a.dX, b.dX), (a.dS, b.dS), (a.w.scales, b.w.scales), (a.m, b.m), (a.v, b.v)):
+        assert torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8))     # (bits: pieces of sums read as bf16 may be NaN)
+    binding.check_status()
+
+
+def test_gradients_of_zero_points_that_meet_dX_keep_the_order():
+    N, K, T = 1024, 1024, 256
+    w, X, dY = _inputs(N, K, 3, 128, T)
+    zf = w.zeros.float() + 0.1
+    dX, dS, dZ = binding.qlinear_bwd_zf(w, zf, X, dY, need_grads=False)[0], *binding.qlinear_bwd_zf(w, zf, X, dY, need_dx=False)[1:]
+    torch.cuda.synchronize()
+    out, got_s = torch.zeros_like(dX), torch.zeros_like(dS)
+    got_z = out.view(torch.float32).view(-1)[:dZ.numel()].view(dZ.shape)
+    q = w.c_struct()
+    assert binding.lib().peqa_qlinear_bwd_zf(ctypes.byref(q), zf.data_ptr(), X.data_ptr(), dY.data_ptr(), T, out.data_ptr(), got_s.data_ptr(),
+                                             got_z.data_ptr(), 0, 0, torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(got_s, dS) and torch.equal(got_z, dZ)
+    assert torch.equal(out.view(-1)[2 * dZ.numel():], dX.view(-1)[2 * dZ.numel():])
