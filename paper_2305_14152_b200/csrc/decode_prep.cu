@@ -204,6 +204,10 @@ __device__ __forceinline__ uint32_t ring_load1(uint32_t addr) {
   return v;
 }
 
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
 __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
   float v;
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr));
@@ -383,14 +387,14 @@ decode_prep_kernel(const PrepParams p) {
   float* tinv = tsum + 16;                                                   // [16] factor of a token's sums, see stage
   const int pair_floats = pair_sums(p.M);
   // the warp that has a pair's first step leaves its sums in the pair's place, a warp whose range begins inside a pair (its
-  // first) leaves them in its own
-  // per pair: see share_bounds; per row: zero-point and scale
-  int* pwarps = reinterpret_cast<int*>(base + kPHeadBytes);                  // [pairs]
-  float2* rowzs = reinterpret_cast<float2*>(pwarps + ((p.pairs_per_cta + 3) & ~3));   // [pairs][16]
-  float* part = reinterpret_cast<float*>(rowzs + (size_t)p.pairs_per_cta * 16);       // [warps][pair_floats]
-  float* ywhole = part + (size_t)kPWarps * pair_floats;                      // [pairs][pair_floats]
-  float* yacc = ywhole + (size_t)p.pairs_per_cta * pair_floats;              // [pairs][pair_floats] (several chunks)
-  float* xshare = yacc + (p.nchunks > 1 ? (size_t)p.pairs_per_cta * pair_floats : 0); // [warps] shares of a token's sum of x
+  // first) leaves them in its own; the pairs' places follow the warps'
+  float* part = reinterpret_cast<float*>(base + kPHeadBytes);                // [warps][pair_floats], 128-byte aligned
+  float* ywhole = part + kPWarps * pair_floats;                              // [pairs][pair_floats]
+  float* yacc = ywhole + p.pairs_per_cta * pair_floats;                      // [pairs][pair_floats] (several chunks)
+  // per row: zero-point and scale; per pair: see share_bounds
+  float2* rowzs = reinterpret_cast<float2*>(p.nchunks > 1 ? yacc + p.pairs_per_cta * pair_floats : yacc);    // [pairs][16]
+  int* pwarps = reinterpret_cast<int*>(rowzs + p.pairs_per_cta * 16);        // [pairs]
+  float* xshare = reinterpret_cast<float*>(pwarps + ((p.pairs_per_cta + 3) & ~3));    // [warps] shares of a token's sum of x
   uint32_t* xmax = reinterpret_cast<uint32_t*>(xshare + kPWarps);        // [warps] largest |x| of a warp's share (bf16 bits)
   // I8, in their place: [steps of the tokens] sum of x and factor of the sums
   float* xsum = xshare;
@@ -827,14 +831,17 @@ decode_prep_kernel(const PrepParams p) {
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
+    // By 32-bit addresses, the halves of a result apart by bits 5 and 6 of its own (a pair's sums begin at multiples of 128
+    // bytes): with pointers the kernels ran out of registers.  us, pointers / this: 16 tokens at 4552 x 1536 6.45 / 6.1, nine
+    // at 22016 x 8192 in groups of 128 37.1 / 34.2, two at 13752 x 3328 in groups of 128 8.0 / 7.65.
     auto park = [&]() {
-      float* mine = cur_pair == own_first ? part + (size_t)warp * pair_floats : ywhole + (size_t)cur_pair * pair_floats;
+      const uint32_t mine = smem_u32(part) + (uint32_t)((cur_pair == own_first ? warp : kPWarps + cur_pair) * pair_floats) * 4;
       if constexpr (I8) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           float v = (c4 & 1) ? yv[0][e] * 65536.0f : yv[0][e];
           v += __shfl_xor_sync(0xffffffffu, v, 1);
-          if ((c4 & 1) == 0 && (c4 >> 1) < p.M) mine[sum_at(c4 >> 1, r8 + 8 * e)] = v;
+          if ((c4 & 1) == 0) st_shared_f32(mine + ((c4 >> 1) * 16 + r8 + 8 * e) * 4, v);      // sum_at; there is room for two tokens
           yv[0][e] = 0.0f;
         }
       } else {
@@ -846,11 +853,11 @@ decode_prep_kernel(const PrepParams p) {
           for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
           if (tk < p.M) {
             const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
-            const int at = nt * 128 + sum_at(c4 * 2, r8);          // the other row and token differ in bits 3 and 4
-            mine[at] = v[0] * f.x;
-            mine[at ^ 8] = v[2] * f.x;
-            mine[at ^ 16] = v[1] * f.y;
-            mine[at ^ 24] = v[3] * f.y;
+            const uint32_t at = mine + (uint32_t)(nt * 128 + sum_at(c4 * 2, r8)) * 4;
+            st_shared_f32(at, v[0] * f.x);
+            st_shared_f32(at ^ 32, v[2] * f.x);
+            st_shared_f32(at ^ 64, v[1] * f.y);
+            st_shared_f32(at ^ 96, v[3] * f.y);
           }
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
@@ -1123,7 +1130,7 @@ decode_prep_kernel(const PrepParams p) {
       const int row = pair_rg(lp) * 8 + lr;
       const int pw = pwarps[lp], wa = pw & 0xFF, wb = pw >> 8;
       const int at0 = sum_at(m, lr), at1 = sum_at(m + 1, lr);
-      float* mine = ywhole + (size_t)lp * pair_floats;
+      float* mine = ywhole + lp * pair_floats;
       float sum[2] = {mine[at0], mine[at1]};
       // four at a time, so that the reads do not wait for one another
 #pragma unroll 1
@@ -1131,7 +1138,7 @@ decode_prep_kernel(const PrepParams p) {
         float v[4][2];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float* from = part + (size_t)(w + q) * pair_floats;
+          const float* from = part + (w + q) * pair_floats;
           v[q][0] = w + q <= wb ? from[at0] : 0.0f;
           v[q][1] = w + q <= wb ? from[at1] : 0.0f;
         }
@@ -1157,7 +1164,7 @@ decode_prep_kernel(const PrepParams p) {
         sum[1] = fmaf(-zs.x, t1, sum[1]) * s1;
       }
       if (p.nchunks > 1) {
-        float* ya = yacc + (size_t)lp * pair_floats;
+        float* ya = yacc + lp * pair_floats;
         if (ch > 0) {
           sum[0] += ya[at0];
           sum[1] += ya[at1];
