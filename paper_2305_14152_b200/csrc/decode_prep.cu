@@ -1333,15 +1333,17 @@ int x_pitch_for(int steps) {
 // adds its sums up through distributed shared memory.  Before / after, 3-bit: 16 tokens at 8192 x 8192 36 / 19 us, at
 // 22016 x 8192 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
 //
-// The estimate, in ns, is fitted to 350 timings (116 random calls, 1 to 16 tokens, prepared and canonical, each with clusters of 1, 2, 4
-// and 8 where these fit): the shape it picks costs 0.9 % more than the best of the four on average, 12 % at worst.  2330 a
-// launch; a warp's step of a pair 1720 (2440 with groups inside the step, 23 % more with two token tiles; integer kernel
-// 1220 and 1700; canonical rows 385 more); staging a token's step 26, 40 in the integer kernel, 83 from canonical rows, whose
-// order takes the activations in half sectors; 8.5 per row group and token for the final pass, 5.5 where a cluster shares
-// it, and 390 for the cluster's exchange, 110 more for each doubling; 2260 per further chunk; 10000 more for a second wave of
-// clusters.  (With 1350 and 12 for the exchange, what it took before its barriers and reads were cut down, it picked single CTAs
-// where clusters are faster, us: 4096 x 4096 in groups of 128, eight tokens of several tasks 7.9 / 7.4, 2064 x 5760, three tokens
-// 6.1 / 5.6.)
+// The estimate, in ns: 2330 a launch; a step of a pair, per turn of the busiest warp, 1440 (2120 with groups inside the step, 9 % more
+// where these have little L1; 13 % less with two token tiles; integer kernel 1180 and 1360; canonical rows 330 more); staging
+// a token's step 31, 63 in the integer kernel, 91 from canonical rows, whose order takes the activations in half sectors; 2.4 per
+// row group, token and chunk for the final pass, 3.6 where a cluster shares it, and 370 for the cluster's exchange, 170 more for each
+// doubling; 5500 per further chunk; 10000 more for a second wave of clusters.  The constants are those that choose best, not
+// each what its part was measured to take (nine of ten estimates are 0.7 to 1.2 of the time): over 942 random calls (1 to 16 tokens, prepared, of several tasks and
+// canonical), each timed with clusters of 1, 2, 4 and 8, one wave and two, as one launch and as two where these fit, the
+// choice costs 0.45 % more than the best on average, 12 % at worst.  (Turns are counted chunk by chunk, since each chunk is
+// dealt to the warps anew: with the steps of all chunks dealt out once, nine chunks of five steps counted as ten turns instead of
+// eighteen, and 13 tokens of 4-bit weights took one launch where two are faster, us: 8192 x 22016 in groups of 128 99 / 56,
+// 8192 x 16384 in groups of 64 82 / 51.)
 //
 // i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
 // staged at once, at most four steps to a half-warp.
@@ -1382,8 +1384,8 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       };
       // ring shapes in order of preference: bytes in flight first, larger copies on a tie
       const int shapes[4][2] = {{2, 2}, {4, 1}, {3, 1}, {2, 1}};   // {slots, steps per slot}
-      // all of the CTA's K staged at once, with the best ring that fits, groups inside the step: that fits and leaves L1 the 28 KB
-      // more that shared memory takes from 195 KB on.  A row's scales are read a vector a step and found there again (us, all /
+      // all of the CTA's K staged at once, with the best ring that fits, groups inside the step: that fits and leaves L1 60 KB
+      // instead of 28, which is what it has from 195 KB of shared memory on.  A row's scales are read a vector a step and found there again (us, all /
       // this: eight tokens of several tasks, 8192 x 8192 in groups of 64 24.4 / 21.0, seven, 4096 x 11008 in groups of
       // 128 17.5 / 14.5; one token, 8192 x 22016 in groups of 64 23.3 / 22.2) ...
       if ((grouped || one_group) && (!i8 || M * Tl <= kI8Units)) {
@@ -1413,11 +1415,13 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       c.x_pitch = pitch_for(c.spc);
       c.i8 = i8;
       c.smem = need(c.spc, c.slots, c.sps);
-      const long long steps = ((long long)c.rg_per_cta * Tl + 1) / 2;
-      const long long per_step = (i8 ? (grouped ? 1700 : 1220) : (grouped ? 2440 : 1720) * (NT == 2 ? 123 : 100) / 100) + (canon ? 385 : 0);
-      const long long per_unit = canon ? 83 : i8 ? 40 : 26;
-      c.ns = waves * (2330 + (steps + kPWarps - 1) / kPWarps * per_step + (long long)M * Tl * per_unit +
-                      (long long)c.rg_per_cta * M * (ci ? 55 : 85) / 10 + (ci ? 280 + 110 * ci : 0) + (c.nchunks - 1) * 2260) +
+      auto turns = [&](int spc) { return (((long long)c.rg_per_cta * spc + 1) / 2 + kPWarps - 1) / kPWarps; };
+      const long long all_turns = Tl / c.spc * turns(c.spc) + turns(Tl % c.spc);
+      long long per_step = (i8 ? (grouped ? 1360 : 1180) : (grouped ? 2120 : 1440) * (NT == 2 ? 87 : 100) / 100) + (canon ? 330 : 0);
+      if (grouped && c.smem > (size_t)kPSmemL1) per_step = per_step * 109 / 100;
+      const long long per_unit = canon ? 91 : i8 ? 63 : 31;
+      c.ns = waves * (2330 + all_turns * per_step + (long long)M * Tl * per_unit +
+                      (long long)c.rg_per_cta * M * c.nchunks * (ci ? 36 : 24) / 10 + (ci ? 370 + 170 * ci : 0) + (c.nchunks - 1) * 5500) +
              (waves - 1) * 10000;
       if (plan->ns < 0 || c.ns < plan->ns) *plan = c;
     }
@@ -1511,7 +1515,8 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
     // table per task (the scales of four tokens per lane do not fit in registers), where all tokens
     // at once would be worked through in more chunks or waves, and where their parked sums leave no
-    // room in shared memory (from about 105000 rows on for 16 tokens, 150000 for 12, 186000 for 9).
+    // room in shared memory (beside many columns, from about 105000 rows of 3-bit weights on for 16 tokens, 150000 for 12, 186000
+    // for 9; of 4-bit weights, whose rings are larger, 70000, 103000 and 131000; with 512 columns about 1.9 times as many).
     const int h = (M + 1) / 2;
     const size_t K = (size_t)w->in_features, N = (size_t)w->out_features;
     PEQA_TRY(run_decode(w, weights, false, g, X, h, Y, scale_table, n_tasks, task_ids, st));

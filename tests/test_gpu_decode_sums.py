@@ -40,3 +40,11 @@ def test_sixteen_tokens_of_many_rows_take_one_launch():
     binding.qlinear_decode_prepared(w, prepared, X)
     names = [n for n in kernels_of(lambda: binding.qlinear_decode_prepared(w, prepared, X)) if "decode_prep_kernel" in n]
     assert len(names) == 1, names
+
+
+def test_many_columns_of_grouped_weights_take_two_launches():
+    """13 tokens at once would be worked through in nine chunks of K, seven and six fit a cluster's CTAs."""
+    w = binding.quantize_rtn(torch.randn((8192, 22016), device="cuda"), 4, 128)
+    prepared, X = binding.decode_prepare(w), torch.randn((13, 22016), device="cuda").bfloat16()
+    names = [n for n in kernels_of(lambda: binding.qlinear_decode_prepared(w, prepared, X)) if "decode_prep_kernel" in n]
+    assert len(names) == 2, names
