@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2305_14152_b200 import binding, synth
-from gpu_util import assert_close, bf16_to_dev, dev_to_f64, to_qweight
+from gpu_util import assert_close, bf16_to_dev, dev_to_f64, kernels_of, to_qweight
 
 pytestmark = pytest.mark.gpu
 
@@ -14,8 +14,8 @@ BITS, TASKS = 4, 3
 
 
 # all at once does not fit for 16 tokens, for 16, for 12 and 16
-@pytest.mark.parametrize("N,K,g", [(50400, 1536, 64), (128256, 512, 0), (128256, 1536, 0)])
-def test_rows_of_an_output_head(N, K, g):
+@pytest.mark.parametrize("N,K,g,two", [(102400, 1536, 64, (16,)), (151936, 512, 0, (16,)), (151936, 2560, 0, (12, 16))])
+def test_rows_of_an_output_head(N, K, g, two):
     rng = np.random.default_rng(N + g)
     G = K // g if g else 1
     packed = rng.integers(0, 1 << 32, size=(N, K * BITS // 32), dtype=np.uint32)     # every word is eight codes
@@ -34,5 +34,7 @@ def test_rows_of_an_output_head(N, K, g):
         Y = binding.qlinear_decode_prepared(qw, prep, X)
         Yt = binding.qlinear_decode_prepared(qw, prep, X, scale_table=tab, task_ids=torch.from_numpy(ids[:M]).cuda())
         binding.check_status()
+        if M in two:
+            assert len(kernels_of(lambda: binding.qlinear_decode_prepared(qw, prep, X))) == 2
         assert_close(dev_to_f64(Y), ref[:M], f"M={M}")
         assert_close(dev_to_f64(Yt), ref_tasks[:M], f"tasks, M={M}")
