@@ -184,7 +184,7 @@ int peqa_qlinear_bwd_ds_adamw(const peqa_qweight_t* w, const void* X_bf16, const
  * first and then calls peqa_scale_adamw.
  *   workspace: peqa_workspace_bytes(PEQA_OP_BWD, T, &w) bytes per linear, 256-byte
  *   aligned (may be NULL when that is 0); the linears may share one workspace,
- *   since their kernels run in stream order.
+ *   since a linear's kernels have ended before the next one's touch memory.
  * 1 <= n_linears <= PEQA_LAYER_MAX_LINEARS.  Shape rules and return codes as for
  * the single calls; nothing is enqueued when a check fails.
  * A large linear with one scale per channel takes its dS from the forward's fp32

@@ -673,11 +673,10 @@ long long split_ns(const peqa_qweight_t* w, int T, bool trans) {
   return (long long)p.waves * (3600 + p.stages * (720 + p.nt * 5 / 6) + p.nt * (34 + (p.cshift ? 0 : 9) + (p.q > 1 ? 27 : 0)));
 }
 
-// The estimates were fitted before MMAs were issued by an elected lane and weights published by a restricted release; both
-// kernels are a tenth faster since.  Over 140 random calls (40 to 2600 tokens) the choice still costs 0.3 % on average, dX 7560 x 14848 in
-// groups of 64 at 254 tokens the most (us, pair / here 67 / 89); over 60 (17 to 300) the cluster shapes cost 0.3 %.
-// Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  Of 150 forwards
-// the choice is more than 3 % off the faster one for two, of 150 dX for four (worst 8 %).  Pair / here, in us:
+// Whether a call is served faster by this kernel than by the pair kernels; 3 % in doubt go to those.  The estimates of both were fitted before MMAs
+// were issued by an elected lane and weights published by a restricted release, which made both kernels a tenth faster.  Over
+// 140 random calls (40 to 2600 tokens) the choice costs 0.3 % on average; it is a third off at worst, dX 7560 x 14848 in groups of 64 at 254
+// tokens (us, pair / here 67 / 89).  Over 60 (17 to 300) the choice of cluster shapes costs 0.3 %.  Pair / here, in us, before that:
 // 4096 x 11008 forward at 1001 tokens 116 / 77, its dX (86 row tiles: three waves) 90 / 124; 4096 x 4096
 // forward at 77 tokens 42 / 12.5, at 2048 52 / 71; 22016 x 8192 at 256 tokens forward 174 / 109, dX 217 / 91;
 // 2360 x 256 forward at 1134 tokens 10.0 / 13.0.
