@@ -154,7 +154,7 @@ extern "C" size_t peqa_workspace_bytes(int op, int T, const peqa_qweight_t* w) {
   }
 }
 
-// Whether contractions of one call may run side by side (`beside` in common.cuh): nothing that one of them writes (`out`; no
+// Whether contractions of one call may run side by side (Side in common.cuh): kernels that hand over, and nothing that one of them writes (`out`; no
 // bytes: unused) is read or written by another.  Called one after the other they may share buffers, and then stay in that order.
 struct Span {
   const void* at;
@@ -164,6 +164,7 @@ static size_t act_bytes(int T, int features) { return (size_t)T * features * 2; 
 static size_t scale_bytes(const peqa_qweight_t* w, int G) { return (size_t)w->out_features * G * sizeof(float); }
 static bool independent(const peqa_qweight_t* w, const float* zeros_f, int G, int T, const void* X, const void* dY,
                         std::initializer_list<Span> out) {
+  if (!fwd_pair_supported(w) || !dx_pair_supported(w)) return false;
   const size_t rows = (size_t)w->out_features;
   const Span in[] = {{X, act_bytes(T, w->in_features)}, {dY, act_bytes(T, w->out_features)},
                      {w->qweight, rows * w->in_features * w->bits / 8}, {w->scales, scale_bytes(w, G)},
@@ -217,12 +218,12 @@ extern "C" int peqa_qlinear_bwd(const peqa_qweight_t* w, const void* X, const vo
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T, 0));
-  if (dS) {
-    const bool beside = dX && independent(w, nullptr, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
-                                                                    {workspace, ds_workspace_bytes(w, g, T)}});
-    PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream), beside));
-  }
+  const bool both = dX && dS && independent(w, nullptr, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
+                                                                      {workspace, ds_workspace_bytes(w, g, T)}});
+  if (dX) PEQA_TRY(launch_dx(w, nullptr, g, dY, T, dX, as_stream(stream), T, 0, both ? kFollowed : kInOrder));
+  if (dS)
+    PEQA_TRY(launch_ds(w, nullptr, g, X, dY, T, dS, nullptr, nullptr, workspace, workspace_bytes, as_stream(stream),
+                       both ? kBeside : kInOrder));
   return PEQA_OK;
 }
 
@@ -288,21 +289,22 @@ extern "C" int peqa_layer_train_step(const peqa_layer_linear_t* linears, int n_l
     adam.v = L->v;
     const int G = L->w.in_features / g[i];
     const size_t opt = apply_adamw ? scale_bytes(&L->w, G) : 0;
-    const bool beside = independent(&L->w, nullptr, G, T, L->X_bf16, L->dY_bf16,
-                                    {{L->Y_bf16, act_bytes(T, L->w.out_features)}, {L->dX_bf16, act_bytes(T, L->w.in_features)},
-                                     {L->dS, scale_bytes(&L->w, G)}, {L->m, opt}, {L->v, opt}, {L->workspace, ds_workspace_bytes(&L->w, g[i], T)}});
+    const bool all = independent(&L->w, nullptr, G, T, L->X_bf16, L->dY_bf16,
+                                 {{L->Y_bf16, act_bytes(T, L->w.out_features)}, {L->dX_bf16, act_bytes(T, L->w.in_features)},
+                                  {L->dS, scale_bytes(&L->w, G)}, {L->m, opt}, {L->v, opt}, {L->workspace, ds_workspace_bytes(&L->w, g[i], T)}});
+    const Side first = all ? kFollowed : kInOrder, next = all ? kBeside : kInOrder;
     const int slots = fwd_ds_slots(&L->w, g[i], T);
     if (slots > 0) {
       float* ds_part = static_cast<float*>(L->workspace);
-      PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st));
-      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, beside));   // before the scales change
+      PEQA_TRY(launch_fwd_ds(&L->w, L->X_bf16, L->dY_bf16, T, L->Y_bf16, ds_part, st, first));
+      PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, next));   // before the scales change
       PEQA_TRY(launch_ds_channel(&L->w, ds_part, slots, L->dS, apply_adamw ? &adam : nullptr, st));
       continue;
     }
-    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T, 0));
-    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, beside));
+    PEQA_TRY(launch_fwd(&L->w, nullptr, g[i], L->X_bf16, T, L->Y_bf16, st, T, 0, first));
+    PEQA_TRY(launch_dx(&L->w, nullptr, g[i], L->dY_bf16, T, L->dX_bf16, st, T, 0, next));
     PEQA_TRY(launch_ds(&L->w, nullptr, g[i], L->X_bf16, L->dY_bf16, T, L->dS, nullptr, apply_adamw ? &adam : nullptr,
-                       L->workspace, L->workspace_bytes, st, beside));
+                       L->workspace, L->workspace_bytes, st, next));
   }
   return PEQA_OK;
 }
@@ -371,12 +373,12 @@ extern "C" int peqa_qlinear_bwd_zf(const peqa_qweight_t* w, const float* zeros_f
       if (reinterpret_cast<uintptr_t>(workspace) & 255u) return PEQA_ERR_ALIGNMENT;
     }
   }
-  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T, 0));
-  if (dS) {
-    const bool beside = dX && independent(w, zeros_f, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
-                                                                    {dZ, scale_bytes(w, G)}, {workspace, dsdz_workspace_bytes(w, g, T)}});
-    PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream), beside));
-  }
+  const bool both = dX && dS && independent(w, zeros_f, G, T, X, dY, {{dX, act_bytes(T, w->in_features)}, {dS, scale_bytes(w, G)},
+                                                                      {dZ, scale_bytes(w, G)}, {workspace, dsdz_workspace_bytes(w, g, T)}});
+  if (dX) PEQA_TRY(launch_dx(w, zeros_f, g, dY, T, dX, as_stream(stream), T, 0, both ? kFollowed : kInOrder));
+  if (dS)
+    PEQA_TRY(launch_ds(w, zeros_f, g, X, dY, T, dS, dZ, nullptr, workspace, workspace_bytes, as_stream(stream),
+                       both ? kBeside : kInOrder));
   return PEQA_OK;
 }
 

@@ -185,13 +185,26 @@ __device__ __forceinline__ void pair_item(const PairItems& it, int item, int T, 
 }
 #endif
 
+// Contractions side by side: launched behind kernels of the same entry point whose results it does not read and whose operands it does
+// not write (but AdamW, which waits for them), a contraction need not wait for them to end (kBeside) and fills the SMs they leave
+// idle.  The first of them (kFollowed) lets it in only behind its own wait for what came before, so
+// all of that is complete, and hands on that it is visible (let_next_in, begin_beside in sm100_ptx.cuh); and one that ran beside another does not
+// end before it, so whoever waits for the last waits for all.  Training step, us, one after the other / side by side: 256 x 256
+// at 64 tokens 15.2 / 10.5, 1024 x 1024 in groups of 64 at 200 24.3 / 20.2, 4096 x 4096 in groups of 128 at 2048 166 / 153; gradients
+// with real zero-points 4096 x 11008 at 1001 164 / 135.
+enum Side : int {
+  kInOrder,     // waits for the kernel before, and whatever comes behind waits for this one
+  kFollowed,    // waits; the next one is kBeside
+  kBeside       // begins beside the one before, as the next one may beside this one
+};
+
 // Entry points implemented in the individual translation units.
 // zeros_f != nullptr: real-valued zero-points [N, G] (App. K) replace w->zeros.  A call of T_call tokens may
 // be launched in parts of T tokens from t0 on (X, Y: of the part; t0 a multiple of part_tokens(w, T_call)): every
 // part takes the route of the whole call and sums in its order, so its results are the same bits.
 int part_tokens(const peqa_qweight_t* w, int T_call);
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
-               cudaStream_t st, int T_call, int t0);
+               cudaStream_t st, int T_call, int t0, Side side = kInOrder);
 // Forward and, from its fp32 sums, the scale gradient of a layer with one scale per channel in two
 // launches: the forward leaves partial sums per channel, launch_ds_channel adds them (and makes the
 // AdamW step).  fwd_ds_slots: rows of N floats that takes, at most ds_workspace_bytes; 0 when the
@@ -199,25 +212,18 @@ int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void*
 int fwd_ds_slots(const peqa_qweight_t* w, int g, int T);
 struct DsAdam;
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
-                  cudaStream_t st);
+                  cudaStream_t st, Side side);
 int launch_ds_channel(const peqa_qweight_t* w, const float* ds_part, int slots, float* dS, const DsAdam* adam,
                       cudaStream_t st);
 bool fwd_pair_supported(const peqa_qweight_t* w);
 // ds_part != nullptr (one scale per channel): sums of dY * u per channel, see fwd_pair_sm100.cu
 int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T,
-                    void* Y, const void* dY, float* ds_part, cudaStream_t st);
+                    void* Y, const void* dY, float* ds_part, cudaStream_t st, Side side);
 bool dx_pair_supported(const peqa_qweight_t* w);
-// beside (dX, dS): launched behind kernels of the same entry point whose results it does not read and whose operands it does
-// not write (but AdamW, which waits for them), a contraction need not wait for them to end and fills the SMs they leave
-// idle.  A kernel that may have another beside it lets that one in only behind its own wait for what came before, so
-// all of that is complete, and hands on that it is visible (let_next_in, begin_beside in sm100_ptx.cuh); and one that ran beside another does not
-// end before it, so whoever waits for the last waits for all.  Training step, us, one after the other / side by side: 256 x 256
-// at 64 tokens 15.2 / 10.5, 1024 x 1024 in groups of 64 at 200 24.3 / 20.2, 4096 x 4096 in groups of 128 at 2048 166 / 153; gradients
-// with real zero-points 4096 x 11008 at 1001 164 / 135.
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
-                   void* dX, bool beside, cudaStream_t st);
+                   void* dX, Side side, cudaStream_t st);
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call, int t0, bool beside = false);
+              cudaStream_t st, int T_call, int t0, Side side = kInOrder);
 // forward (trans = false) or dX (true) for few tokens; same shapes as the pair kernels.
 // channel_scales: a forward that multiplies by one scale per channel at the end
 long long split_ns(const peqa_qweight_t* w, int T, bool trans);
@@ -225,7 +231,7 @@ bool split_is_faster(const peqa_qweight_t* w, int T, bool trans, bool channel_sc
 int split_ds_slots(const peqa_qweight_t* w, int T);
 int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans);
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, bool beside = false);
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, Side side = kInOrder);
 // adam != nullptr: the AdamW step on (w->scales, m, v) is applied where dS is produced
 struct DsAdam {
   AdamWConsts c;
@@ -236,7 +242,7 @@ struct DsAdam {
 // zeros_f != nullptr needs dZ: dS is then taken with the real-valued zero-point
 int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, const void* dY,
               int T, float* dS, float* dZ, const DsAdam* adam, void* workspace,
-              size_t workspace_bytes, cudaStream_t st, bool beside = false);
+              size_t workspace_bytes, cudaStream_t st, Side side = kInOrder);
 size_t dsdz_workspace_bytes(const peqa_qweight_t* w, int g, int T);
 size_t ds_workspace_bytes(const peqa_qweight_t* w, int g, int T);
 size_t ds_from_y_workspace_bytes(const peqa_qweight_t* w, int T);

@@ -67,7 +67,7 @@ struct DxParams {
   int N, K, G, g, g_shift, T;
   int j_tiles, t_tiles, k_blocks;   // 256-column tiles, 512-token tiles, 64-row stages over N
   PairItems items;
-  int beside;           // see common.cuh
+  Side side;           // see common.cuh
   int* status;
 };
 
@@ -92,7 +92,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   const bool leader = rank == 0;
   volatile int* abort_flag = &bars->abort_flag;
 
-  begin_beside(p.beside);
+  const bool beside = p.side == kBeside;
+  begin_beside(beside);
   if (threadIdx.x == 0) {
     for (int s = 0; s < XSTAGES; ++s) {
       mbar_init(smem_u32(&bars->full[s]), 1 + 8);         // the dY copies, 4 warps of one group in each CTA
@@ -121,8 +122,8 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
   // launched beside it (common.cuh).
-  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  let_next_in(p.beside);
+  if (!beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+  let_next_in(p.side == kFollowed);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.items.total_items;      // work items: whole tiles, then halves
   const int pair = blockIdx.x >> 1;
@@ -388,7 +389,7 @@ qdx_pair_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_consta
     p.status[1] = (int)blockIdx.x;
   }
   // beside another kernel: this one has not ended before that one has
-  if (p.beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int BITS, bool ZF>
@@ -424,9 +425,9 @@ bool dx_pair_supported(const peqa_qweight_t* w) {
 }
 
 int launch_dx_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T,
-                   void* dX, bool beside, cudaStream_t st) {
+                   void* dX, Side side, cudaStream_t st) {
   DxParams p;
-  p.beside = beside;
+  p.side = side;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;

@@ -71,6 +71,7 @@ struct PairParams {
   int N, K, G, g, g_shift, T;
   int n_tiles, t_tiles, k_blocks;   // 256-channel tiles, 512-token tiles, 64-deep stages
   PairItems items;
+  Side side;            // see common.cuh
   const __nv_bfloat16* dY;   // DS: [T, N]
   float* ds_part;            // DS: [2 * ceil(T / 256)][N]
   int* status;
@@ -132,7 +133,7 @@ qfwd_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  let_next_in(false);
+  let_next_in(p.side == kFollowed);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.items.total_items;      // work items: whole tiles, then halves
   const int pair = blockIdx.x >> 1;
@@ -554,8 +555,9 @@ bool fwd_pair_supported(const peqa_qweight_t* w) {
 }
 
 int launch_fwd_pair(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T,
-                    void* Y, const void* dY, float* ds_part, cudaStream_t st) {
+                    void* Y, const void* dY, float* ds_part, cudaStream_t st, Side side) {
   PairParams p;
+  p.side = side;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;

@@ -377,7 +377,7 @@ struct DsParams {
   int vec_ok;        // out, out_z, adam_s, adam_m, adam_v are 16-byte aligned
   int i_tiles, j_tiles, k_blocks;
   int band, band_rows;   // tile order: tiles per band and which dimension is banded (see ds_tile)
-  int beside;           // see common.cuh
+  Side side;           // see common.cuh
   int* status;
 };
 
@@ -480,7 +480,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   volatile int* abort_flag = &bars->abort_flag;
-  begin_beside(p.beside);
+  const bool beside = p.side == kBeside;
+  begin_beside(beside);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < DS_STAGES; ++s) {
@@ -519,8 +520,8 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
   // launched beside it (common.cuh).
-  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  let_next_in(p.beside);
+  if (!beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+  let_next_in(p.side == kFollowed);
   const uint32_t tmem_base = bars->tmem_base;
   const int total_tiles = p.i_tiles * p.j_tiles;   // pair tiles (256 x 256)
   const int pair = blockIdx.x >> 1;
@@ -760,7 +761,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
         for (int k = 0; k < 4; ++k)
           if (k < n_pieces) adamw_update(ms[k], r[k], mm[k], mv[k], p.adam);
         // the kernels this one runs beside read the scales
-        if (p.beside && local == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (beside && local == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
         store_pieces(p.adam_s + e0, n_pieces, vec, ms);
         store_pieces(p.adam_m + e0, n_pieces, vec, mm);
         store_pieces(p.adam_v + e0, n_pieces, vec, mv);
@@ -793,7 +794,7 @@ ds_kernel(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ C
     p.status[1] = (int)blockIdx.x;
   }
   // beside another kernel: this one has not ended before that one has (any CTA but the running ones may have been taken over)
-  if (p.beside && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (beside && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // An output's pieces lie side by side.  A thread that adds up its own reads every line of memory as often as the
@@ -1010,19 +1011,19 @@ int part_tokens(const peqa_qweight_t* w, int T_call) {
 }
 
 int launch_fwd(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, int T, void* Y,
-               cudaStream_t st, int T_call, int t0) {
+               cudaStream_t st, int T_call, int t0, Side side) {
   const bool channel_scales = g == w->in_features && !zeros_f;
   if (fwd_pair_supported(w) && split_is_faster(w, T_call, false, channel_scales))
-    return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call, t0);
-  if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st);
+    return launch_split(w, zeros_f, g, X, T, Y, false, nullptr, nullptr, st, T_call, t0, side);
+  if (fwd_pair_supported(w)) return launch_fwd_pair(w, zeros_f, g, X, T, Y, nullptr, nullptr, st, side);
   return launch_qgemm(w, zeros_f, g, X, T, Y, false, st);
 }
 
 int launch_dx(const peqa_qweight_t* w, const float* zeros_f, int g, const void* dY, int T, void* dX,
-              cudaStream_t st, int T_call, int t0, bool beside) {
+              cudaStream_t st, int T_call, int t0, Side side) {
   if (dx_pair_supported(w) && split_is_faster(w, T_call, true, false))
-    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call, t0, beside);
-  if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, beside, st);
+    return launch_split(w, zeros_f, g, dY, T, dX, true, nullptr, nullptr, st, T_call, t0, side);
+  if (dx_pair_supported(w)) return launch_dx_pair(w, zeros_f, g, dY, T, dX, side, st);
   return launch_qgemm(w, zeros_f, g, dY, T, dX, true, st);
 }
 
@@ -1044,10 +1045,10 @@ int fwd_ds_slots(const peqa_qweight_t* w, int g, int T) {
 }
 
 int launch_fwd_ds(const peqa_qweight_t* w, const void* X, const void* dY, int T, void* Y, float* ds_part,
-                  cudaStream_t st) {
+                  cudaStream_t st, Side side) {
   const int g = w->in_features;
-  if (split_is_faster(w, T, false, true)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T, 0);
-  return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st);
+  if (split_is_faster(w, T, false, true)) return launch_split(w, nullptr, g, X, T, Y, false, dY, ds_part, st, T, 0, side);
+  return launch_fwd_pair(w, nullptr, g, X, T, Y, dY, ds_part, st, side);
 }
 
 int launch_ds_channel(const peqa_qweight_t* w, const float* ds_part, int slots, float* dS, const DsAdam* adam,
@@ -1080,12 +1081,12 @@ size_t dsdz_workspace_bytes(const peqa_qweight_t* w, int g, int T) {
 
 int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* X, const void* dY,
               int T, float* dS, float* dZ, const DsAdam* adam, void* workspace,
-              size_t workspace_bytes, cudaStream_t st, bool beside) {
+              size_t workspace_bytes, cudaStream_t st, Side side) {
   if (adam && dZ) return PEQA_ERR_BAD_SHAPE;   // dZ reads the scales the step would be rewriting
   if (zeros_f && !dZ) return PEQA_ERR_NULL;    // the correction needs the sums dZ is made of
   (void)workspace_bytes;
   DsParams p;
-  p.beside = beside;
+  p.side = side;
   p.qw = w->qweight;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
@@ -1137,7 +1138,7 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   // zero-points, 2304 x 2304 in groups of 64 at 64 14.8 / 12.8, at 200 20.5 / 14.4, 4096 x 4096 per channel at 64 27.5 / 27.8, at 384 39.7 /
   // 38.6, 4096 x 11008 in groups of 128 at 40 47.6 / 45.3, at 256 67.3 / 61.9; step in groups of 256, 4096 x 4096 at 64 34.4 / 34.7, at 384 53.9 / 51.1.
   const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;   // 4-bit: always; 3-bit: K % 128 == 0
-  const bool dynamic = beside && pktma && tiles > max_pairs && (!adam_in_kernel || p.k_blocks >= 13);
+  const bool dynamic = side == kBeside && pktma && tiles > max_pairs && (!adam_in_kernel || p.k_blocks >= 13);
   const int pairs = tiles < max_pairs || dynamic ? tiles : max_pairs;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs, 1, 1);

@@ -238,7 +238,7 @@ __device__ __forceinline__ void tc_fence_after() {
 // The warp's index, which the compiler may hold in a uniform register (threadIdx.x >> 5 differs between threads as far
 // as it can tell).
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
-// A kernel that begins beside another (`beside` in common.cuh) was let in by it and has no wait that makes visible to it what kernels
+// A kernel that begins beside another (Side in common.cuh) was let in by it and has no wait that makes visible to it what kernels
 // before both have written.  The hand-over is a release and an acquire of its own: the thread that lets the next kernel in
 // fences before it does, behind its wait or, in a kernel that itself began beside another, behind having begun; and every
 // thread of a kernel that begins beside another fences before its first access (whatever its SM's L1 still held is not
@@ -254,11 +254,12 @@ __device__ __forceinline__ void begin_beside(bool beside) {
     asm volatile("fence.proxy.async.global;" ::: "memory");
   }
 }
-// Lets the next kernel of the stream in, behind the set-up and, if there is one, the wait.  One thread does, which counts for its CTA,
-// and of a warp that has nothing else to begin with: fencing threads of the others, a forward of 256 x 256 took 0.5 us longer.
-__device__ __forceinline__ void let_next_in(bool beside) {
+// Lets the next kernel of the stream in, behind the set-up and, if there is one, the wait; followed: by one that begins beside this
+// kernel, which waited.  One thread does, which counts for its CTA, and of a warp that has nothing else to begin with: with fencing threads of the
+// others a forward of 256 x 256 took 0.5 us longer.
+__device__ __forceinline__ void let_next_in(bool followed) {
   if (threadIdx.x == 64) {
-    if (!beside) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    if (followed) asm volatile("fence.acq_rel.gpu;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   __syncwarp();

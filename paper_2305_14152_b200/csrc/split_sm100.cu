@@ -83,7 +83,7 @@ struct SplitParams {
   int q, cshift;          // tiles per cluster, log2 of the CTAs per cluster (q <= 1 << cshift)
   const __nv_bfloat16* dY;   // DS: [T, N]
   float* ds_part;            // DS: [token tiles * passes][N]
-  int beside;                // see common.cuh
+  Side side;                 // see common.cuh
   int* status;
 };
 
@@ -159,7 +159,8 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   auto r0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) % p.r_tiles) * SM_ROWS; };
   auto t0_of = [&](int it) { return ((first_tile + j0 + (it < split_at ? 0 : 1)) / p.r_tiles - p.t_first) * p.nt; };
 
-  begin_beside(p.beside);
+  const bool beside = TRANS && p.side == kBeside;     // (a forward is the first of its call)
+  begin_beside(beside);
   // Forward: the first codes, scales and zero-points are asked for in L2 at once.  (Nothing is read: the preceding
   // kernel may still be writing them, and L2 is where it writes.)  us before / after: 256 x 256 at 64 tokens 5.8 / 5.4,
   // 4096 x 4096 at 77 12.55 / 12.3; dX gained nothing (13.0 / 13.2).
@@ -204,8 +205,8 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
   tc_fence_after();
   // Set-up is done.  Everything below touches memory that the preceding kernel may still be writing, unless this one was
   // launched beside it (common.cuh).
-  if (!p.beside) asm volatile("griddepcontrol.wait;" ::: "memory");
-  let_next_in(p.beside);
+  if (!beside) asm volatile("griddepcontrol.wait;" ::: "memory");
+  let_next_in(p.side == kFollowed);
   const uint32_t tmem_base = bars->tmem_base;
 
   if (warp == 0) {
@@ -551,7 +552,7 @@ qsplit_kernel(const __grid_constant__ CUtensorMap tmap_act, const __grid_constan
     p.status[1] = (int)blockIdx.x;
   }
   // beside another kernel: this one has not ended before that one has
-  if (p.beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (beside && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int BITS, bool TRANS, bool FOLD, bool ZF, bool DS = false>
@@ -700,9 +701,9 @@ int split_part_tokens(const peqa_qweight_t* w, int T_call, bool trans) {
 // The T tokens from t0 on of a call of T_call tokens (act, out: of the part).  Plan and cut are those of the
 // whole call, so a token's sums are added in the same order in whichever part it comes.
 int launch_split(const peqa_qweight_t* w, const float* zeros_f, int g, const void* act, int T, void* out,
-                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, bool beside) {
+                 bool trans, const void* dY, float* ds_part, cudaStream_t st, int T_call, int t0, Side side) {
   SplitParams p;
-  p.beside = beside;
+  p.side = side;
   p.zeros = w->zeros;
   p.zeros_f = zeros_f;
   p.scales = w->scales;

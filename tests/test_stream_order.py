@@ -36,24 +36,24 @@ def test_kernels_side_by_side_hand_over_what_came_before():
     """A kernel that begins without the wait (`beside`) acquires what the one that let it in has released.  Hardware
     that happens to order both shows no difference, so the sources are checked."""
     helpers = open(os.path.join(CSRC, "sm100_ptx.cuh")).read()
-    body = lambda name: re.search(r"void %s\(bool beside\) \{(.*?)\n\}" % name, helpers, re.S).group(1)
+    body = lambda name: re.search(r"void %s\(bool \w+\) \{(.*?)\n\}" % name, helpers, re.S).group(1)
     begins, lets_in = body("begin_beside"), body("let_next_in")
     assert 0 < begins.index("if (beside)") < begins.index("fence.acq_rel.gpu") < begins.index("fence.proxy.async.global")
-    assert 0 < lets_in.index("if (!beside)") < lets_in.index("fence.acq_rel.gpu") < lets_in.index("griddepcontrol.launch_dependents")
+    assert 0 < lets_in.index("if (followed)") < lets_in.index("fence.acq_rel.gpu") < lets_in.index("griddepcontrol.launch_dependents")
     beside = first = 0
     for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
         text = re.sub(r"//[^\n]*", "", open(path).read())
         for k in re.split(r"(?=\b__global__\b)", text)[1:]:
             k = k[:k.index("\n}\n")]                               # the kernel, without what follows it
-            wait = 'asm volatile("griddepcontrol.wait;" ::: "memory");\n  let_next_in('
-            if "p.beside" in k:
+            wait = 'asm volatile("griddepcontrol.wait;" ::: "memory");\n  let_next_in(p.side == kFollowed);'
+            if "kBeside" in k:
                 beside += 1
-                assert k.index("begin_beside(p.beside);") < k.index("__syncthreads()") < k.index("if (!p.beside) " + wait + "p.beside);")
-                assert k.index("p.beside") == k.index("begin_beside(p.beside);") + len("begin_beside(")
+                assert k.index("begin_beside(beside);") < k.index("__syncthreads()") < k.index("if (!beside) " + wait)
+                assert len(re.findall(r"const bool beside = (TRANS && )?p\.side == kBeside;\s+begin_beside\(beside\);", k)) == k.count("kBeside") == 1
                 assert "launch_dependents" not in k
-            elif "let_next_in(" in k:
+            elif "kFollowed" in k:
                 first += 1
-                assert wait + "false);" in k and "launch_dependents" not in k
+                assert "\n  " + wait in k and "launch_dependents" not in k
     assert beside == 3 and first == 1          # dX, dS and the kernel of few tokens; the forward
 
 
