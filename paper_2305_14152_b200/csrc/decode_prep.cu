@@ -1503,13 +1503,16 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
                const float* scale_table, int n_tasks, const int32_t* task_ids, cudaStream_t st) {
   PrepPlan plan;
   bool two = false;
+  // A row that is one group of 64, 128 or 256 columns is taken for one with groups inside the step, but for canonical rows with a
+  // table per task: their instances look the table up where a row's sums are added, which is for one scale per row.
+  const int gcols = canon && task_ids && g < kStepCols ? kStepCols : g;
   if (M > 8) {
     PrepPlan half;
     PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, false, false, &half));
     two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, false, false, &plan) != PEQA_OK ||
           2 * half.ns < plan.ns;
-  } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, true, &plan) != PEQA_OK) {
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, g, canon, false, &plan));
+  } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, true, &plan) != PEQA_OK) {
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, false, &plan));
   }
   if (two) {
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
@@ -1550,7 +1553,7 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
   p.m_magic[0] = quotient_magic(M);
   p.m_magic[1] = quotient_magic((M + 1) / 2);
   PEQA_TRY(status_word(st, &p.status));
-  const int gsh = g == 64 ? 1 : g == 128 ? 2 : g == 256 ? 3 : 0;
+  const int gsh = gcols == 64 ? 1 : gcols == 128 ? 2 : gcols == 256 ? 3 : 0;
   if (canon)
     return w->bits == 3 ? launch_prep_b<3, true>(p, plan.i8, gsh, plan.grid, plan.smem, st)
                         : launch_prep_b<4, true>(p, plan.i8, gsh, plan.grid, plan.smem, st);

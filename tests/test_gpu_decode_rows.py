@@ -32,6 +32,25 @@ def test_canonical_rows(N, K, bits, g):
         assert_close(dev_to_f64(Y), ref[:M], f"M={M}")
 
 
+@pytest.mark.parametrize("N,K,bits", [(4744, 128, 4), (4744, 256, 3), (4752, 384, 4), (5008, 512, 3), (6120, 128, 3), (6120, 640, 4), (264, 256, 4),
+                                      (4744, 4096, 3)])
+def test_canonical_rows_of_several_tasks(N, K, bits):
+    """One scale per row, also where the row is as long as a group of 128 or 256 columns; by rows from 4744 rows on."""
+    rng = np.random.default_rng(N + K)
+    d = synth.custom(N + K, N, K, 16, bits, 0, outliers=True)
+    codes, zeros, scales, packed = oracle_layer(d, bits, 0)
+    qw = to_qweight(packed, zeros, scales, bits, 0, K)
+    table = rng.uniform(0.01, 0.02, size=(3, N, 1)).astype(np.float32)
+    ids = rng.integers(0, 3, size=8).astype(np.int32)
+    ids[:2] = (2, 1)
+    ref = oracle.fwd_multitask(d["X"][:8], packed, zeros, table, ids, bits, 0)
+    tab = torch.from_numpy(table[:, :, 0].copy()).cuda()
+    for M in (1, 2, 3, 8):
+        Y = binding.qlinear_decode_multitask(qw, tab, torch.from_numpy(ids[:M]).cuda(), bf16_to_dev(d["X"][:M]))
+        binding.check_status()
+        assert_close(dev_to_f64(Y), ref[:M], f"M={M}")
+
+
 @pytest.mark.parametrize("bits,g", [(3, 0), (4, 0), (3, 64), (4, 128), (3, 256)])
 def test_tokens_of_any_magnitude(bits, g):
     """A token (in a call of one or two: a step of it) is brought to the range of its operands by a power of two of
