@@ -377,6 +377,7 @@ decode_prep_kernel(const PrepParams p) {
   constexpr bool GROUPED = GSH != 0;
   constexpr int RUNS_PER_GROUP = GROUPED ? (1 << GSH) : 16;
   constexpr int GPS = 16 / RUNS_PER_GROUP;           // groups per step (GROUPED)
+  constexpr bool kIndexed = GSH == 1 && NT == 2 && BITS == 4, kWideIndex = kIndexed || (GSH == 1 && TASKS);    // see park
   extern __shared__ uint8_t prep_smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(prep_smem_raw) + 127) &
                                              ~static_cast<uintptr_t>(127));
@@ -831,9 +832,12 @@ decode_prep_kernel(const PrepParams p) {
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
-    // By 32-bit addresses, the halves of a result apart by bits 5 and 6 of its own (a pair's sums begin at multiples of 128
+    // By 32-bit addresses, the parts of a result apart by bits 5 and 6 of its own (a pair's sums begin at multiples of 128
     // bytes): with pointers the kernels ran out of registers.  us, pointers / this: 16 tokens at 4552 x 1536 6.45 / 6.1, nine
-    // at 22016 x 8192 in groups of 128 37.1 / 34.2, two at 13752 x 3328 in groups of 128 8.0 / 7.65.
+    // at 22016 x 8192 in groups of 128 37.1 / 34.2, two at 13752 x 3328 in groups of 128 8.0 / 7.65.  What a loop of 128 registers spills depends on
+    // the arithmetic around it, so two kinds of kernel, whose scales of a step take the most registers, have it in another form
+    // (kIndexed here, kWideIndex in the final pass; us, without / with them: 4 bits in groups of 64, 11 tokens at 22016 x 8192 51.4 / 47.4, 16 at
+    // 4096 x 11008 22.1 / 20.9; 3 bits in groups of 64, nine tokens of several tasks at 17048 x 7040 92 / 84).
     auto park = [&]() {
       const uint32_t mine = smem_u32(part) + (uint32_t)((cur_pair == own_first ? warp : kPWarps + cur_pair) * pair_floats) * 4;
       if constexpr (I8) {
@@ -853,11 +857,11 @@ decode_prep_kernel(const PrepParams p) {
           for (int e = 0; e < 4; ++e) v[e] = (GROUPED ? yv[nt][e] : acc[nt][e] + acc2[nt][e]) * 4096.0f;
           if (tk < p.M) {
             const float2 f = *reinterpret_cast<const float2*>(tinv + tk);
-            const uint32_t at = mine + (uint32_t)(nt * 128 + sum_at(c4 * 2, r8)) * 4;
+            const uint32_t i = (uint32_t)(nt * 128 + sum_at(c4 * 2, r8)), at = mine + i * 4;
             st_shared_f32(at, v[0] * f.x);
-            st_shared_f32(at ^ 32, v[2] * f.x);
-            st_shared_f32(at ^ 64, v[1] * f.y);
-            st_shared_f32(at ^ 96, v[3] * f.y);
+            st_shared_f32(kIndexed ? mine + (i ^ 8) * 4 : at ^ 32, v[2] * f.x);
+            st_shared_f32(kIndexed ? mine + (i ^ 16) * 4 : at ^ 64, v[1] * f.y);
+            st_shared_f32(kIndexed ? mine + (i ^ 24) * 4 : at ^ 96, v[3] * f.y);
           }
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[nt][e] = acc2[nt][e] = yv[nt][e] = 0.0f;
@@ -1138,7 +1142,7 @@ decode_prep_kernel(const PrepParams p) {
         float v[4][2];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float* from = part + (w + q) * pair_floats;
+          const float* from = part + (kWideIndex ? (size_t)(w + q) * pair_floats : (size_t)((w + q) * pair_floats));
           v[q][0] = w + q <= wb ? from[at0] : 0.0f;
           v[q][1] = w + q <= wb ? from[at1] : 0.0f;
         }
