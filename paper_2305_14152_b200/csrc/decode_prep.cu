@@ -1338,7 +1338,8 @@ int x_pitch_for(int steps) {
 // 22016 x 8192 65 / 50, in groups of 64 at 8192 x 8192 97 / 28.
 //
 // The estimate, in ns: 2330 a launch; a step of a pair, per turn of the busiest warp, 1440 (2120 with groups inside the step, 9 % more
-// where these have little L1; 13 % less with two token tiles; integer kernel 1180 and 1360; canonical rows 330 more); staging
+// where these have little L1, 25 with a table per task, whose tokens read scales of their own each; 13 % less with two token
+// tiles; integer kernel 1180 and 1360; canonical rows 330 more); staging
 // a token's step 31, 63 in the integer kernel, 91 from canonical rows, whose order takes the activations in half sectors; 2.4 per
 // row group, token and chunk for the final pass, 3.6 where a cluster shares it, and 370 for the cluster's exchange, 170 more for each
 // doubling; 5500 per further chunk; 10000 more for a second wave of clusters.  The constants are those that choose best, not
@@ -1349,9 +1350,12 @@ int x_pitch_for(int steps) {
 // eighteen, and 13 tokens of 4-bit weights took one launch where two are faster, us: 8192 x 22016 in groups of 128 99 / 56,
 // 8192 x 16384 in groups of 64 82 / 51.)
 //
+// tasks: a table per task.  (With 9 % for it too, eight tokens at 17128 x 11904 in groups of 64, 3 bits, took 163 us on two CTAs a range, whose
+// rings leave 28 KB of L1, where four a range take 87.)
+//
 // i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
 // staged at once, at most four steps to a half-warp.
-int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, PrepPlan* plan) {
+int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, bool tasks, PrepPlan* plan) {
   const int sms = sm_count_or(148);
   const int rgs = N / 8;
   const int NT = M <= 8 ? 1 : 2, TOKP = 8 * NT;
@@ -1422,7 +1426,7 @@ int plan_prep(int N, int K, int M, int bits, int gcols, bool canon, bool i8, Pre
       auto turns = [&](int spc) { return (((long long)c.rg_per_cta * spc + 1) / 2 + kPWarps - 1) / kPWarps; };
       const long long all_turns = Tl / c.spc * turns(c.spc) + turns(Tl % c.spc);
       long long per_step = (i8 ? (grouped ? 1360 : 1180) : (grouped ? 2120 : 1440) * (NT == 2 ? 87 : 100) / 100) + (canon ? 330 : 0);
-      if (grouped && c.smem > (size_t)kPSmemL1) per_step = per_step * 109 / 100;
+      if (grouped && c.smem > (size_t)kPSmemL1) per_step = per_step * (tasks && !i8 ? 125 : 109) / 100;
       const long long per_unit = canon ? 91 : i8 ? 63 : 31;
       c.ns = waves * (2330 + all_turns * per_step + (long long)M * Tl * per_unit +
                       (long long)c.rg_per_cta * M * c.nchunks * (ci ? 36 : 24) / 10 + (ci ? 370 + 170 * ci : 0) + (c.nchunks - 1) * 5500) +
@@ -1512,11 +1516,11 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
   const int gcols = canon && task_ids && g < kStepCols ? kStepCols : g;
   if (M > 8) {
     PrepPlan half;
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, false, false, &half));
-    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, false, false, &plan) != PEQA_OK ||
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, (M + 1) / 2, w->bits, g, false, false, task_ids != nullptr, &half));
+    two = task_ids || plan_prep(w->out_features, w->in_features, M, w->bits, g, false, false, false, &plan) != PEQA_OK ||
           2 * half.ns < plan.ns;
-  } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, true, &plan) != PEQA_OK) {
-    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, false, &plan));
+  } else if (M > 2 || plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, true, task_ids != nullptr, &plan) != PEQA_OK) {
+    PEQA_TRY(plan_prep(w->out_features, w->in_features, M, w->bits, gcols, canon, false, task_ids != nullptr, &plan));
   }
   if (two) {
     // Two launches of at most eight tokens each, the second of which finds the weights in L2: with a
@@ -1570,7 +1574,7 @@ int run_decode(const peqa_qweight_t* w, const void* weights, bool canon, int g, 
 bool decode_rows_supported(const peqa_qweight_t* w, int g, int M) {
   PrepPlan plan;
   return M <= 8 && w->in_features % 128 == 0 && w->out_features % 8 == 0 && (g == w->in_features || g == 128 || g == 256) &&
-         plan_prep(w->out_features, w->in_features, M, w->bits, g, true, false, &plan) == PEQA_OK;
+         plan_prep(w->out_features, w->in_features, M, w->bits, g, true, false, false, &plan) == PEQA_OK;
 }
 
 int launch_decode_rows(const peqa_qweight_t* w, int g, const void* X, int M, void* Y, const float* scale_table,
