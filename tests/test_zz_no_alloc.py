@@ -7,6 +7,7 @@ a caller-provided workspace, on two consecutive calls that reuse that array with
 data.  This file sorts last on purpose so that a failure here cannot hide another test.
 """
 import ctypes
+import gc
 
 import numpy as np
 import pytest
@@ -17,6 +18,12 @@ from paper_2305_14152_b200 import binding, synth
 from gpu_util import assert_close, bf16_to_dev, dev_to_f64, oracle_layer, to_qweight
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _garbage_of_earlier_tests():
+    """Tensors that a caught exception's frames hold in a cycle are freed now, and not between two readings of what is allocated."""
+    gc.collect()
 
 
 def _layer(seed, N, K, T, bits, g):
