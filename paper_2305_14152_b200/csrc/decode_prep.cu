@@ -1339,19 +1339,18 @@ int x_pitch_for(int steps) {
 //
 // The estimate, in ns: 2330 a launch; a step of a pair, per turn of the busiest warp, 1440 (2120 with groups inside the step, 9 % more
 // where these have little L1, 25 with a table per task, whose tokens read scales of their own each; 13 % less with two token
-// tiles; integer kernel 1180 and 1360; canonical rows 330 more); staging
-// a token's step 31, 63 in the integer kernel, 91 from canonical rows, whose order takes the activations in half sectors; 2.4 per
-// row group, token and chunk for the final pass, 3.6 where a cluster shares it, and 370 for the cluster's exchange, 170 more for each
-// doubling; 5500 per further chunk; 10000 more for a second wave of clusters.  The constants are those that choose best, not
-// each what its part was measured to take (nine of ten estimates are 0.7 to 1.2 of the time): over 942 random calls (1 to 16 tokens, prepared, of several tasks and
-// canonical), each timed with clusters of 1, 2, 4 and 8, one wave and two, as one launch and as two where these fit, the
-// choice costs 0.45 % more than the best on average, 12 % at worst.  (Turns are counted chunk by chunk, since each chunk is
-// dealt to the warps anew: with the steps of all chunks dealt out once, nine chunks of five steps counted as ten turns instead of
-// eighteen, and 13 tokens of 4-bit weights took one launch where two are faster, us: 8192 x 22016 in groups of 128 99 / 56,
-// 8192 x 16384 in groups of 64 82 / 51.)
+// tiles; integer kernel 1180 and 1360; canonical rows 330 more); staging a token's step 31, 63 in the integer kernel, 91 from canonical
+// rows, whose order takes the activations in half sectors; 2.4 per row group, token and chunk for the final pass, 3.6 where a
+// cluster shares it, and 370 for the cluster's exchange, 170 more for each doubling; 5500 per further chunk; 10000 more for a
+// second wave of clusters.  The constants are those that choose best, not each what its part was measured to take (nine of ten
+// estimates are 0.7 to 1.2 of the time): over 942 random calls (1 to 16 tokens, prepared, of several tasks and canonical), each timed
+// with clusters of 1, 2, 4 and 8, one wave and two, as one launch and as two where these fit, the choice costs 0.45 % more
+// than the best on average, 12 % at worst.  (Turns are counted chunk by chunk, since each chunk is dealt to the warps anew: with
+// the steps of all chunks dealt out once, nine chunks of five steps counted as ten turns instead of eighteen, and 13 tokens of 4-bit
+// weights took one launch where two are faster, us: 8192 x 22016 in groups of 128 99 / 56, 8192 x 16384 in groups of 64 82 / 51.)
 //
-// tasks: a table per task.  (With 9 % for it too, eight tokens at 17128 x 11904 in groups of 64, 3 bits, took 163 us on two CTAs a range, whose
-// rings leave 28 KB of L1, where four a range take 87.)
+// tasks: a table per task.  (With 9 % for it too, eight tokens at 17128 x 11904 in groups of 64, 3 bits, took 163 us on two CTAs a
+// range, whose rings leave 28 KB of L1, where four a range take 87.)
 //
 // i8 (one or two tokens): the plan of the integer kernel, whose activations take four bytes each and are all
 // staged at once, at most four steps to a half-warp.
