@@ -1131,14 +1131,14 @@ int launch_ds(const peqa_qweight_t* w, const float* zeros_f, int g, const void* 
   const int tiles = p.i_tiles * p.j_tiles;
   const int max_pairs = sms / 2;
   // Taking tiles over pays but for short tiles of a step with AdamW in the kernel, where the store of a pair's first tile waits for the
-  // kernels beside.  us, dealt / taken over, steps with AdamW here: 8192 x 8192 in groups of 64 at 64 tokens 99 / 102, at 256 134.7 /
+  // kernels beside: there from where shapes that lose and shapes that gain come to the same.  us, dealt / taken over, steps with AdamW here: 8192 x 8192 in groups of 64 at 64 tokens 99 / 102, at 256 134.7 /
   // 136.5, at 384 187.5 / 190.3, at 512 215.5 / 215.8, at 2048 633 / 609; 2304 x 2304 in groups of 64 at 64 22.3 / 21.5, at 256
   // 31.4 / 33.8, at 384 39.6 / 41.4, at 512 45.2 / 46.3, at 1000 47.3 / 45.7; 4096 x 4096 in groups of 128 at 384 59.0 / 57.6, at
-  // 700 87.2 / 87.5, at 2048 174 / 164; five shapes lose 1.8 % at 256, 0.2 at 512, 0.5 at 700, nine gain 2.1 % at 1000.  Without AdamW here: real
+  // 700 87.2 / 87.5, at 2048 174 / 164; five shapes lose 1.8 % at 256, seven 0.3 % at 384, five 0.2 % at 512, nine gain 2.1 % at 1000.  Without AdamW here: real
   // zero-points, 2304 x 2304 in groups of 64 at 64 14.8 / 12.8, at 200 20.5 / 14.4, 4096 x 4096 per channel at 64 27.5 / 27.8, at 384 39.7 /
   // 38.6, 4096 x 11008 in groups of 128 at 40 47.6 / 45.3, at 256 67.3 / 61.9; step in groups of 256, 4096 x 4096 at 64 34.4 / 34.7, at 384 53.9 / 51.1.
   const bool pktma = ((size_t)p.wpr * 4) % 16 == 0;   // 4-bit: always; 3-bit: K % 128 == 0
-  const bool dynamic = side == kBeside && pktma && tiles > max_pairs && (!adam_in_kernel || p.k_blocks >= 13);
+  const bool dynamic = side == kBeside && pktma && tiles > max_pairs && (!adam_in_kernel || p.k_blocks >= 6);
   const int pairs = tiles < max_pairs || dynamic ? tiles : max_pairs;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs, 1, 1);
